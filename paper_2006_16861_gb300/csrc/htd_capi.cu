@@ -146,7 +146,10 @@ struct htd_ctx {
     StepCoef<double> C{};
     // FP64 operator data
     double *kap64 = nullptr, *imH = nullptr;
-    double *coefP = nullptr;    // assembled operator, h_planes(d) planes of N
+    double *coefP = nullptr;    // assembled operator, h_planes(d) planes of N, ...
+    double hmul = 1.0;          // ... times hmul (-q where the FP64 step reads it too, else 1)
+    bool asm_step = false;      // the one-step kernel reads coefP (FP64 I_acd, 3-D)
+    double c2 = 0.0;            // 2 - p (asm_step)
     double *coefI = nullptr;    // assembled Im H (cell damping only), same layout
     // Krylov workspace
     int m = 20;
@@ -238,6 +241,28 @@ void free_ctx(htd_ctx *c)
     delete c;
 }
 
+// 1/h^2 as a factor of the assembled planes
+double h_factor(const htd_ctx *c)
+{
+    return 1.0 / (c->h * c->h) / c->hmul;
+}
+
+// one step by the handle's one-step kernel: u_{j+1} over um = u_{j-1}
+template <typename T>
+void one_step(htd_ctx *c, const T *u, T *um, const T *fre, const T *fim, const StepCoef<T> &C, T a,
+              T b, int flags, cudaStream_t s, const htd::RhsSet &R)
+{
+    if constexpr (std::is_same<T, double>::value) {
+        if (c->asm_step) {
+            htd::launch_step_asm(c->Lr, u, um, c->coefP, (const double *)c->dco, fre, fim, c->c2,
+                                 a, b, c->slot, flags, s, R);
+            return;
+        }
+    }
+    htd::launch_step<T>(c->Lr, u, um, (const T *)c->kap, (const T *)c->dco, fre, fim, C, a, b,
+                        c->slot, flags, s, R);
+}
+
 // Consecutive launches of the blocked 2-D and the streamed 3-D step overlap
 // (programmatic dependent launch) unless the handle's options say
 // HTD_LAUNCH_NO_OVERLAP.
@@ -306,9 +331,8 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
             int flags = 0;
             if (j + 1 == jim) flags |= 1;
             if (j + 1 == jfin) flags |= 2;
-            htd::launch_step<T>(L, cur, oth, (const T *)c->kap, (const T *)c->dco,
-                                (const T *)c->fre, (const T *)c->fim, C, (T)c->atab[j],
-                                (T)c->btab[j], c->slot, flags, s, c->Rs);
+            one_step<T>(c, cur, oth, (const T *)c->fre, (const T *)c->fim, C, (T)c->atab[j],
+                        (T)c->btab[j], flags, s, c->Rs);
             if (project && j >= j_acc) accumulate(j, oth);
             std::swap(cur, oth);
         }
@@ -498,7 +522,7 @@ htd_status precond(htd_ctx *c, const double2 *F, double2 *U, cudaStream_t s)
 
 void apply_H(htd_ctx *c, const double2 *X, const double2 *F, double2 *Y, cudaStream_t s)
 {
-    htd::launch_apply_H(c->L64, c->coefP, c->imH, 1.0 / (c->h * c->h), X, F, Y, s, c->coefI);
+    htd::launch_apply_H(c->L64, c->coefP, c->imH, h_factor(c), X, F, Y, s, c->coefI);
 }
 
 // dots of w with V_0..V_{k-1} into hdev + off (device); does not synchronise
@@ -973,8 +997,7 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
     std::vector<double2> res(nrec > 0 ? nrec : 1);
     double J = 0.0;
     auto step = [&](const T *u, T *um, const T *fre, const T *fim, T a, T b) {
-        htd::launch_step<T>(L, u, um, (const T *)c->kap, (const T *)c->dco, fre, fim, Cf, a, b,
-                            c->slot, 0, s, one);
+        one_step<T>(c, u, um, fre, fim, Cf, a, b, 0, s, one);
     };
     for (int src = 0; src < nsrc; ++src) {
         const double2 *Fs = F + (size_t)src * N;
@@ -1340,10 +1363,17 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
     if (st != HTD_OK) return st;
     HTD_CUDA(cudaMemcpy(c->kap64, k64.data(), sizeof(double) * c->L64.total, cudaMemcpyHostToDevice));
     {
-        double S2[4];
-        for (int k = 0; k < 4; ++k) S2[k] = std::ldexp(c->S[k], d - k);
+        // the FP64 step reads the same planes, scaled by -q
+        c->asm_step = d == 3 && !mixed && !abd;
+        c->hmul = c->asm_step ? -q : 1.0;
+        c->c2 = 2.0 - p;
+        double S2[4], M2[4];
+        for (int k = 0; k < 4; ++k) {
+            S2[k] = c->hmul * std::ldexp(c->S[k], d - k);
+            M2[k] = c->hmul * c->M[k];
+        }
         HTD_CUDA(htd::dev_malloc((void **)&c->coefP, sizeof(double) * htd::h_planes(d) * (size_t)N));
-        htd::launch_assemble_H(c->L64, c->kap64, S2, c->M, c->coefP, 0);
+        htd::launch_assemble_H(c->L64, c->kap64, S2, M2, c->coefP, 0);
         HTD_CUDA(cudaGetLastError());
         if (cell_damp) {
             // Im H = sum_o M_s (sum of omega_phys R over the shared cells): the same
@@ -1485,7 +1515,7 @@ void operator_view(const htd_ctx *c, OperatorView *out)
         out->S2[k] = std::ldexp(c->S[k], c->d - k);
         out->M[k] = c->M[k];
     }
-    out->ih2 = 1.0 / (c->h * c->h);
+    out->ih2 = h_factor(c);
     out->device = c->device;
 }
 

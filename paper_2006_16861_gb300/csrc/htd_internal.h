@@ -202,6 +202,13 @@ void launch_step(const Layout &L, const T *u, T *um, const T *kap, const T *dco,
                  const T *fre, const T *fim, const StepCoef<T> &C, T a, T b,
                  const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R = RhsSet{});
 
+// The FP64 step from the assembled planes of launch_assemble_H scaled by -q
+// (see step3d_asm_kernel); c2 = 2 - p.
+void launch_step_asm(const Layout &L, const double *u, double *um, const double *coefP,
+                     const double *dco, const double *fre, const double *fim, double c2, double a,
+                     double b, const OutSlot *slot, int flags, cudaStream_t s,
+                     const RhsSet &R = RhsSet{});
+
 template <typename T>
 void launch_split(const Layout &L, const double2 *F, T *fre, T *fim, int flip, cudaStream_t s);
 

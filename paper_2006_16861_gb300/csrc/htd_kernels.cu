@@ -33,6 +33,25 @@ namespace htd {
 
 long long g_launches = 0;
 
+// SMs of the current device, looked up once per device (1 if the lookup fails)
+static int sm_count()
+{
+    static int count[64] = {0};
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        (void)cudaGetLastError();
+        return 1;
+    }
+    if (count[dev] > 0) return count[dev];
+    if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        nsm < 1) {
+        (void)cudaGetLastError();
+        return 1;
+    }
+    count[dev] = nsm;
+    return nsm;
+}
+
 // ---------------------------------------------------------------------------
 // recurrence step
 // ---------------------------------------------------------------------------
@@ -223,6 +242,117 @@ template void launch_step<double>(const Layout &, const double *, double *, cons
                                   const double *, const double *, const double *,
                                   const StepCoef<double> &, double, double, const OutSlot *,
                                   int, cudaStream_t, const RhsSet &);
+
+// One step of I_acd in FP64 from the assembled stencil.  GB300 retires two FP64
+// operations per clock and SM (1.26 TFLOP/s as FMAs on 152 SMs) beside
+// 6.8 TB/s, so the FP64 step is bound by its FP64 instruction count, not by its
+// bytes: the cell form's sums of q kappa and coefficients (about 50 of the 81
+// operations per 3-D node) are not recomputed in every step but read back, from
+// the same assembled planes that apply_H uses (the centre and the positive
+// offsets; a negative offset is the neighbour's positive one).  For FP64 handles
+// those planes hold -q (2^{d-s} S_s - M_s sum kappa), so that with c2 = 2 - p
+//   (2 - K) u_j = c2 u_j + sum_o coef_o u_{j, beta + o}
+// is one multiply-add per offset: 32 FP64 operations per 3-D node.  The planes
+// are compact (N values each) and padded nowhere: where an offset leaves the
+// grid u is the zero ghost ring, and the index is clamped into the plane (any
+// finite coefficient times the ghost's zero).
+// Own-node terms open the chain, the neighbours follow in (oz, oy, ox) order.
+// A thread marches up a column of zc planes with the 3 x 3 x 3 window of u in
+// registers; zc is chosen by the launcher so that every SM gets about eight
+// blocks (the last wave of an FP64-bound kernel costs as much as it holds).
+// Measured on GB300, 96^3: 59 us per step (cell form: 179 us), 76 % of the
+// FP64 pipe's 45 us.
+constexpr int kAsmTY = 4;
+
+__global__ void __launch_bounds__(32 * kAsmTY)
+step3d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
+                  const double *__restrict__ coefP, const double *__restrict__ dco,
+                  const double *__restrict__ fre, const double *__restrict__ fim, Layout L,
+                  double c2, double a, double b, const OutSlot *__restrict__ slot, int flags,
+                  RhsSet R, int zc, int nchunks)
+{
+    const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    const int64_t iy = (int64_t)blockIdx.y * kAsmTY + threadIdx.y;
+    int rhs;
+    if (!rhs_of_slot(R, (int)blockIdx.z / nchunks, rhs)) return;
+    const int64_t z0 = (int64_t)(blockIdx.z % nchunks) * zc;
+    const int64_t z1 = min((int64_t)L.nz, z0 + zc);
+    if (ix >= L.nx || iy >= L.ny) return;
+    u += rhs * R.stride;
+    um += rhs * R.stride;
+    fre += rhs * R.stride;
+    fim += rhs * R.stride;
+    slot += rhs;
+    const int64_t P = L.pitch, Q = L.plane, N = L.N;
+    const int64_t col = (iy + 1) * P + L.xl + ix;     // offset of the column in a stored plane
+    // w[p][oy][ox]: u_j at stored plane iz + p, row offset oy - 1, column offset ox - 1
+    double w[3][3][3];
+#pragma unroll
+    for (int p = 0; p < 2; ++p)
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy)
+#pragma unroll
+            for (int ox = 0; ox < 3; ++ox)
+                w[p][oy][ox] = u[(z0 + p) * Q + col + (oy - 1) * P + (ox - 1)];
+    for (int64_t iz = z0; iz < z1; ++iz) {
+        const int64_t i = (iz + 1) * Q + col;
+        const int64_t c = (iz * L.ny + iy) * L.nx + ix;
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy)
+#pragma unroll
+            for (int ox = 0; ox < 3; ++ox)
+                w[2][oy][ox] = u[i + Q + (oy - 1) * P + (ox - 1)];
+        const double uprev = um[i];
+        double acc = fma(a, fre[i], -b * fim[i]);
+        acc = fma(-2.0, uprev, acc);
+        acc = fma(c2, w[1][1][1], acc);
+        acc = fma(coefP[c], w[1][1][1], acc);
+#pragma unroll
+        for (int oz = 0; oz < 3; ++oz)
+#pragma unroll
+            for (int oy = 0; oy < 3; ++oy)
+#pragma unroll
+                for (int ox = 0; ox < 3; ++ox) {
+                    const int lin = oz * 9 + oy * 3 + ox;
+                    if (lin == 13) continue;
+                    int64_t ci = c;
+                    if (lin < 13) {
+                        ci += ((int64_t)(oz - 1) * L.ny + (oy - 1)) * L.nx + (ox - 1);
+                        ci = ci > 0 ? ci : 0;
+                    }
+                    acc = fma(coefP[(lin < 13 ? 13 - lin : lin - 13) * N + ci], w[oz][oy][ox], acc);
+                }
+        const double unew = fma(dco[i], acc, uprev);
+        um[i] = unew;
+        if (flags) {
+            if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = unew;
+            if ((flags & 2) && slot->final_part) slot->final_part[2 * c] = unew;
+        }
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy)
+#pragma unroll
+            for (int ox = 0; ox < 3; ++ox) {
+                w[0][oy][ox] = w[1][oy][ox];
+                w[1][oy][ox] = w[2][oy][ox];
+            }
+    }
+}
+
+void launch_step_asm(const Layout &L, const double *u, double *um, const double *coefP,
+                     const double *dco, const double *fre, const double *fim, double c2, double a,
+                     double b, const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R)
+{
+    const int64_t tiles = ((L.nx + 31) / 32) * ((L.ny + kAsmTY - 1) / kAsmTY) * R.slots;
+    const int64_t want = 8 * (int64_t)sm_count();
+    int zc = (int)std::min<int64_t>(16, std::max<int64_t>(1, L.nz * tiles / want));
+    zc = (int)std::min<int64_t>(zc, L.nz);
+    const int nchunks = (int)((L.nz + zc - 1) / zc);
+    dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + kAsmTY - 1) / kAsmTY),
+             (unsigned)(nchunks * R.slots));
+    step3d_asm_kernel<<<grd, dim3(32, kAsmTY), 0, s>>>(u, um, coefP, dco, fre, fim, L, c2, a, b,
+                                                       slot, flags, R, zc, nchunks);
+    ++g_launches;
+}
 
 // ---------------------------------------------------------------------------
 // frequency-adapted backward-differences damped leapfrog (Def. of I_abd)
@@ -793,24 +923,7 @@ dots_kernel(const double2 *__restrict__ V, int64_t ldv, int kcount, const double
 
 int dots_blocks(int64_t N)
 {
-    // 4 blocks per SM of the current device, looked up once per device
-    static int sm_count[64] = {0};
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
-        (void)cudaGetLastError();
-        dev = -1;
-    }
-    if (dev >= 0 && sm_count[dev] > 0) {
-        nsm = sm_count[dev];
-    } else if (dev >= 0 &&
-               cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-               nsm > 0) {
-        sm_count[dev] = nsm;
-    } else {
-        (void)cudaGetLastError();
-        nsm = 1;
-    }
-    const int64_t cap = std::min<int64_t>(4 * (int64_t)nsm, kMaxDotBlocks);
+    const int64_t cap = std::min<int64_t>(4 * (int64_t)sm_count(), kMaxDotBlocks);
     int64_t nb = (N + 8 * kRedThreads - 1) / (8 * kRedThreads);
     if (nb > cap) nb = cap;
     if (nb < 1) nb = 1;
