@@ -148,8 +148,7 @@ struct htd_ctx {
     double *kap64 = nullptr, *imH = nullptr;
     double *coefP = nullptr;    // assembled operator, h_planes(d) planes of N, ...
     double hmul = 1.0;          // ... times hmul (-q where the FP64 step reads it too, else 1)
-    bool asm_step = false;      // the one-step kernel reads coefP (FP64 I_acd, 3-D)
-    double c2 = 0.0;            // 2 - p (asm_step)
+    double c2 = 0.0;            // 2 - p (FP64 step)
     double *coefI = nullptr;    // assembled Im H (cell damping only), same layout
     // Krylov workspace
     int m = 20;
@@ -252,15 +251,27 @@ template <typename T>
 void one_step(htd_ctx *c, const T *u, T *um, const T *fre, const T *fim, const StepCoef<T> &C, T a,
               T b, int flags, cudaStream_t s, const htd::RhsSet &R)
 {
-    if constexpr (std::is_same<T, double>::value) {
-        if (c->asm_step) {
-            htd::launch_step_asm(c->Lr, u, um, c->coefP, (const double *)c->dco, fre, fim, c->c2,
-                                 a, b, c->slot, flags, s, R);
-            return;
-        }
-    }
-    htd::launch_step<T>(c->Lr, u, um, (const T *)c->kap, (const T *)c->dco, fre, fim, C, a, b,
-                        c->slot, flags, s, R);
+    if constexpr (std::is_same<T, double>::value)
+        htd::launch_step_asm(c->Lr, u, um, c->coefP, (const double *)c->dco, fre, fim, c->c2, a, b,
+                             c->slot, flags, s, R);
+    else
+        htd::launch_step<T>(c->Lr, u, um, (const T *)c->kap, (const T *)c->dco, fre, fim, C, a, b,
+                            c->slot, flags, s, R);
+}
+
+// one run of the resident-grid kernel from the handle's planes
+template <typename T>
+void run_resident(htd_ctx *c, const StepCoef<T> &C, int jim, int jfin, cudaStream_t s,
+                  const htd::Res2dProj<T> &P)
+{
+    if constexpr (std::is_same<T, double>::value)
+        htd::launch_res2d64(c->res, c->coefP, (const double *)c->dco, (const double *)c->fre,
+                            (const double *)c->fim, c->Lr, c->c2, (const double *)c->res_ab,
+                            (int)c->nsteps, jim, jfin, c->slot, c->res_x, c->err_dev, s, P);
+    else
+        htd::launch_res2d<T>(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
+                             (const T *)c->fim, c->Lr, C, (const T *)c->res_ab, (int)c->nsteps, jim,
+                             jfin, c->slot, c->res_x, c->err_dev, s, P);
 }
 
 // Consecutive launches of the blocked 2-D and the streamed 3-D step overlap
@@ -299,9 +310,7 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
             P.N = L.N;
             HTD_CUDA(cudaMemsetAsync(c->acc, 0, sizeof(T) * 4 * L.N, s));
         }
-        htd::launch_res2d<T>(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
-                             (const T *)c->fim, L, C, (const T *)c->res_ab, (int)c->nsteps,
-                             (int)jim, (int)jfin, c->slot, c->res_x, c->err_dev, s, P);
+        run_resident<T>(c, C, (int)jim, (int)jfin, s, P);
         if (project)
             htd::launch_project_finish<T>(L.N, (const T *)c->acc, 4 * L.N, 2.0 / (double)n_res,
                                           c->slot, c->Rs, s);
@@ -701,7 +710,9 @@ template <typename T>
 htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1)
 {
     if (c->rcap != 1 || c->nsteps >= (1LL << 30)) return HTD_OK;
-    if (!htd::res2d_plan<T>(c->Lr, &c->res)) return HTD_OK;
+    if (!(std::is_same<T, double>::value ? htd::res2d64_plan(c->Lr, &c->res)
+                                         : htd::res2d_plan<float>(c->Lr, &c->res)))
+        return HTD_OK;
     if (c->opt.mode == HTD_MODE_PROJECT) {
         // projection weights per phase k of the new state: cos and -sin of
         // 2 pi k / nP, rounded as for the separate accumulation kernel
@@ -725,9 +736,7 @@ htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cud
     const StepCoef<T> C = cast_coef<T>(c->C);
     for (int r = 0; r < 2; ++r) {
         if (r == 1) HTD_CUDA(cudaEventRecord(e0, s));
-        htd::launch_res2d<T>(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
-                             (const T *)c->fim, c->Lr, C, (const T *)c->res_ab, (int)c->nsteps,
-                             -1, -1, c->slot, c->res_x, c->err_dev, s);
+        run_resident<T>(c, C, -1, -1, s, htd::Res2dProj<T>{});
     }
     HTD_CUDA(cudaEventRecord(e1, s));
     HTD_CUDA(cudaEventSynchronize(e1));
@@ -764,10 +773,8 @@ htd_status autotune_fp64_2d(htd_ctx *c)
     const int reps = 64;
     for (int r = 0; r < 2 + reps; ++r) {
         if (r == 2) HTD_CUDA(cudaEventRecord(e0, s));
-        htd::launch_step<double>(c->Lr, (const double *)c->u0, (double *)c->u1,
-                                 (const double *)c->kap, (const double *)c->dco,
-                                 (const double *)c->fre, (const double *)c->fim, C, 0.0, 0.0,
-                                 c->slot, 0, s);
+        one_step<double>(c, (const double *)c->u0, (double *)c->u1, (const double *)c->fre,
+                         (const double *)c->fim, C, 0.0, 0.0, 0, s, htd::RhsSet{});
     }
     HTD_CUDA(cudaEventRecord(e1, s));
     HTD_CUDA(cudaEventSynchronize(e1));
@@ -1364,8 +1371,7 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
     HTD_CUDA(cudaMemcpy(c->kap64, k64.data(), sizeof(double) * c->L64.total, cudaMemcpyHostToDevice));
     {
         // the FP64 step reads the same planes, scaled by -q
-        c->asm_step = d == 3 && !mixed && !abd;
-        c->hmul = c->asm_step ? -q : 1.0;
+        c->hmul = (!mixed && !abd) ? -q : 1.0;
         c->c2 = 2.0 - p;
         double S2[4], M2[4];
         for (int k = 0; k < 4; ++k) {
@@ -1776,7 +1782,7 @@ htd_status htd_get_params(htd_handle h, htd_params *out)
     P.steps_per_launch = h->use_res ? (int)h->nsteps : h->use_tb ? h->tb.B : 1;
     P.tile[0] = h->use_res ? h->res.W : h->use_tb ? h->tb.TX : 0;
     P.tile[1] = h->use_res ? h->res.H : h->use_tb ? h->tb.TY : 0;
-    P.tile[2] = h->use_res ? 2 : h->use_tb ? (h->tb.pair ? 2 : 1) : 0;
+    P.tile[2] = h->use_res ? (h->esz == 8 ? 1 : 2) : h->use_tb ? (h->tb.pair ? 2 : 1) : 0;
     P.ctas_per_sm = h->use_res ? 1 : h->use_tb ? h->tb.occ : 0;
     P.waves = h->use_res ? 1 : h->use_tb ? h->tb.waves : 0;
     if (h->use_s3) {

@@ -100,6 +100,35 @@ __device__ __forceinline__ V stencil2d(const Stencil2dCoef<V> &C, V umm, V um0, 
     return vadd(r1, r2);
 }
 
+// The 2-D assembled stencil at a node: the centre, then the neighbours in
+// (oy, ox) order (see step3d_asm_kernel; planes scaled by -q).
+struct Asm9 {
+    double c0, kmm, km0, kmp, k0m, k0p, kpm, kp0, kpp;
+};
+
+// u_{j+1} at a node in FP64: own-node terms first, then one multiply-add per
+// neighbour.  The one-step and the resident-grid kernel share it, so their
+// results are bit-identical.  nb = -b_j.
+__device__ __forceinline__ double asm2d_step(const Asm9 &k, double umm, double um0, double ump,
+                                             double u0m, double u00, double u0p, double upm,
+                                             double up0, double upp, double uprev, double d,
+                                             double fr, double fi, double c2, double a, double nb)
+{
+    double t = __fma_rn(a, fr, __dmul_rn(nb, fi));
+    t = __fma_rn(-2.0, uprev, t);
+    t = __fma_rn(c2, u00, t);
+    t = __fma_rn(k.c0, u00, t);
+    t = __fma_rn(k.kmm, umm, t);
+    t = __fma_rn(k.km0, um0, t);
+    t = __fma_rn(k.kmp, ump, t);
+    t = __fma_rn(k.k0m, u0m, t);
+    t = __fma_rn(k.k0p, u0p, t);
+    t = __fma_rn(k.kpm, upm, t);
+    t = __fma_rn(k.kp0, up0, t);
+    t = __fma_rn(k.kpp, upp, t);
+    return __fma_rn(d, t, uprev);
+}
+
 // Output targets of a preconditioner run, read by the step kernels from device
 // memory so that a captured graph can be replayed for any output vector.
 struct OutSlot {
@@ -368,7 +397,7 @@ void launch_tb2d(const TbPlan &p, const TbMaps &maps, int in0, int in1, const La
 
 // ---- resident-grid 2-D step (htd_res2d.cu) ------------------------------------
 //
-// A whole run (all steps, one rhs, FP32 or FP64) in one cooperative launch:
+// A whole run (all steps, one rhs, FP32) in one cooperative launch:
 // ntx x nty tiles of W x H nodes, one CTA per tile and at most one per SM,
 // every tile's states, cells, d and forcing in shared memory; neighbouring
 // tiles swap edge values through `xbuf` (xwords 64-bit words, zeroed by the
@@ -378,6 +407,7 @@ struct Res2dPlan {
     int ntx = 0, nty = 0;        // tiles (CTAs) per axis
     int rpt = 0;                 // interior rows per thread and strip (3, 5 or 8)
     int sw = 0;                  // row stride of the shared-memory arrays (72 or 136)
+    int threads = 0;             // threads per CTA (FP64 form)
     size_t smem = 0;             // dynamic shared memory per CTA
     size_t xwords = 0;           // exchange buffer words
 };
@@ -410,6 +440,14 @@ void launch_res2d(const Res2dPlan &p, const T *kap, const T *dco, const T *fre, 
                   const Layout &L, const StepCoef<T> &C, const T *ab, int nsteps, int jim,
                   int jfin, const OutSlot *slot, unsigned long long *xbuf, int *err,
                   cudaStream_t s, const Res2dProj<T> &P = Res2dProj<T>{});
+
+// The FP64 form (htd_res2d64.cu): reads the assembled planes (see
+// launch_step_asm), two steps per exchange of edge values; nsteps is even.
+bool res2d64_plan(const Layout &L, Res2dPlan *p);
+void launch_res2d64(const Res2dPlan &p, const double *coefP, const double *dco, const double *fre,
+                    const double *fim, const Layout &L, double c2, const double *ab, int nsteps,
+                    int jim, int jfin, const OutSlot *slot, unsigned long long *xbuf, int *err,
+                    cudaStream_t s, const Res2dProj<double> &P = Res2dProj<double>{});
 
 // ---- one persistent launch for many 2-D instances (htd_tblock.cu) -----------
 //

@@ -1,4 +1,4 @@
-// Resident-grid 2-D recurrence (FP32 or FP64, node pairs): the whole grid
+// Resident-grid 2-D recurrence (FP32, node pairs): the whole grid
 // stays in shared memory, spread over the SMs, for all T n_P steps of a run.
 //
 // One cooperative launch runs a whole preconditioner run (Def. of I_acd with
@@ -9,9 +9,8 @@
 // the tile, and in every step
 //  - computes the new state of its edge nodes first (one edge pair per
 //    thread) and publishes each edge value to a global exchange buffer as
-//    tagged 64-bit words (tag = index of the state + 1; an FP32 value in one
-//    word with its bits, an FP64 value in two words, one per 32-bit half; one
-//    buffer per state parity);
+//    tagged 64-bit words (tag = index of the state + 1, beside the value's
+//    bits; one buffer per state parity);
 //  - computes its interior nodes in row strips with a 3 x 3 register window;
 //    the strip threads also read the neighbours' edge words of the new state
 //    into the ring: each read is issued two rows into the thread's strip and
@@ -42,31 +41,18 @@ namespace htd {
 
 namespace {
 
-// threads per CTA: 768 for FP32 (80 registers each), 512 for FP64 (its
-// register windows are twice as wide)
+// threads per CTA (80 registers each)
 template <typename T>
 __host__ __device__ constexpr int res_threads()
 {
-    return sizeof(T) == 8 ? 512 : 768;
+    return 768;
 }
 
-// A node pair (lx, lx + 1) as one value: float2 for the FP32 recurrence
-// (paired FP32 instructions), DPair for FP64 (two scalar FP64 operations, each
-// lane rounded like the one-step kernel's scalar).
-struct __align__(16) DPair {
-    double x, y;
-};
-// (the FP32 and scalar overloads of the enclosing namespace stay visible)
 using htd::vadd;
 using htd::vfma;
 using htd::vmul;
-__device__ __forceinline__ DPair vadd(DPair a, DPair b) { return {__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y)}; }
-__device__ __forceinline__ DPair vmul(DPair a, DPair b) { return {__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y)}; }
-__device__ __forceinline__ DPair vfma(DPair a, DPair b, DPair c)
-{
-    return {__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y)};
-}
 
+// A node pair (lx, lx + 1) as one value (paired FP32 instructions)
 template <typename T>
 struct PairOf;
 template <>
@@ -74,12 +60,6 @@ struct PairOf<float> {
     typedef float2 V;
     __device__ static V make(float a, float b) { return make_float2(a, b); }
 };
-template <>
-struct PairOf<double> {
-    typedef DPair V;
-    __device__ static V make(double a, double b) { return {a, b}; }
-};
-
 template <typename T>
 __device__ __forceinline__ typename PairOf<T>::V ld2(const T *p)
 {
@@ -113,9 +93,7 @@ __device__ __forceinline__ void st_word(unsigned long long *p, unsigned bits, un
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
 }
 
-// An exchanged value as tagged words: an FP32 value in one word, an FP64 value
-// in two (low and high halves, each with the tag), valid when every tag is the
-// expected one.
+// An exchanged FP32 value as a tagged word, valid when the tag is the expected one.
 template <typename T>
 struct Xword;
 template <>
@@ -132,39 +110,10 @@ struct Xword<float> {
     __device__ static bool ok(const Raw &r, unsigned want) { return (unsigned)(r.w >> 32) == want; }
     __device__ static float value(const Raw &r) { return __uint_as_float((unsigned)r.w); }
 };
-template <>
-struct Xword<double> {
-    static constexpr int kPer = 2;
-    struct Raw {
-        unsigned long long lo, hi;
-    };
-    __device__ static void put(unsigned long long *p, double v, unsigned tag)
-    {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-        st_word(p, (unsigned)b, tag);
-        st_word(p + 1, (unsigned)(b >> 32), tag);
-    }
-    __device__ static Raw get(const unsigned long long *p) { return {ld_word(p), ld_word(p + 1)}; }
-    __device__ static bool ok(const Raw &r, unsigned want)
-    {
-        return (unsigned)(r.lo >> 32) == want && (unsigned)(r.hi >> 32) == want;
-    }
-    __device__ static double value(const Raw &r)
-    {
-        return __longlong_as_double((long long)((r.hi << 32) | (r.lo & 0xffffffffull)));
-    }
-};
-
 // the step coefficients broadcast to node pairs
 __device__ __forceinline__ Stencil2dCoef<float2> pair_coef(const StepCoef<float> &C)
 {
     return stencil2d_coef2(C);
-}
-
-__device__ __forceinline__ Stencil2dCoef<DPair> pair_coef(const StepCoef<double> &C)
-{
-    auto b = [](double x) { return DPair{x, x}; };
-    return {b(C.c0), b(C.mt[0]), b(C.mt[1]), b(C.mt[2]), b(-C.cs[1]), b(-C.cs[2])};
 }
 
 // row strides of the shared-memory arrays the kernel is built for (8 banks of
@@ -517,30 +466,19 @@ res2d_kernel(const T *__restrict__ kap, const T *__restrict__ dco, const T *__re
     }
 }
 
-// Rows per strip a plan may choose: FP32 3, 5 or 8; FP64 also 1 -- its
-// long-latency FP64 pipe makes a thread's chain of dependent rows, not the
-// register window's saved loads, what sets the step time on small tiles
-// (one-row strips in FP32 measured no faster at 101^2).
-constexpr int kRpts[] = {1, 3, 5, 8};
-
-template <typename T>
-bool rpt_allowed(int r)
-{
-    return r != 1 || sizeof(T) == 8;
-}
+// Rows per strip a plan may choose (one-row strips measured no faster at 101^2)
+constexpr int kRpts[] = {3, 5, 8};
 
 // fn(the kernel for precision T, RPT rows per strip, row stride SW)
 template <typename T, typename Fn>
 void with_kernel(int rpt, int sw, Fn &&fn)
 {
     if (sw == 72) {
-        if (rpt == 1) fn(res2d_kernel<T, 1, 72>);
-        else if (rpt == 3) fn(res2d_kernel<T, 3, 72>);
+        if (rpt == 3) fn(res2d_kernel<T, 3, 72>);
         else if (rpt == 5) fn(res2d_kernel<T, 5, 72>);
         else fn(res2d_kernel<T, 8, 72>);
     } else {
-        if (rpt == 1) fn(res2d_kernel<T, 1, 136>);
-        else if (rpt == 3) fn(res2d_kernel<T, 3, 136>);
+        if (rpt == 3) fn(res2d_kernel<T, 3, 136>);
         else if (rpt == 5) fn(res2d_kernel<T, 5, 136>);
         else fn(res2d_kernel<T, 8, 136>);
     }
@@ -581,7 +519,6 @@ bool plan_impl(const Layout &L, Res2dPlan *out)
     bool attr_ok = true;
     for (int sw : kStrides)
         for (int r : kRpts) {
-            if (!rpt_allowed<T>(r)) continue;
             with_kernel<T>(r, sw, [&](auto kern) {
                 cudaFuncAttributes fa;
                 if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
@@ -633,7 +570,6 @@ bool plan_impl(const Layout &L, Res2dPlan *out)
     best.rpt = kRpts[sizeof(kRpts) / sizeof(kRpts[0]) - 1];
     int best_load = -1;
     for (int r : kRpts) {
-        if (!rpt_allowed<T>(r)) continue;
         const int ld = res2d_load(best.W, best.H, r, res_threads<T>());
         if (ld >= 0 && (best_load < 0 || ld < best_load)) {
             best_load = ld;
@@ -690,16 +626,10 @@ void launch_res2d(const Res2dPlan &p, const T *kap, const T *dco, const T *fre, 
 }
 
 template bool res2d_plan<float>(const Layout &, Res2dPlan *);
-template bool res2d_plan<double>(const Layout &, Res2dPlan *);
 template void launch_res2d<float>(const Res2dPlan &, const float *, const float *, const float *,
                                   const float *, const Layout &, const StepCoef<float> &,
                                   const float *, int, int, int, const OutSlot *,
                                   unsigned long long *, int *, cudaStream_t,
                                   const Res2dProj<float> &);
-template void launch_res2d<double>(const Res2dPlan &, const double *, const double *,
-                                   const double *, const double *, const Layout &,
-                                   const StepCoef<double> &, const double *, int, int, int,
-                                   const OutSlot *, unsigned long long *, int *, cudaStream_t,
-                                   const Res2dProj<double> &);
 
 }  // namespace htd

@@ -49,3 +49,28 @@ def test_fp64_3d_step_in_a_batch_equals_single():
         assert np.array_equal(U[r], host(s.precond(dev(F[r]))))
     b.close()
     s.close()
+
+
+# one tile, one tile row or column, tiles two nodes wide or high, last tiles of one
+# node, the ring reaching past the domain, and tiles of many nodes per thread
+SIZES_2D = [(1, 1), (1, 7), (2, 3), (5, 5), (3, 400), (400, 3), (305, 5), (31, 33), (153, 77),
+            (97, 613), (500, 501)]
+
+
+@pytest.mark.parametrize("n", SIZES_2D, ids=lambda n: "x".join(map(str, n)))
+@pytest.mark.parametrize("mode", ["table1", "project"])
+def test_fp64_2d_resident_and_one_step_match_the_oracle(n, mode):
+    p = het_problem(2, n, T=2, layer=2, seed=5)
+    o = oracle.Oracle(p)
+    F = W.random_rhs(8, n)
+    want = o.precond(F, mode).reshape(-1)
+    got = []
+    for kw in (dict(tblock=1), dict(tb_form=htd.TB_RESIDENT)):
+        s = htd.Solver(p, precision="fp64", mode=mode, **kw)
+        assert s.params["step_kernel"] == (0 if "tblock" in kw else 4)
+        U = host(s.precond(dev(F)))
+        assert rel_l2(U.reshape(-1), want) <= 1e-10
+        got.append(U)
+        s.close()
+    if mode == "table1":
+        assert np.array_equal(got[0], got[1])
