@@ -269,7 +269,7 @@ void run_resident(htd_ctx *c, const StepCoef<T> &C, int jim, int jfin, cudaStrea
                             (const double *)c->fim, c->Lr, c->c2, (const double *)c->res_ab,
                             (int)c->nsteps, jim, jfin, c->slot, c->res_x, c->err_dev, s, P);
     else
-        htd::launch_res2d<T>(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
+        htd::launch_res2d(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
                              (const T *)c->fim, c->Lr, C, (const T *)c->res_ab, (int)c->nsteps, jim,
                              jfin, c->slot, c->res_x, c->err_dev, s, P);
 }
@@ -711,7 +711,7 @@ htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cud
 {
     if (c->rcap != 1 || c->nsteps >= (1LL << 30)) return HTD_OK;
     if (!(std::is_same<T, double>::value ? htd::res2d64_plan(c->Lr, &c->res)
-                                         : htd::res2d_plan<float>(c->Lr, &c->res)))
+                                         : htd::res2d_plan(c->Lr, &c->res)))
         return HTD_OK;
     if (c->opt.mode == HTD_MODE_PROJECT) {
         // projection weights per phase k of the new state: cos and -sin of

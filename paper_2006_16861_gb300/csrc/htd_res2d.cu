@@ -1,34 +1,50 @@
-// Resident-grid 2-D recurrence (FP32, node pairs): the whole grid
-// stays in shared memory, spread over the SMs, for all T n_P steps of a run.
+// Resident-grid 2-D recurrence in FP32: the whole grid stays on chip, spread
+// over the SMs, for all T n_P steps of a run, with one exchange of edge values
+// for every two steps.
 //
 // One cooperative launch runs a whole preconditioner run (Def. of I_acd with
 // Table 1's windowed forcing and read-out).  The grid is cut into ntx x nty
 // tiles of W x H nodes, one CTA per tile and at most one CTA per SM, every CTA
-// resident at once.  A CTA loads its tile's q*kappa cells, d and forcing once,
-// keeps both recurrence states in shared memory with a one-node ring around
-// the tile, and in every step
-//  - computes the new state of its edge nodes first (one edge pair per
-//    thread) and publishes each edge value to a global exchange buffer as
-//    tagged 64-bit words (tag = index of the state + 1, beside the value's
-//    bits; one buffer per state parity);
-//  - computes its interior nodes in row strips with a 3 x 3 register window;
-//    the strip threads also read the neighbours' edge words of the new state
-//    into the ring: each read is issued two rows into the thread's strip and
-//    its tags checked after the strip, re-reading until they are the expected
-//    ones (bounded by the handle's wait limit);
-//  - passes one CTA barrier.
-// Each exchanged word carries its own tag and moves as one 64-bit access, so
-// no fence has to order data before a flag.  A CTA cannot run more than one
-// step ahead of a neighbour (it needs the neighbour's edges of the previous
-// state), so two buffers per tile suffice; they are zeroed before every run
-// (tag 0 is never expected).  Nothing else touches global memory between the
-// first load and the two output steps; no CTA waits for another except
-// through these words, and a CTA whose wait runs out sets the handle's error
-// word, which every other waiting CTA polls, so that all of them return.
+// resident at once.  Two steps make a block:
+//  A  u_{j+1} on the tile and one ring layer around it, from u_j with a ring two
+//     layers deep (the neighbours compute the same ring nodes with the same
+//     arithmetic);
+//  B  u_{j+2} on the tile; then the neighbours' values of u_{j+2} fill both ring
+//     layers of that state.
+// A thread owns 2 RPT rows of one column of the tile with its ring layer in every
+// step, as the RPT pairs (row i, row i + RPT) in paired FP32 instructions: both
+// states and d stay in registers for the whole run.  The state and cell arrays
+// in shared memory, which serve the neighbouring threads, interleave the two
+// rows of a pair, so that an operand of a pair is one 64-bit load into a register
+// pair: 6 shared-memory accesses per pair and step (pairs of adjacent columns
+// need register moves for every shifted operand, and scalar loads of the two
+// rows still moves: 87 and 81 instructions per pair and step measured, against
+// 66).
+// Edge values (nodes within two of the tile's edge) are what the neighbours
+// wait for: a pass before step B computes them one node per thread and publishes
+// them at once, so that the exchange (about a microsecond) runs under the
+// strips, which compute them again.  Publishing from the strips instead was
+// slower at every size (257 x 193: 0.87 us per step against 0.75).
+//
+// What bounds it: on small grids the exchange (257 x 193: 0.45 us per step
+// without its wait, 0.72 with it), on large ones shared memory (69 % of its
+// wavefronts at 1001^2), FP32 (47 %) and issue (46 %) together.  Measured on
+// GB300, us per step, against one exchange per step with every operand in
+// shared memory: 0.72 / 1.6 at 257 x 193, 1.90 / 2.34 at 1001^2.  Holding the
+// forcing and the cells in registers as well (256 threads) spilled from 8 rows up
+// and gained at few sizes (640^2: 1.11 against 1.20); computing the edge pass as
+// node pairs, and taking the halo pairs' own halves from registers, cost moves
+// (1001^2: 2.12).
+//
+// An exchanged value is one 64-bit word, its bits beside a tag (index of the
+// exchange + 1), so no fence orders data before a flag.  Before a CTA publishes
+// exchange e + 2 it has read its neighbours' e + 1, which they published after
+// reading its e: two buffers suffice.  They are zeroed before every run (tag 0 is
+// never expected).  A wait that runs out sets the handle's error word, which
+// every waiting CTA polls, so that all of them return.
 //
 // Per node the arithmetic is that of step2d_kernel and of the blocked kernels
-// (stencil2d, the same expression in the same order), so the results are
-// bit-identical to theirs.
+// (stencil2d, the same expression in the same order): results bit-identical.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -41,36 +57,9 @@ namespace htd {
 
 namespace {
 
-// threads per CTA (80 registers each)
-template <typename T>
-__host__ __device__ constexpr int res_threads()
-{
-    return 768;
-}
-
-using htd::vadd;
-using htd::vfma;
-using htd::vmul;
-
-// A node pair (lx, lx + 1) as one value (paired FP32 instructions)
-template <typename T>
-struct PairOf;
-template <>
-struct PairOf<float> {
-    typedef float2 V;
-    __device__ static V make(float a, float b) { return make_float2(a, b); }
-};
-template <typename T>
-__device__ __forceinline__ typename PairOf<T>::V ld2(const T *p)
-{
-    return *reinterpret_cast<const typename PairOf<T>::V *>(p);
-}
-
-template <typename T>
-__device__ __forceinline__ void st2(T *p, typename PairOf<T>::V v)
-{
-    *reinterpret_cast<typename PairOf<T>::V *>(p) = v;
-}
+constexpr int kThreads = 512;        // at most; 128 registers each
+constexpr int kMaxRows = 10;         // row pairs per thread, 1 .. kMaxRows
+constexpr int kPer = 2;              // edge nodes and ring slots per thread kept in registers
 
 __device__ __forceinline__ unsigned long long global_ns()
 {
@@ -87,195 +76,212 @@ __device__ __forceinline__ unsigned long long ld_word(const unsigned long long *
     return v;
 }
 
-__device__ __forceinline__ void st_word(unsigned long long *p, unsigned bits, unsigned tag)
+__device__ __forceinline__ void st_word(unsigned long long *p, float v, unsigned tag)
 {
-    const unsigned long long w = ((unsigned long long)tag << 32) | bits;
+    const unsigned long long w = ((unsigned long long)tag << 32) | __float_as_uint(v);
     asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
 }
 
-// An exchanged FP32 value as a tagged word, valid when the tag is the expected one.
-template <typename T>
-struct Xword;
-template <>
-struct Xword<float> {
-    static constexpr int kPer = 1;
-    struct Raw {
-        unsigned long long w;
-    };
-    __device__ static void put(unsigned long long *p, float v, unsigned tag)
+__device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
+
+// Geometry of a plan, shared by the kernel and the planner.  Threads cover the
+// columns lx = -1 .. W in NB blocks of 2 rpt rows from ly = -1.  The state and cell
+// arrays hold pairs: row ly = -1 + 2 rpt b + i (+ rpt for the second of the pair) at
+// pair row b rpt + i + 1, column lx + 2; pair row 0 and the last one carry the
+// outermost ring rows.
+struct Res2dGeom {
+    int NC, NB, S, rpt;
+    size_t plane;                    // floats per array
+    __host__ __device__ Res2dGeom(int W, int H, int r)
     {
-        st_word(p, __float_as_uint(v), tag);
+        rpt = r;
+        NC = W + 2;
+        NB = (H + 2 + 2 * r - 1) / (2 * r);
+        S = 2 * (W + 4);
+        plane = (size_t)(NB * r + 2) * S;
     }
-    __device__ static Raw get(const unsigned long long *p) { return {ld_word(p)}; }
-    __device__ static bool ok(const Raw &r, unsigned want) { return (unsigned)(r.w >> 32) == want; }
-    __device__ static float value(const Raw &r) { return __uint_as_float((unsigned)r.w); }
+    // float of node (lx, ly), ly >= -2
+    __host__ __device__ int at(int lx, int ly) const
+    {
+        const int t = ly + 1 + 2 * rpt, b = t / (2 * rpt), k = t - b * 2 * rpt;
+        const int half = k >= rpt ? 1 : 0;
+        return ((b - 1) * rpt + (k - half * rpt) + 1) * S + 2 * (lx + 2) + half;
+    }
+    // edge nodes of a full tile
+    __host__ __device__ static int edges(int W, int H)
+    {
+        const int br = H < 4 ? H : 4, bc = W < 4 ? W : 4;
+        return br * W + (H - br) * bc;
+    }
 };
-// the step coefficients broadcast to node pairs
-__device__ __forceinline__ Stencil2dCoef<float2> pair_coef(const StepCoef<float> &C)
+
+// Exchange words of a tile and parity, one per edge node in this order: rows 0,
+// 1, h-2, h-1, then columns 0, 1, w-2, w-1 of the other rows.
+__device__ __forceinline__ int edge_rank(int lx, int ly, int w, int h)
 {
-    return stencil2d_coef2(C);
+    const int br = min(h, 4), bc = min(w, 4);
+    if (ly < 2) return ly * w + lx;
+    if (ly >= h - 2) return (br - h + ly) * w + lx;
+    if (lx < 2) return br * w + (ly - 2) * bc + lx;
+    if (lx >= w - 2) return br * w + (ly - 2) * bc + (bc - w + lx);
+    return -1;
 }
 
-// row strides of the shared-memory arrays the kernel is built for (8 banks of
-// 4 bytes apart from row to row for FP32); a tile of width W uses the smallest
-// one >= W + 4
-constexpr int kStrides[] = {72, 136};
-
-__host__ __device__ constexpr size_t res2d_elems(int SW, int H)
-{
-    return 6 * (size_t)(H + 2) * SW;
-}
-
-// Shared memory: six arrays of (H + 2) rows of SW elements of T -- the states
-// U0, U1, the cells K, and d, Re F, Im F -- with node (lx, ly) of the tile at
-// row ly + 1, column lx + 2 of each (so the pair (lx, lx + 1), lx even, is
-// aligned for one vector access, and one offset addresses a node in all six),
-// the state ring at rows 0 and h + 1 and columns 1 and w + 2, and cell
-// (cx, cy) (its lower corner node) at the place of node (cx, cy).  Exchange
-// buffer of a tile and parity: E = 2W + 2H values (X::kPer words each) --
-// bottom row [0, W), top row [W, 2W), left column [2W, 2W + H), right column
-// [2W + H, 2W + 2H).
-template <typename T, int RPT, int SW>
-__global__ void __launch_bounds__(res_threads<T>(), 1)
-res2d_kernel(const T *__restrict__ kap, const T *__restrict__ dco, const T *__restrict__ fre,
-             const T *__restrict__ fim, Layout L, StepCoef<T> C,
-             const typename PairOf<T>::V *__restrict__ ab, int nsteps, int jim, int jfin,
+template <int RPT>
+__global__ void __launch_bounds__(kThreads, 1)
+res2d_kernel(const float *__restrict__ kap, const float *__restrict__ dco,
+             const float *__restrict__ fre, const float *__restrict__ fim, Layout L,
+             StepCoef<float> C, const float2 *__restrict__ ab, int nsteps, int jim, int jfin,
              const OutSlot *__restrict__ slot, unsigned long long *__restrict__ xbuf,
-             int *__restrict__ err, int W, int H, Res2dProj<T> P)
+             int *__restrict__ err, int W, int H, Res2dProj<float> P)
 {
-    typedef typename PairOf<T>::V V;
-    typedef Xword<T> X;
-    constexpr int NT = res_threads<T>();
     extern __shared__ __align__(16) unsigned char smraw[];
-    T *sm = reinterpret_cast<T *>(smraw);
     __shared__ int s_abort;
-    auto pr = [](T a, T b) { return PairOf<T>::make(a, b); };
-    const int tid = threadIdx.x;
+    const Res2dGeom G(W, H, RPT);
+    const int tid = threadIdx.x, NT = blockDim.x;
     const int tx = blockIdx.x, ty = blockIdx.y;
-    const int ntx = gridDim.x, nty = gridDim.y;
-    const int64_t x0 = (int64_t)tx * W, y0 = (int64_t)ty * H;
-    const int w = (int)min((int64_t)W, L.nx - x0);
-    const int h = (int)min((int64_t)H, L.ny - y0);
-    const int NA = (H + 2) * SW;
-    T *U0 = sm, *U1 = sm + NA, *K = sm + 2 * NA;
-    T *D = sm + 3 * NA, *FR = sm + 4 * NA, *FI = sm + 5 * NA;
-    const int EW = (2 * W + 2 * H) * X::kPer;          // exchange words per tile and parity
+    const int ntx = gridDim.x;
+    const int x0 = tx * W, y0 = ty * H;
+    const int nx = (int)L.nx, ny = (int)L.ny;
+    const int w = min(W, nx - x0), h = min(H, ny - y0);
+    const int NC = G.NC, S = G.S;
+    float4 *F4 = reinterpret_cast<float4 *>(smraw);            // forcing of the pairs, thread rows
+    float4 *EC = F4 + G.NB * RPT * NC;                         // (d, Re F, Im F) of the edge nodes
+    int4 *EI = reinterpret_cast<int4 *>(EC + Res2dGeom::edges(W, H));   // and their elements
+    float *U0 = reinterpret_cast<float *>(EI + Res2dGeom::edges(W, H));
+    float *U1 = U0 + G.plane, *K = U1 + G.plane;
+    const int E = Res2dGeom::edges(W, H);                      // words per tile and parity
 
+    auto in_domain = [&](int lx, int ly) {
+        return x0 + lx >= 0 && x0 + lx < nx && y0 + ly >= 0 && y0 + ly < ny;
+    };
+    auto gidx = [&](int lx, int ly) {
+        return (int64_t)(y0 + ly + 1) * L.pitch + L.xl + x0 + lx;
+    };
     if (tid == 0) s_abort = 0;
-    for (int i = tid; i < NA; i += NT) {
-        const int ly = i / SW - 1, lx = i % SW - 2;
-        T k = 0, dv = 0, fr = 0, fi = 0;
-        if (lx >= -1 && lx < w && ly >= -1 && ly < h) {
-            const int64_t g = (y0 + ly + 1) * L.pitch + L.xl + x0 + lx;
-            k = kap[g];                                // cell (lx, ly)
-            if (lx >= 0 && ly >= 0) {
-                dv = dco[g];
-                fr = fre[g];
-                fi = fim[g];
-            }
-        }
+    for (int i = tid; i < (int)G.plane; i += NT) {
         U0[i] = 0.f;
         U1[i] = 0.f;
-        K[i] = k;
-        D[i] = dv;
-        FR[i] = fr;
-        FI[i] = fi;
+        K[i] = 0.f;
+    }
+    __syncthreads();
+    // cells (lower corner lx, ly), those of the domain's nodes
+    for (int i = tid; i < (W + 4) * (H + 4); i += NT) {
+        const int lx = i % (W + 4) - 2, ly = i / (W + 4) - 2;
+        if (x0 + lx >= -1 && x0 + lx < nx && y0 + ly >= -1 && y0 + ly < ny)
+            K[G.at(lx, ly)] = kap[gidx(lx, ly)];
+    }
+    // this thread's strip: column lx, rows ly0 + i and ly0 + RPT + i.  Nodes
+    // outside the domain or beyond the ring layer have d = 0 and no forcing, so
+    // they stay exactly zero.
+    const bool has = tid < NC * G.NB;
+    const int q = has ? tid % NC : 0, blk = has ? tid / NC : 0;
+    const int lx = q - 1, ly0 = blk * 2 * RPT - 1;
+    const bool sx = has && lx >= 0 && lx < w;      // a tile column
+    float4 *fp = F4 + blk * RPT * NC + q;
+    float2 za[RPT], zb[RPT], dd[RPT];
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        za[i] = zb[i] = dd[i] = f2(0.f, 0.f);
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int la = ly0 + i, lb = ly0 + RPT + i;
+        if (has && lx <= w && la <= h && in_domain(lx, la)) {
+            const int64_t g = gidx(lx, la);
+            dd[i].x = dco[g];
+            f.x = fre[g];
+            f.z = fim[g];
+        }
+        if (has && lx <= w && lb <= h && in_domain(lx, lb)) {
+            const int64_t g = gidx(lx, lb);
+            dd[i].y = dco[g];
+            f.y = fre[g];
+            f.w = fim[g];
+        }
+        if (has) fp[i * NC] = f;
+    }
+    const int o0 = (blk * RPT + 1) * S + 2 * q;    // pair left of the strip's first pair
+    // pairs whose two nodes, and whose one or the other node, are in the tile
+    unsigned in2 = 0, in1a = 0, in1b = 0;
+#pragma unroll
+    for (int i = 0; i < RPT; ++i) {
+        const bool ra = sx && (unsigned)(ly0 + i) < (unsigned)h;
+        const bool rb = sx && (unsigned)(ly0 + RPT + i) < (unsigned)h;
+        if (ra && rb) in2 |= 1u << i;
+        else if (ra) in1a |= 1u << i;
+        else if (rb) in1b |= 1u << i;
     }
 
-    // Work of a step, per thread in this order: (1) an edge pair -- rows 0 and
-    // h-1, then the pairs 0 and PL of rows 1 .. h-2 -- dealt one per thread
-    // from the last thread down, so that threads without interior work take
-    // them first (several edge pairs on one thread publish the later ones too
-    // late for the neighbours); each new edge value is published at once; (2) one strip of up to RPT interior
-    // rows of an interior column pair 1 .. PL-1 (strip t on thread t); (3) the
-    // ring slot of the next state (slot k on thread k): the read of the
-    // neighbour's word is issued two rows into the thread's strip and its tag
-    // checked after the strip, so that the exchange overlaps the interior
-    // work; the word is read again only if the neighbour had not published it.
-    // The geometry of all three is the same in every step.
-    const int PW = (w + 1) >> 1, PL = PW - 1;
-    const int ncp = max(0, PL - 1);
-    const int nrow = max(0, h - 2);
-    const int nS = ncp * ((nrow + RPT - 1) / RPT);
-    const int nEr = (h >= 2) ? 2 : 1;
-    const int nEc = (PL > 0) ? 2 : 1;
-    const int nA = nEr * PW + nrow * nEc;
-    const int nslot = 2 * w + 2 * h + 4;
-    // (1) the edge pair of task a as (node offset, lx, ly)
-    auto edge_of = [&](int a, int &lx, int &ly) {
-        int p;
-        if (a < nEr * PW) {
-            ly = (a < PW) ? 0 : h - 1;
-            p = (a < PW) ? a : a - PW;
+    // edge nodes: rank t on thread t
+    const int br = min(h, 4), bc = min(w, 4);
+    const int nE = br * w + (h - br) * bc;
+    auto edge_node = [&](int t, int &lx, int &ly) {
+        if (t < br * w) {
+            const int r = t / w;
+            ly = r < 2 ? r : h - br + r;
+            lx = t % w;
         } else {
-            const int b = a - nEr * PW;
-            ly = 1 + b / nEc;
-            p = (b % nEc) ? PL : 0;
+            const int s = t - br * w, cc = s % bc;
+            ly = 2 + s / bc;
+            lx = cc < 2 ? cc : w - bc + cc;
         }
-        lx = 2 * p;
     };
-    const int ea = NT - 1 - tid;              // this thread's first edge task
-    int e_lx = 0, e_ly = 0;
-    if (ea < nA) edge_of(ea, e_lx, e_ly);
-    // (2) strip t: column pair, first row, rows
-    auto strip_of = [&](int t, int &lx, int &r0, int &nr) -> bool {
-        lx = 2 * (1 + t % ncp);
-        r0 = 1 + (t / ncp) * RPT;
-        nr = min(RPT, h - 1 - r0);
-        return true;
-    };
-    int s_lx = 0, s_r0 = 1, s_nr = 0;
-    const bool has_strip = tid < nS && strip_of(tid, s_lx, s_r0, s_nr);
-    // (3) the ring slot: the neighbour's word (offset in xbuf for parity 0, or
-    // -1 on the domain boundary, where the ring stays zero) and its place in a
-    // state array
+    float e_prev[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        e_prev[k] = 0.f;
+        const int t = tid + k * NT;
+        if (t < nE) {
+            int ex, ey;
+            edge_node(t, ex, ey);
+            EI[t] = make_int4(G.at(ex, ey), G.at(ex, ey - 1), G.at(ex, ey + 1), 0);
+            const int64_t g = gidx(ex, ey);
+            EC[t] = make_float4(dco[g], fre[g], fim[g], 0.f);
+        }
+    }
+    // ring slot k: rows -2, -1, h, h+1 over w + 4 columns, then columns -2, -1, w,
+    // w+1 of the tile's rows: the neighbour's word (-1 outside the domain, where
+    // the ring stays zero) and the place in a state array
+    const int nslot = 4 * (w + 4) + 4 * h;
     auto slot_of = [&](int k, int &dst) -> int {
-        int nbx = tx, nby = ty, idx;
-        if (k < w) {                                   // below the tile: the top row of (tx, ty-1)
-            nby = ty - 1;
-            idx = W + k;
-            dst = k + 2;
-        } else if (k < 2 * w) {                        // above: the bottom row of (tx, ty+1)
-            nby = ty + 1;
-            idx = k - w;
-            dst = (h + 1) * SW + (k - w) + 2;
-        } else if (k < 2 * w + h) {                    // left: the right column of (tx-1, ty)
-            const int ly = k - 2 * w;
-            nbx = tx - 1;
-            idx = 2 * W + H + ly;
-            dst = (ly + 1) * SW + 1;
-        } else if (k < 2 * w + 2 * h) {                // right: the left column of (tx+1, ty)
-            const int ly = k - 2 * w - h;
-            nbx = tx + 1;
-            idx = 2 * W + ly;
-            dst = (ly + 1) * SW + w + 2;
-        } else {                                       // corners, from the diagonal tiles' rows
-            const int c = k - 2 * w - 2 * h;           // 0 (-1,-1), 1 (w,-1), 2 (-1,h), 3 (w,h)
-            nbx = (c & 1) ? tx + 1 : tx - 1;
-            nby = (c & 2) ? ty + 1 : ty - 1;
-            idx = (c & 2) ? ((c & 1) ? 0 : W - 1) : ((c & 1) ? W : 2 * W - 1);
-            dst = ((c & 2) ? h + 1 : 0) * SW + ((c & 1) ? w + 2 : 1);
+        int rx, ry;
+        if (k < 4 * (w + 4)) {
+            const int r = k / (w + 4);
+            ry = r < 2 ? r - 2 : h + r - 2;
+            rx = k % (w + 4) - 2;
+        } else {
+            const int s = k - 4 * (w + 4), cc = s / h;
+            ry = s % h;
+            rx = cc < 2 ? cc - 2 : w + cc - 2;
         }
-        if (nbx < 0 || nbx >= ntx || nby < 0 || nby >= nty) return -1;
-        return (nby * ntx + nbx) * 2 * EW + idx * X::kPer;
+        dst = G.at(rx, ry);
+        if (!in_domain(rx, ry)) return -1;
+        const int dx = rx < 0 ? -1 : rx >= w ? 1 : 0, dy = ry < 0 ? -1 : ry >= h ? 1 : 0;
+        const int wn = min(W, nx - (tx + dx) * W), hn = min(H, ny - (ty + dy) * H);
+        const int lx = dx < 0 ? wn + rx : dx > 0 ? rx - w : rx;
+        const int ly = dy < 0 ? hn + ry : dy > 0 ? ry - h : ry;
+        return ((ty + dy) * ntx + tx + dx) * 2 * E + edge_rank(lx, ly, wn, hn);
     };
-    int r_dst = 0;
-    const int r_src = (tid < nslot) ? slot_of(tid, r_dst) : -1;
+    int r_dst[kPer], r_src[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        r_dst[k] = 0;
+        r_src[k] = tid + k * NT < nslot ? slot_of(tid + k * NT, r_dst[k]) : -1;
+    }
 
-    // store slot value v (read from p) of state s into U at dst, reading it again
-    // until its words carry the tag of state s (bounded by the handle's limit;
-    // with the stall test the first wait of CTA (0, 0) expects a tag no word has)
-    auto complete = [&](const unsigned long long *p, typename X::Raw v, int s, int dst, T *U) {
-        unsigned want = (unsigned)(s + 1);
-        if (s == 1 && tx == 0 && ty == 0 && *(volatile const int *)(err + 1) != 0)
+    // word v (read from p) of exchange e into U0[dst], read again until it carries
+    // the tag (bounded by the handle's limit; with the stall test the first wait
+    // of CTA (0, 0) expects a tag no word has)
+    auto complete = [&](const unsigned long long *p, unsigned long long v, int e, int dst) {
+        unsigned want = (unsigned)(e + 1);
+        if (e == 0 && tx == 0 && ty == 0 && *(volatile const int *)(err + 1) != 0)
             want = 0xffffffffu;
-        if (!X::ok(v, want)) {
+        if ((unsigned)(v >> 32) != want) {
             unsigned long long lim = *reinterpret_cast<volatile const unsigned long long *>(err + 2);
             if (lim == 0) lim = kDefaultWaitNs;
             const unsigned long long t0 = global_ns();
             for (int it = 1;; ++it) {
-                v = X::get(p);
-                if (X::ok(v, want)) break;
+                v = ld_word(p);
+                if ((unsigned)(v >> 32) == want) break;
                 if ((it & 31) == 0 && *(volatile int *)err) {
                     s_abort = 1;
                     return;
@@ -287,219 +293,183 @@ res2d_kernel(const T *__restrict__ kap, const T *__restrict__ dco, const T *__re
                 }
             }
         }
-        U[dst] = X::value(v);
+        U0[dst] = __uint_as_float((unsigned)v);
     };
 
-    const Stencil2dCoef<V> SC = pair_coef(C);
-    const V n2 = pr(T(-2), T(-2));
-    // u row at q (the node lx - 1 of the row) as the pairs (m, 0, p) =
-    // (u(lx-1+o), u(lx+o)), o = 0, 1, 2
-    auto urow = [&](const T *q, V &m, V &z, V &p) {
-        const T l = q[0];
-        z = ld2(q + 1);
-        const T r = q[3];
-        m = pr(l, z.x);
-        p = pr(z.y, r);
-    };
-    // cells at q (the cell lx - 1 of a cell row): k0 = cells left of the nodes
-    // (lx-1, lx), k1 = cells right of them
-    auto krow = [&](const T *q, V &k0, V &k1) {
-        k1 = ld2(q + 1);
-        k0 = pr(q[0], k1.x);
-    };
-    auto output = [&](int lx, int ly, V u, int fl, bool two) {
-        const int64_t c = ((int64_t)blockIdx.y * H + ly) * L.nx + (int64_t)blockIdx.x * W + lx;
-        if ((fl & 1) && slot->snap_part) {
-            slot->snap_part[2 * c] = (double)u.x;
-            if (two) slot->snap_part[2 * c + 2] = (double)u.y;
-        }
-        if ((fl & 2) && slot->final_part) {
-            slot->final_part[2 * c] = (double)u.x;
-            if (two) slot->final_part[2 * c + 2] = (double)u.y;
-        }
-    };
-    // the new state of the pair at node offset o (row ly + 1, column lx + 2)
-    // from its stencil sum
-    auto update = [&](int o, V acc, V a2, V nb2, T *nxt) -> V {
-        const V ag = vfma(a2, ld2(FR + o), vfma(nb2, ld2(FI + o), acc));
-        const V uprev = ld2(nxt + o);
-        return vfma(ld2(D + o), vfma(n2, uprev, ag), uprev);
-    };
-    // nr <= RPT interior rows r0 .. r0+nr-1 of the column pair lx; the read of
-    // the ring word at rp (if any) is issued before the third row
-    // (kFull: nr == RPT, so the unrolled rows need no test; kOut: a step with
-    // output flags)
-    auto strip = [&](int lx, int r0, int nr, const T *cur, T *nxt, V a2, V nb2, int fl,
-                     const unsigned long long *rp, typename X::Raw &rv, bool &issued,
-                     auto full_tag, auto out_tag) {
-        constexpr bool kFull = decltype(full_tag)::value, kOut = decltype(out_tag)::value;
-        const int o0 = r0 * SW + lx + 1;               // node (lx - 1, r0 - 1)
-        const T *qc = cur + o0, *qk = K + o0;
-        V umm, um0, ump, u0m, u00, u0p, k00, k01;
-        urow(qc, umm, um0, ump);
-        urow(qc + SW, u0m, u00, u0p);
-        V pm = vadd(umm, ump), p0 = vadd(u0m, u0p);
-        krow(qk, k00, k01);
-        V hk0 = vadd(k00, k01);
+    const Stencil2dCoef<float2> SC = stencil2d_coef2(C);
+    // The strip's new states over zo from zc (own nodes) and cur (the neighbours).
+    // kB: step B stores tile nodes only, and issues the reads of this thread's
+    // ring words half way down.
+    unsigned long long rv[kPer];
+    auto strip = [&](const float2 (&zc)[RPT], float2 (&zo)[RPT], const float *cur, float *nxt,
+                     float2 abj, auto is_b, const unsigned long long *xr) {
+        constexpr bool kB = decltype(is_b)::value;
+        const float2 a2 = f2(abj.x, abj.x), nb2 = f2(-abj.y, -abj.y), n2 = f2(-2.f, -2.f);
+        const float *u = cur + o0, *k = K + o0;
+        // operand pair i, c columns right of lx - 1
+        auto pair = [&](const float *b, int i, int c) {
+            return *reinterpret_cast<const float2 *>(b + i * S + 2 * c);
+        };
+        // The pairs above the first one -- (row before the strip, row RPT - 1) -- and
+        // below the last one -- (row RPT, row after the strip)
+        auto above = [&](const float *b, int c) {
+            return f2(b[-S + 2 * c + 1], b[(RPT - 1) * S + 2 * c]);
+        };
+        auto below = [&](const float *b, int c) {
+            return f2(b[2 * c + 1], b[RPT * S + 2 * c]);
+        };
+        float2 umm = above(u, 0), um0 = above(u, 1), ump = above(u, 2);
+        float2 u0m = pair(u, 0, 0), u0p = pair(u, 0, 2);
+        float2 k00 = above(k, 0), k01 = above(k, 1);
+        float2 pm = vadd(umm, ump), p0 = vadd(u0m, u0p), hk0 = vadd(k00, k01);
 #pragma unroll
         for (int i = 0; i < RPT; ++i) {
-            if (!kFull && i >= nr) break;
-            if (i == 2 && rp) {
-                rv = X::get(rp);
-                issued = true;
+            if (kB && i == RPT / 2) {
+#pragma unroll
+                for (int s = 0; s < kPer; ++s)
+                    if (xr && r_src[s] >= 0) rv[s] = ld_word(xr + r_src[s]);
             }
-            V upm, up0, upp, k10, k11;
-            urow(qc + (i + 2) * SW, upm, up0, upp);
-            krow(qk + (i + 1) * SW, k10, k11);
-            const V pp = vadd(upm, upp);
-            const V hk1 = vadd(k10, k11);
-            const V acc = stencil2d(SC, umm, um0, ump, u0m, u00, u0p, upm, up0, upp, k00, k01,
-                                         k10, k11, pm, p0, pp, hk0, hk1);
-            const int o = o0 + (i + 1) * SW + 1;       // node (lx, r0 + i)
-            const V unew = update(o, acc, a2, nb2, nxt);
-            st2(nxt + o, unew);
-            if (kOut) output(lx, r0 + i, unew, fl, true);
-            umm = u0m; um0 = u00; ump = u0p; pm = p0;
-            u0m = upm; u00 = up0; u0p = upp; p0 = pp;
+            float2 upm, up0, upp;
+            if (i + 1 < RPT) {
+                upm = pair(u, i + 1, 0);
+                up0 = zc[i + 1 < RPT ? i + 1 : 0];
+                upp = pair(u, i + 1, 2);
+            } else {
+                upm = below(u, 0);
+                up0 = below(u, 1);
+                upp = below(u, 2);
+            }
+            const float2 k10 = pair(k, i, 0), k11 = pair(k, i, 1);
+            const float2 pp = vadd(upm, upp), hk1 = vadd(k10, k11);
+            const float2 acc = stencil2d(SC, umm, um0, ump, u0m, zc[i], u0p, upm, up0, upp, k00,
+                                         k01, k10, k11, pm, p0, pp, hk0, hk1);
+            const float4 f = fp[i * NC];
+            const float2 ag = vfma(a2, f2(f.x, f.y), vfma(nb2, f2(f.z, f.w), acc));
+            const float2 un = vfma(dd[i], vfma(n2, zo[i], ag), zo[i]);
+            zo[i] = un;
+            float *o = nxt + o0 + i * S + 2;
+            if (!kB || (in2 >> i & 1)) {
+                *reinterpret_cast<float2 *>(o) = un;
+            } else {
+                if (in1a >> i & 1) o[0] = un.x;
+                if (in1b >> i & 1) o[1] = un.y;
+            }
+            umm = u0m; um0 = zc[i]; ump = u0p; pm = p0;
+            u0m = upm; u0p = upp; p0 = pp;
             k00 = k10; k01 = k11; hk0 = hk1;
         }
     };
+    // the new value of an edge node in step B (o: its element, those above and below;
+    // e: d, Re F, Im F)
+    auto edge_value = [&](int4 o, float4 e, float prev, float2 abj) -> float {
+        const Stencil2dCoef<float> c = stencil2d_coef(C);
+        const float *u0 = U1 + o.x, *um = U1 + o.y, *up = U1 + o.z;
+        const float *k0 = K + o.x, *km = K + o.y;
+        const float umm = um[-2], um0 = um[0], ump = um[2];
+        const float u0m = u0[-2], u00 = u0[0], u0p = u0[2];
+        const float upm = up[-2], up0 = up[0], upp = up[2];
+        const float k00 = km[-2], k01 = km[0], k10 = k0[-2], k11 = k0[0];
+        const float acc = stencil2d(c, umm, um0, ump, u0m, u00, u0p, upm, up0, upp, k00, k01, k10,
+                                    k11, vadd(umm, ump), vadd(u0m, u0p), vadd(upm, upp),
+                                    vadd(k00, k01), vadd(k10, k11));
+        const float ag = vfma(abj.x, e.y, vfma(-abj.y, e.z, acc));
+        return vfma(e.x, vfma(-2.f, prev, ag), prev);
+    };
+    // outputs of the new state of step j (tile nodes of U): snapshot, final state,
+    // and in projection mode the compensated sums of the window's states (as the
+    // separate accumulation kernel adds them)
+    auto read_out = [&](const float *U, int j) {
+        const bool acc = j >= P.j_acc;
+        const int ph = acc ? (j + 1) % P.nP : 0;
+        const float wc = acc ? P.w[2 * ph] : 0.f, ws = acc ? P.w[2 * ph + 1] : 0.f;
+        for (int i = tid; i < w * h; i += NT) {
+            const int ly = i / w, lx = i - ly * w;
+            const int64_t c = (int64_t)(y0 + ly) * nx + x0 + lx;
+            const float v = U[G.at(lx, ly)];
+            if (j + 1 == jim && slot->snap_part) slot->snap_part[2 * c] = (double)v;
+            if (j + 1 == jfin && slot->final_part) slot->final_part[2 * c] = (double)v;
+            if (acc) {
+                float *s = P.acc + c;
+                const float sr = s[0], si = s[P.N], cr = s[2 * P.N], ci = s[3 * P.N];
+                const float yr = wc * v - cr, yi = ws * v - ci;
+                const float tr = sr + yr, ti = si + yi;
+                s[2 * P.N] = (tr - sr) - yr;
+                s[3 * P.N] = (ti - si) - yi;
+                s[0] = tr;
+                s[P.N] = ti;
+            }
+        }
+    };
+    auto reads = [&](int j) { return j + 1 == jim || j + 1 == jfin || j >= P.j_acc; };
 
     __syncthreads();
-    for (int j = 0; j < nsteps; ++j) {
-        const T *cur = (j & 1) ? U1 : U0;              // u_j (ring filled)
-        T *nxt = (j & 1) ? U0 : U1;                    // u_{j-1}, becomes u_{j+1}
-        const V abj = ab[j];
-        const V a2 = pr(abj.x, abj.x), nb2 = pr(-abj.y, -abj.y);
-        const int fl = ((j + 1 == jim) ? 1 : 0) | ((j + 1 == jfin) ? 2 : 0);
-        const bool more = j + 1 < nsteps;
-
-        // (1) edge pairs, published as they are computed
-        if (ea < nA) {
-            const unsigned tag = (unsigned)(j + 2);
-            unsigned long long *pub = xbuf + (size_t)((ty * ntx + tx) * 2 + ((j + 1) & 1)) * EW;
-            auto publish = [&](int lx, int ly, T v) {
-                if (ly == 0) X::put(pub + X::kPer * lx, v, tag);
-                if (ly == h - 1) X::put(pub + X::kPer * (W + lx), v, tag);
-                if (lx == 0) X::put(pub + X::kPer * (2 * W + ly), v, tag);
-                if (lx == w - 1) X::put(pub + X::kPer * (2 * W + H + ly), v, tag);
-            };
-            for (int a = ea; a < nA; a += NT) {
-                int lx = e_lx, ly = e_ly;
-                if (a != ea) edge_of(a, lx, ly);
-                const int o = (ly + 1) * SW + lx + 2;
-                V umm, um0, ump, u0m, u00, u0p, upm, up0, upp, k00, k01, k10, k11;
-                urow(cur + o - SW - 1, umm, um0, ump);
-                urow(cur + o - 1, u0m, u00, u0p);
-                urow(cur + o + SW - 1, upm, up0, upp);
-                krow(K + o - SW - 1, k00, k01);
-                krow(K + o - 1, k10, k11);
-                const V acc =
-                    stencil2d(SC, umm, um0, ump, u0m, u00, u0p, upm, up0, upp, k00, k01, k10, k11,
-                              vadd(umm, ump), vadd(u0m, u0p), vadd(upm, upp), vadd(k00, k01),
-                              vadd(k10, k11));
-                const V unew = update(o, acc, a2, nb2, nxt);
-                const bool two = lx + 1 < w;                // the second node is in the tile
-                if (two) st2(nxt + o, unew);
-                else nxt[o] = unew.x;
-                publish(lx, ly, unew.x);
-                if (two) publish(lx + 1, ly, unew.y);
-                if (fl) output(lx, ly, unew, fl, two);
+    for (int j = 0; j < nsteps; j += 2) {
+        const float2 abA = ab[j], abB = ab[j + 1];
+        // A: the ring nodes a thread owns come from the exchange
+        if (has) {
+#pragma unroll
+            for (int i = 0; i < RPT; ++i)
+                if (!(in2 >> i & 1)) za[i] = *reinterpret_cast<const float2 *>(U0 + o0 + i * S + 2);
+            strip(za, zb, U0, U1, abA, std::false_type{}, nullptr);
+        }
+        __syncthreads();
+        if (reads(j)) read_out(U1, j);
+        // B
+        const int e = j >> 1;
+        const bool more = j + 2 < nsteps;
+        const unsigned long long *xr = more ? xbuf + (size_t)(e & 1) * E : nullptr;
+        if (more) {
+            unsigned long long *pub = xbuf + (size_t)((ty * ntx + tx) * 2 + (e & 1)) * E;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int t = tid + k * NT;
+                if (t < nE) {
+                    e_prev[k] = edge_value(EI[t], EC[t], e_prev[k], abB);
+                    st_word(pub + t, e_prev[k], (unsigned)(e + 1));
+                }
             }
         }
-
-        // (2) the interior strip, with the read of this thread's ring slot
-        const unsigned long long *rp =
-            (more && r_src >= 0) ? xbuf + r_src + ((j + 1) & 1) * EW : nullptr;
-        typename X::Raw rv{};
-        bool issued = false;
-        using T_ = std::true_type;
-        using F_ = std::false_type;
-        if (has_strip) {
-            if (s_nr == RPT) {
-                if (fl) strip(s_lx, s_r0, s_nr, cur, nxt, a2, nb2, fl, rp, rv, issued, T_{}, T_{});
-                else strip(s_lx, s_r0, s_nr, cur, nxt, a2, nb2, fl, rp, rv, issued, T_{}, F_{});
-            } else {
-                strip(s_lx, s_r0, s_nr, cur, nxt, a2, nb2, fl, rp, rv, issued, F_{}, T_{});
-            }
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) rv[k] = 0;
+        if (has) strip(zb, za, U1, U0, abB, std::true_type{}, xr);
+        if (more) {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k)
+                if (r_src[k] >= 0) complete(xr + r_src[k], rv[k], e, r_dst[k]);
         }
-        for (int t = tid + NT; t < nS; t += NT) {
-            int lx, r0, nr;
-            if (strip_of(t, lx, r0, nr))
-                strip(lx, r0, nr, cur, nxt, a2, nb2, fl, nullptr, rv, issued, F_{}, T_{});
-        }
-
-        // (3) the ring of u_{j+1}
-        if (rp) complete(rp, issued ? rv : X::get(rp), j + 1, r_dst, nxt);
-        if (more)
-            for (int k = tid + NT; k < nslot; k += NT) {
-                int dst = 0;
-                const int src = slot_of(k, dst);
-                if (src < 0) continue;
-                const unsigned long long *p = xbuf + src + ((j + 1) & 1) * EW;
-                complete(p, X::get(p), j + 1, dst, nxt);
-            }
         __syncthreads();
         if (s_abort) break;
-        // projection read-out: the compensated accumulation of u_{j+1} (complete
-        // in nxt, which the next step only reads) into the sums and
-        // compensations (re, im), as the separate accumulation kernel does it,
-        // the tile's nodes in compact order
-        if (j >= P.j_acc) {
-            const int k = (j + 1) % P.nP;
-            const T wc = P.w[2 * k], ws = P.w[2 * k + 1];
-            T *a = P.acc;
-            for (int i = tid; i < w * h; i += NT) {
-                const int ly = i / w, lx = i - ly * w;
-                const int64_t c = ((int64_t)blockIdx.y * H + ly) * L.nx +
-                                  (int64_t)blockIdx.x * W + lx;
-                const T v = nxt[(ly + 1) * SW + lx + 2];
-                T sr = a[c], si = a[P.N + c], cr = a[2 * P.N + c], ci = a[3 * P.N + c];
-                const T yr = wc * v - cr, yi = ws * v - ci;
-                const T tr = sr + yr, ti = si + yi;
-                a[2 * P.N + c] = (tr - sr) - yr;
-                a[3 * P.N + c] = (ti - si) - yi;
-                a[c] = tr;
-                a[P.N + c] = ti;
-            }
-        }
+        if (reads(j + 1)) read_out(U0, j + 1);
     }
 }
 
-// Rows per strip a plan may choose (one-row strips measured no faster at 101^2)
-constexpr int kRpts[] = {3, 5, 8};
-
-// fn(the kernel for precision T, RPT rows per strip, row stride SW)
-template <typename T, typename Fn>
-void with_kernel(int rpt, int sw, Fn &&fn)
+template <typename Fn>
+void with_kernel(int rpt, Fn &&fn)
 {
-    if (sw == 72) {
-        if (rpt == 3) fn(res2d_kernel<T, 3, 72>);
-        else if (rpt == 5) fn(res2d_kernel<T, 5, 72>);
-        else fn(res2d_kernel<T, 8, 72>);
-    } else {
-        if (rpt == 3) fn(res2d_kernel<T, 3, 136>);
-        else if (rpt == 5) fn(res2d_kernel<T, 5, 136>);
-        else fn(res2d_kernel<T, 8, 136>);
+    switch (rpt) {
+    case 1: fn(res2d_kernel<1>); break;
+    case 2: fn(res2d_kernel<2>); break;
+    case 3: fn(res2d_kernel<3>); break;
+    case 4: fn(res2d_kernel<4>); break;
+    case 5: fn(res2d_kernel<5>); break;
+    case 6: fn(res2d_kernel<6>); break;
+    case 7: fn(res2d_kernel<7>); break;
+    case 8: fn(res2d_kernel<8>); break;
+    case 9: fn(res2d_kernel<9>); break;
+    default: fn(res2d_kernel<10>); break;
     }
 }
 
-// Rows of work of the busiest thread of a full W x H tile with RPT rows per
-// strip (an edge pair counted as two rows: it has no register window), or -1
-// if there are more strips than threads.
-int res2d_load(int W, int H, int rpt, int NT)
+size_t res2d_smem(int W, int H, int rpt)
 {
-    const int PW = (W + 1) / 2, PL = PW - 1;
-    const int nrow = std::max(0, H - 2);
-    const int nS = std::max(0, PL - 1) * ((nrow + rpt - 1) / rpt);
-    const int nA = ((H >= 2) ? 2 : 1) * PW + nrow * ((PL > 0) ? 2 : 1);
-    if (nS > NT) return -1;
-    const int edges = (nA + NT - 1) / NT;                       // edge pairs per thread
-    return std::min(rpt, nrow) + 2 * (nS + nA > NT ? edges : 0);
+    const Res2dGeom G(W, H, rpt);
+    return 3 * G.plane * sizeof(float) +
+           ((size_t)G.NB * rpt * G.NC + 2 * (size_t)Res2dGeom::edges(W, H)) * sizeof(float4);
 }
 
-template <typename T>
-bool plan_impl(const Layout &L, Res2dPlan *out)
+}  // namespace
+
+bool res2d_plan(const Layout &L, Res2dPlan *out)
 {
     if (L.d != 2 || L.nx < 1 || L.ny < 1) return false;
     int dev = 0, nsm = 0, coop = 0, maxsm = 0;
@@ -513,103 +483,91 @@ bool plan_impl(const Layout &L, Res2dPlan *out)
     if (!coop || nsm < 1) return false;
     // the limit is a property of the kernel, shared by every handle: raise it
     // to what the device allows beside the kernel's static shared memory,
-    // rather than to this plan's size (a smaller plan made later must not
-    // shrink it under an earlier handle's launches)
+    // rather than to this plan's size
     int avail = maxsm;
     bool attr_ok = true;
-    for (int sw : kStrides)
-        for (int r : kRpts) {
-            with_kernel<T>(r, sw, [&](auto kern) {
-                cudaFuncAttributes fa;
-                if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
-                    attr_ok = false;
-                    return;
-                }
-                const int dyn = maxsm - (int)fa.sharedSizeBytes;
-                avail = std::min(avail, dyn);
-                attr_ok = attr_ok && dyn > 0 &&
-                          cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               dyn) == cudaSuccess;
-            });
-        }
+    for (int r = 1; r <= kMaxRows; ++r)
+        with_kernel(r, [&](auto kern) {
+            cudaFuncAttributes fa;
+            if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
+                attr_ok = false;
+                return;
+            }
+            const int dyn = maxsm - (int)fa.sharedSizeBytes;
+            avail = std::min(avail, dyn);
+            attr_ok = attr_ok && dyn > 0 &&
+                      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           dyn) == cudaSuccess;
+        });
     if (!attr_ok) {
         (void)cudaGetLastError();
         return false;
     }
-    // the tiling with the smallest largest tile (then the shortest edges) that
-    // fits one tile per CTA, one CTA per SM
+    // Tiles of W x H nodes (inner tiles at least 2 x 2: the ring reaches one tile
+    // only) with RPT row pairs per thread, at most one tile per SM.  Cost of two
+    // steps in cycles of an SM's quarter: a row pair takes about 60 issue cycles
+    // per warp, 120 when no other warp fills its latency; the edge pass about 60
+    // per warp and pass.
     Res2dPlan best;
-    long long best_area = -1, best_edge = 0;
-    for (int a = 1; a <= nsm; ++a) {
-        long long W = (L.nx + a - 1) / a;
-        W += W & 1;
+    long long best_cost = -1;
+    for (int a = 1; a <= nsm && (a == 1 || 2 * (a - 1) < L.nx); ++a) {
+        const long long W = std::max<long long>(2, (L.nx + a - 1) / a);
         const long long ntx = (L.nx + W - 1) / W;
         const long long tiles_y = nsm / ntx;
         if (tiles_y < 1) break;
-        const long long H = (L.ny + tiles_y - 1) / tiles_y;
+        const long long H = std::max<long long>(2, (L.ny + tiles_y - 1) / tiles_y);
         const long long nty = (L.ny + H - 1) / H;
-        int sw = 0;
-        for (int s : kStrides)
-            if (sw == 0 && W + 4 <= s) sw = s;
-        if (sw == 0 || H > 4096) continue;
-        const size_t smem = res2d_elems(sw, (int)H) * sizeof(T);
-        if (smem > (size_t)avail) continue;
-        const long long area = W * H, edge = W + H;
-        if (best_area < 0 || area < best_area || (area == best_area && edge < best_edge)) {
-            best_area = area;
-            best_edge = edge;
-            best.W = (int)W;
-            best.H = (int)H;
-            best.sw = sw;
-            best.ntx = (int)ntx;
-            best.nty = (int)nty;
-            best.smem = smem;
+        if (H > 8192 || W > kThreads) continue;
+        for (int rpt = 1; rpt <= kMaxRows; ++rpt) {
+            const Res2dGeom G((int)W, (int)H, rpt);
+            const long long strips = (long long)G.NC * G.NB;
+            const long long nedge = Res2dGeom::edges((int)W, (int)H);
+            const long long slots = 4 * (W + 4) + 4 * H;
+            // the edge pass and the ring keep kPer entries per thread
+            long long threads = std::max(strips, (std::max(slots, nedge) + kPer - 1) / kPer);
+            threads = (threads + 31) / 32 * 32;
+            const size_t smem = res2d_smem((int)W, (int)H, rpt);
+            if (threads > kThreads || smem > (size_t)avail) continue;
+            const long long row = std::max<long long>(120, 60 * ((strips + 127) / 128));
+            const long long cost = 2 * rpt * row + 60 * ((nedge + 127) / 128) +
+                                   120 * ((nedge + threads - 1) / threads);
+            if (best_cost < 0 || cost < best_cost ||
+                (cost == best_cost && W + H < (long long)best.W + best.H)) {
+                best_cost = cost;
+                best.W = (int)W;
+                best.H = (int)H;
+                best.rpt = rpt;
+                best.ntx = (int)ntx;
+                best.nty = (int)nty;
+                best.smem = smem;
+                best.threads = (int)threads;
+            }
         }
     }
-    if (best_area < 0) return false;
-    best.rpt = kRpts[sizeof(kRpts) / sizeof(kRpts[0]) - 1];
-    int best_load = -1;
-    for (int r : kRpts) {
-        const int ld = res2d_load(best.W, best.H, r, res_threads<T>());
-        if (ld >= 0 && (best_load < 0 || ld < best_load)) {
-            best_load = ld;
-            best.rpt = r;
-        }
-    }
+    if (best_cost < 0) return false;
     int occ = 0;
     cudaError_t oe = cudaSuccess;
-    with_kernel<T>(best.rpt, best.sw, [&](auto kern) {
-        oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, res_threads<T>(),
-                                                           best.smem);
+    with_kernel(best.rpt, [&](auto kern) {
+        oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, best.threads, best.smem);
     });
     if (oe != cudaSuccess || occ < 1 || (long long)best.ntx * best.nty > (long long)occ * nsm) {
         (void)cudaGetLastError();
         return false;
     }
-    best.xwords = (size_t)best.ntx * best.nty * 2 * (2 * (size_t)best.W + 2 * (size_t)best.H) *
-                  Xword<T>::kPer;
+    best.xwords = (size_t)best.ntx * best.nty * 2 * Res2dGeom::edges(best.W, best.H);
     *out = best;
     return true;
 }
 
-}  // namespace
-
-template <typename T>
-bool res2d_plan(const Layout &L, Res2dPlan *p)
-{
-    return plan_impl<T>(L, p);
-}
-
-template <typename T>
-void launch_res2d(const Res2dPlan &p, const T *kap, const T *dco, const T *fre, const T *fim,
-                  const Layout &L, const StepCoef<T> &C, const T *ab, int nsteps, int jim,
-                  int jfin, const OutSlot *slot, unsigned long long *xbuf, int *err,
-                  cudaStream_t s, const Res2dProj<T> &P)
+void launch_res2d(const Res2dPlan &p, const float *kap, const float *dco, const float *fre,
+                  const float *fim, const Layout &L, const StepCoef<float> &C, const float *ab,
+                  int nsteps, int jim, int jfin, const OutSlot *slot, unsigned long long *xbuf,
+                  int *err, cudaStream_t s, const Res2dProj<float> &P)
 {
     (void)cudaMemsetAsync(xbuf, 0, p.xwords * sizeof(unsigned long long), s);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)p.ntx, (unsigned)p.nty);
-    cfg.blockDim = dim3(res_threads<T>());
+    cfg.blockDim = dim3((unsigned)p.threads);
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -617,19 +575,12 @@ void launch_res2d(const Res2dPlan &p, const T *kap, const T *dco, const T *fre, 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const auto *abv = reinterpret_cast<const typename PairOf<T>::V *>(ab);
-    with_kernel<T>(p.rpt, p.sw, [&](auto kern) {
-        (void)cudaLaunchKernelEx(&cfg, kern, kap, dco, fre, fim, L, C, abv, nsteps, jim, jfin,
-                                 slot, xbuf, err, p.W, p.H, P);
+    with_kernel(p.rpt, [&](auto kern) {
+        (void)cudaLaunchKernelEx(&cfg, kern, kap, dco, fre, fim, L, C,
+                                 reinterpret_cast<const float2 *>(ab), nsteps, jim, jfin, slot,
+                                 xbuf, err, p.W, p.H, P);
     });
     ++g_launches;
 }
-
-template bool res2d_plan<float>(const Layout &, Res2dPlan *);
-template void launch_res2d<float>(const Res2dPlan &, const float *, const float *, const float *,
-                                  const float *, const Layout &, const StepCoef<float> &,
-                                  const float *, int, int, int, const OutSlot *,
-                                  unsigned long long *, int *, cudaStream_t,
-                                  const Res2dProj<float> &);
 
 }  // namespace htd

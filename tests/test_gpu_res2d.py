@@ -255,3 +255,26 @@ def test_resident_projection_matches_the_oracle(precision, periods):
                                                              else 1e-13)
     sr.close()
     s1.close()
+
+
+# tiles whose strips end inside a row block, one-node last tiles in x or y, tiles two
+# nodes wide, one tile in all, and one, two and many row pairs per thread
+EDGE_SHAPES = [(1, 2), (1, 9), (9, 1), (3, 3), (305, 3), (3, 305), (153, 153), (305, 307),
+               (421, 389), (613, 640), (1100, 1200)]
+
+
+@pytest.mark.parametrize("n", EDGE_SHAPES)
+@pytest.mark.parametrize("mode", ["table1", "project"])
+def test_resident_strips_equal_one_step_kernel(n, mode):
+    """Two steps per exchange, row pairs per thread: bit-identical to the one-step
+    kernel (Table 1); the projection sums of the same states agree to FP32 rounding
+    of the window's compensated sums (contraction may differ between kernels)."""
+    p = _problem(n, T=2)
+    U1, _ = precond(p, mode=mode, tblock=1)
+    Ur, prm = precond(p, mode=mode, tb_form=htd.TB_RESIDENT)
+    assert prm["step_kernel"] == 4
+    assert np.isfinite(Ur).all() and np.abs(Ur).max() > 0
+    if mode == "table1":
+        assert np.array_equal(Ur, U1)
+    else:
+        assert np.linalg.norm(Ur - U1) <= 1e-6 * np.linalg.norm(U1)
