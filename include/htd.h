@@ -507,7 +507,9 @@ void htd_test_fail_alloc(long long after);
 /* How a batch runs its preconditioner applications (filled after the first
  * application or solve; zeros before).  A batch with a group of 2-D handles
  * has two forms of a run that give the same bits: every handle's own step
- * sequence as a child graph (plain), or the group's persistent launch beside
+ * sequence as a child graph (plain; 2-D FP32 handles whose grids fit the SMs'
+ * shared memory together run as one resident-grid launch after the other
+ * sequences), or the group's persistent launch beside
  * the other handles' sequences (group).  The first two rounds of a solve run
  * one form each; the one with the smaller device time per point update is
  * kept for the batch from then on. */

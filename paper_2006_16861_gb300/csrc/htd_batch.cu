@@ -19,7 +19,10 @@
 //    its 3 x 3 neighbourhood has finished the previous one (htd_tblock.cu);
 //  - the other handles' captured step sequences (different sizes, kernels and
 //    step counts T n_P) are child graphs of one graph beside it, launched once
-//    per run.
+//    per run;
+//  - in the form without that persistent launch, the 2-D FP32 handles whose grids
+//    fit the SMs' shared memory together run as one resident-grid launch
+//    (htd_res2d.cu), each on its share of the SMs.
 //
 // The paper treats one system at a time (Sec. 5); the batch changes only the
 // schedule, not the arithmetic of any system.
@@ -107,6 +110,14 @@ struct htd_batch_s {
     size_t gdone_n = 0;
     unsigned long long *ghead = nullptr;
     float *gab = nullptr;
+    // the 2-D handles whose grids fit the SMs together: one resident-grid launch
+    // per run in the plain form
+    std::vector<char> in_res;            // per instance (empty: no such launch)
+    htd::Res2dInst *rinst = nullptr;
+    float *rab = nullptr;
+    unsigned long long *rx = nullptr;
+    size_t rx_words = 0, rsmem = 0;
+    int rn = 0, rctas = 0;
 };
 
 namespace {
@@ -116,7 +127,8 @@ void free_batch(htd_batch b)
     if (!b) return;
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->exec_plain) cudaGraphExecDestroy(b->exec_plain);
-    void *gp[] = {b->ginst, b->glev, b->goff, b->gdone, b->gabort, b->ghead, b->gab};
+    void *gp[] = {b->ginst, b->glev, b->goff, b->gdone, b->gabort, b->ghead, b->gab,
+                  b->rinst, b->rab, b->rx};
     for (void *q : gp)
         if (q) cudaFree(q);
     if (b->ws) cudaFree(b->ws);
@@ -224,6 +236,95 @@ htd_status build_group(htd_batch b)
     return HTD_OK;
 }
 
+// The resident launch of the plain form: every 2-D FP32 handle (each rhs slot an
+// instance of its own), if their grids fit the SMs' shared memory together and no
+// other handle of the batch is one whose launches leave most of the GPU idle -- the
+// resident launch holds every SM, so it runs after the others, not beside them.
+// Measured against the handles' own blocked sequences side by side: five handles of
+// 200^2 .. 640^2 2.04 ms per application (2.70), with a 64^3 handle of 8 rhs 2.94 (3.63).
+htd_status build_resident(htd_batch b)
+{
+    const int ninst = (int)b->ctx.size();
+    std::vector<char> in(ninst, 0);
+    std::vector<htd::CtxGroupView> views;
+    std::vector<htd::Layout> L;
+    std::vector<long long> steps;
+    size_t ab_n = 0;
+    for (int i = 0; i < ninst; ++i) {
+        htd::CtxGroupView v;
+        if (!htd::ctx_group_view(b->ctx[i], &v)) {
+            if (!htd::ctx_fills_device(b->ctx[i])) return HTD_OK;
+            continue;
+        }
+        in[i] = 1;
+        ab_n += v.ab.size();
+        views.push_back(v);
+        for (int k = 0; k < v.R.slots && L.size() <= 256; ++k) {
+            L.push_back(v.L);
+            steps.push_back(v.nsteps);
+        }
+    }
+    std::vector<htd::Res2dPlan> plans;
+    if (views.empty() || !htd::res2d_group_plan(L, steps, &plans)) return HTD_OK;
+    const int n = (int)L.size();
+    size_t xw = 0, smem = 0;
+    int ctas = 0;
+    for (const htd::Res2dPlan &p : plans) {
+        xw += p.xwords;
+        smem = std::max(smem, p.smem);
+        ctas += p.ntx * p.nty;
+    }
+    HTD_CUDA(htd::dev_malloc(&b->rab, sizeof(float) * ab_n));
+    HTD_CUDA(htd::dev_malloc(&b->rx, sizeof(unsigned long long) * xw));
+    HTD_CUDA(htd::dev_malloc(&b->rinst, sizeof(htd::Res2dInst) * n));
+    std::vector<htd::Res2dInst> inst;
+    std::vector<float> ab(ab_n);
+    size_t ab_at = 0, x_at = 0;
+    int cta = 0;
+    for (const htd::CtxGroupView &v : views) {
+        for (long long j = 0; j < v.nsteps; ++j) {
+            ab[ab_at + 2 * j] = v.ab[j];
+            ab[ab_at + 2 * j + 1] = v.ab[v.nsteps + j];
+        }
+        for (int k = 0; k < v.R.slots; ++k) {
+            const htd::Res2dPlan &p = plans[inst.size()];
+            htd::Res2dInst I;
+            I.kap = v.kap;
+            I.dco = v.dco;
+            I.fre = v.fre;
+            I.fim = v.fim;
+            I.L = v.L;
+            I.C = v.C;
+            I.ab = b->rab + ab_at;
+            I.nsteps = (int)v.nsteps;
+            I.jim = (int)v.jim;
+            I.jfin = (int)v.jfin;
+            I.slot = v.slot;
+            I.xbuf = b->rx + x_at;
+            I.err = v.err;
+            I.W = p.W;
+            I.H = p.H;
+            I.ntx = p.ntx;
+            I.rpt = p.rpt;
+            I.cta0 = cta;
+            I.R = v.R;
+            I.k = k;
+            inst.push_back(I);
+            x_at += p.xwords;
+            cta += p.ntx * p.nty;
+        }
+        ab_at += v.ab.size();
+    }
+    HTD_CUDA(cudaMemcpy(b->rab, ab.data(), sizeof(float) * ab_n, cudaMemcpyHostToDevice));
+    HTD_CUDA(cudaMemcpy(b->rinst, inst.data(), sizeof(htd::Res2dInst) * n, cudaMemcpyHostToDevice));
+    b->rn = n;
+    b->rctas = ctas;
+    b->rsmem = smem;
+    b->rx_words = xw;
+    b->in_res = in;
+    return HTD_OK;
+}
+
 // one run of the group: every member starts from rest, the queue and the
 // counters start at zero, then the persistent launch
 htd_status run_group(htd_batch b, cudaStream_t s)
@@ -241,19 +342,26 @@ htd_status run_group(htd_batch b, cudaStream_t s)
 }
 
 // Instantiate a graph whose children (no dependencies between them, so they
-// may run concurrently) are the given graphs.
-htd_status make_parent(const std::vector<cudaGraph_t> &kids, cudaGraphExec_t *out)
+// may run concurrently) are the given graphs, with `last` (if any) after all of
+// them.
+htd_status make_parent(const std::vector<cudaGraph_t> &kids, cudaGraph_t last, cudaGraphExec_t *out)
 {
     cudaGraph_t parent = nullptr;
     HTD_CUDA(cudaGraphCreate(&parent, 0));
     bool ok = true;
+    std::vector<cudaGraphNode_t> nodes;
     for (cudaGraph_t g : kids) {
         cudaGraphNode_t node;
         if (cudaGraphAddChildGraphNode(&node, parent, nullptr, 0, g) != cudaSuccess) {
             ok = false;
             break;
         }
+        nodes.push_back(node);
     }
+    cudaGraphNode_t end;
+    if (ok && last &&
+        cudaGraphAddChildGraphNode(&end, parent, nodes.data(), nodes.size(), last) != cudaSuccess)
+        ok = false;
     if (ok && cudaGraphInstantiate(out, parent, 0) != cudaSuccess) {
         *out = nullptr;
         ok = false;
@@ -263,42 +371,74 @@ htd_status make_parent(const std::vector<cudaGraph_t> &kids, cudaGraphExec_t *ou
     return HTD_OK;
 }
 
-// The batch graphs: every handle's captured step sequence as a child graph
-// (the plain form), and, when the batch has a group of 2-D handles, the group
-// launch beside the other handles' sequences.  Both give the same bits; the
-// first rounds of a solve time them and the faster one is kept.
+// what `run` enqueues on a stream as a graph, or null if the capture fails
+template <typename Run>
+cudaGraph_t capture(Run &&run)
+{
+    cudaGraph_t g = nullptr;
+    cudaStream_t cs;
+    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return nullptr;
+    }
+    if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        const long long before = htd::g_launches;
+        const htd_status st = run(cs);
+        const cudaError_t e = cudaStreamEndCapture(cs, &g);
+        htd::g_launches = before;        // captured, not launched
+        if (e != cudaSuccess || st != HTD_OK) {
+            if (g) cudaGraphDestroy(g);
+            g = nullptr;
+        }
+    }
+    cudaStreamDestroy(cs);
+    (void)cudaGetLastError();
+    return g;
+}
+
+// The batch graphs.  Plain form: every handle's captured step sequence as a child
+// graph, the 2-D handles that fit the SMs together as one resident launch after
+// the others (build_resident).  Group form, when the batch has a group of 2-D
+// handles: the group launch beside the other handles' sequences.  Both give the
+// same bits; the first rounds of a solve time them and the faster one is kept.
 htd_status build_graph(htd_batch b)
 {
     if (b->graph_tried) return HTD_OK;
     b->graph_tried = true;
     htd_status gst = build_group(b);
     if (gst != HTD_OK) return gst;
-    std::vector<cudaGraph_t> all, others;
+    if ((gst = build_resident(b)) != HTD_OK) return gst;
+    std::vector<cudaGraph_t> plain, others;
     for (size_t i = 0; i < b->ctx.size(); ++i) {
+        const bool res = !b->in_res.empty() && b->in_res[i];
+        // no graphs or no capture: run the handles one by one
+        if (!b->ci[i].graphs) return HTD_OK;
+        if (res && (b->in_group[i] || b->group.empty())) continue;   // no graph of its own
         cudaGraph_t g = htd::ctx_step_graph(b->ctx[i]);
-        if (!g) return HTD_OK;               // no capture: run the handles one by one
-        all.push_back(g);
+        if (!g) return HTD_OK;
+        if (!res) plain.push_back(g);
         if (!b->in_group[i]) others.push_back(g);
     }
-    if ((gst = make_parent(all, &b->exec_plain)) != HTD_OK) return gst;
+    cudaGraph_t rgraph = nullptr;
+    if (!b->in_res.empty()) {
+        rgraph = capture([&](cudaStream_t cs) -> htd_status {
+            htd::launch_res2d_group(b->rinst, b->rn, b->rctas, b->rsmem, b->rx, b->rx_words, cs);
+            HTD_CUDA(cudaGetLastError());
+            return HTD_OK;
+        });
+        if (!rgraph) return HTD_OK;
+    }
+    gst = make_parent(plain, rgraph, &b->exec_plain);
+    if (rgraph) cudaGraphDestroy(rgraph);    // the parent holds its own copy
+    if (gst != HTD_OK) return gst;
     if (!b->group.empty()) {
-        cudaGraph_t ggraph = nullptr;
-        cudaStream_t cs;
-        HTD_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-        if (ok) {
-            const long long before = htd::g_launches;
-            htd_status st = run_group(b, cs);
-            ok = cudaStreamEndCapture(cs, &ggraph) == cudaSuccess && st == HTD_OK;
-            htd::g_launches = before;        // captured, not launched
-        }
-        cudaStreamDestroy(cs);
-        (void)cudaGetLastError();
-        if (ok) {
+        cudaGraph_t ggraph = capture([&](cudaStream_t cs) { return run_group(b, cs); });
+        if (ggraph) {
             others.push_back(ggraph);
-            if ((gst = make_parent(others, &b->exec)) != HTD_OK) return gst;
+            gst = make_parent(others, nullptr, &b->exec);
+            cudaGraphDestroy(ggraph);
+            if (gst != HTD_OK) return gst;
         }
-        if (ggraph) cudaGraphDestroy(ggraph);  // the parent holds its own copy
     }
     if (!b->exec) b->form = 1;               // no group: the plain form only
     return HTD_OK;
@@ -370,9 +510,11 @@ htd_status precond_round(htd_batch b, const std::vector<char> &sel,
         if (ex) {
             HTD_CUDA(cudaGraphLaunch(ex, s));
             b->round_form = use;
-            for (int i = 0; i < ninst; ++i)
-                if (use == 1 || !b->in_group[i]) htd::g_launches += b->ci[i].nsteps;
-            if (use == 2) htd::g_launches += 1;
+            for (int i = 0; i < ninst; ++i) {
+                const bool own = use == 1 ? b->in_res.empty() || !b->in_res[i] : !b->in_group[i];
+                if (own) htd::g_launches += b->ci[i].nsteps;
+            }
+            if (use == 2 || !b->in_res.empty()) htd::g_launches += 1;
         } else {
             b->round_form = 0;
             for (int i = 0; i < ninst; ++i) {

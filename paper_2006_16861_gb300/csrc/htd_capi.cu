@@ -173,6 +173,7 @@ struct htd_ctx {
     bool use_s3 = false;
     int s3_zchunk = 0;
     int s3_shape = 0;
+    int s3_tx = 64;             // tile width of the pair kernel
     int s3_stages = 5;
     int s3_rpc = 1;             // right-hand sides per CTA of the streamed pair kernel
     // right-hand-side batch: rcap rhs slots in every per-rhs array (u0, u1, u2,
@@ -411,7 +412,7 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
                 if (j + 1 == jfin) flags |= 2;
                 T *um = (j & 1) ? A : B;                    // receives u_{j+1}
                 if (c->s3_shape == kS3Pair)
-                    htd::launch_stream3d_pair(c->s3maps, (int)(j & 1), L, um, C,
+                    htd::launch_stream3d_pair(c->s3maps, (int)(j & 1), c->s3_tx, L, um, C,
                                               (T)c->atab[j], (T)c->btab[j], c->slot, flags,
                                               c->s3_zchunk, c->s3_stages, c->err_dev, s, c->Rs,
                                               j > 0 && step_overlap(c), c->s3_rpc);
@@ -891,20 +892,30 @@ htd_status autotune_tb2d(htd_ctx *c, int want_B, int want_RPT)
 }
 
 // z-chunk length of the streamed 3-D step, chosen by timing: every chunk count k
-// whose chunk length ceil(nz / k) lies in [16, 128] (nz itself when nz < 16),
-// one step each on the context's own buffers with zero forcing and no outputs.
+// whose chunk length ceil(nz / k) lies in [16, 128], and shorter ones while the
+// launch has at most six CTAs per SM (two waves); none that gives fewer CTAs than
+// SMs while a shorter chunk is left.  A CTA marches through its planes one after
+// the other, so on a small grid the chunk sets the step's time (64^3: 9.4 us with 16
+// planes, 4.0 with 2).
+// One step each on the context's own buffers with zero forcing and no outputs.
 // How the CTAs of the last wave fill the GPU decides the best length, which no
 // simple rule predicts well (at 256^3: 37 planes beats 32 and 64 by 3-8 %).
 htd_status autotune_s3_zchunk(htd_ctx *c, const htd::RhsSet &R = htd::RhsSet{})
 {
     const Layout &L = c->Lr;
     std::vector<int> cands;
+    static const int txs[3] = {32, 64, 128};
+    const int tx = c->s3_shape == kS3Pair ? c->s3_tx : txs[c->s3_shape];
+    const int ty = c->s3_shape == kS3Pair ? 512 / tx : 256 / tx;
+    int nsm = 1;
+    HTD_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device));
+    const int64_t groups = (c->s3_rpc == 2) ? (R.slots + 1) / 2 : R.slots;
+    const int64_t tiles = ((L.nx + tx - 1) / tx) * ((L.ny + ty - 1) / ty) * groups;
     for (int64_t k = 1; k <= L.nz; ++k) {
         const int64_t zc = (L.nz + k - 1) / k;
-        if (zc > 128) continue;
-        if (zc < 16 && !cands.empty()) break;
+        if (zc > 128 || (tiles * k < nsm && zc > 1)) continue;
+        if (zc < 16 && !cands.empty() && tiles * k > 6 * (int64_t)nsm) break;
         if (cands.empty() || cands.back() != (int)zc) cands.push_back((int)zc);
-        if (zc < 16) break;
     }
     if (cands.size() < 2) {
         if (!cands.empty()) c->s3_zchunk = cands[0];
@@ -916,36 +927,60 @@ htd_status autotune_s3_zchunk(htd_ctx *c, const htd::RhsSet &R = htd::RhsSet{})
     HTD_CUDA(cudaEventCreate(&e0));
     HTD_CUDA(cudaEventCreate(&e1));
     const StepCoef<float> C = cast_coef<float>(c->C);
-    const int reps = 4;
     float best_us = INFINITY;
     int best = c->s3_zchunk;
-    // two passes over the candidates, each candidate's best kept: neighbouring
-    // chunk lengths differ by 1-2 %, about the spread of a single timing
-    for (int pass = 0; pass < 2; ++pass)
-    for (int zc : cands) {
-        for (int r = 0; r < 2 + reps; ++r) {
-            if (r == 2) HTD_CUDA(cudaEventRecord(e0, s));
+    auto enqueue = [&](int zc, int n) {      // n steps
+        for (int r = 0; r < n; ++r) {
+            float *um = (r & 1) ? (float *)c->u0 : (float *)c->u1;
             if (c->s3_shape == kS3Pair)
-                htd::launch_stream3d_pair(c->s3maps, r & 1, L, (r & 1) ? (float *)c->u0
-                                                                        : (float *)c->u1,
-                                          C, 0.f, 0.f, c->slot, 0, zc, c->s3_stages, c->err_dev, s,
-                                          R, r > 0 && step_overlap(c), c->s3_rpc);
+                htd::launch_stream3d_pair(c->s3maps, r & 1, c->s3_tx, L, um, C, 0.f, 0.f, c->slot,
+                                          0, zc, c->s3_stages, c->err_dev, s, R,
+                                          r > 0 && step_overlap(c), c->s3_rpc);
             else
-                htd::launch_stream3d(c->s3maps, r & 1, c->s3_shape, L,
-                                     (r & 1) ? (float *)c->u0 : (float *)c->u1, C, 0.f, 0.f,
-                                     c->slot, 0, zc, c->err_dev, s);
+                htd::launch_stream3d(c->s3maps, r & 1, c->s3_shape, L, um, C, 0.f, 0.f, c->slot, 0,
+                                     zc, c->err_dev, s);
         }
-        HTD_CUDA(cudaEventRecord(e1, s));
-        HTD_CUDA(cudaEventSynchronize(e1));
-        HTD_CUDA(cudaGetLastError());
-        float ms = 0.f;
-        HTD_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-        const float us = 1e3f * ms / reps;
-        if (us < best_us) {
-            best_us = us;
-            best = zc;
+    };
+    // two passes over the candidates, each candidate's best kept: neighbouring
+    // chunk lengths differ by 1-2 %, about the spread of a single timing.  Short
+    // steps would be timed at the host's launch rate, so on small grids each
+    // candidate's steps replay from a graph, as a run's do.
+    const bool small = L.N * R.slots <= (1 << 20);
+    const int reps = small ? 16 : 4;
+    std::vector<cudaGraphExec_t> ex(cands.size(), nullptr);
+    for (size_t k = 0; small && k < cands.size(); ++k) {
+        cudaGraph_t g = nullptr;
+        if (cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+            enqueue(cands[k], reps);
+            if (cudaStreamEndCapture(s, &g) == cudaSuccess &&
+                cudaGraphInstantiate(&ex[k], g, 0) != cudaSuccess)
+                ex[k] = nullptr;
+            if (g) cudaGraphDestroy(g);
         }
+        (void)cudaGetLastError();
     }
+    cudaError_t te = cudaSuccess;
+    for (int pass = 0; pass < 2; ++pass)
+        for (size_t k = 0; k < cands.size(); ++k) {
+            for (int r = 0; r < 2 && te == cudaSuccess; ++r) {
+                if (r == 1) te = cudaEventRecord(e0, s);
+                if (ex[k]) te = cudaGraphLaunch(ex[k], s);
+                else enqueue(cands[k], reps);
+            }
+            float ms = 0.f;
+            if (te == cudaSuccess) te = cudaEventRecord(e1, s);
+            if (te == cudaSuccess) te = cudaEventSynchronize(e1);
+            if (te == cudaSuccess) te = cudaGetLastError();
+            if (te == cudaSuccess) te = cudaEventElapsedTime(&ms, e0, e1);
+            const float us = 1e3f * ms / reps;
+            if (te == cudaSuccess && us < best_us) {
+                best_us = us;
+                best = cands[k];
+            }
+        }
+    for (cudaGraphExec_t x : ex)
+        if (x) cudaGraphExecDestroy(x);
+    HTD_CUDA(te);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaStreamDestroy(s);
@@ -1428,7 +1463,8 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
             c->s3_shape = (opt.s3_kernel == HTD_S3_PAIR) ? kS3Default : opt.s3_kernel - HTD_S3_NODE_32x8;
             if (c->s3_shape != kS3Pair && c->rcap > 1) c->s3_shape = kS3Pair;   // rhs batches
             if (c->s3_shape == kS3Pair) {
-                c->use_s3 = htd::make_stream3d_pair_maps(L, planes, &c->s3maps, c->rcap);
+                c->s3_tx = htd::stream3d_pair_tx(L);
+                c->use_s3 = htd::make_stream3d_pair_maps(L, c->s3_tx, planes, &c->s3maps, c->rcap);
                 if (!c->use_s3) {                                  // odd layout: one node per thread
                     (void)cudaGetLastError();
                     c->s3_shape = 0;
@@ -1439,7 +1475,7 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
             if (c->use_s3) {
                 c->s3_stages = (opt.s3_stages == 0) ? 5 : opt.s3_stages;
                 c->s3_rpc = 1;
-                c->s3_zchunk = c->s3_shape == kS3Pair ? htd::stream3d_pair_zchunk(L, c->s3_stages)
+                c->s3_zchunk = c->s3_shape == kS3Pair ? htd::stream3d_pair_zchunk(L, c->s3_tx, c->s3_stages)
                                                       : htd::stream3d_zchunk(L, c->s3_shape);
                 // right-hand sides per CTA (pair kernel, handles with several rhs):
                 // 2 when asked, or the faster of 1 and 2 timed with every rhs slot
@@ -1467,7 +1503,7 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
                     const float us1 = c->step_us;
                     c->s3_rpc = 2;
                     c->s3_stages = 4;
-                    c->s3_zchunk = htd::stream3d_pair_zchunk(L, 4, 2);
+                    c->s3_zchunk = htd::stream3d_pair_zchunk(L, c->s3_tx, 4, 2);
                     if ((ts = autotune_s3_zchunk(c, all)) != HTD_OK) return ts;
                     if (!(c->step_us < us1)) {
                         c->s3_rpc = 1;
@@ -1479,7 +1515,7 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
                     if (want_rpc == 2) {
                         c->s3_rpc = 2;
                         c->s3_stages = 4;
-                        c->s3_zchunk = htd::stream3d_pair_zchunk(L, 4, 2);
+                        c->s3_zchunk = htd::stream3d_pair_zchunk(L, c->s3_tx, 4, 2);
                     }
                     htd_status ts = autotune_s3_zchunk(c, all);
                     if (ts != HTD_OK) return ts;
@@ -1534,6 +1570,7 @@ void ctx_info(const htd_ctx *c, CtxInfo *out)
     out->krylov = c->opt.krylov;
     out->device = c->device;
     out->nsteps = c->nsteps;
+    out->graphs = !graphs_disabled(c);
 }
 
 htd_status ctx_stage_run(htd_ctx *c, int run, int n, const int *idx, const double2 *const *Fp,
@@ -1629,6 +1666,21 @@ bool ctx_group_view(htd_ctx *c, CtxGroupView *out)
     out->err = c->err_dev;
     out->rcap = c->rcap;
     return true;
+}
+
+bool ctx_fills_device(const htd_ctx *c)
+{
+    htd_params p;
+    int nsm = 0;
+    if (!c->use_s3 || htd_get_params(const_cast<htd_ctx *>(c), &p) != HTD_OK ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    const Layout &L = c->Lr;
+    const int64_t ctas = ((L.nx + p.tile[0] - 1) / p.tile[0]) * ((L.ny + p.tile[1] - 1) / p.tile[1]) *
+                         ((L.nz + p.tile[2] - 1) / p.tile[2]) * ((c->rcap + c->s3_rpc - 1) / c->s3_rpc);
+    return ctas >= nsm;
 }
 
 htd_status ctx_zero_states(htd_ctx *c, cudaStream_t s)
@@ -1789,14 +1841,15 @@ htd_status htd_get_params(htd_handle h, htd_params *out)
         static const int tx[4] = {32, 64, 128, 64}, ty[4] = {8, 4, 2, 8};
         const int sh = (h->s3_shape >= 0 && h->s3_shape < 4) ? h->s3_shape : 0;
         const Layout &L = h->Lr;
-        P.tile[0] = tx[sh];
-        P.tile[1] = ty[sh];
+        P.tile[0] = sh == kS3Pair ? h->s3_tx : tx[sh];
+        P.tile[1] = sh == kS3Pair ? 512 / h->s3_tx : ty[sh];
         P.tile[2] = h->s3_zchunk;
         P.ctas_per_sm = (sh == kS3Pair && h->s3_stages <= 5 && h->s3_rpc == 1) ? 3 : 2;
         int dev = 0, nsm = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        const int64_t ctas = ((L.nx + tx[sh] - 1) / tx[sh]) * ((L.ny + ty[sh] - 1) / ty[sh]) *
+        const int64_t ctas = ((L.nx + P.tile[0] - 1) / P.tile[0]) *
+                             ((L.ny + P.tile[1] - 1) / P.tile[1]) *
                              ((L.nz + h->s3_zchunk - 1) / h->s3_zchunk);
         const int64_t slots = (int64_t)P.ctas_per_sm * nsm;
         P.waves = (int)((ctas + slots - 1) / slots);

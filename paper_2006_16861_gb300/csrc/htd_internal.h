@@ -291,6 +291,7 @@ struct CtxInfo {
     int krylov;         // HTD_FGMRES or HTD_LEFT_GMRES
     int device;
     long long nsteps;   // recurrence steps per run
+    bool graphs;        // the handle's steps may run from a graph
 };
 void ctx_info(const htd_ctx *c, CtxInfo *out);
 // stage run `run` of one application for the rhs idx[0..n) (n = 0: the
@@ -334,6 +335,9 @@ struct CtxGroupView {
     int rcap;
 };
 bool ctx_group_view(htd_ctx *c, CtxGroupView *out);
+// whether the handle's step launches fill the device (the streamed 3-D step with
+// at least one CTA per SM)
+bool ctx_fills_device(const htd_ctx *c);
 // zero the first state pair of every rhs slot (a run starts from rest)
 htd_status ctx_zero_states(htd_ctx *c, cudaStream_t s);
 
@@ -422,6 +426,32 @@ struct Res2dProj {
     T *acc = nullptr;
     int64_t N = 0;
 };
+
+// A run of the resident kernel: the operands of launch_res2d and the tiling.  A
+// group launch runs slot k of the handle's active list (R) on the CTAs from cta0.
+struct Res2dInst {
+    const float *kap = nullptr, *dco = nullptr, *fre = nullptr, *fim = nullptr;
+    Layout L;
+    StepCoef<float> C;
+    const float *ab = nullptr;
+    int nsteps = 0, jim = 0, jfin = 0;
+    const OutSlot *slot = nullptr;
+    unsigned long long *xbuf = nullptr;
+    int *err = nullptr;
+    int W = 0, H = 0, ntx = 0, rpt = 0;
+    int cta0 = 0;
+    RhsSet R;
+    int k = 0;
+};
+
+// Plans for several instances run by one launch (each on its share of the SMs), or
+// false if they do not fit the device together.
+bool res2d_group_plan(const std::vector<Layout> &L, const std::vector<long long> &nsteps,
+                      std::vector<Res2dPlan> *plans);
+// inst: device array of n instances, cta0 ascending; xbuf: the exchange buffers of
+// all of them (xwords words).  Threads and shared memory are the largest plan's.
+void launch_res2d_group(const Res2dInst *inst, int n, int ctas, size_t smem,
+                        unsigned long long *xbuf, size_t xwords, cudaStream_t s);
 
 // The plan for a 2-D grid, or false if the grid does not fit the SMs at one
 // tile per SM, or the device cannot launch cooperatively.
@@ -535,15 +565,16 @@ void launch_stream3d(const Stream3Maps &maps, int from, int shape, const Layout 
                      int zchunk, int *err, cudaStream_t s);
 
 // Same step with two x-adjacent nodes per thread in paired FP32 instructions
-// (htd_stream3d_pair.cu): 64 x 8 column tiles, same maps layout (halo boxes
-// 72 x 10).  Needs an even x lead and pitch.  The per-rhs planes (u0, u1,
+// (htd_stream3d_pair.cu): 64 x 8 or 32 x 16 column tiles (tx = 64 or 32; the width
+// for a grid: stream3d_pair_tx), same maps layout (halo boxes of 720 nodes).  Needs an even x lead and pitch.  The per-rhs planes (u0, u1,
 // Re F, Im F) are nrhs stacks L.total elements apart (4-D maps, rhs
 // outermost); q*kappa and d are shared.
-bool make_stream3d_pair_maps(const Layout &L, float *const planes[6], Stream3Maps *maps,
+int stream3d_pair_tx(const Layout &L);
+bool make_stream3d_pair_maps(const Layout &L, int tx, float *const planes[6], Stream3Maps *maps,
                              int nrhs = 1);
 // first z chunk to try for a ring of `stages` stages and `rpc` right-hand sides
 // per CTA (3 CTAs per SM for rpc 1 with 4-5 stages, else 2)
-int stream3d_pair_zchunk(const Layout &L, int stages, int rpc = 1);
+int stream3d_pair_zchunk(const Layout &L, int tx, int stages, int rpc = 1);
 size_t stream3d_pair_smem_bytes(int stages, int rpc = 1);
 // overlap: the launch may start while the previous kernel of the stream drains
 // (its prologue loads q*kappa, d and the forcing, which no step writes; the
@@ -551,7 +582,7 @@ size_t stream3d_pair_smem_bytes(int stages, int rpc = 1);
 // sides per CTA, 1 (any stages) or 2 (4 stages): a CTA then streams one column
 // tile for two rhs slots, loading q*kappa and d once and computing each
 // stencil coefficient once for both.
-void launch_stream3d_pair(const Stream3Maps &maps, int from, const Layout &L, float *um,
+void launch_stream3d_pair(const Stream3Maps &maps, int from, int tx, const Layout &L, float *um,
                           const StepCoef<float> &C, float a, float b, const OutSlot *slot,
                           int flags, int zchunk, int stages, int *err, cudaStream_t s,
                           const RhsSet &R = RhsSet{}, bool overlap = false, int rpc = 1);

@@ -50,6 +50,7 @@
 
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "htd_internal.h"
 
@@ -127,20 +128,28 @@ __device__ __forceinline__ int edge_rank(int lx, int ly, int w, int h)
     return -1;
 }
 
-template <int RPT>
-__global__ void __launch_bounds__(kThreads, 1)
-res2d_kernel(const float *__restrict__ kap, const float *__restrict__ dco,
-             const float *__restrict__ fre, const float *__restrict__ fim, Layout L,
-             StepCoef<float> C, const float2 *__restrict__ ab, int nsteps, int jim, int jfin,
-             const OutSlot *__restrict__ slot, unsigned long long *__restrict__ xbuf,
-             int *__restrict__ err, int W, int H, Res2dProj<float> P)
+// One run of the instance I, as the CTA of its tile (tx, ty).  kGroup: for slot I.k of
+// the handle's active list, else for its only rhs.
+template <int RPT, bool kGroup>
+__device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, const Res2dProj<float> &P)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ int s_abort;
+    const Layout &L = I.L;
+    const StepCoef<float> &C = I.C;
+    const int W = I.W, H = I.H, ntx = I.ntx;
+    const int nsteps = I.nsteps, jim = I.jim, jfin = I.jfin;
+    int rhs = 0;
+    if (kGroup && !rhs_of_slot(I.R, I.k, rhs)) return;   // an idle slot: all its tiles return
+    const float *__restrict__ kap = I.kap, *__restrict__ dco = I.dco;
+    const float *__restrict__ fre = I.fre + (kGroup ? rhs * I.R.stride : 0);
+    const float *__restrict__ fim = I.fim + (kGroup ? rhs * I.R.stride : 0);
+    const float2 *__restrict__ ab = reinterpret_cast<const float2 *>(I.ab);
+    const OutSlot *__restrict__ slot = I.slot + (kGroup ? rhs : 0);
+    unsigned long long *__restrict__ xbuf = I.xbuf;
+    int *__restrict__ err = I.err;
     const Res2dGeom G(W, H, RPT);
     const int tid = threadIdx.x, NT = blockDim.x;
-    const int tx = blockIdx.x, ty = blockIdx.y;
-    const int ntx = gridDim.x;
     const int x0 = tx * W, y0 = ty * H;
     const int nx = (int)L.nx, ny = (int)L.ny;
     const int w = min(W, nx - x0), h = min(H, ny - y0);
@@ -443,6 +452,44 @@ res2d_kernel(const float *__restrict__ kap, const float *__restrict__ dco,
     }
 }
 
+template <int RPT>
+__global__ void __launch_bounds__(kThreads, 1)
+res2d_kernel(const __grid_constant__ Res2dInst I, const __grid_constant__ Res2dProj<float> P)
+{
+    res2d_run<RPT, false>(I, blockIdx.x, blockIdx.y, P);
+}
+
+// Several instances in one launch, instance i on the CTAs from inst[i].cta0 up to
+// the next one's: every instance's tiles resident at once, each with the plan made
+// for its share of the SMs.
+__global__ void __launch_bounds__(kThreads, 1)
+res2d_group_kernel(const Res2dInst *__restrict__ inst, int n)
+{
+    __shared__ __align__(16) unsigned char raw[sizeof(Res2dInst)];
+    int i = 0;
+    while (i + 1 < n && inst[i + 1].cta0 <= (int)blockIdx.x) ++i;
+    static_assert(sizeof(Res2dInst) % 4 == 0, "copied by words");
+    for (int k = threadIdx.x; k < (int)sizeof(Res2dInst) / 4; k += blockDim.x)
+        reinterpret_cast<int *>(raw)[k] = reinterpret_cast<const int *>(inst + i)[k];
+    __syncthreads();
+    const Res2dInst &I = *reinterpret_cast<const Res2dInst *>(raw);
+    const int t = (int)blockIdx.x - I.cta0;
+    const int tx = t % I.ntx, ty = t / I.ntx;
+    const Res2dProj<float> P;
+    switch (I.rpt) {
+    case 1: res2d_run<1, true>(I, tx, ty, P); break;
+    case 2: res2d_run<2, true>(I, tx, ty, P); break;
+    case 3: res2d_run<3, true>(I, tx, ty, P); break;
+    case 4: res2d_run<4, true>(I, tx, ty, P); break;
+    case 5: res2d_run<5, true>(I, tx, ty, P); break;
+    case 6: res2d_run<6, true>(I, tx, ty, P); break;
+    case 7: res2d_run<7, true>(I, tx, ty, P); break;
+    case 8: res2d_run<8, true>(I, tx, ty, P); break;
+    case 9: res2d_run<9, true>(I, tx, ty, P); break;
+    default: res2d_run<10, true>(I, tx, ty, P); break;
+    }
+}
+
 template <typename Fn>
 void with_kernel(int rpt, Fn &&fn)
 {
@@ -467,53 +514,55 @@ size_t res2d_smem(int W, int H, int rpt)
            ((size_t)G.NB * rpt * G.NC + 2 * (size_t)Res2dGeom::edges(W, H)) * sizeof(float4);
 }
 
-}  // namespace
-
-bool res2d_plan(const Layout &L, Res2dPlan *out)
+// Device limits for the kernels: SMs, and the dynamic shared memory every one of
+// them may use.  The limit is a property of a kernel, shared by every handle: it is
+// raised to what the device allows beside the kernel's static shared memory.
+bool res2d_device(int *nsm, int *avail)
 {
-    if (L.d != 2 || L.nx < 1 || L.ny < 1) return false;
-    int dev = 0, nsm = 0, coop = 0, maxsm = 0;
+    int dev = 0, coop = 0, maxsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
         (void)cudaGetLastError();
         return false;
     }
-    if (!coop || nsm < 1) return false;
-    // the limit is a property of the kernel, shared by every handle: raise it
-    // to what the device allows beside the kernel's static shared memory,
-    // rather than to this plan's size
-    int avail = maxsm;
-    bool attr_ok = true;
-    for (int r = 1; r <= kMaxRows; ++r)
-        with_kernel(r, [&](auto kern) {
-            cudaFuncAttributes fa;
-            if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
-                attr_ok = false;
-                return;
-            }
-            const int dyn = maxsm - (int)fa.sharedSizeBytes;
-            avail = std::min(avail, dyn);
-            attr_ok = attr_ok && dyn > 0 &&
-                      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           dyn) == cudaSuccess;
-        });
-    if (!attr_ok) {
-        (void)cudaGetLastError();
-        return false;
-    }
-    // Tiles of W x H nodes (inner tiles at least 2 x 2: the ring reaches one tile
-    // only) with RPT row pairs per thread, at most one tile per SM.  Cost of two
-    // steps in cycles of an SM's quarter: a row pair takes about 60 issue cycles
-    // per warp, 120 when no other warp fills its latency; the edge pass about 60
-    // per warp and pass.
+    if (!coop || *nsm < 1) return false;
+    *avail = maxsm;
+    bool ok = true;
+    auto limit = [&](auto kern) {
+        cudaFuncAttributes fa;
+        if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) {
+            ok = false;
+            return;
+        }
+        const int dyn = maxsm - (int)fa.sharedSizeBytes;
+        *avail = std::min(*avail, dyn);
+        ok = ok && dyn > 0 &&
+             cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) ==
+                 cudaSuccess;
+    };
+    for (int r = 1; r <= kMaxRows; ++r) with_kernel(r, limit);
+    limit(res2d_group_kernel);
+    if (!ok) (void)cudaGetLastError();
+    return ok;
+}
+
+// The best plan of a grid on `ctas` CTAs and its cost, -1 if it does not fit.
+// Tiles of W x H nodes (inner tiles at least 2 x 2: the ring reaches one tile
+// only) with RPT row pairs per thread.  Cost of two steps in cycles of an SM's
+// quarter: a row pair takes about 60 issue cycles per warp, 120 when no other warp
+// fills its latency; the edge pass about 60 per warp and pass.  Against the
+// measured times of the 14 cheapest plans at nine sizes from 101^2 to 1101^2 the
+// chosen one was within 5 % of the best.
+long long res2d_best(const Layout &L, int ctas, int avail, Res2dPlan *out)
+{
     Res2dPlan best;
     long long best_cost = -1;
-    for (int a = 1; a <= nsm && (a == 1 || 2 * (a - 1) < L.nx); ++a) {
+    for (int a = 1; a <= ctas && (a == 1 || 2 * (a - 1) < L.nx); ++a) {
         const long long W = std::max<long long>(2, (L.nx + a - 1) / a);
         const long long ntx = (L.nx + W - 1) / W;
-        const long long tiles_y = nsm / ntx;
+        const long long tiles_y = ctas / ntx;
         if (tiles_y < 1) break;
         const long long H = std::max<long long>(2, (L.ny + tiles_y - 1) / tiles_y);
         const long long nty = (L.ny + H - 1) / H;
@@ -544,7 +593,24 @@ bool res2d_plan(const Layout &L, Res2dPlan *out)
             }
         }
     }
-    if (best_cost < 0) return false;
+    if (best_cost >= 0) {
+        best.xwords = (size_t)best.ntx * best.nty * 2 * Res2dGeom::edges(best.W, best.H);
+        *out = best;
+    }
+    return best_cost;
+}
+
+// cost of the exchange that no work hides, per two steps (about 0.7 us)
+constexpr long long kExchangeCost = 1400;
+
+}  // namespace
+
+bool res2d_plan(const Layout &L, Res2dPlan *out)
+{
+    if (L.d != 2 || L.nx < 1 || L.ny < 1) return false;
+    int nsm = 0, avail = 0;
+    Res2dPlan best;
+    if (!res2d_device(&nsm, &avail) || res2d_best(L, nsm, avail, &best) < 0) return false;
     int occ = 0;
     cudaError_t oe = cudaSuccess;
     with_kernel(best.rpt, [&](auto kern) {
@@ -554,10 +620,107 @@ bool res2d_plan(const Layout &L, Res2dPlan *out)
         (void)cudaGetLastError();
         return false;
     }
-    best.xwords = (size_t)best.ntx * best.nty * 2 * Res2dGeom::edges(best.W, best.H);
     *out = best;
     return true;
 }
+
+// Shares of the SMs for several instances (layout, steps per run) in one launch, so
+// that the slowest one ends as early as possible: in proportion to their work
+// first, then SM by SM from the fastest instance to the slowest.
+bool res2d_group_plan(const std::vector<Layout> &L, const std::vector<long long> &nsteps,
+                      std::vector<Res2dPlan> *plans)
+{
+    const int n = (int)L.size();
+    int nsm = 0, avail = 0;
+    if (n < 1 || !res2d_device(&nsm, &avail) || n > nsm) return false;
+    std::vector<Res2dPlan> p(n), q(1);
+    std::vector<int> c(n), least(n);
+    std::vector<double> t(n);
+    double work = 0.0;
+    int sum = 0;
+    auto time = [&](int i, int ctas, Res2dPlan *out) -> double {
+        const long long cost = res2d_best(L[i], ctas, avail, out);
+        return cost < 0 ? -1.0 : (double)nsteps[i] * (double)(cost + kExchangeCost);
+    };
+    for (int i = 0; i < n; ++i) {
+        if (L[i].d != 2 || nsteps[i] >= (1LL << 30)) return false;
+        work += (double)L[i].N * (double)nsteps[i];
+        // 10 row pairs of 512 threads hold 10240 nodes with the ring
+        least[i] = (int)std::max<int64_t>(1, L[i].N / 10000);
+        while (least[i] <= nsm && time(i, least[i], &p[i]) < 0.0) ++least[i];
+        if ((sum += least[i]) > nsm) return false;
+    }
+    sum = 0;
+    for (int i = 0; i < n; ++i) {
+        c[i] = std::max(least[i], (int)(nsm * ((double)L[i].N * (double)nsteps[i] / work)));
+        sum += c[i];
+    }
+    for (int i = 0; i < n; ++i) t[i] = time(i, c[i], &p[i]);
+    auto pick = [&](bool slowest, bool spare) {
+        int b = -1;
+        for (int i = 0; i < n; ++i)
+            if ((!spare || c[i] > least[i]) && (b < 0 || (slowest ? t[i] > t[b] : t[i] < t[b])))
+                b = i;
+        return b;
+    };
+    while (sum > nsm) {
+        const int f = pick(false, true);
+        if (f < 0) return false;
+        t[f] = time(f, --c[f], &p[f]);
+        --sum;
+    }
+    for (int it = 0; it < 64; ++it) {
+        const int b = pick(true, false);
+        if (sum == nsm) {
+            const int f = pick(false, true);
+            if (f < 0 || f == b) break;
+            const double tf = time(f, c[f] - 1, &q[0]);
+            if (tf < 0.0 || tf >= t[b]) break;
+            --c[f];
+            t[f] = tf;
+            p[f] = q[0];
+            --sum;
+        }
+        t[b] = time(b, ++c[b], &p[b]);
+        ++sum;
+    }
+    size_t smem = 0;
+    int used = 0, occ = 0;
+    for (int i = 0; i < n; ++i) {
+        smem = std::max(smem, p[i].smem);
+        used += p[i].ntx * p[i].nty;
+    }
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, res2d_group_kernel, kThreads, smem) !=
+            cudaSuccess ||
+        occ < 1 || used > occ * nsm) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    *plans = p;
+    return true;
+}
+
+namespace {
+
+template <typename Kern, typename... Args>
+void launch_cooperative(Kern kern, dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                        Args &&...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
+    ++g_launches;
+}
+
+}  // namespace
 
 void launch_res2d(const Res2dPlan &p, const float *kap, const float *dco, const float *fre,
                   const float *fim, const Layout &L, const StepCoef<float> &C, const float *ab,
@@ -565,22 +728,35 @@ void launch_res2d(const Res2dPlan &p, const float *kap, const float *dco, const 
                   int *err, cudaStream_t s, const Res2dProj<float> &P)
 {
     (void)cudaMemsetAsync(xbuf, 0, p.xwords * sizeof(unsigned long long), s);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)p.ntx, (unsigned)p.nty);
-    cfg.blockDim = dim3((unsigned)p.threads);
-    cfg.dynamicSmemBytes = p.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    Res2dInst I;
+    I.kap = kap;
+    I.dco = dco;
+    I.fre = fre;
+    I.fim = fim;
+    I.L = L;
+    I.C = C;
+    I.ab = ab;
+    I.nsteps = nsteps;
+    I.jim = jim;
+    I.jfin = jfin;
+    I.slot = slot;
+    I.xbuf = xbuf;
+    I.err = err;
+    I.W = p.W;
+    I.H = p.H;
+    I.ntx = p.ntx;
+    I.rpt = p.rpt;
     with_kernel(p.rpt, [&](auto kern) {
-        (void)cudaLaunchKernelEx(&cfg, kern, kap, dco, fre, fim, L, C,
-                                 reinterpret_cast<const float2 *>(ab), nsteps, jim, jfin, slot,
-                                 xbuf, err, p.W, p.H, P);
+        launch_cooperative(kern, dim3((unsigned)p.ntx, (unsigned)p.nty), (unsigned)p.threads,
+                           p.smem, s, I, P);
     });
-    ++g_launches;
+}
+
+void launch_res2d_group(const Res2dInst *inst, int n, int ctas, size_t smem,
+                        unsigned long long *xbuf, size_t xwords, cudaStream_t s)
+{
+    (void)cudaMemsetAsync(xbuf, 0, xwords * sizeof(unsigned long long), s);
+    launch_cooperative(res2d_group_kernel, dim3((unsigned)ctas), kThreads, smem, s, inst, n);
 }
 
 }  // namespace htd

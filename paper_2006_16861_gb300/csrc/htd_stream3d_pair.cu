@@ -1,23 +1,31 @@
-// 3-D recurrence step streamed by TMA, two x-adjacent nodes per thread (FP32).
+// 3-D recurrence step streamed by TMA, 2 x 2 nodes per thread (FP32).
 //
 // Same method and pipeline as stream3d_kernel (one step of I_acd with Table 1's
 // windowed forcing; a producer warp streams z planes of a column tile through
-// a ring of shared-memory stages with full/empty mbarriers; consumer warps keep
-// register windows over three planes), but each consumer thread updates the
-// pair of nodes (x, x+1), x = x0 + 2 tx, so that the 27-term stencil sum, the
-// cell sums of q*kappa and the update run on float2 pairs with the paired FP32
-// instructions of sm_100+ (__ffma2_rn, __fadd2_rn, __fmul2_rn): about half the
-// FP instructions and half the per-node bookkeeping of the one-node kernel.
+// a ring of shared-memory stages with full/empty mbarriers), but each of the 128
+// consumer threads updates the node pairs (x, x+1) of two rows, x = x0 + 2 tx, so
+// that the 27-term stencil sum, the cell sums of q*kappa and the update run on
+// float2 pairs with the paired FP32 instructions of sm_100+ (__ffma2_rn,
+// __fadd2_rn, __fmul2_rn), and the two rows share their u_j rows, their middle
+// cell row and every coefficient between them: 45 coefficients, 54 stencil
+// products and 12 u_j loads per two pairs, where one row per thread took 54, 54 and
+// 18.  The loop over planes is unrolled by two, so that the cell sums of the
+// previous plane stay in their registers.
 //
-// Tile: 64 x 8 columns (256 consumer threads).  Stage = u_j box and q*kappa box
-// (72 x 10: columns x0-1 .. x0+64 with the 16-byte aligned start, rows
-// y0-1 .. y0+8) and exact 64 x 8 boxes of d, Re F, Im F, u_{j-1}.  In the halo
-// boxes node column x sits at box column x - x0 + 1 + off with off = 3 (the
-// padded layout puts column x0 - 1 at 3 mod 4), so (x, x+1) for even x - x0
-// is an aligned 64-bit pair and x - 1, x + 2 are single loads.  The two halo
-// planes of a z chunk (below and above its node planes) load only u_j, plus
-// q*kappa for the lower one: their node boxes would never be read, and as the
-// neighbouring chunk runs in another wave they would come from DRAM.
+// What bounds it: HBM on grids beyond L2 (256^3: 78.1 us per step, 6.02 TB/s
+// algorithmic, 0.886 of the measured copy bandwidth; 80.8 with one row per thread),
+// issue and the ramp of a launch below (106 x 200 x 200: 161 instructions per pair
+// and plane, 213 before; 25.2 us per step on the same tiles, 28.0 before).
+//
+// Tile: 64 x 8 or 32 x 16 columns.  Stage = u_j box and q*kappa box (for 64 x 8: 72 x
+// 10, columns x0-1 .. x0+64 with the 16-byte aligned start, rows y0-1 .. y0+8) and
+// exact boxes of d, Re F, Im F, u_{j-1}.  In the halo boxes node column x sits at
+// box column x - x0 + 1 + off with off = 3 (the padded layout puts column x0 - 1 at
+// 3 mod 4), so (x, x+1) for even x - x0 is an aligned 64-bit pair and x - 1, x + 2
+// are single loads.  The two halo planes of a z chunk (below and above its node
+// planes) load only u_j, plus q*kappa for the lower one: their node boxes would
+// never be read, and as the neighbouring chunk runs in another wave they would
+// come from DRAM.
 //
 // Per node the arithmetic is the one-node kernel's, in the same order, with
 // each scalar operation replaced by the same operation on a pair; paired
@@ -33,12 +41,15 @@ namespace htd {
 
 namespace {
 
-constexpr int kTX = 64, kTY = 8;
-constexpr int kThreads = 256;                   // consumer threads, 2 nodes each
-constexpr int kHaloW = 72, kHaloH = kTY + 2;
-constexpr int kHaloElems = kHaloW * kHaloH;     // 720 floats copied
+// Column tiles of 512 nodes: 64 x 8 or 32 x 16, whose halo boxes have the same size
+constexpr int tile_y(int tx) { return 512 / tx; }
+constexpr int kThreads = 128;                   // consumer threads, 2 x 2 nodes each
+constexpr int halo_w(int tx) { return tx + 8; }
+constexpr int halo_h(int tx) { return tile_y(tx) + 2; }
+constexpr int kHaloElems = 720;                 // floats copied
+static_assert(halo_w(64) * halo_h(64) == kHaloElems && halo_w(32) * halo_h(32) == kHaloElems, "");
 constexpr int kHaloStride = 768;                // padded to 3072 bytes (128-byte multiple)
-constexpr int kNodeElems = kTX * kTY;           // 512 floats
+constexpr int kNodeElems = 512;
 // Stage layout for RPC right-hand sides per CTA: the u_j halo box of each rhs,
 // the q*kappa halo box, d, then Re F, Im F, u_{j-1} of each rhs.  RPC = 1 is the
 // single-rhs layout [u_j | q*kappa | d | Re F | Im F | u_{j-1}].
@@ -190,13 +201,14 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // fit 3 CTAs per SM (the default, 5), 6 or 7 stages (86 / 100 KB) fit 2.
 // RPC = 2 (two right-hand sides per CTA sharing the q*kappa and d boxes and
 // every stencil coefficient): 4 stages (94 KB), 2 CTAs per SM.
-template <int NS, int RPC>
+template <int NS, int RPC, int kTX>
 __global__ void __launch_bounds__(kThreads + 32, RPC == 2 ? 2 : (NS >= 6 ? 2 : 3))
 stream3d_pair_kernel(const __grid_constant__ Stream3Maps maps, int iu, int ium,
                      float *__restrict__ um, Layout L, StepCoef<float> C, float a, float b,
                      const OutSlot *__restrict__ slot, int flags, int zchunk, int *__restrict__ err,
                      RhsSet R)
 {
+    constexpr int kTY = tile_y(kTX), kHaloW = halo_w(kTX);
     constexpr int kSE = stage_elems<RPC>();
     extern __shared__ __align__(128) float ring[];
     uint64_t *full = reinterpret_cast<uint64_t *>(ring + NS * kSE);
@@ -283,13 +295,13 @@ stream3d_pair_kernel(const __grid_constant__ Stream3Maps maps, int iu, int ium,
         return;
     }
 
-    // ---- consumer warps: nodes (x, x+1), x = x0 + 2 tx, row y = y0 + ty ----
+    // ---- consumer warps: nodes (x, x+1), x = x0 + 2 tx, rows y = y0 + 2 ty and y + 1
     grid_dep_wait();         // before any write of a plane the previous step reads
-    const int tx = tid & 31, ty = tid >> 5;
+    const int tx = tid % (kTX / 2), ty = tid / (kTX / 2);
     const int lane = tid & 31;
-    const int64_t gx = x0 + 2 * tx, gy = y0 + ty;
-    const bool rowok = gy < L.ny;
-    const bool actA = rowok && gx < L.nx, actB = rowok && gx + 1 < L.nx;
+    const int64_t gx = x0 + 2 * tx, gy = y0 + 2 * ty;
+    const bool okA = gx < L.nx, okB = gx + 1 < L.nx;       // the pair's nodes
+    const bool row0 = gy < L.ny, row1 = gy + 1 < L.ny;
     const float2 cc0 = bc(C.c0), m0 = bc(C.mt[0]);
     const float2 mf[4] = {bc(C.mt[0]), bc(C.mt[1]), bc(C.mt[2]), bc(C.mt[3])};
     const float2 ncf[4] = {bc(0.f), bc(-C.cs[1]), bc(-C.cs[2]), bc(-C.cs[3])};
@@ -309,10 +321,10 @@ stream3d_pair_kernel(const __grid_constant__ Stream3Maps maps, int iu, int ium,
         if (lane == 0) mbar_arrive(&empty[rst]);
         if (++rst == NS) rst = 0;
     };
-    // box offsets: row ty (= node row - 1), column of node x - 1 in the halo boxes,
-    // (ty, 2 tx) in the node boxes
-    const int uo = ty * kHaloW + 2 * tx + 3;
-    const int no = ty * kTX + 2 * tx;
+    // box offsets: row 2 ty (= first node row - 1), column of node x - 1 in the halo
+    // boxes, (2 ty, 2 tx) in the node boxes
+    const int uo = 2 * ty * kHaloW + 2 * tx + 3;
+    const int no = 2 * ty * kTX + 2 * tx;
     float *ump[RPC];                                   // u_{j+1} at node zb, per rhs
 #pragma unroll
     for (int q = 0; q < RPC; ++q)
@@ -320,7 +332,7 @@ stream3d_pair_kernel(const __grid_constant__ Stream3Maps maps, int iu, int ium,
     int64_t cidx = (zb * L.ny + gy) * L.nx + gx;
     const int64_t cstride = L.ny * L.nx;
 
-    // u_j of one stored plane at row oy as the three pairs (u(x-1+ox), u(x+ox))
+    // u_j of one stored plane at box row oy as the three pairs (u(x-1+ox), u(x+ox))
     auto load_u = [&](float2 (&w)[3], const float *ubox, int oy) {
         const float *r = ubox + uo + oy * kHaloW;
         const float um1 = r[0];
@@ -330,25 +342,25 @@ stream3d_pair_kernel(const __grid_constant__ Stream3Maps maps, int iu, int ium,
         w[1] = mid;
         w[2] = f2(mid.y, up2);
     };
-    // sums of q*kappa of one cell plane over the cells shared with the neighbour at
-    // (oy, ox) - 1 (-1 keeps the lower cell, +1 the upper, 0 both), same order of
-    // additions as the one-node kernel: along x first, then across y
-    auto load_k = [&](float2 (&kk)[3][3], const float *stage) {
+    // Sums of q*kappa of one cell plane over the cells shared with the neighbour at
+    // (oy, ox) - 1 (-1 keeps the lower cell, +1 the upper, 0 both): along x first,
+    // then across y.  The thread's two node rows touch three cell rows; entry 2 r is
+    // cell row r (the upper row of node row r - 1 and the lower one of node row r),
+    // entry 2 r + 1 the sum of rows r and r + 1 (the middle of node row r).
+    auto load_k = [&](float2 (&kk)[5][3], const float *stage) {
         const float *r = stage + RPC * kHaloStride + uo;
-        float2 kx[2][3];
 #pragma unroll
-        for (int ay = 0; ay < 2; ++ay) {
+        for (int ay = 0; ay < 3; ++ay) {
             const float km = r[ay * kHaloW];
             const float2 k2 = *reinterpret_cast<const float2 *>(r + ay * kHaloW + 1);
-            kx[ay][0] = f2(km, k2.x);
-            kx[ay][2] = k2;
-            kx[ay][1] = add2(kx[ay][0], kx[ay][2]);
+            kk[2 * ay][0] = f2(km, k2.x);
+            kk[2 * ay][2] = k2;
+            kk[2 * ay][1] = add2(kk[2 * ay][0], k2);
         }
 #pragma unroll
         for (int ox = 0; ox < 3; ++ox) {
-            kk[0][ox] = kx[0][ox];
-            kk[1][ox] = add2(kx[0][ox], kx[1][ox]);
-            kk[2][ox] = kx[1][ox];
+            kk[1][ox] = add2(kk[0][ox], kk[2][ox]);
+            kk[3][ox] = add2(kk[2][ox], kk[4][ox]);
         }
     };
     // Each stored plane P is read from the ring once: its u_j rows are pushed
@@ -357,117 +369,141 @@ stream3d_pair_kernel(const __grid_constant__ Stream3Maps maps, int iu, int ium,
     // c(P)) and P - 1 (upper plane, c(P-1)) -- where c(P) is the cell plane
     // stored with P.  A node plane receives its lower, middle and upper terms in
     // that order, each in (oy, ox) order, so the sums are those of the one-node
-    // kernel bit for bit.  accL, accM, accU: node planes P + 1, P, P - 1, one
-    // set per rhs; every coefficient is computed once and used for each rhs.
-    float2 kprev[3][3], kcur[3][3];
+    // kernel bit for bit.  accL, accM, accU: node planes P + 1, P, P - 1, two
+    // rows, one set per rhs; every coefficient is computed once and used for each
+    // rhs and, between the two node rows, for both of them.
+    float2 kA[5][3], kB[5][3];
 #pragma unroll
-    for (int oy = 0; oy < 3; ++oy)
+    for (int e = 0; e < 5; ++e)
 #pragma unroll
-        for (int ox = 0; ox < 3; ++ox) kprev[oy][ox] = bc(0.f);
-    float2 accL[RPC], accM[RPC], accU[RPC];
+        for (int ox = 0; ox < 3; ++ox) kB[e][ox] = bc(0.f);
+    float2 accL[RPC][2], accM[RPC][2], accU[RPC][2];
 #pragma unroll
-    for (int q = 0; q < RPC; ++q) accL[q] = accM[q] = accU[q] = bc(0.f);
-    auto coef = [&](int oz, int oy, int ox, float2 ks) -> float2 {
-        const int sh = (oz != 1) + (oy != 1) + (ox != 1);
+    for (int q = 0; q < RPC; ++q)
+#pragma unroll
+        for (int y = 0; y < 2; ++y) accL[q][y] = accM[q][y] = accU[q][y] = bc(0.f);
+    auto coef = [&](int oz, int e, int ox, float2 ks) -> float2 {
+        const int sh = (oz != 1) + (e % 2 == 0) + (ox != 1);
         return (sh == 0) ? fma2(m0, ks, cc0) : fma2(mf[sh], ks, ncf[sh]);
     };
-    // the terms of stored plane `st` for the node planes flagged
-    auto push = [&](const float *st, auto doL, auto doM, auto doU) {
-        constexpr bool kL = decltype(doL)::value, kM = decltype(doM)::value,
-                       kU = decltype(doU)::value;
+    // the terms of stored plane `st`: box row oy is row oy - 1 of node row 0 (entry
+    // oy) and row oy - 2 of node row 1 (entry oy + 1)
+    auto push = [&](const float *st, const float2 (&kprev)[5][3], const float2 (&kcur)[5][3],
+                    auto all) {
+        constexpr bool kAll = decltype(all)::value;      // false: upper terms only
 #pragma unroll
-        for (int oy = 0; oy < 3; ++oy) {
+        for (int oy = 0; oy < 4; ++oy) {
             float2 uv[RPC][3];
 #pragma unroll
             for (int q = 0; q < RPC; ++q) load_u(uv[q], st + q * kHaloStride, oy);
 #pragma unroll
-            for (int ox = 0; ox < 3; ++ox) {
-                if (kL) {
-                    const float2 cL = coef(0, oy, ox, kcur[oy][ox]);
+            for (int y = 0; y < 2; ++y) {
+                if (oy - y < 0 || oy - y > 2) continue;
+                const int e = oy + y;
 #pragma unroll
-                    for (int q = 0; q < RPC; ++q) accL[q] = fma2(cL, uv[q][ox], accL[q]);
-                }
-                if (kM) {
-                    const float2 cM = coef(1, oy, ox, add2(kprev[oy][ox], kcur[oy][ox]));
+                for (int ox = 0; ox < 3; ++ox) {
+                    if (kAll) {
+                        const float2 cL = coef(0, e, ox, kcur[e][ox]);
+                        const float2 cM = coef(1, e, ox, add2(kprev[e][ox], kcur[e][ox]));
 #pragma unroll
-                    for (int q = 0; q < RPC; ++q) accM[q] = fma2(cM, uv[q][ox], accM[q]);
-                }
-                if (kU) {
-                    const float2 cU = coef(2, oy, ox, kprev[oy][ox]);
+                        for (int q = 0; q < RPC; ++q) {
+                            accL[q][y] = fma2(cL, uv[q][ox], accL[q][y]);
+                            accM[q][y] = fma2(cM, uv[q][ox], accM[q][y]);
+                        }
+                    }
+                    const float2 cU = coef(2, e, ox, kprev[e][ox]);
 #pragma unroll
-                    for (int q = 0; q < RPC; ++q) accU[q] = fma2(cU, uv[q][ox], accU[q]);
+                    for (int q = 0; q < RPC; ++q)
+                        accU[q][y] = fma2(cU, uv[q][ox], accU[q][y]);
                 }
             }
         }
     };
     // node plane of stored plane `sn` complete: update, store, outputs
     auto finish = [&](const float *sn) {
-        const float *nd = sn + (RPC + 1) * kHaloStride + no;
-        const float2 d = *reinterpret_cast<const float2 *>(nd);
 #pragma unroll
-        for (int q = 0; q < RPC; ++q) {
-            const float *nq = nd + kNodeElems + q * 3 * kNodeElems;
-            const float2 fr = *reinterpret_cast<const float2 *>(nq);
-            const float2 fi = *reinterpret_cast<const float2 *>(nq + kNodeElems);
-            const float2 uprev = *reinterpret_cast<const float2 *>(nq + 2 * kNodeElems);
-            const float2 g = fma2(a2, fr, mul2(nb2, fi));
-            const float2 t = fma2(ntwo, uprev, add2(accU[q], g));
-            const float2 unew = fma2(d, t, uprev);
-            if (q < nr) {
-                if (actB) {
-                    *reinterpret_cast<float2 *>(ump[q]) = unew;
-                } else if (actA) {
-                    *ump[q] = unew.x;
-                }
-                if (flags && actA) {
-                    const OutSlot *sl = slot + rr[q];
-                    if ((flags & 1) && sl->snap_part) {
-                        sl->snap_part[2 * cidx] = (double)unew.x;
-                        if (actB) sl->snap_part[2 * cidx + 2] = (double)unew.y;
+        for (int y = 0; y < 2; ++y) {
+            const float *nd = sn + (RPC + 1) * kHaloStride + no + y * kTX;
+            const float2 d = *reinterpret_cast<const float2 *>(nd);
+            const bool rowok = y ? row1 : row0;
+            const bool actA = rowok && okA, actB = rowok && okB;
+#pragma unroll
+            for (int q = 0; q < RPC; ++q) {
+                const float *nq = nd + kNodeElems + q * 3 * kNodeElems;
+                const float2 fr = *reinterpret_cast<const float2 *>(nq);
+                const float2 fi = *reinterpret_cast<const float2 *>(nq + kNodeElems);
+                const float2 uprev = *reinterpret_cast<const float2 *>(nq + 2 * kNodeElems);
+                const float2 g = fma2(a2, fr, mul2(nb2, fi));
+                const float2 t = fma2(ntwo, uprev, add2(accU[q][y], g));
+                const float2 unew = fma2(d, t, uprev);
+                if (q < nr) {
+                    float *out = ump[q] + y * L.pitch;
+                    if (actB) {
+                        *reinterpret_cast<float2 *>(out) = unew;
+                    } else if (actA) {
+                        *out = unew.x;
                     }
-                    if ((flags & 2) && sl->final_part) {
-                        sl->final_part[2 * cidx] = (double)unew.x;
-                        if (actB) sl->final_part[2 * cidx + 2] = (double)unew.y;
+                    if (flags && actA) {
+                        const OutSlot *sl = slot + rr[q];
+                        const int64_t c = cidx + y * L.nx;
+                        if ((flags & 1) && sl->snap_part) {
+                            sl->snap_part[2 * c] = (double)unew.x;
+                            if (actB) sl->snap_part[2 * c + 2] = (double)unew.y;
+                        }
+                        if ((flags & 2) && sl->final_part) {
+                            sl->final_part[2 * c] = (double)unew.x;
+                            if (actB) sl->final_part[2 * c + 2] = (double)unew.y;
+                        }
                     }
                 }
             }
-            ump[q] += L.plane;
         }
+#pragma unroll
+        for (int q = 0; q < RPC; ++q) ump[q] += L.plane;
         cidx += cstride;
     };
 
     // stored planes zb + p, p = 0 .. nplanes - 1; node planes are stored planes
-    // 1 .. nplanes - 2.  Plane p feeds node p + 1 if p <= nplanes - 3, node p if
-    // 1 <= p <= nplanes - 2, node p - 1 if p >= 2 (which it completes); after
-    // plane p the stage of plane p - 1 is no longer needed.
-    using T_ = std::true_type;
-    using F_ = std::false_type;
-    bool ok = true;
-    for (int p = 0; p < nplanes; ++p) {
-        if (!(ok = full_wait_next())) break;
-        const float *st = ring + (p % NS) * kSE;
-        if (p < nplanes - 1) load_k(kcur, st);
-        const bool hL = p <= nplanes - 3, hM = p >= 1 && p <= nplanes - 2, hU = p >= 2;
-        if (hL && hM && hU) push(st, T_{}, T_{}, T_{});
-        else if (hL && hM) push(st, T_{}, T_{}, F_{});
-        else if (hL && hU) push(st, T_{}, F_{}, T_{});
-        else if (hM && hU) push(st, F_{}, T_{}, T_{});
-        else if (hL) push(st, T_{}, F_{}, F_{});
-        else if (hM) push(st, F_{}, T_{}, F_{});
-        else push(st, F_{}, F_{}, T_{});
-        if (hU) finish(ring + ((p - 1) % NS) * kSE);
+    // 1 .. nplanes - 2.  Every plane but the last is pushed into all three sums
+    // (the ones no node plane uses are dropped), the last one into the upper
+    // only; plane p >= 2 completes node plane p - 1, after which the stage of plane
+    // p - 1 is no longer needed.  The two sets of cell sums swap roles from plane
+    // to plane (unrolled by two, so they stay in their registers).
+    int sprev = 0, scur = 0;
+    auto plane = [&](int p, const float2 (&kprev)[5][3], float2 (&kcur)[5][3]) -> bool {
+        if (!full_wait_next()) return false;
+        const float *st = ring + scur * kSE;
+        load_k(kcur, st);
+        push(st, kprev, kcur, std::true_type{});
+        if (p >= 2) finish(ring + sprev * kSE);
         if (p >= 1) release_next();
+        sprev = scur;
+        if (++scur == NS) scur = 0;
 #pragma unroll
-        for (int q = 0; q < RPC; ++q) {
-            accU[q] = accM[q];
-            accM[q] = accL[q];
-            accL[q] = bc(0.f);
-        }
+        for (int q = 0; q < RPC; ++q)
 #pragma unroll
-        for (int oy = 0; oy < 3; ++oy)
-#pragma unroll
-            for (int ox = 0; ox < 3; ++ox) kprev[oy][ox] = kcur[oy][ox];
+            for (int y = 0; y < 2; ++y) {
+                accU[q][y] = accM[q][y];
+                accM[q][y] = accL[q][y];
+                accL[q][y] = bc(0.f);
+            }
+        return true;
+    };
+    int p = 0;
+    for (; p + 1 < nplanes - 1; p += 2) {
+        if (!plane(p, kB, kA)) return;
+        if (!plane(p + 1, kA, kB)) return;
     }
+    if (p < nplanes - 1) {
+        if (!plane(p, kB, kA)) return;
+#pragma unroll
+        for (int e = 0; e < 5; ++e)
+#pragma unroll
+            for (int ox = 0; ox < 3; ++ox) kB[e][ox] = kA[e][ox];
+    }
+    if (!full_wait_next()) return;
+    push(ring + scur * kSE, kB, kB, std::false_type{});
+    finish(ring + sprev * kSE);
 }
 
 }  // namespace
@@ -478,7 +514,38 @@ size_t stream3d_pair_smem_bytes(int stages, int rpc)
     return (size_t)stages * se * sizeof(float) + 2 * stages * sizeof(uint64_t);
 }
 
-bool make_stream3d_pair_maps(const Layout &L, float *const planes[6], Stream3Maps *maps, int nrhs)
+// fn(the kernel for the given ring stages, right-hand sides per CTA and tile width)
+template <typename Fn>
+static void with_pair_kernel(int stages, int rpc, int tx, Fn &&fn)
+{
+    if (tx == 64) {
+        if (rpc == 2) fn(stream3d_pair_kernel<4, 2, 64>);
+        else if (stages == 7) fn(stream3d_pair_kernel<7, 1, 64>);
+        else if (stages == 6) fn(stream3d_pair_kernel<6, 1, 64>);
+        else if (stages == 5) fn(stream3d_pair_kernel<5, 1, 64>);
+        else fn(stream3d_pair_kernel<4, 1, 64>);
+    } else {
+        if (rpc == 2) fn(stream3d_pair_kernel<4, 2, 32>);
+        else if (stages == 7) fn(stream3d_pair_kernel<7, 1, 32>);
+        else if (stages == 6) fn(stream3d_pair_kernel<6, 1, 32>);
+        else if (stages == 5) fn(stream3d_pair_kernel<5, 1, 32>);
+        else fn(stream3d_pair_kernel<4, 1, 32>);
+    }
+}
+
+// Tile width: 32 (32 x 16 columns) where it covers the grid with fewer columns than
+// 64 (64 x 8), else 64.  Measured, 32 x 16 against 64 x 8: 106 x 200 x 200 22.1 / 25.2
+// us per step (9 % fewer columns), 160^3 19.0 / 23.3 (17 %), 96^3 5.8 / 7.3 (25 %).
+int stream3d_pair_tx(const Layout &L)
+{
+    auto cover = [&](int tx) {
+        return (L.nx + tx - 1) / tx * tx * ((L.ny + tile_y(tx) - 1) / tile_y(tx) * tile_y(tx));
+    };
+    return cover(32) < cover(64) ? 32 : 64;
+}
+
+bool make_stream3d_pair_maps(const Layout &L, int tx, float *const planes[6], Stream3Maps *maps,
+                             int nrhs)
 {
     typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
@@ -500,8 +567,8 @@ bool make_stream3d_pair_maps(const Layout &L, float *const planes[6], Stream3Map
     const cuuint64_t strides[3] = {(cuuint64_t)(L.pitch * sizeof(float)),
                                    (cuuint64_t)(L.plane * sizeof(float)),
                                    (cuuint64_t)(L.total * sizeof(float))};
-    const cuuint32_t halo[4] = {(cuuint32_t)kHaloW, (cuuint32_t)kHaloH, 1, 1};
-    const cuuint32_t node[4] = {(cuuint32_t)kTX, (cuuint32_t)kTY, 1, 1};
+    const cuuint32_t halo[4] = {(cuuint32_t)halo_w(tx), (cuuint32_t)halo_h(tx), 1, 1};
+    const cuuint32_t node[4] = {(cuuint32_t)tx, (cuuint32_t)tile_y(tx), 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     float *src[8] = {planes[0], planes[1], planes[2], planes[3], planes[4], planes[5], planes[0],
                      planes[1]};
@@ -514,25 +581,26 @@ bool make_stream3d_pair_maps(const Layout &L, float *const planes[6], Stream3Map
             CUDA_SUCCESS)
             return false;
     }
-    const int smem_attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    return cudaFuncSetAttribute(stream3d_pair_kernel<7, 1>, (cudaFuncAttribute)smem_attr,
-                                (int)stream3d_pair_smem_bytes(7, 1)) == cudaSuccess &&
-           cudaFuncSetAttribute(stream3d_pair_kernel<6, 1>, (cudaFuncAttribute)smem_attr,
-                                (int)stream3d_pair_smem_bytes(6, 1)) == cudaSuccess &&
-           cudaFuncSetAttribute(stream3d_pair_kernel<5, 1>, (cudaFuncAttribute)smem_attr,
-                                (int)stream3d_pair_smem_bytes(5, 1)) == cudaSuccess &&
-           cudaFuncSetAttribute(stream3d_pair_kernel<4, 1>, (cudaFuncAttribute)smem_attr,
-                                (int)stream3d_pair_smem_bytes(4, 1)) == cudaSuccess &&
-           cudaFuncSetAttribute(stream3d_pair_kernel<4, 2>, (cudaFuncAttribute)smem_attr,
-                                (int)stream3d_pair_smem_bytes(4, 2)) == cudaSuccess;
+    // the limit is a property of each kernel, shared by every handle
+    bool ok = true;
+    for (int w : {32, 64})
+        for (int v = 0; v < 5; ++v) {
+            const int rpc = v == 4 ? 2 : 1, stages = v == 4 ? 4 : 4 + v;
+            with_pair_kernel(stages, rpc, w, [&](auto kern) {
+                ok = ok && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)stream3d_pair_smem_bytes(stages, rpc)) ==
+                               cudaSuccess;
+            });
+        }
+    return ok;
 }
 
-int stream3d_pair_zchunk(const Layout &L, int stages, int rpc)
+int stream3d_pair_zchunk(const Layout &L, int tx, int stages, int rpc)
 {
     int dev = 0, nsm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tiles = ((L.nx + kTX - 1) / kTX) * ((L.ny + kTY - 1) / kTY);
+    const int64_t tiles = ((L.nx + tx - 1) / tx) * ((L.ny + tile_y(tx) - 1) / tile_y(tx));
     int64_t zc = 64;
     const int per_sm = (rpc == 2 || stages >= 6) ? 2 : 3;
     while (zc > 16 && tiles * ((L.nz + zc - 1) / zc) < per_sm * nsm) zc /= 2;
@@ -540,30 +608,21 @@ int stream3d_pair_zchunk(const Layout &L, int stages, int rpc)
     return (int)zc;
 }
 
-void launch_stream3d_pair(const Stream3Maps &maps, int from, const Layout &L, float *um,
+void launch_stream3d_pair(const Stream3Maps &maps, int from, int tx, const Layout &L, float *um,
                           const StepCoef<float> &C, float a, float b, const OutSlot *slot,
                           int flags, int zchunk, int stages, int *err, cudaStream_t s,
                           const RhsSet &R, bool overlap, int rpc)
 {
     const int iu = from ? 1 : 0, ium = from ? 6 : 7;
     const int groups = (rpc == 2) ? (R.slots + 1) / 2 : R.slots;
-    dim3 grd((unsigned)(((L.nx + kTX - 1) / kTX) * groups), (unsigned)((L.ny + kTY - 1) / kTY),
+    const int ty = tile_y(tx);
+    if (rpc == 2) stages = 4;
+    dim3 grd((unsigned)(((L.nx + tx - 1) / tx) * groups), (unsigned)((L.ny + ty - 1) / ty),
              (unsigned)((L.nz + zchunk - 1) / zchunk));
-    if (rpc == 2)
-        launch_ex(stream3d_pair_kernel<4, 2>, grd, kThreads + 32, stream3d_pair_smem_bytes(4, 2),
-                  s, overlap, maps, iu, ium, um, L, C, a, b, slot, flags, zchunk, err, R);
-    else if (stages == 7)
-        launch_ex(stream3d_pair_kernel<7, 1>, grd, kThreads + 32, stream3d_pair_smem_bytes(7, 1),
-                  s, overlap, maps, iu, ium, um, L, C, a, b, slot, flags, zchunk, err, R);
-    else if (stages == 5)
-        launch_ex(stream3d_pair_kernel<5, 1>, grd, kThreads + 32, stream3d_pair_smem_bytes(5, 1),
-                  s, overlap, maps, iu, ium, um, L, C, a, b, slot, flags, zchunk, err, R);
-    else if (stages == 4)
-        launch_ex(stream3d_pair_kernel<4, 1>, grd, kThreads + 32, stream3d_pair_smem_bytes(4, 1),
-                  s, overlap, maps, iu, ium, um, L, C, a, b, slot, flags, zchunk, err, R);
-    else
-        launch_ex(stream3d_pair_kernel<6, 1>, grd, kThreads + 32, stream3d_pair_smem_bytes(6, 1),
-                  s, overlap, maps, iu, ium, um, L, C, a, b, slot, flags, zchunk, err, R);
+    with_pair_kernel(stages, rpc, tx, [&](auto kern) {
+        launch_ex(kern, grd, kThreads + 32, stream3d_pair_smem_bytes(stages, rpc), s, overlap, maps,
+                  iu, ium, um, L, C, a, b, slot, flags, zchunk, err, R);
+    });
     ++g_launches;
 }
 
