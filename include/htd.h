@@ -419,8 +419,11 @@ htd_status htd_grad(htd_handle h, int nsrc, const void *F_dev, int nrec,
  *               as in htd_grad.
  *   checkpoint_every  C: (u_j, u_{j-1}) are kept every C steps and each
  *               segment is recomputed once on the way back; 0 chooses
- *               ceil(sqrt(2 T n_P)).  Device memory 2 ceil(T n_P / C) + C + 6
- *               state planes (the handle keeps the largest workspace asked).
+ *               ceil(sqrt(2 T n_P)).  Device memory 2 ceil(T n_P / C) + 2 C + 8
+ *               state planes and the two gradients in FP64 for each of the
+ *               sources that run together (as many as fit 1 GiB, at least one);
+ *               where that does not fit the device, 2 ceil(T n_P / C) + C + 6
+ *               planes (the handle keeps the largest workspace asked).
  * The states and multipliers are in the handle's recurrence precision (FP32 in
  * mixed mode), the gradient sums in FP64.  Synchronises the stream.  Errors:
  * HTD_ERR_ARG (bad sizes or indices, mode PROJECT), HTD_ERR_OOM, HTD_ERR_CUDA,

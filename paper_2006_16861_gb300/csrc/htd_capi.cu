@@ -148,7 +148,7 @@ struct htd_ctx {
     double *kap64 = nullptr, *imH = nullptr;
     double *coefP = nullptr;    // assembled operator, h_planes(d) planes of N, ...
     double hmul = 1.0;          // ... times hmul (-q where the FP64 step reads it too, else 1)
-    double c2 = 0.0;            // 2 - p (FP64 step)
+    double h0 = 0.0;            // ... the centre plane less h0
     double *coefI = nullptr;    // assembled Im H (cell damping only), same layout
     // Krylov workspace
     int m = 20;
@@ -192,6 +192,14 @@ struct htd_ctx {
     // htd_grad_td workspace (checkpoints, segment states, multipliers), grown on demand
     void *td_ws = nullptr;
     size_t td_ws_bytes = 0;
+    // captured passes of htd_grad_td: a group's forward pass and, per real run, its
+    // backward sweep, for the workspace and settings of the last call (two group
+    // sizes: whole groups and the last one)
+    struct TdGraph {
+        long long key[5] = {0, 0, 0, 0, 0};
+        cudaGraphExec_t ex[3] = {nullptr, nullptr, nullptr};
+        long long launches[3] = {0, 0, 0};
+    } td_graph[2];
     // captured step sequence
     cudaGraph_t graph = nullptr;          // kept for batches (child graph nodes)
     cudaGraphExec_t exec = nullptr;
@@ -231,6 +239,9 @@ void free_ctx(htd_ctx *c)
     if (c->graph) cudaGraphDestroy(c->graph);
     for (cudaEvent_t e : c->pev)
         if (e) cudaEventDestroy(e);
+    for (htd_ctx::TdGraph &g : c->td_graph)
+        for (cudaGraphExec_t x : g.ex)
+            if (x) cudaGraphExecDestroy(x);
     void *dev[] = {c->kap, c->dco, c->fre, c->fim, c->u0, c->u1, c->kap64, c->imH, c->coefP, c->coefI, c->V, c->Z,
                    c->w, c->t, c->r, c->partial, c->hdev, c->slot, c->Fh, c->Uh, c->u2, c->u3,
                    c->err_dev, c->gU, c->gMu, c->gR, c->gres, c->grec, c->act_dev,
@@ -247,17 +258,18 @@ double h_factor(const htd_ctx *c)
     return 1.0 / (c->h * c->h) / c->hmul;
 }
 
-// one step by the handle's one-step kernel: u_{j+1} over um = u_{j-1}
+// one step by the handle's one-step kernel: u_{j+1} -> out (which may be um = u_{j-1})
 template <typename T>
-void one_step(htd_ctx *c, const T *u, T *um, const T *fre, const T *fim, const StepCoef<T> &C, T a,
-              T b, int flags, cudaStream_t s, const htd::RhsSet &R)
+void one_step(htd_ctx *c, const T *u, const T *um, T *out, const T *fre, const T *fim,
+              const StepCoef<T> &C, T a, T b, const OutSlot *slot, int flags, cudaStream_t s,
+              const htd::RhsSet &R, bool force = true)
 {
     if constexpr (std::is_same<T, double>::value)
-        htd::launch_step_asm(c->Lr, u, um, c->coefP, (const double *)c->dco, fre, fim, c->c2, a, b,
-                             c->slot, flags, s, R);
+        htd::launch_step_asm(c->Lr, u, um, out, c->coefP, (const double *)c->dco, fre, fim, c->C.c0,
+                             a, b, slot, flags, s, R);
     else
-        htd::launch_step<T>(c->Lr, u, um, (const T *)c->kap, (const T *)c->dco, fre, fim, C, a, b,
-                            c->slot, flags, s, R);
+        htd::launch_step(c->Lr, u, um, out, (const T *)c->kap, (const T *)c->dco, fre, fim, C, a, b,
+                         slot, flags, s, R, force);
 }
 
 // one run of the resident-grid kernel from the handle's planes
@@ -267,7 +279,7 @@ void run_resident(htd_ctx *c, const StepCoef<T> &C, int jim, int jfin, cudaStrea
 {
     if constexpr (std::is_same<T, double>::value)
         htd::launch_res2d64(c->res, c->coefP, (const double *)c->dco, (const double *)c->fre,
-                            (const double *)c->fim, c->Lr, c->c2, (const double *)c->res_ab,
+                            (const double *)c->fim, c->Lr, c->C.c0, (const double *)c->res_ab,
                             (int)c->nsteps, jim, jfin, c->slot, c->res_x, c->err_dev, s, P);
     else
         htd::launch_res2d(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
@@ -341,8 +353,8 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
             int flags = 0;
             if (j + 1 == jim) flags |= 1;
             if (j + 1 == jfin) flags |= 2;
-            one_step<T>(c, cur, oth, (const T *)c->fre, (const T *)c->fim, C, (T)c->atab[j],
-                        (T)c->btab[j], flags, s, c->Rs);
+            one_step<T>(c, cur, oth, oth, (const T *)c->fre, (const T *)c->fim, C, (T)c->atab[j],
+                        (T)c->btab[j], c->slot, flags, s, c->Rs);
             if (project && j >= j_acc) accumulate(j, oth);
             std::swap(cur, oth);
         }
@@ -532,7 +544,7 @@ htd_status precond(htd_ctx *c, const double2 *F, double2 *U, cudaStream_t s)
 
 void apply_H(htd_ctx *c, const double2 *X, const double2 *F, double2 *Y, cudaStream_t s)
 {
-    htd::launch_apply_H(c->L64, c->coefP, c->imH, h_factor(c), X, F, Y, s, c->coefI);
+    htd::launch_apply_H(c->L64, c->coefP, c->imH, c->h0, h_factor(c), X, F, Y, s, c->coefI);
 }
 
 // dots of w with V_0..V_{k-1} into hdev + off (device); does not synchronise
@@ -774,8 +786,9 @@ htd_status autotune_fp64_2d(htd_ctx *c)
     const int reps = 64;
     for (int r = 0; r < 2 + reps; ++r) {
         if (r == 2) HTD_CUDA(cudaEventRecord(e0, s));
-        one_step<double>(c, (const double *)c->u0, (double *)c->u1, (const double *)c->fre,
-                         (const double *)c->fim, C, 0.0, 0.0, 0, s, htd::RhsSet{});
+        one_step<double>(c, (const double *)c->u0, (double *)c->u1, (double *)c->u1,
+                         (const double *)c->fre, (const double *)c->fim, C, 0.0, 0.0, c->slot, 0,
+                         s, htd::RhsSet{});
     }
     HTD_CUDA(cudaEventRecord(e1, s));
     HTD_CUDA(cudaEventSynchronize(e1));
@@ -830,9 +843,9 @@ htd_status autotune_tb2d(htd_ctx *c, int want_B, int want_RPT)
     {
         for (int r = 0; r < 2 + reps * 4; ++r) {
             if (r == 2) HTD_CUDA(cudaEventRecord(e0, s));
-            htd::launch_step<float>(L, (const float *)c->u0, (float *)c->u1, (const float *)c->kap,
-                                    (const float *)c->dco, (const float *)c->fre,
-                                    (const float *)c->fim, C, 0.f, 0.f, c->slot, 0, s);
+            htd::launch_step(L, (const float *)c->u0, (float *)c->u1, (float *)c->u1,
+                             (const float *)c->kap, (const float *)c->dco, (const float *)c->fre,
+                             (const float *)c->fim, C, 0.f, 0.f, c->slot, 0, s);
         }
         HTD_CUDA(cudaEventRecord(e1, s));
         HTD_CUDA(cudaEventSynchronize(e1));
@@ -993,19 +1006,63 @@ htd_status autotune_s3_zchunk(htd_ctx *c, const htd::RhsSet &R = htd::RhsSet{})
 }
 
 // Misfit of the preconditioner's own output and its gradient through the
-// recurrence (htd_grad_td).  Per source: U = P F by the handle's fast path for
-// the misfit; then per real run a forward pass of one-step launches that keeps
-// (u_j, u_{j-1}) every C steps, and a backward sweep over the segments from the
-// last: recompute the segment's states from its checkpoint, run the adjoint
-// recurrence (the same step kernel on the multipliers, forcing -dJ/du_k at the
-// read-out steps) and add each step's gradient term.  Memory: 2 ceil(N/C) +
-// C + 6 planes.
+// recurrence (htd_grad_td).  Per source U = P F by the handle's fast path for the
+// misfit (2-D Table 1 runs take it from the forward pass); then, for a group of sources at once (a one-step launch of one source
+// leaves most of the GPU idle at the sizes of an inversion), per real run a forward
+// pass of one-step launches that keeps (u_j, u_{j-1}) every C steps, and a backward
+// sweep over the segments from the last: recompute the segment's states from its
+// checkpoint, run the adjoint recurrence (the same step kernel on the multipliers,
+// forcing -dJ/du_k at the read-out steps) keeping the segment's multipliers, and add
+// the segment's gradient terms in one launch.  The sums are kept per source and
+// added in order, so the gradient depends neither on C nor on the group.
+// Workspace of a group: per source 2 ceil(N/C) + 2 (C + 2) + 4 planes and the sums.
+// Where not even one source's fits, one source at a time with two multiplier
+// planes, a gradient launch per step into gm and gR, and the handle's forcing
+// planes: 2 ceil(N/C) + C + 6 planes.
+// Measured on GB300, 512^2 mixed, 768 steps, 4 sources: 17.2 ms; one source at a time,
+// launch by launch, 86.8.
+constexpr size_t kTdGroupBytes = (size_t)1 << 30;   // a group's workspace, at most (or one source's)
+// planes that a group's steps read and write, at most: 512^2 (5.7 MB per source) took
+// 9.0, 6.4 and 7.1 ms per source in groups of 2, 4 and 7 -- beyond, a step's operands
+// no longer stay in L2 beside the states it leaves behind
+constexpr size_t kTdHotBytes = (size_t)24 << 20;
+
+// Replays a pass of htd_grad_td from graph `*ex`, capturing it first if need be; run
+// directly where that fails or the handle's options ask for no graphs.
+template <typename Run>
+htd_status replay(htd_ctx *c, cudaGraphExec_t *ex, long long *launches, cudaStream_t s, Run &&run)
+{
+    if (c->opt.launch & HTD_LAUNCH_NO_GRAPH) return run(s);
+    if (!*ex) {
+        cudaStream_t cs;
+        HTD_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
+        cudaGraph_t g = nullptr;
+        const long long before = htd::g_launches;
+        bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+        if (ok) {
+            const htd_status st = run(cs);
+            ok = cudaStreamEndCapture(cs, &g) == cudaSuccess && st == HTD_OK;
+        }
+        *launches = htd::g_launches - before;
+        htd::g_launches = before;
+        if (!ok || cudaGraphInstantiate(ex, g, 0) != cudaSuccess) *ex = nullptr;
+        if (g) cudaGraphDestroy(g);
+        cudaStreamDestroy(cs);
+        (void)cudaGetLastError();
+        if (!*ex) return run(s);
+    }
+    HTD_CUDA(cudaGraphLaunch(*ex, s));
+    htd::g_launches += *launches;
+    return HTD_OK;
+}
+
 template <typename T>
 htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const double2 *d,
                         int ckpt, double *gm, double *gR, double *misfit, cudaStream_t s)
 {
     const Layout &L = c->Lr;
     const int64_t N = L.N;
+    const int64_t ncell = (L.nx + 1) * (L.ny + 1) * (L.d == 3 ? L.nz + 1 : 1);
     const long long ns = c->nsteps;
     const long long jim = ns - c->nP / 4;
     const int runs = (c->opt.mode == HTD_MODE_EXACT) ? 2 : 1;
@@ -1013,80 +1070,143 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
                                  : std::max<long long>(1, (long long)std::ceil(std::sqrt(2.0 * ns)));
     const long long nseg = (ns + C - 1) / C;
     const size_t plane = sizeof(T) * (size_t)L.total;
-    const size_t nplanes = (size_t)(2 * nseg + C + 2 + 2 + 2);
-    const size_t need = plane * nplanes + sizeof(double2) * (size_t)N;
-    if (need > c->td_ws_bytes) {
+    const bool want = gm || gR;
+    // group size, multiplier planes, planes and FP64 sums per source
+    int g = 1, nlam = (int)C + 2;
+    size_t npl = (size_t)(2 * nseg + C + 2 + nlam + 4);
+    int64_t nsum = ncell + N;
+    const size_t vec = sizeof(double2) * ((size_t)nrec * nsrc + 1) + sizeof(int) * (1 + htd::kMaxRhs);
+    auto bytes = [&](int k) {
+        return (plane * npl + sizeof(double) * (size_t)nsum + sizeof(double2) * (size_t)N +
+                sizeof(OutSlot)) * k + vec;
+    };
+    while (g < std::min(nsrc, htd::kMaxRhs) && bytes(g + 1) <= kTdGroupBytes &&
+           5 * plane * (g + 1) <= kTdHotBytes)
+        ++g;
+    if (c->td_ws_bytes < bytes(g)) {
         if (c->td_ws) cudaFree(c->td_ws);
         c->td_ws = nullptr;
         c->td_ws_bytes = 0;
-        HTD_CUDA(htd::dev_malloc(&c->td_ws, need));
-        c->td_ws_bytes = need;
+        cudaError_t e = htd::dev_malloc(&c->td_ws, bytes(g));
+        if (e == cudaErrorMemoryAllocation && g > 1) {
+            (void)cudaGetLastError();
+            g = 1;
+            e = htd::dev_malloc(&c->td_ws, bytes(g));
+        }
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            nlam = 2;
+            npl = (size_t)(2 * nseg + C + 2 + nlam + 2);
+            nsum = 0;
+            e = htd::dev_malloc(&c->td_ws, bytes(g));
+        }
+        HTD_CUDA(e);
+        c->td_ws_bytes = bytes(g);
     }
+    const bool lean = nsum == 0;
+    const int64_t sstride = (int64_t)npl * L.total;         // from source to source
     T *base = static_cast<T *>(c->td_ws);
-    auto P = [&](size_t k) { return base + k * (size_t)L.total; };
-    T *ck = P(0);                                   // checkpoint m: planes 2m (u_{mC}), 2m+1 (u_{mC-1})
-    T *seg = P(2 * nseg);                           // u_{s0-2+i} in plane i, i = 0 .. C+1
-    T *lam0 = P(2 * nseg + C + 2), *lam1 = P(2 * nseg + C + 3);
-    T *are = P(2 * nseg + C + 4), *aim = P(2 * nseg + C + 5);
-    double2 *U = reinterpret_cast<double2 *>(P(nplanes));
+    auto P = [&](long long k) { return base + (size_t)k * L.total; };
+    T *seg = P(2 * nseg);                     // u_{s0-2+i} in plane i, i = 0 .. C+1 (checkpoint m: planes
+                                              // 2m (u_{mC}), 2m+1 (u_{mC-1}))
+    T *lam = P(2 * nseg + C + 2);             // lam_k in plane k % nlam
+    T *are = lam + (size_t)nlam * L.total, *aim = are + L.total;
+    T *fre = lean ? (T *)c->fre : aim + L.total, *fim = lean ? (T *)c->fim : aim + 2 * L.total;
+    double2 *U = reinterpret_cast<double2 *>(base + (size_t)sstride * g);      // per source
+    OutSlot *slots = reinterpret_cast<OutSlot *>(U + (size_t)N * g);
+    double *sums = reinterpret_cast<double *>(slots + g);
+    double2 *resd = reinterpret_cast<double2 *>(sums + (((size_t)nsum * g + 1) & ~(size_t)1));
+    int *act = reinterpret_cast<int *>(resd + (size_t)nrec * nsrc);   // (resd: receiver
+                                                                      // residuals of all sources)
+    // Table 1 in 2-D: the forward pass ends in the application's own result, bit for
+    // bit (every 2-D kernel evaluates the same expression), so it gives U itself
+    const bool forward_U = want && !lean && c->d == 2 && runs == 1;
     auto seg_of = [&](long long i, long long s0) { return seg + (size_t)(i - s0 + 2) * L.total; };
-    HTD_CUDA(cudaMemsetAsync(c->td_ws, 0, plane * nplanes, s));   // ghost rings stay zero
+    auto lam_of = [&](long long k) { return lam + (size_t)(k % nlam) * L.total; };
+    HTD_CUDA(cudaMemsetAsync(c->td_ws, 0, plane * npl * g, s));   // ghost rings stay zero
     const StepCoef<T> Cf = cast_coef<T>(c->C);
     const double cK = c->dt * c->dt / c->alpha;
     const double cm = -cK * c->omega_phys * c->omega_phys;
     const double cR = c->beta * c->dt / (2.0 * c->alpha * c->omega) * c->omega_phys;
-    const htd::RhsSet one{};
-    std::vector<double2> res(nrec > 0 ? nrec : 1);
-    double J = 0.0;
-    auto step = [&](const T *u, T *um, const T *fre, const T *fim, T a, T b) {
-        one_step<T>(c, u, um, fre, fim, Cf, a, b, 0, s, one);
+    htd::RhsSet set;
+    set.stride = sstride;
+    // plane `from` of every source of the group -> plane `to`
+    // (the pitch of a 2-D copy has to stay below 2 GiB: that of a group does)
+    auto copy = [&](T *to, const T *from, int n, cudaStream_t t) {
+        if (n == 1) return cudaMemcpyAsync(to, from, plane, cudaMemcpyDeviceToDevice, t);
+        return cudaMemcpy2DAsync(to, sizeof(T) * sstride, from, sizeof(T) * sstride, plane, n,
+                                 cudaMemcpyDeviceToDevice, t);
     };
-    for (int src = 0; src < nsrc; ++src) {
-        const double2 *Fs = F + (size_t)src * N;
-        htd_status st = precond(c, Fs, U, s);
-        if (st != HTD_OK) return st;
-        HTD_CUDA(cudaMemsetAsync(are, 0, 2 * plane, s));     // are, aim adjacent
-        if (nrec > 0) {
-            htd::launch_residual_planes<T>(L, U, d + (size_t)src * nrec, c->grec, nrec, c->gres,
-                                           are, aim, s);
+    auto zero = [&](T *p, size_t planes, int n, cudaStream_t t) {
+        if (n == 1) return cudaMemsetAsync(p, 0, plane * planes, t);
+        return cudaMemset2DAsync(p, sizeof(T) * sstride, 0, plane * planes, n, t);
+    };
+    std::vector<double2> res(nrec > 0 ? (size_t)nrec * nsrc : 1);
+    for (int first = 0; first < nsrc; first += g) {
+        const int n = std::min(g, nsrc - first);
+        HTD_CUDA(zero(are, 2, n, s));                        // are, aim adjacent
+        // receiver residuals and the adjoint forcing planes from U
+        auto residuals = [&]() -> htd_status {
+            for (int q = 0; q < n && nrec > 0; ++q) {
+                const size_t at = (size_t)(first + q) * nrec;
+                htd::launch_residual_planes<T>(L, U + (size_t)q * N, d + at, c->grec, nrec, resd + at,
+                                               are + q * sstride, aim + q * sstride, s);
+            }
             HTD_CUDA(cudaGetLastError());
-            HTD_CUDA(cudaMemcpyAsync(res.data(), c->gres, sizeof(double2) * nrec,
-                                     cudaMemcpyDeviceToHost, s));
-            HTD_CUDA(cudaStreamSynchronize(s));
-            for (int k = 0; k < nrec; ++k) J += 0.5 * (res[k].x * res[k].x + res[k].y * res[k].y);
+            return HTD_OK;
+        };
+        for (int q = 0; q < n; ++q) {
+            double *Ure = reinterpret_cast<double *>(U + (size_t)q * N);
+            if (forward_U) {
+                htd::launch_set_slot(slots + q, Ure, Ure + 1, s);
+                continue;
+            }
+            const htd_status st = precond(c, F + (size_t)(first + q) * N, U + (size_t)q * N, s);
+            if (st != HTD_OK) return st;
         }
-        if (!gm && !gR) continue;
-        for (int run = 0; run < runs; ++run) {
-            // the run's forcing planes (Table 1: F; EXACT run 1: -iF)
-            htd::launch_split<T>(L, Fs, (T *)c->fre, (T *)c->fim, run, s);
-            // forward, keeping (u_j, u_{j-1}) at j = m C
+        htd_status rst;
+        if (!forward_U && (rst = residuals()) != HTD_OK) return rst;
+        if (!want) continue;
+        // the sources of the group as the rhs slots of a step launch
+        set.slots = n;
+        set.act = nullptr;
+        if (n > 1) {
+            std::vector<int> idx(n);
+            for (int q = 0; q < n; ++q) idx[q] = q;
+            htd::launch_set_act(act, n, idx.data(), s);
+            set.act = act;
+        }
+        if (!lean) HTD_CUDA(cudaMemsetAsync(sums, 0, sizeof(double) * nsum * n, s));
+        double *gms = !gm ? nullptr : lean ? gm : sums;
+        double *gRs = !gR ? nullptr : lean ? gR : sums + ncell;
+        // forward, keeping (u_j, u_{j-1}) at j = m C
+        auto forward = [&](cudaStream_t t) -> htd_status {
             T *cur = seg, *oth = seg + L.total;
-            HTD_CUDA(cudaMemsetAsync(seg, 0, 2 * plane, s));
+            HTD_CUDA(zero(seg, 2, n, t));
             for (long long j = 0; j < ns; ++j) {
                 if (j % C == 0) {
                     const long long m = j / C;
-                    HTD_CUDA(cudaMemcpyAsync(P(2 * m), cur, plane, cudaMemcpyDeviceToDevice, s));
-                    HTD_CUDA(cudaMemcpyAsync(P(2 * m + 1), oth, plane, cudaMemcpyDeviceToDevice, s));
+                    HTD_CUDA(copy(P(2 * m), cur, n, t));
+                    HTD_CUDA(copy(P(2 * m + 1), oth, n, t));
                 }
-                step(cur, oth, (const T *)c->fre, (const T *)c->fim, (T)c->atab[j], (T)c->btab[j]);
+                const int flags = !forward_U ? 0 : (j + 1 == jim ? 1 : 0) | (j + 1 == ns ? 2 : 0);
+                one_step<T>(c, cur, oth, oth, fre, fim, Cf, (T)c->atab[j], (T)c->btab[j], slots,
+                            flags, t, set);
                 std::swap(cur, oth);
             }
-            // backward over the segments [s0, s1], s0 = 1 + m C
-            HTD_CUDA(cudaMemsetAsync(lam0, 0, 2 * plane, s));     // lam_{k+1}, lam_{k+2}
-            T *la = lam0, *lb = lam1;
+            HTD_CUDA(cudaGetLastError());
+            return HTD_OK;
+        };
+        // backward over the segments [s0, s1], s0 = 1 + m C
+        auto backward = [&](int run, cudaStream_t t) -> htd_status {
+            HTD_CUDA(zero(lam, nlam, n, t));                  // lam_{ns+1}, lam_{ns+2} among them
             for (long long m = nseg - 1; m >= 0; --m) {
                 const long long s0 = 1 + m * C, s1 = std::min(s0 + C - 1, ns);
-                HTD_CUDA(cudaMemcpyAsync(seg_of(s0 - 2, s0), P(2 * m + 1), plane,
-                                         cudaMemcpyDeviceToDevice, s));
-                HTD_CUDA(cudaMemcpyAsync(seg_of(s0 - 1, s0), P(2 * m), plane,
-                                         cudaMemcpyDeviceToDevice, s));
-                for (long long j = s0 - 1; j < s1; ++j) {
-                    T *dst = seg_of(j + 1, s0);
-                    HTD_CUDA(cudaMemcpyAsync(dst, seg_of(j - 1, s0), plane,
-                                             cudaMemcpyDeviceToDevice, s));
-                    step(seg_of(j, s0), dst, (const T *)c->fre, (const T *)c->fim, (T)c->atab[j],
-                         (T)c->btab[j]);
-                }
+                HTD_CUDA(copy(seg_of(s0 - 2, s0), P(2 * m + 1), n, t));
+                HTD_CUDA(copy(seg_of(s0 - 1, s0), P(2 * m), n, t));
+                for (long long j = s0 - 1; j < s1; ++j)
+                    one_step<T>(c, seg_of(j, s0), seg_of(j - 1, s0), seg_of(j + 1, s0), fre, fim, Cf,
+                                (T)c->atab[j], (T)c->btab[j], slots, 0, t, set);
                 for (long long k = s1; k >= s0; --k) {
                     // forcing -dJ/du_k: Table 1 reads Re U at N and Im U at jim; EXACT
                     // reads Re U (run 0) or Im U (run 1) at N
@@ -1097,16 +1217,56 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
                     } else if (k == ns) {
                         if (run == 0) a = T(-1); else b = T(1);
                     }
-                    step(la, lb, are, aim, a, b);          // lb <- lam_k
-                    std::swap(la, lb);                     // la = lam_k, lb = lam_{k+1}
-                    htd::launch_grad_td<T>(L, c->M, cm, cR, la, seg_of(k, s0), seg_of(k - 1, s0),
-                                           seg_of(k - 2, s0), gm, gR, s);
+                    one_step<T>(c, lam_of(k + 1), lam_of(k + 2), lam_of(k), are, aim, Cf, a, b, slots,
+                                0, t, set, a != T(0) || b != T(0));
+                    if (lean)
+                        htd::launch_grad_td<T>(L, c->M, cm, cR, lam, nlam, seg, sstride, 1, s0, k, k,
+                                               gms, gRs, 0, t);
                 }
+                if (!lean)
+                    htd::launch_grad_td<T>(L, c->M, cm, cR, lam, nlam, seg, sstride, n, s0, s1, s0,
+                                           gms, gRs, nsum, t);
             }
             HTD_CUDA(cudaGetLastError());
+            return HTD_OK;
+        };
+        // the captured passes of this workspace, group size and settings
+        const long long key[5] = {(long long)(intptr_t)c->td_ws, ((long long)g << 32) | n, C,
+                                  (gms ? 1 : 0) | (gRs ? 2 : 0) | (want ? 4 : 0),
+                                  (long long)(intptr_t)act};
+        htd_ctx::TdGraph &tg = c->td_graph[n == g ? 0 : 1];
+        if (std::memcmp(tg.key, key, sizeof(key)) != 0) {
+            for (cudaGraphExec_t &x : tg.ex) {
+                if (x) cudaGraphExecDestroy(x);
+                x = nullptr;
+            }
+            std::memcpy(tg.key, key, sizeof(key));
         }
+        for (int run = 0; run < runs; ++run) {
+            // the run's forcing planes (Table 1: F; EXACT run 1: -iF)
+            for (int q = 0; q < n; ++q)
+                htd::launch_split<T>(L, F + (size_t)(first + q) * N, fre + (lean ? 0 : q * sstride),
+                                     fim + (lean ? 0 : q * sstride), run, s);
+            // (the lean form writes to the caller's gradients: not captured)
+            htd_status st = lean ? forward(s) : replay(c, &tg.ex[0], &tg.launches[0], s, forward);
+            if (st == HTD_OK && forward_U) st = residuals();
+            if (st == HTD_OK)
+                st = lean ? backward(run, s)
+                          : replay(c, &tg.ex[1 + run], &tg.launches[1 + run], s,
+                                   [&](cudaStream_t t) { return backward(run, t); });
+            if (st != HTD_OK) return st;
+        }
+        if (!lean && gm) htd::launch_add_sources(gm, sums, nsum, n, ncell, s);
+        if (!lean && gR) htd::launch_add_sources(gR, sums + ncell, nsum, n, N, s);
+        HTD_CUDA(cudaGetLastError());
     }
+    if (nrec > 0)
+        HTD_CUDA(cudaMemcpyAsync(res.data(), resd, sizeof(double2) * nrec * nsrc,
+                                 cudaMemcpyDeviceToHost, s));
     HTD_CUDA(cudaStreamSynchronize(s));
+    double J = 0.0;
+    for (size_t k = 0; k < (size_t)nrec * nsrc; ++k)
+        J += 0.5 * (res[k].x * res[k].x + res[k].y * res[k].y);
     *misfit = J;
     return std::isfinite(J) ? HTD_OK : HTD_ERR_NONFINITE;
 }
@@ -1407,11 +1567,14 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
     {
         // the FP64 step reads the same planes, scaled by -q
         c->hmul = (!mixed && !abd) ? -q : 1.0;
-        c->c2 = 2.0 - p;
         double S2[4], M2[4];
         for (int k = 0; k < 4; ++k) {
             S2[k] = c->hmul * std::ldexp(c->S[k], d - k);
             M2[k] = c->hmul * c->M[k];
+        }
+        if (!mixed && !abd) {                  // the centre's constant is the step's c0
+            c->h0 = S2[0];
+            S2[0] = 0.0;
         }
         HTD_CUDA(htd::dev_malloc((void **)&c->coefP, sizeof(double) * htd::h_planes(d) * (size_t)N));
         htd::launch_assemble_H(c->L64, c->kap64, S2, M2, c->coefP, 0);
@@ -1557,6 +1720,7 @@ void operator_view(const htd_ctx *c, OperatorView *out)
         out->S2[k] = std::ldexp(c->S[k], c->d - k);
         out->M[k] = c->M[k];
     }
+    out->h0 = c->h0;
     out->ih2 = h_factor(c);
     out->device = c->device;
 }

@@ -100,32 +100,36 @@ __device__ __forceinline__ V stencil2d(const Stencil2dCoef<V> &C, V umm, V um0, 
     return vadd(r1, r2);
 }
 
-// The 2-D assembled stencil at a node: the centre, then the neighbours in
-// (oy, ox) order (see step3d_asm_kernel; planes scaled by -q).
+// The 2-D assembled stencil at a node: the centre's and the neighbours' coefficients
+// by (oy, ox) (see step3d_asm_kernel; planes scaled by -q).
 struct Asm9 {
-    double c0, kmm, km0, kmp, k0m, k0p, kpm, kp0, kpp;
+    double c, kmm, km0, kmp, k0m, k0p, kpm, kp0, kpp;
 };
 
-// u_{j+1} at a node in FP64: own-node terms first, then one multiply-add per
-// neighbour.  The one-step and the resident-grid kernel share it, so their
+// u_{j+1} at a node in FP64: one multiply-add per neighbour, the small corner terms
+// first, and the own-node terms beside them (16 operations).  Summed apart, the
+// neighbours' rounding stays at their size: the misfit of a 512^2 run came out with a
+// rounding noise of 3.3e-15 of its value against 5.9e-15 in one chain and 4.6e-15
+// with the cell form.  The one-step and the resident-grid kernel share it, so their
 // results are bit-identical.  nb = -b_j.
 __device__ __forceinline__ double asm2d_step(const Asm9 &k, double umm, double um0, double ump,
                                              double u0m, double u00, double u0p, double upm,
                                              double up0, double upp, double uprev, double d,
-                                             double fr, double fi, double c2, double a, double nb)
+                                             double fr, double fi, double c0, double a, double nb)
 {
-    double t = __fma_rn(a, fr, __dmul_rn(nb, fi));
-    t = __fma_rn(-2.0, uprev, t);
-    t = __fma_rn(c2, u00, t);
-    t = __fma_rn(k.c0, u00, t);
-    t = __fma_rn(k.kmm, umm, t);
-    t = __fma_rn(k.km0, um0, t);
+    double t = __dmul_rn(k.kmm, umm);
     t = __fma_rn(k.kmp, ump, t);
+    t = __fma_rn(k.kpm, upm, t);
+    t = __fma_rn(k.kpp, upp, t);
+    t = __fma_rn(k.km0, um0, t);
     t = __fma_rn(k.k0m, u0m, t);
     t = __fma_rn(k.k0p, u0p, t);
-    t = __fma_rn(k.kpm, upm, t);
     t = __fma_rn(k.kp0, up0, t);
-    t = __fma_rn(k.kpp, upp, t);
+    double v = __fma_rn(a, fr, __dmul_rn(nb, fi));
+    v = __fma_rn(-2.0, uprev, v);
+    v = __fma_rn(c0, u00, v);
+    v = __fma_rn(k.c, u00, v);
+    t = __dadd_rn(t, v);
     return __fma_rn(d, t, uprev);
 }
 
@@ -226,15 +230,18 @@ void launch_ex(void (*kern)(KArgs...), dim3 grd, unsigned threads, size_t smem, 
     (void)cudaLaunchKernelEx(&cfg, kern, static_cast<Args &&>(args)...);
 }
 
-template <typename T>
-void launch_step(const Layout &L, const T *u, T *um, const T *kap, const T *dco,
-                 const T *fre, const T *fim, const StepCoef<T> &C, T a, T b,
-                 const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R = RhsSet{});
+// One FP32 step u_{j+1} -> out from u = u_j and um = u_{j-1} (out may be um); force
+// false: no forcing (a = b = 0).
+void launch_step(const Layout &L, const float *u, const float *um, float *out, const float *kap,
+                 const float *dco, const float *fre, const float *fim, const StepCoef<float> &C,
+                 float a, float b, const OutSlot *slot, int flags, cudaStream_t s,
+                 const RhsSet &R = RhsSet{}, bool force = true);
 
 // The FP64 step from the assembled planes of launch_assemble_H scaled by -q
-// (see step3d_asm_kernel); c2 = 2 - p.
-void launch_step_asm(const Layout &L, const double *u, double *um, const double *coefP,
-                     const double *dco, const double *fre, const double *fim, double c2, double a,
+// (see step3d_asm_kernel); c0 = 2 - p - q 2^d S_0.
+void launch_step_asm(const Layout &L, const double *u, const double *um, double *out,
+                     const double *coefP,
+                     const double *dco, const double *fre, const double *fim, double c0, double a,
                      double b, const OutSlot *slot, int flags, cudaStream_t s,
                      const RhsSet &R = RhsSet{});
 
@@ -469,7 +476,7 @@ void launch_res2d(const Res2dPlan &p, const float *kap, const float *dco, const 
 // launch_step_asm), two steps per exchange of edge values; nsteps is even.
 bool res2d64_plan(const Layout &L, Res2dPlan *p);
 void launch_res2d64(const Res2dPlan &p, const double *coefP, const double *dco, const double *fre,
-                    const double *fim, const Layout &L, double c2, const double *ab, int nsteps,
+                    const double *fim, const Layout &L, double c0, const double *ab, int nsteps,
                     int jim, int jfin, const OutSlot *slot, unsigned long long *xbuf, int *err,
                     cudaStream_t s, const Res2dProj<double> &P = Res2dProj<double>{});
 
@@ -525,9 +532,10 @@ void launch_group2d(const TbPlan &p, const GroupSched &S, int ctas, cudaStream_t
 __host__ __device__ constexpr int h_planes(int d) { return d == 3 ? 14 : 5; }
 void launch_assemble_H(const Layout &L, const double *kap64, const double S2[4], const double M[4],
                        double *coefP, cudaStream_t s);
-// Y = H X (F == null) or Y = F - H X, complex128 compact vectors.  Im H is the
+// Y = H X (F == null) or Y = F - H X, complex128 compact vectors.  h0 is added to
+// the centre plane's coefficients (0 unless the plane holds only their kappa part).  Im H is the
 // diagonal imH, plus the assembled planes coefI if given (cell damping).
-void launch_apply_H(const Layout &L, const double *coefP, const double *imH, double ih2,
+void launch_apply_H(const Layout &L, const double *coefP, const double *imH, double h0, double ih2,
                     const double2 *X, const double2 *F, double2 *Y, cudaStream_t s,
                     const double *coefI = nullptr);
 
@@ -593,11 +601,14 @@ template <typename T>
 void launch_residual_planes(const Layout &L, const double2 *U, const double2 *d,
                             const int64_t *rec, int nrec, double2 *res, T *are, T *aim,
                             cudaStream_t s);
-// gm[cell] += cm sum lam_b M u_{k-1,g};  gR[node] += cR lam (u_k - u_{k-2})
+// The gradient terms k0 .. k1 (descending) of nsrc sources (see grad_td_kernel)
 template <typename T>
-void launch_grad_td(const Layout &L, const double M[4], double cm, double cR, const T *lam,
-                    const T *uk, const T *uk1, const T *uk2, double *gm, double *gR,
-                    cudaStream_t s);
+void launch_grad_td(const Layout &L, const double M[4], double cm, double cR, const T *lam, int nlam,
+                    const T *seg, int64_t sstride, int nsrc, long long s0, long long k0,
+                    long long k1, double *gm, double *gR, int64_t gstride, cudaStream_t s);
+// out[0 .. n) += the sums of nsrc sources, gstride apart, in order
+void launch_add_sources(double *out, const double *g, int64_t gstride, int nsrc, int64_t n,
+                        cudaStream_t s);
 
 // Receiver residual res = U[rec] - d, and r[rec] += conj(res) (r pre-zeroed).
 void launch_receiver_residual(const double2 *U, const double2 *d, const int64_t *rec, int nrec,
@@ -613,7 +624,7 @@ struct OperatorView {
     const double *coefP;    // assembled operator (launch_assemble_H)
     const double *coefI;    // assembled non-diagonal Im H, or null
     const double *imH;      // omega_phys R per node
-    double S2[4], M[4], ih2;
+    double S2[4], M[4], h0, ih2;   // h0, ih2: see launch_apply_H
     int device;
 };
 void operator_view(const htd_ctx *c, OperatorView *out);

@@ -56,47 +56,77 @@ static int sm_count()
 // recurrence step
 // ---------------------------------------------------------------------------
 
-template <typename T>
+// One step in 2-D, FP32: u_{j+1} -> out (which may be the plane um of u_{j-1}).  A
+// thread takes ROWS nodes of one column, so that a node costs 4.5 loads of u_j and 2.5
+// of q*kappa (nine and four with one row), all of them issued before the first sum.
+// ROWS = 4 where that leaves two blocks per SM, else 1.  force: without it the step has no forcing (a = b = 0: the adjoint
+// between its read-out steps).
+template <int ROWS>
 __global__ void __launch_bounds__(256)
-step2d_kernel(const T *__restrict__ u, T *__restrict__ um, const T *__restrict__ kap,
-              const T *__restrict__ dco, const T *__restrict__ fre, const T *__restrict__ fim,
-              Layout L, StepCoef<T> C, T a, T b, const OutSlot *__restrict__ slot, int flags,
-              RhsSet R)
+step2d_kernel(const float *__restrict__ u, const float *um, float *out,
+              const float *__restrict__ kap, const float *__restrict__ dco,
+              const float *__restrict__ fre, const float *__restrict__ fim, Layout L,
+              StepCoef<float> C, float a, float b, const OutSlot *__restrict__ slot, int flags,
+              RhsSet R, bool force)
 {
-    const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
+    const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    const int64_t iy0 = ((int64_t)blockIdx.y * 8 + threadIdx.y) * ROWS;
     int rhs;
     if (!rhs_of_slot(R, (int)blockIdx.z, rhs)) return;
-    if (ix >= L.nx || iy >= L.ny) return;
-    u += rhs * R.stride;
-    um += rhs * R.stride;
-    fre += rhs * R.stride;
-    fim += rhs * R.stride;
+    if (ix >= L.nx || iy0 >= L.ny) return;
+    const int64_t off = rhs * R.stride;
+    u += off;
+    um += off;
+    out += off;
+    fre += off;
+    fim += off;
     slot += rhs;
     const int64_t P = L.pitch;
-    const int64_t i = (iy + 1) * P + L.xl + ix;
-    // u_j on the 3x3 neighbourhood; first index = y offset, second = x offset
-    const T umm = u[i - P - 1], um0 = u[i - P], ump = u[i - P + 1];
-    const T u0m = u[i - 1], u00 = u[i], u0p = u[i + 1];
-    const T upm = u[i + P - 1], up0 = u[i + P], upp = u[i + P + 1];
-    // q*kappa of the four cells around the node, k<ay><ax>: cell at row y-1+ay, column x-1+ax
-    const T k00 = kap[i - P - 1], k01 = kap[i - P], k10 = kap[i - 1], k11 = kap[i];
-    // pair sums shared with the temporally blocked kernel (same order, same result)
-    const T pm = umm + ump, p0 = u0m + u0p, pp = upm + upp;
-    const T hk0 = k00 + k01, hk1 = k10 + k11;
-    const Stencil2dCoef<T> SC = stencil2d_coef(C);
-    const T acc = stencil2d(SC, umm, um0, ump, u0m, u00, u0p, upm, up0, upp, k00, k01, k10, k11,
-                            pm, p0, pp, hk0, hk1);
-    // acc + a Re F - b Im F as two FMAs (the blocked kernels round the same way)
-    const T ag = vfma(a, fre[i], vfma(-b, fim[i], acc));
-    const T d = dco[i];
-    const T uprev = um[i];
-    const T unew = vfma(d, vfma(T(-2), uprev, ag), uprev);
-    um[i] = unew;
-    if (flags) {
-        const int64_t c = iy * L.nx + ix;
-        if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = (double)unew;
-        if ((flags & 2) && slot->final_part) slot->final_part[2 * c] = (double)unew;
+    const Stencil2dCoef<float> SC = stencil2d_coef(C);
+    const int64_t i0 = (iy0 + 1) * P + L.xl + ix;
+    // every operand first: the loads of all rows are in flight together.  (Rows
+    // below the grid are loaded from its last ghost row and not stored.)
+    float w[ROWS + 2][3], k[ROWS + 1][2], um1[ROWS], d[ROWS], fr[ROWS], fi[ROWS];
+    int64_t at[ROWS + 2];                   // u row r - 1
+#pragma unroll
+    for (int r = 0; r < ROWS + 2; ++r) at[r] = i0 + (min(iy0 + r - 1, L.ny) - iy0) * P;
+#pragma unroll
+    for (int r = 0; r < ROWS + 2; ++r)
+#pragma unroll
+        for (int x = 0; x < 3; ++x) w[r][x] = u[at[r] + x - 1];
+#pragma unroll
+    for (int r = 0; r < ROWS + 1; ++r)
+#pragma unroll
+        for (int x = 0; x < 2; ++x) k[r][x] = kap[at[r] + x - 1];
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        um1[r] = um[at[r + 1]];
+        d[r] = dco[at[r + 1]];
+        if (force) {
+            fr[r] = fre[at[r + 1]];
+            fi[r] = fim[at[r + 1]];
+        }
+    }
+    // w[r]: u_j at row offset r - 1 of the first node; k[r]: q*kappa of the cells of
+    // row y - 1 + r.  Pair sums shared with the temporally blocked kernel (same
+    // order, same result)
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        if (r > 0 && iy0 + r >= L.ny) break;
+        const float *a0 = w[r], *a1 = w[r + 1], *a2 = w[r + 2];
+        float ag = stencil2d(SC, a0[0], a0[1], a0[2], a1[0], a1[1], a1[2], a2[0], a2[1], a2[2],
+                             k[r][0], k[r][1], k[r + 1][0], k[r + 1][1], a0[0] + a0[2],
+                             a1[0] + a1[2], a2[0] + a2[2], k[r][0] + k[r][1],
+                             k[r + 1][0] + k[r + 1][1]);
+        // acc + a Re F - b Im F as two FMAs (the blocked kernels round the same way)
+        if (force) ag = vfma(a, fr[r], vfma(-b, fi[r], ag));
+        const float unew = vfma(d[r], vfma(-2.f, um1[r], ag), um1[r]);
+        out[at[r + 1]] = unew;
+        if (flags) {
+            const int64_t c = (iy0 + r) * L.nx + ix;
+            if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = (double)unew;
+            if ((flags & 2) && slot->final_part) slot->final_part[2 * c] = (double)unew;
+        }
     }
 }
 
@@ -106,13 +136,14 @@ step2d_kernel(const T *__restrict__ u, T *__restrict__ um, const T *__restrict__
 // L1, the plane below and the node's own plane from registers).
 constexpr int kZChunk = 16;
 
-template <typename T>
 __global__ void __launch_bounds__(256)
-step3d_kernel(const T *__restrict__ u, T *__restrict__ um, const T *__restrict__ kap,
-              const T *__restrict__ dco, const T *__restrict__ fre, const T *__restrict__ fim,
-              Layout L, StepCoef<T> C, T a, T b, const OutSlot *__restrict__ slot, int flags,
-              RhsSet R, int nchunks)
+step3d_kernel(const float *__restrict__ u, const float *um, float *out,
+              const float *__restrict__ kap, const float *__restrict__ dco,
+              const float *__restrict__ fre, const float *__restrict__ fim, Layout L,
+              StepCoef<float> C, float a, float b, const OutSlot *__restrict__ slot, int flags,
+              RhsSet R, int nchunks, bool force)
 {
+    typedef float T;
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -122,6 +153,7 @@ step3d_kernel(const T *__restrict__ u, T *__restrict__ um, const T *__restrict__
     if (ix >= L.nx || iy >= L.ny) return;
     u += rhs * R.stride;
     um += rhs * R.stride;
+    out += rhs * R.stride;
     fre += rhs * R.stride;
     fim += rhs * R.stride;
     slot += rhs;
@@ -188,11 +220,11 @@ step3d_kernel(const T *__restrict__ u, T *__restrict__ um, const T *__restrict__
                     acc += coef * w[oz][oy][ox];
                 }
         const int64_t i = (iz + 1) * Q + col;
-        const T g = a * fre[i] - b * fim[i];
+        const T g = force ? a * fre[i] - b * fim[i] : 0.f;
         const T d = dco[i];
         const T uprev = um[i];
         const T unew = d * (acc + g - T(2) * uprev) + uprev;
-        um[i] = unew;
+        out[i] = unew;
         if (flags) {
             const int64_t c = (iz * L.ny + iy) * L.nx + ix;
             if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = (double)unew;
@@ -212,32 +244,31 @@ step3d_kernel(const T *__restrict__ u, T *__restrict__ um, const T *__restrict__
     }
 }
 
-template <typename T>
-void launch_step(const Layout &L, const T *u, T *um, const T *kap, const T *dco,
-                 const T *fre, const T *fim, const StepCoef<T> &C, T a, T b,
-                 const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R)
+void launch_step(const Layout &L, const float *u, const float *um, float *out, const float *kap,
+                 const float *dco, const float *fre, const float *fim, const StepCoef<float> &C,
+                 float a, float b, const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R,
+                 bool force)
 {
+    const unsigned gx = (unsigned)((L.nx + 31) / 32);
     if (L.d == 2) {
-        dim3 blk(32, 8);
-        dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
-        step2d_kernel<T><<<grd, blk, 0, s>>>(u, um, kap, dco, fre, fim, L, C, a, b, slot, flags,
-                                             R);
-        ++g_launches;
+        const int64_t blocks4 = gx * ((L.ny + 31) / 32) * R.slots;
+        if (blocks4 >= 2 * (int64_t)sm_count()) {
+            dim3 grd(gx, (unsigned)((L.ny + 31) / 32), (unsigned)R.slots);
+            step2d_kernel<4><<<grd, dim3(32, 8), 0, s>>>(u, um, out, kap, dco, fre, fim, L, C, a,
+                                                         b, slot, flags, R, force);
+        } else {
+            dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
+            step2d_kernel<1><<<grd, dim3(32, 8), 0, s>>>(u, um, out, kap, dco, fre, fim, L, C, a,
+                                                         b, slot, flags, R, force);
+        }
     } else {
         const int nchunks = (int)((L.nz + kZChunk - 1) / kZChunk);
-        dim3 blk(32, 8);
-        dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8),
-                 (unsigned)(nchunks * R.slots));
-        step3d_kernel<T><<<grd, blk, 0, s>>>(u, um, kap, dco, fre, fim, L, C, a, b, slot, flags,
-                                             R, nchunks);
-        ++g_launches;
+        dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)(nchunks * R.slots));
+        step3d_kernel<<<grd, dim3(32, 8), 0, s>>>(u, um, out, kap, dco, fre, fim, L, C, a, b, slot,
+                                                  flags, R, nchunks, force);
     }
+    ++g_launches;
 }
-
-template void launch_step<float>(const Layout &, const float *, float *, const float *,
-                                 const float *, const float *, const float *,
-                                 const StepCoef<float> &, float, float, const OutSlot *, int,
-                                 cudaStream_t, const RhsSet &);
 
 // One step of I_acd in FP64 from the assembled stencil.  GB300 retires two FP64
 // operations per clock and SM (1.26 TFLOP/s as FMAs on 152 SMs) beside
@@ -246,13 +277,16 @@ template void launch_step<float>(const Layout &, const float *, float *, const f
 // operations per 3-D node) are not recomputed in every step but read back, from
 // the same assembled planes that apply_H uses (the centre and the positive
 // offsets; a negative offset is the neighbour's positive one).  For FP64 handles
-// those planes hold -q (2^{d-s} S_s - M_s sum kappa), so that with c2 = 2 - p
-//   (2 - K) u_j = c2 u_j + sum_o coef_o u_{j, beta + o}
-// is one multiply-add per offset: 32 FP64 operations per 3-D node.  The planes
+// those planes hold -q (2^{d-s} S_s - M_s sum kappa) off the centre and q M_0 sum
+// kappa at the centre, so that with c0 = 2 - p - q 2^d S_0
+//   (2 - K) u_j = c0 u_j + sum_o coef_o u_{j, beta + o}
+// is one multiply-add per offset: 33 FP64 operations per 3-D node.  (The centre's
+// constant stays a scalar because a stored coefficient's rounding is the same in
+// every step and so adds up: the centre's, about 1, would round five times as
+// coarsely as the others.)  The planes
 // are compact (N values each) and padded nowhere: where an offset leaves the
 // grid u is the zero ghost ring, and the index is clamped into the plane (any
 // finite coefficient times the ghost's zero).
-// Own-node terms open the chain, the neighbours follow in (oz, oy, ox) order.
 // A thread marches up a column of zc planes with the 3 x 3 x 3 window of u in
 // registers; zc is chosen by the launcher so that every SM gets about eight
 // blocks (the last wave of an FP64-bound kernel costs as much as it holds).
@@ -261,10 +295,10 @@ template void launch_step<float>(const Layout &, const float *, float *, const f
 constexpr int kAsmTY = 4;
 
 __global__ void __launch_bounds__(32 * kAsmTY)
-step3d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
+step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   const double *__restrict__ coefP, const double *__restrict__ dco,
                   const double *__restrict__ fre, const double *__restrict__ fim, Layout L,
-                  double c2, double a, double b, const OutSlot *__restrict__ slot, int flags,
+                  double c0, double a, double b, const OutSlot *__restrict__ slot, int flags,
                   RhsSet R, int zc, int nchunks)
 {
     const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
@@ -276,6 +310,7 @@ step3d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
     if (ix >= L.nx || iy >= L.ny) return;
     u += rhs * R.stride;
     um += rhs * R.stride;
+    out += rhs * R.stride;
     fre += rhs * R.stride;
     fim += rhs * R.stride;
     slot += rhs;
@@ -299,27 +334,28 @@ step3d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
             for (int ox = 0; ox < 3; ++ox)
                 w[2][oy][ox] = u[i + Q + (oy - 1) * P + (ox - 1)];
         const double uprev = um[i];
-        double acc = fma(a, fre[i], -b * fim[i]);
-        acc = fma(-2.0, uprev, acc);
-        acc = fma(c2, w[1][1][1], acc);
-        acc = fma(coefP[c], w[1][1][1], acc);
+        // own-node terms beside the neighbours', corners first (as in asm2d_step)
+        double own = fma(a, fre[i], -b * fim[i]);
+        own = fma(-2.0, uprev, own);
+        own = fma(c0, w[1][1][1], own);
+        own = fma(coefP[c], w[1][1][1], own);
+        double acc = coefP[13 * N + c] * w[2][2][2];
 #pragma unroll
-        for (int oz = 0; oz < 3; ++oz)
+        for (int sh = 3; sh >= 1; --sh)
 #pragma unroll
-            for (int oy = 0; oy < 3; ++oy)
-#pragma unroll
-                for (int ox = 0; ox < 3; ++ox) {
-                    const int lin = oz * 9 + oy * 3 + ox;
-                    if (lin == 13) continue;
-                    int64_t ci = c;
-                    if (lin < 13) {
-                        ci += ((int64_t)(oz - 1) * L.ny + (oy - 1)) * L.nx + (ox - 1);
-                        ci = ci > 0 ? ci : 0;
-                    }
-                    acc = fma(coefP[(lin < 13 ? 13 - lin : lin - 13) * N + ci], w[oz][oy][ox], acc);
+            for (int lin = 0; lin < 26; ++lin) {
+                const int oz = lin / 9, oy = lin / 3 % 3, ox = lin % 3;
+                if ((oz != 1) + (oy != 1) + (ox != 1) != sh) continue;
+                int64_t ci = c;
+                if (lin < 13) {
+                    ci += ((int64_t)(oz - 1) * L.ny + (oy - 1)) * L.nx + (ox - 1);
+                    ci = ci > 0 ? ci : 0;
                 }
+                acc = fma(coefP[(lin < 13 ? 13 - lin : lin - 13) * N + ci], w[oz][oy][ox], acc);
+            }
+        acc += own;
         const double unew = fma(dco[i], acc, uprev);
-        um[i] = unew;
+        out[i] = unew;
         if (flags) {
             if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = unew;
             if ((flags & 2) && slot->final_part) slot->final_part[2 * c] = unew;
@@ -334,13 +370,13 @@ step3d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
     }
 }
 
-// the 2-D form: one node per thread, 14 FP64 operations (the cell form: 33);
+// the 2-D form: one node per thread, 16 FP64 operations (the cell form: 33);
 // 801^2: 18.9 us per step (cell form: 43 us), 14.3 us at the FP64 pipe's rate
 __global__ void __launch_bounds__(256)
-step2d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
+step2d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   const double *__restrict__ coefP, const double *__restrict__ dco,
                   const double *__restrict__ fre, const double *__restrict__ fim, Layout L,
-                  double c2, double a, double b, const OutSlot *__restrict__ slot, int flags,
+                  double c0, double a, double b, const OutSlot *__restrict__ slot, int flags,
                   RhsSet R)
 {
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -350,6 +386,7 @@ step2d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
     if (ix >= L.nx || iy >= L.ny) return;
     u += rhs * R.stride;
     um += rhs * R.stride;
+    out += rhs * R.stride;
     fre += rhs * R.stride;
     fim += rhs * R.stride;
     slot += rhs;
@@ -364,21 +401,22 @@ step2d_asm_kernel(const double *__restrict__ u, double *__restrict__ um,
                     c2p[c],           c3[c],                c4[c]};
     const double unew =
         asm2d_step(k, u[i - P - 1], u[i - P], u[i - P + 1], u[i - 1], u[i], u[i + 1], u[i + P - 1],
-                   u[i + P], u[i + P + 1], um[i], dco[i], fre[i], fim[i], c2, a, -b);
-    um[i] = unew;
+                   u[i + P], u[i + P + 1], um[i], dco[i], fre[i], fim[i], c0, a, -b);
+    out[i] = unew;
     if (flags) {
         if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = unew;
         if ((flags & 2) && slot->final_part) slot->final_part[2 * c] = unew;
     }
 }
 
-void launch_step_asm(const Layout &L, const double *u, double *um, const double *coefP,
-                     const double *dco, const double *fre, const double *fim, double c2, double a,
+void launch_step_asm(const Layout &L, const double *u, const double *um, double *out,
+                     const double *coefP,
+                     const double *dco, const double *fre, const double *fim, double c0, double a,
                      double b, const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R)
 {
     if (L.d == 2) {
         dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
-        step2d_asm_kernel<<<grd, dim3(32, 8), 0, s>>>(u, um, coefP, dco, fre, fim, L, c2, a, b,
+        step2d_asm_kernel<<<grd, dim3(32, 8), 0, s>>>(u, um, out, coefP, dco, fre, fim, L, c0, a, b,
                                                       slot, flags, R);
         ++g_launches;
         return;
@@ -390,7 +428,7 @@ void launch_step_asm(const Layout &L, const double *u, double *um, const double 
     const int nchunks = (int)((L.nz + zc - 1) / zc);
     dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + kAsmTY - 1) / kAsmTY),
              (unsigned)(nchunks * R.slots));
-    step3d_asm_kernel<<<grd, dim3(32, kAsmTY), 0, s>>>(u, um, coefP, dco, fre, fim, L, c2, a, b,
+    step3d_asm_kernel<<<grd, dim3(32, kAsmTY), 0, s>>>(u, um, out, coefP, dco, fre, fim, L, c0, a, b,
                                                        slot, flags, R, zc, nchunks);
     ++g_launches;
 }
@@ -798,8 +836,8 @@ void launch_assemble_H(const Layout &L, const double *kap64, const double S2[4],
 template <int D, bool kImH>
 __global__ void __launch_bounds__(256)
 apply_H_asm_kernel(int64_t nx, int64_t ny, int64_t nz, const double *__restrict__ coefP,
-                   const double *__restrict__ coefI, const double *__restrict__ imH, double ih2,
-                   const double2 *__restrict__ X, const double2 *__restrict__ F,
+                   const double *__restrict__ coefI, const double *__restrict__ imH, double h0,
+                   double ih2, const double2 *__restrict__ X, const double2 *__restrict__ F,
                    double2 *__restrict__ Y)
 {
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -821,7 +859,7 @@ apply_H_asm_kernel(int64_t nx, int64_t ny, int64_t nz, const double *__restrict_
                 const int64_t cn = c + ((int64_t)oz * ny + oy) * nx + ox;
                 const int lin = hlin(oz, oy, ox);
                 const int64_t ci = (lin >= 13) ? (lin - 13) * N + c : (13 - lin) * N + cn;
-                const double w = coefP[ci];
+                const double w = lin == 13 ? coefP[ci] + h0 : coefP[ci];
                 const double2 x = X[cn];
                 re = fma(w, x.x, re);
                 im = fma(w, x.y, im);
@@ -845,14 +883,14 @@ apply_H_asm_kernel(int64_t nx, int64_t ny, int64_t nz, const double *__restrict_
     Y[c] = y;
 }
 
-void launch_apply_H(const Layout &L, const double *coefP, const double *imH, double ih2,
+void launch_apply_H(const Layout &L, const double *coefP, const double *imH, double h0, double ih2,
                     const double2 *X, const double2 *F, double2 *Y, cudaStream_t s,
                     const double *coefI)
 {
     dim3 blk(32, 8);
     dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)L.nz);
 #define HTD_AH(DD, II) \
-    apply_H_asm_kernel<DD, II><<<grd, blk, 0, s>>>(L.nx, L.ny, L.nz, coefP, coefI, imH, ih2, X, F, Y)
+    apply_H_asm_kernel<DD, II><<<grd, blk, 0, s>>>(L.nx, L.ny, L.nz, coefP, coefI, imH, h0, ih2, X, F, Y)
     if (L.d == 3) {
         if (coefI) HTD_AH(3, true); else HTD_AH(3, false);
     } else {
@@ -1163,6 +1201,26 @@ template void launch_residual_planes<double>(const Layout &, const double2 *, co
                                              const int64_t *, int, double2 *, double *, double *,
                                              cudaStream_t);
 
+// (a call, not inlined: a conversion under a predicate takes the FP64 pipe for every
+// x, taken or not)
+__device__ __noinline__ double convert(float x) { return (double)x; }
+
+// (double)x without the conversion instruction, which GB300 issues at the FP64
+// pipe's two per clock and SM: the exponent rebiased and the mantissa moved by
+// integer instructions, exact for every finite x (a denormal, frequent ahead of a
+// wave front, is scaled by 2^24 first); infinities and NaNs are converted.
+__device__ __forceinline__ double widen(float x)
+{
+    const bool tiny = (__float_as_uint(x) & 0x7f800000u) == 0u;
+    const unsigned b = __float_as_uint(tiny ? __fmul_rn(x, 16777216.f) : x);
+    const unsigned bias = tiny ? 0x38000000u - (24u << 20) : 0x38000000u;
+    const unsigned hi = ((b & 0x7fffffffu) >> 3) + bias;
+    double r = __hiloint2double((int)((b & 0x80000000u) | ((b << 1) ? hi : 0u)), (int)(b << 29));
+    if ((b & 0x7f800000u) == 0x7f800000u) r = convert(x);
+    return r;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 template <typename T>
 struct TdGradCoef {
     T M[4];
@@ -1170,17 +1228,26 @@ struct TdGradCoef {
     double cR;      // beta dt omega_phys / (2 alpha omega)
 };
 
-// One term of the gradient sum, for the multiplier lam = lam_k and the states
-// u_k, u_{k-1}, u_{k-2} (all padded; the ghost ring is zero):
+// The terms k = k0, k0 - 1, .. k1 of the gradient sum of every source (grid.y), for
+// the multipliers lam_k and the states u_k, u_{k-1}, u_{k-2} (all padded; the ghost
+// ring is zero):
 //   gm[cell] += cm sum_{b,g corners} lam_b M_{|b-g|} u_{k-1,g}
 //   gR[node] += cR lam (u_k - u_{k-2})
-// One thread per cell (compact (n+1)^d order); the thread of cell a >= 0 also
-// does node a.  Products in the recurrence precision, sums in double.
+// lam_k is plane k % nlam of lam, u_k plane k - s0 + 2 of seg; a source's planes lie
+// sstride after the one's before, its sums gstride.  One thread per cell (compact
+// (n+1)^d order) keeps the cell's sum over all the terms; the thread of cell a >= 0
+// also does node a.  Products in the recurrence precision, sums in double, one
+// term after the other, so the result does not depend on how the run is cut.
+// One launch per segment instead of one per step: the sums are read and written once
+// per segment, and two FP64 multiply-adds per term are left of that pipe's work
+// (with the conversion instruction four: 334 us per segment of 40 steps at 512^2 with 4
+// sources, 83 % of the pipe; 270 without it, and waiting on the loads until the next
+// term's were issued ahead).
 template <typename T, int D>
 __global__ void __launch_bounds__(256)
-grad_td_kernel(Layout L, TdGradCoef<T> G, const T *__restrict__ lam, const T *__restrict__ uk,
-               const T *__restrict__ uk1, const T *__restrict__ uk2, double *__restrict__ gm,
-               double *__restrict__ gR)
+grad_td_kernel(Layout L, TdGradCoef<T> G, const T *__restrict__ lam, int nlam,
+               const T *__restrict__ seg, int64_t sstride, long long s0, long long k0, long long k1,
+               double *__restrict__ gm, double *__restrict__ gR, int64_t gstride)
 {
     const int64_t cx_n = L.nx + 1, cy_n = L.ny + 1, cz_n = (D == 3) ? L.nz + 1 : 1;
     const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1190,57 +1257,117 @@ grad_td_kernel(Layout L, TdGradCoef<T> G, const T *__restrict__ lam, const T *__
     const int64_t ay = rr % cy_n - 1;
     const int64_t az = (D == 3) ? rr / cy_n - 1 : 0;
     constexpr int nc = (D == 3) ? 8 : 4;
+    lam += blockIdx.y * sstride;
+    seg += blockIdx.y * sstride;
+    int64_t o[nc];                                 // corners from corner 0
+#pragma unroll
+    for (int b = 0; b < nc; ++b)
+        o[b] = (b & 1) + ((b >> 1) & 1) * L.pitch + ((b >> 2) & 1) * L.plane;
+    const int64_t i0 = L.node(ax, ay, az);
+    const bool node = gR && ax >= 0 && ay >= 0 && (D == 2 || az >= 0) && ax < L.nx && ay < L.ny &&
+                      (D == 2 || az < L.nz);
+    const int64_t n = (az * L.ny + ay) * L.nx + ax;
+    double sm = 0.0, sR = 0.0;
     if (gm) {
+        gm += blockIdx.y * gstride;
+        sm = gm[c];
+    }
+    T uk = T(0), uk1 = T(0);
+    if (node) {
+        gR += blockIdx.y * gstride;
+        sR = gR[n];
+        uk = seg[(k0 - s0 + 2) * L.total + i0];
+        uk1 = seg[(k0 - s0 + 1) * L.total + i0];
+    }
+    // the next term's operands are loaded before the present one is summed
+    int kl = (int)(k0 % nlam);
+    T ln[nc], un[nc], u2n = T(0);
+    auto load = [&](long long k) {
+        const T *lk = lam + kl * L.total + i0, *uq = seg + (k - s0 + 1) * L.total + i0;
+        if (--kl < 0) kl = nlam - 1;
+#pragma unroll
+        for (int b = 0; b < nc; ++b) {
+            ln[b] = lk[o[b]];
+            un[b] = uq[o[b]];
+        }
+        if (node) u2n = uq[-L.total];
+    };
+    load(k0);
+    for (long long k = k0; k >= k1; --k) {
         T l8[nc], u8[nc];
+        const T uk2 = u2n;
 #pragma unroll
         for (int b = 0; b < nc; ++b) {
-            const int64_t i = L.node(ax + (b & 1), ay + ((b >> 1) & 1), az + ((b >> 2) & 1));
-            l8[b] = lam[i];
-            u8[b] = uk1[i];
+            l8[b] = ln[b];
+            u8[b] = un[b];
         }
-        T acc = T(0);
+        if (k > k1) load(k - 1);
+        if (gm) {
+            T acc = T(0);
 #pragma unroll
-        for (int b = 0; b < nc; ++b) {
-            T row = T(0);
+            for (int b = 0; b < nc; ++b) {
+                T row = T(0);
 #pragma unroll
-            for (int g = 0; g < nc; ++g) row += G.M[__popc(b ^ g)] * u8[g];
-            acc += l8[b] * row;
+                for (int g = 0; g < nc; ++g) row += G.M[__popc(b ^ g)] * u8[g];
+                acc += l8[b] * row;
+            }
+            sm = fma(G.cm, widen(acc), sm);
         }
-        gm[c] += G.cm * (double)acc;
+        if (node) {
+            sR = fma(G.cR, widen(l8[0] * (uk - uk2)), sR);
+            uk = uk1;
+            uk1 = uk2;
+        }
     }
-    if (gR && ax >= 0 && ay >= 0 && (D == 2 || az >= 0) && ax < L.nx && ay < L.ny &&
-        (D == 2 || az < L.nz)) {
-        const int64_t i = L.node(ax, ay, az);
-        const int64_t n = (az * L.ny + ay) * L.nx + ax;
-        gR[n] += G.cR * (double)(lam[i] * (uk[i] - uk2[i]));
-    }
+    if (gm) gm[c] = sm;
+    if (node) gR[n] = sR;
 }
 
 template <typename T>
-void launch_grad_td(const Layout &L, const double M[4], double cm, double cR, const T *lam,
-                    const T *uk, const T *uk1, const T *uk2, double *gm, double *gR,
-                    cudaStream_t s)
+void launch_grad_td(const Layout &L, const double M[4], double cm, double cR, const T *lam, int nlam,
+                    const T *seg, int64_t sstride, int nsrc, long long s0, long long k0,
+                    long long k1, double *gm, double *gR, int64_t gstride, cudaStream_t s)
 {
     TdGradCoef<T> G;
     for (int k = 0; k < 4; ++k) G.M[k] = (T)M[k];
     G.cm = cm;
     G.cR = cR;
     const int64_t ncell = (L.nx + 1) * (L.ny + 1) * ((L.d == 3) ? L.nz + 1 : 1);
-    const int bs = 256;
+    const dim3 grd((unsigned)((ncell + 255) / 256), (unsigned)nsrc);
     if (L.d == 3)
-        grad_td_kernel<T, 3><<<(unsigned)((ncell + bs - 1) / bs), bs, 0, s>>>(L, G, lam, uk, uk1,
-                                                                             uk2, gm, gR);
+        grad_td_kernel<T, 3><<<grd, 256, 0, s>>>(L, G, lam, nlam, seg, sstride, s0, k0, k1, gm, gR,
+                                                 gstride);
     else
-        grad_td_kernel<T, 2><<<(unsigned)((ncell + bs - 1) / bs), bs, 0, s>>>(L, G, lam, uk, uk1,
-                                                                             uk2, gm, gR);
+        grad_td_kernel<T, 2><<<grd, 256, 0, s>>>(L, G, lam, nlam, seg, sstride, s0, k0, k1, gm, gR,
+                                                 gstride);
     ++g_launches;
 }
 template void launch_grad_td<float>(const Layout &, const double[4], double, double, const float *,
-                                    const float *, const float *, const float *, double *,
-                                    double *, cudaStream_t);
+                                    int, const float *, int64_t, int, long long, long long,
+                                    long long, double *, double *, int64_t, cudaStream_t);
 template void launch_grad_td<double>(const Layout &, const double[4], double, double,
-                                     const double *, const double *, const double *,
-                                     const double *, double *, double *, cudaStream_t);
+                                     const double *, int, const double *, int64_t, int, long long,
+                                     long long, long long, double *, double *, int64_t,
+                                     cudaStream_t);
+
+// out[i] += the sources' sums in order (nsrc of them, gstride apart)
+__global__ void __launch_bounds__(256)
+add_sources_kernel(double *__restrict__ out, const double *__restrict__ g, int64_t gstride, int nsrc,
+                   int64_t n)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    double v = out[i];
+    for (int q = 0; q < nsrc; ++q) v += g[q * gstride + i];
+    out[i] = v;
+}
+
+void launch_add_sources(double *out, const double *g, int64_t gstride, int nsrc, int64_t n,
+                        cudaStream_t s)
+{
+    add_sources_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(out, g, gstride, nsrc, n);
+    ++g_launches;
+}
 
 struct GradCoef {
     double M[4];

@@ -106,7 +106,7 @@ extern "C" htd_status htd_residual_norm_noalloc(htd_handle h, const void *F_dev,
     // every element read below is written first by this call: r by apply_H,
     // the partials by the dot kernels, the sums by the reductions; each
     // launch is checked as soon as it is made
-    htd::launch_apply_H(op.L64, op.coefP, op.imH, op.ih2,
+    htd::launch_apply_H(op.L64, op.coefP, op.imH, op.h0, op.ih2,
                         static_cast<const double2 *>(U_dev), static_cast<const double2 *>(F_dev),
                         r, s, op.coefI);
     if (failed(cudaGetLastError())) return HTD_ERR_CUDA;

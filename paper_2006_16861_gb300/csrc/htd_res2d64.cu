@@ -16,7 +16,7 @@
 // What bounds it: on small tiles the exchange (store, L2, load across the
 // chip: about a microsecond, which an exchange in every step paid twice as
 // often), on large ones the FP64 pipe (two operations per clock and SM).  One
-// node per thread keeps the dependent chain at 14 FP64 operations.  Measured on
+// node per thread keeps the dependent chain at 10 FP64 operations.  Measured on
 // GB300: a 101^2 Table 1 application (120 steps) 159 us; with one exchange per
 // step, node pairs and cell sums (33 operations per node) it took 429 us.
 //
@@ -85,7 +85,7 @@ __device__ __forceinline__ double value(const Raw &r)
 // [2 W, 4 W), columns 0, 1 at [4 W, 4 W + 2 H), columns w-1, w-2 behind them.
 __global__ void __launch_bounds__(kMaxThreads, 1)
 res2d64_kernel(const double *__restrict__ coefP, const double *__restrict__ dco,
-               const double *__restrict__ fre, const double *__restrict__ fim, Layout L, double c2,
+               const double *__restrict__ fre, const double *__restrict__ fim, Layout L, double c0,
                const double2 *__restrict__ ab, int nsteps, int jim, int jfin,
                const OutSlot *__restrict__ slot, unsigned long long *__restrict__ xbuf,
                int *__restrict__ err, int W, int H, Res2dProj<double> P)
@@ -208,7 +208,7 @@ res2d64_kernel(const double *__restrict__ coefP, const double *__restrict__ dco,
                         c[NA - 1],      c[NA],              c[2 * NA],      c[3 * NA],
                         c[4 * NA]};
         const double un = asm2d_step(k, u[-SW - 1], u[-SW], u[-SW + 1], u[-1], u[0], u[1], u[SW - 1],
-                                     u[SW], u[SW + 1], nxt[o], D[o], FR[o], FI[o], c2, a, nb);
+                                     u[SW], u[SW + 1], nxt[o], D[o], FR[o], FI[o], c0, a, nb);
         nxt[o] = un;
         return un;
     };
@@ -352,7 +352,7 @@ bool res2d64_plan(const Layout &L, Res2dPlan *out)
 }
 
 void launch_res2d64(const Res2dPlan &p, const double *coefP, const double *dco, const double *fre,
-                    const double *fim, const Layout &L, double c2, const double *ab, int nsteps,
+                    const double *fim, const Layout &L, double c0, const double *ab, int nsteps,
                     int jim, int jfin, const OutSlot *slot, unsigned long long *xbuf, int *err,
                     cudaStream_t s, const Res2dProj<double> &P)
 {
@@ -367,7 +367,7 @@ void launch_res2d64(const Res2dPlan &p, const double *coefP, const double *dco, 
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    (void)cudaLaunchKernelEx(&cfg, res2d64_kernel, coefP, dco, fre, fim, L, c2,
+    (void)cudaLaunchKernelEx(&cfg, res2d64_kernel, coefP, dco, fre, fim, L, c0,
                              reinterpret_cast<const double2 *>(ab), nsteps, jim, jfin, slot, xbuf,
                              err, p.W, p.H, P);
     ++g_launches;
