@@ -252,6 +252,13 @@ void free_ctx(htd_ctx *c)
     delete c;
 }
 
+// Consecutive step launches overlap (programmatic dependent launch) unless the handle's options say
+// HTD_LAUNCH_NO_OVERLAP.
+bool step_overlap(const htd_ctx *c)
+{
+    return !(c->opt.launch & HTD_LAUNCH_NO_OVERLAP);
+}
+
 // 1/h^2 as a factor of the assembled planes
 double h_factor(const htd_ctx *c)
 {
@@ -266,10 +273,10 @@ void one_step(htd_ctx *c, const T *u, const T *um, T *out, const T *fre, const T
 {
     if constexpr (std::is_same<T, double>::value)
         htd::launch_step_asm(c->Lr, u, um, out, c->coefP, (const double *)c->dco, fre, fim, c->C.c0,
-                             a, b, slot, flags, s, R);
+                             a, b, slot, flags, s, R, step_overlap(c));
     else
         htd::launch_step(c->Lr, u, um, out, (const T *)c->kap, (const T *)c->dco, fre, fim, C, a, b,
-                         slot, flags, s, R, force);
+                         slot, flags, s, R, force, step_overlap(c));
 }
 
 // one run of the resident-grid kernel from the handle's planes
@@ -287,13 +294,6 @@ void run_resident(htd_ctx *c, const StepCoef<T> &C, int jim, int jfin, cudaStrea
                              jfin, c->slot, c->res_x, c->err_dev, s, P);
 }
 
-// Consecutive launches of the blocked 2-D and the streamed 3-D step overlap
-// (programmatic dependent launch) unless the handle's options say
-// HTD_LAUNCH_NO_OVERLAP.
-bool step_overlap(const htd_ctx *c)
-{
-    return !(c->opt.launch & HTD_LAUNCH_NO_OVERLAP);
-}
 
 // One preconditioner run of T n_P steps; the forcing planes are already filled.
 // Table 1 / EXACT: the step kernels write the snapshot and final state into the
@@ -371,7 +371,8 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
             if (j + 1 == jfin) flags |= 2;
             htd::launch_abd_step<T>(L, cur, prv, nxt, (const T *)c->kap, (const T *)c->dco, cell,
                                     (const T *)c->fre, (const T *)c->fim, C, (T)c->atab[j],
-                                    (T)c->btab[j], cth, c->slot, flags, s, c->Rs);
+                                    (T)c->btab[j], cth, c->slot, flags, s, c->Rs,
+                                    step_overlap(c));
             if (project && j >= j_acc) accumulate(j, nxt);
             T *t = prv;
             prv = cur;

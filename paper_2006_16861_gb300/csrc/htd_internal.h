@@ -214,12 +214,12 @@ extern long long g_launches;
 // kernel writes or writes anything that kernel reads.  Launch errors are left
 // for cudaGetLastError.
 template <typename... KArgs, typename... Args>
-void launch_ex(void (*kern)(KArgs...), dim3 grd, unsigned threads, size_t smem, cudaStream_t s,
+void launch_ex(void (*kern)(KArgs...), dim3 grd, dim3 threads, size_t smem, cudaStream_t s,
                bool overlap, Args &&...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grd;
-    cfg.blockDim = dim3(threads);
+    cfg.blockDim = threads;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -231,11 +231,13 @@ void launch_ex(void (*kern)(KArgs...), dim3 grd, unsigned threads, size_t smem, 
 }
 
 // One FP32 step u_{j+1} -> out from u = u_j and um = u_{j-1} (out may be um); force
-// false: no forcing (a = b = 0).
+// false: no forcing (a = b = 0).  overlap (here and below): the launch may start
+// while the kernel before it drains; the one-step kernels wait for it before they
+// read or write a state.
 void launch_step(const Layout &L, const float *u, const float *um, float *out, const float *kap,
                  const float *dco, const float *fre, const float *fim, const StepCoef<float> &C,
                  float a, float b, const OutSlot *slot, int flags, cudaStream_t s,
-                 const RhsSet &R = RhsSet{}, bool force = true);
+                 const RhsSet &R = RhsSet{}, bool force = true, bool overlap = false);
 
 // The FP64 step from the assembled planes of launch_assemble_H scaled by -q
 // (see step3d_asm_kernel); c0 = 2 - p - q 2^d S_0.
@@ -243,7 +245,7 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
                      const double *coefP,
                      const double *dco, const double *fre, const double *fim, double c0, double a,
                      double b, const OutSlot *slot, int flags, cudaStream_t s,
-                     const RhsSet &R = RhsSet{});
+                     const RhsSet &R = RhsSet{}, bool overlap = false);
 
 template <typename T>
 void launch_split(const Layout &L, const double2 *F, T *fre, T *fim, int flip, cudaStream_t s);
@@ -258,7 +260,7 @@ template <typename T>
 void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *kap,
                      const T *damp, bool cell, const T *fre, const T *fim, const StepCoef<T> &C,
                      T a, T b, T cth, const OutSlot *slot, int flags, cudaStream_t s,
-                     const RhsSet &R = RhsSet{});
+                     const RhsSet &R = RhsSet{}, bool overlap = false);
 
 // ---- projection read-out (mode HTD_MODE_PROJECT) ------------------------------
 

@@ -56,6 +56,15 @@ static int sm_count()
 // recurrence step
 // ---------------------------------------------------------------------------
 
+// Programmatic dependent launch (no-op for an ordinary launch): the next kernel of
+// the stream may be scheduled as this one's blocks retire; from here on everything
+// the previous kernel wrote is visible.
+__device__ __forceinline__ void grid_dep_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // One step in 2-D, FP32: u_{j+1} -> out (which may be the plane um of u_{j-1}).  A
 // thread takes ROWS nodes of one column, so that a node costs 4.5 loads of u_j and 2.5
 // of q*kappa (nine and four with one row), all of them issued before the first sum.
@@ -69,6 +78,7 @@ step2d_kernel(const float *__restrict__ u, const float *um, float *out,
               StepCoef<float> C, float a, float b, const OutSlot *__restrict__ slot, int flags,
               RhsSet R, bool force)
 {
+    grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int64_t iy0 = ((int64_t)blockIdx.y * 8 + threadIdx.y) * ROWS;
     int rhs;
@@ -144,6 +154,7 @@ step3d_kernel(const float *__restrict__ u, const float *um, float *out,
               RhsSet R, int nchunks, bool force)
 {
     typedef float T;
+    grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -247,25 +258,25 @@ step3d_kernel(const float *__restrict__ u, const float *um, float *out,
 void launch_step(const Layout &L, const float *u, const float *um, float *out, const float *kap,
                  const float *dco, const float *fre, const float *fim, const StepCoef<float> &C,
                  float a, float b, const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R,
-                 bool force)
+                 bool force, bool overlap)
 {
     const unsigned gx = (unsigned)((L.nx + 31) / 32);
     if (L.d == 2) {
         const int64_t blocks4 = gx * ((L.ny + 31) / 32) * R.slots;
         if (blocks4 >= 2 * (int64_t)sm_count()) {
             dim3 grd(gx, (unsigned)((L.ny + 31) / 32), (unsigned)R.slots);
-            step2d_kernel<4><<<grd, dim3(32, 8), 0, s>>>(u, um, out, kap, dco, fre, fim, L, C, a,
-                                                         b, slot, flags, R, force);
+            launch_ex(step2d_kernel<4>, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre,
+                      fim, L, C, a, b, slot, flags, R, force);
         } else {
             dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
-            step2d_kernel<1><<<grd, dim3(32, 8), 0, s>>>(u, um, out, kap, dco, fre, fim, L, C, a,
-                                                         b, slot, flags, R, force);
+            launch_ex(step2d_kernel<1>, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre,
+                      fim, L, C, a, b, slot, flags, R, force);
         }
     } else {
         const int nchunks = (int)((L.nz + kZChunk - 1) / kZChunk);
         dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)(nchunks * R.slots));
-        step3d_kernel<<<grd, dim3(32, 8), 0, s>>>(u, um, out, kap, dco, fre, fim, L, C, a, b, slot,
-                                                  flags, R, nchunks, force);
+        launch_ex(step3d_kernel, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre, fim, L,
+                  C, a, b, slot, flags, R, nchunks, force);
     }
     ++g_launches;
 }
@@ -301,6 +312,7 @@ step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   double c0, double a, double b, const OutSlot *__restrict__ slot, int flags,
                   RhsSet R, int zc, int nchunks)
 {
+    grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * kAsmTY + threadIdx.y;
     int rhs;
@@ -379,6 +391,7 @@ step2d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   double c0, double a, double b, const OutSlot *__restrict__ slot, int flags,
                   RhsSet R)
 {
+    grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -412,12 +425,13 @@ step2d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
 void launch_step_asm(const Layout &L, const double *u, const double *um, double *out,
                      const double *coefP,
                      const double *dco, const double *fre, const double *fim, double c0, double a,
-                     double b, const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R)
+                     double b, const OutSlot *slot, int flags, cudaStream_t s, const RhsSet &R,
+                     bool overlap)
 {
     if (L.d == 2) {
         dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
-        step2d_asm_kernel<<<grd, dim3(32, 8), 0, s>>>(u, um, out, coefP, dco, fre, fim, L, c0, a, b,
-                                                      slot, flags, R);
+        launch_ex(step2d_asm_kernel, grd, dim3(32, 8), 0, s, overlap, u, um, out, coefP, dco, fre,
+                  fim, L, c0, a, b, slot, flags, R);
         ++g_launches;
         return;
     }
@@ -428,8 +442,8 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
     const int nchunks = (int)((L.nz + zc - 1) / zc);
     dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + kAsmTY - 1) / kAsmTY),
              (unsigned)(nchunks * R.slots));
-    step3d_asm_kernel<<<grd, dim3(32, kAsmTY), 0, s>>>(u, um, out, coefP, dco, fre, fim, L, c0, a, b,
-                                                       slot, flags, R, zc, nchunks);
+    launch_ex(step3d_asm_kernel, grd, dim3(32, kAsmTY), 0, s, overlap, u, um, out, coefP, dco, fre,
+              fim, L, c0, a, b, slot, flags, R, zc, nchunks);
     ++g_launches;
 }
 
@@ -457,6 +471,7 @@ abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict
                 const T *__restrict__ fre, const T *__restrict__ fim, Layout L, StepCoef<T> C,
                 T a, T b, T cth, const OutSlot *__restrict__ slot, int flags, RhsSet R, int nz)
 {
+    grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -524,14 +539,14 @@ template <typename T>
 void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *kap,
                      const T *damp, bool cell, const T *fre, const T *fim, const StepCoef<T> &C,
                      T a, T b, T cth, const OutSlot *slot, int flags, cudaStream_t s,
-                     const RhsSet &R)
+                     const RhsSet &R, bool overlap)
 {
     const int nz = (int)L.nz;
     dim3 blk(32, 8);
     dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)(nz * R.slots));
 #define HTD_ABD_LAUNCH(DD, CC)                                                                  \
-    abd_step_kernel<T, DD, CC><<<grd, blk, 0, s>>>(u, um, out, kap, damp, fre, fim, L, C, a, b, \
-                                                   cth, slot, flags, R, nz)
+    launch_ex(abd_step_kernel<T, DD, CC>, grd, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, \
+              L, C, a, b, cth, slot, flags, R, nz)
     if (L.d == 3) {
         if (cell) HTD_ABD_LAUNCH(3, true); else HTD_ABD_LAUNCH(3, false);
     } else {
@@ -543,11 +558,12 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
 template void launch_abd_step<float>(const Layout &, const float *, const float *, float *,
                                      const float *, const float *, bool, const float *,
                                      const float *, const StepCoef<float> &, float, float, float,
-                                     const OutSlot *, int, cudaStream_t, const RhsSet &);
+                                     const OutSlot *, int, cudaStream_t, const RhsSet &, bool);
 template void launch_abd_step<double>(const Layout &, const double *, const double *, double *,
                                       const double *, const double *, bool, const double *,
                                       const double *, const StepCoef<double> &, double, double,
-                                      double, const OutSlot *, int, cudaStream_t, const RhsSet &);
+                                      double, const OutSlot *, int, cudaStream_t, const RhsSet &,
+                                      bool);
 
 // ---------------------------------------------------------------------------
 // projection read-out: compensated sums of e^{-i theta_j} u_j
