@@ -464,7 +464,7 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
 // sum_o M_s (sum of damp over the shared cells) w_{beta+o}).  Reads u_{n-1} at
 // the neighbours in the cell case, so u_{n+1} goes to a third plane.
 
-template <typename T, int D, bool kCell>
+template <typename T, bool kCell>
 __global__ void __launch_bounds__(256)
 abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict__ out,
                 const T *__restrict__ kap, const T *__restrict__ damp,
@@ -487,7 +487,7 @@ abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict
     slot += rhs;
     const int64_t P = L.pitch, Q = L.plane;
     const int64_t i = L.node(ix, iy, iz);
-    constexpr int NC = 1 << D;
+    constexpr int D = 3, NC = 1 << D;
     // the node's cells, bit t of index c: upper (1) or lower (0) cell along axis t
     // (t = 0: x, 1: y, 2: z)
     T kc[NC], dc[NC];
@@ -535,6 +535,97 @@ abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict
     }
 }
 
+// The 2-D step, ROWS nodes of a column per thread with all operands loaded before
+// the first sum (a row of u_n and u_{n-1} serves the nodes above and below it too);
+// the expressions and their order are abd_step_kernel's.  ROWS: the most of 4, 2, 1
+// that leaves two blocks per SM.  401^2 cell damping: 2.0 us per step (two rows), 3.0 with
+// the per-node loads of the 3-D form.
+template <typename T, bool kCell, int ROWS>
+__global__ void __launch_bounds__(256)
+abd_step2d_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict__ out,
+                  const T *__restrict__ kap, const T *__restrict__ damp,
+                  const T *__restrict__ fre, const T *__restrict__ fim, Layout L, StepCoef<T> C,
+                  T a, T b, T cth, const OutSlot *__restrict__ slot, int flags, RhsSet R)
+{
+    const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    const int64_t iy0 = ((int64_t)blockIdx.y * 8 + threadIdx.y) * ROWS;
+    const bool in = ix < L.nx && iy0 < L.ny;
+    const int64_t P = L.pitch, i0 = (iy0 + 1) * P + L.xl + ix;
+    int64_t at[ROWS + 2];                   // row r - 1; rows below the grid: its last ghost row
+#pragma unroll
+    for (int r = 0; r < ROWS + 2; ++r) at[r] = i0 + (min(iy0 + r - 1, L.ny) - iy0) * P;
+    // the coefficients, which no step writes, before the wait for the previous step
+    T k[ROWS + 1][2], dc[ROWS + 1][2], dn[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS + 1; ++r)
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+            k[r][x] = in ? kap[at[r] + x - 1] : T(0);
+            dc[r][x] = kCell && in ? damp[at[r] + x - 1] : T(0);
+        }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) dn[r] = !kCell && in ? damp[at[r + 1]] : T(0);
+    grid_dep_begin();
+    int rhs;
+    if (!rhs_of_slot(R, (int)blockIdx.z, rhs)) return;
+    if (!in) return;
+    const int64_t off = rhs * R.stride;
+    u += off;
+    um += off;
+    out += off;
+    fre += off;
+    fim += off;
+    slot += rhs;
+    constexpr int MX = kCell ? 3 : 1;       // columns of u_{n-1} read
+    T w[ROWS + 2][3], wm[ROWS + 2][3], fr[ROWS], fi[ROWS];
+#pragma unroll
+    for (int r = 0; r < ROWS + 2; ++r) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x) w[r][x] = u[at[r] + x - 1];
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+            wm[r][x] = (MX == 3 || (x == 1 && r >= 1 && r <= ROWS)) ? um[at[r] + x - 1] : T(0);
+    }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        fr[r] = fre[at[r + 1]];
+        fi[r] = fim[at[r + 1]];
+    }
+#pragma unroll
+    for (int r = 0; r < ROWS; ++r) {
+        if (r > 0 && iy0 + r >= L.ny) break;
+        T accA = T(0), accB = T(0);
+#pragma unroll
+        for (int oy = -1; oy <= 1; ++oy)
+#pragma unroll
+            for (int ox = -1; ox <= 1; ++ox) {
+                const int sh = (ox != 0) + (oy != 0);
+                T ks = T(0), ds = T(0);
+#pragma unroll
+                for (int cidx = 0; cidx < 4; ++cidx) {
+                    const int ax = cidx & 1, ay = cidx >> 1;
+                    if ((ox == 0 || ox == 2 * ax - 1) && (oy == 0 || oy == 2 * ay - 1)) {
+                        ks += k[r + ay][ax];
+                        if (kCell) ds += dc[r + ay][ax];
+                    }
+                }
+                const T v = w[r + 1 + oy][1 + ox];
+                const T coef = (sh == 0) ? C.c0 + C.mt[0] * ks : C.mt[sh] * ks - C.cs[sh];
+                accA += coef * v;
+                if (kCell) accB += C.mt[sh] * ds * (cth * v - wm[r + 1 + oy][1 + ox]);
+            }
+        const T prev = wm[r + 1][1];
+        if (!kCell) accB = dn[r] * (cth * w[r + 1][1] - prev);
+        const T unew = accA - prev - accB + (a * fr[r] - b * fi[r]);
+        out[at[r + 1]] = unew;
+        if (flags) {
+            const int64_t c = (iy0 + r) * L.nx + ix;
+            if ((flags & 1) && slot->snap_part) slot->snap_part[2 * c] = (double)unew;
+            if ((flags & 2) && slot->final_part) slot->final_part[2 * c] = (double)unew;
+        }
+    }
+}
+
 template <typename T>
 void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *kap,
                      const T *damp, bool cell, const T *fre, const T *fim, const StepCoef<T> &C,
@@ -544,15 +635,34 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
     const int nz = (int)L.nz;
     dim3 blk(32, 8);
     dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)(nz * R.slots));
-#define HTD_ABD_LAUNCH(DD, CC)                                                                  \
-    launch_ex(abd_step_kernel<T, DD, CC>, grd, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, \
-              L, C, a, b, cth, slot, flags, R, nz)
-    if (L.d == 3) {
-        if (cell) HTD_ABD_LAUNCH(3, true); else HTD_ABD_LAUNCH(3, false);
+    if (L.d == 2) {
+        const unsigned gx = (unsigned)((L.nx + 31) / 32);
+        auto blocks = [&](int rows) { return (L.ny + 8 * rows - 1) / (8 * rows); };
+        auto fits = [&](int rows) {
+            return gx * blocks(rows) * R.slots >= 2 * (int64_t)sm_count();
+        };
+        const int rows = fits(4) ? 4 : fits(2) ? 2 : 1;
+        const dim3 grd2(gx, (unsigned)blocks(rows), (unsigned)R.slots);
+        auto go = [&](auto kern) {
+            launch_ex(kern, grd2, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, L, C, a, b,
+                      cth, slot, flags, R);
+        };
+        if (cell) {
+            if (rows == 4) go(abd_step2d_kernel<T, true, 4>);
+            else if (rows == 2) go(abd_step2d_kernel<T, true, 2>);
+            else go(abd_step2d_kernel<T, true, 1>);
+        } else {
+            if (rows == 4) go(abd_step2d_kernel<T, false, 4>);
+            else if (rows == 2) go(abd_step2d_kernel<T, false, 2>);
+            else go(abd_step2d_kernel<T, false, 1>);
+        }
+    } else if (cell) {
+        launch_ex(abd_step_kernel<T, true>, grd, blk, 0, s, overlap, u, um, out, kap, damp, fre,
+                  fim, L, C, a, b, cth, slot, flags, R, nz);
     } else {
-        if (cell) HTD_ABD_LAUNCH(2, true); else HTD_ABD_LAUNCH(2, false);
+        launch_ex(abd_step_kernel<T, false>, grd, blk, 0, s, overlap, u, um, out, kap, damp, fre,
+                  fim, L, C, a, b, cth, slot, flags, R, nz);
     }
-#undef HTD_ABD_LAUNCH
     ++g_launches;
 }
 template void launch_abd_step<float>(const Layout &, const float *, const float *, float *,
