@@ -274,9 +274,14 @@ htd_status build_resident(htd_batch b)
         smem = std::max(smem, p.smem);
         ctas += p.ntx * p.nty;
     }
-    HTD_CUDA(htd::dev_malloc(&b->rab, sizeof(float) * ab_n));
-    HTD_CUDA(htd::dev_malloc(&b->rx, sizeof(unsigned long long) * xw));
-    HTD_CUDA(htd::dev_malloc(&b->rinst, sizeof(htd::Res2dInst) * n));
+    cudaError_t e = htd::dev_malloc(&b->rab, sizeof(float) * ab_n);
+    if (e == cudaSuccess) e = htd::dev_malloc(&b->rx, sizeof(unsigned long long) * xw);
+    if (e == cudaSuccess) e = htd::dev_malloc(&b->rinst, sizeof(htd::Res2dInst) * n);
+    if (e == cudaErrorMemoryAllocation) {    // the handles' own sequences need none of it
+        (void)cudaGetLastError();
+        return HTD_OK;
+    }
+    HTD_CUDA(e);
     std::vector<htd::Res2dInst> inst;
     std::vector<float> ab(ab_n);
     size_t ab_at = 0, x_at = 0;

@@ -48,3 +48,32 @@ def test_batch_equals_single_handles(name, mode):
             assert np.isfinite(u[q]).all() and np.abs(u[q]).max() > 0
             assert np.array_equal(u[q], host(s.precond(f[q])))
         s.close()
+
+
+def test_no_memory_for_the_resident_launch_leaves_the_handles_sequences():
+    """An allocation that fails while a batch is built is reported as before (2: out of
+    memory), except those of the resident launch, which the handles' own sequences
+    replace: same outputs."""
+    solvers, F = [], []
+    for k, n in enumerate([(65, 70), (120, 33)]):
+        solvers.append(htd.Solver(het_problem(2, n, T=2, layer=2, seed=30 + k), precision="mixed"))
+        F.append(dev(W.random_rhs(60 + k, n)[None]))
+    want = [host(s.precond(f[0])) for s, f in zip(solvers, F)]
+    built = 0
+    for k in range(24):
+        htd.htd_test_fail_alloc(k)
+        try:
+            b = htd.Batch(solvers, [1, 1])
+        except htd.HtdError as e:
+            assert e.status == 2
+            continue
+        finally:
+            htd.htd_test_fail_alloc(-1)
+        built += 1
+        b.set_form(1)
+        for u, w in zip(b.precond(F), want):
+            assert np.array_equal(host(u)[0], w)
+        b.close()
+    assert built >= 4                       # the three of the resident launch, and none
+    for s in solvers:
+        s.close()
