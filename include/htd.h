@@ -253,7 +253,8 @@ typedef struct {
     long long steps;         /* recurrence steps per real run: T * nP */
     int steps_per_launch;    /* recurrence steps per kernel launch (temporal
                                 blocking; 1 = one step per launch; T * nP for the
-                                resident-grid kernel; 0 in htd_plan, which does not
+                                resident-grid kernel, fewer where it runs over
+                                windows of a larger grid; 0 in htd_plan, which does not
                                 look at the device) */
     int tile[3];             /* owned tile (x, y) of the blocked or resident-grid
                                 2-D step kernel and its columns per thread (1, or
@@ -266,7 +267,8 @@ typedef struct {
                                 (gather / z-march), 1 temporally blocked 2-D
                                 (TMA tiles), 2 TMA-streamed 3-D, 3 one-step
                                 backward differences (HTD_ABD), 4 resident-grid
-                                2-D (one launch per run); -1 in htd_plan */
+                                2-D (one launch per run, or per window and pass
+                                of a larger grid); -1 in htd_plan */
     int rhs_per_cta;         /* right-hand sides one CTA of the step kernel works
                                 on (1 or 2); 0 in htd_plan */
 } htd_params;

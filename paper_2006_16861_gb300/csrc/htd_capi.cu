@@ -165,6 +165,7 @@ struct htd_ctx {
     // resident-grid 2-D step (FP32, one rhs): a whole run in one cooperative launch
     htd::Res2dPlan res{};
     bool use_res = false;
+    htd::Res2dWin win;          // n > 0: over windows of the grid (FP32)
     void *res_ab = nullptr;                 // a_j, b_j per step, in the recurrence precision
     void *res_w = nullptr;                  // projection weights per phase (PROJECT)
     unsigned long long *res_x = nullptr;    // edge exchange buffer
@@ -279,18 +280,23 @@ void one_step(htd_ctx *c, const T *u, const T *um, T *out, const T *fre, const T
                          slot, flags, s, R, force, step_overlap(c));
 }
 
-// one run of the resident-grid kernel from the handle's planes
+// one run of the resident-grid kernel (its first nsteps steps) from the handle's planes
 template <typename T>
-void run_resident(htd_ctx *c, const StepCoef<T> &C, int jim, int jfin, cudaStream_t s,
+void run_resident(htd_ctx *c, const StepCoef<T> &C, int nsteps, int jim, int jfin, cudaStream_t s,
                   const htd::Res2dProj<T> &P)
 {
     if constexpr (std::is_same<T, double>::value)
         htd::launch_res2d64(c->res, c->coefP, (const double *)c->dco, (const double *)c->fre,
                             (const double *)c->fim, c->Lr, c->C.c0, (const double *)c->res_ab,
-                            (int)c->nsteps, jim, jfin, c->slot, c->res_x, c->err_dev, s, P);
-    else
+                            nsteps, jim, jfin, c->slot, c->res_x, c->err_dev, s, P);
+    else if (c->win.n) {
+        float *planes[4] = {(float *)c->u0, (float *)c->u1, (float *)c->u2, (float *)c->u3};
+        htd::launch_res2d_win(c->win, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
+                              (const T *)c->fim, c->Lr, C, (const T *)c->res_ab, nsteps, jim, jfin,
+                              c->slot, c->res_x, c->err_dev, planes, s, P);
+    } else
         htd::launch_res2d(c->res, (const T *)c->kap, (const T *)c->dco, (const T *)c->fre,
-                             (const T *)c->fim, c->Lr, C, (const T *)c->res_ab, (int)c->nsteps, jim,
+                             (const T *)c->fim, c->Lr, C, (const T *)c->res_ab, nsteps, jim,
                              jfin, c->slot, c->res_x, c->err_dev, s, P);
 }
 
@@ -310,7 +316,8 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
     const long long jim = project ? -1 : c->nsteps - c->nP / 4;
     const long long jfin = project ? -1 : c->nsteps;
     if (c->use_res) {
-        // the whole run in one launch; the global state planes are not used.
+        // the whole run in one launch, the global state planes not used, or in one per
+        // window and pass.
         // PROJECT: the kernel accumulates the window's states itself, then the
         // finishing kernel writes (2 / n_acc) times the sums
         htd::Res2dProj<T> P;
@@ -323,7 +330,7 @@ htd_status run_steps_direct(htd_ctx *c, cudaStream_t s)
             P.N = L.N;
             HTD_CUDA(cudaMemsetAsync(c->acc, 0, sizeof(T) * 4 * L.N, s));
         }
-        run_resident<T>(c, C, (int)jim, (int)jfin, s, P);
+        run_resident<T>(c, C, (int)c->nsteps, (int)jim, (int)jfin, s, P);
         if (project)
             htd::launch_project_finish<T>(L.N, (const T *)c->acc, 4 * L.N, 2.0 / (double)n_res,
                                           c->slot, c->Rs, s);
@@ -724,9 +731,16 @@ template <typename T>
 htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1)
 {
     if (c->rcap != 1 || c->nsteps >= (1LL << 30)) return HTD_OK;
-    if (!(std::is_same<T, double>::value ? htd::res2d64_plan(c->Lr, &c->res)
-                                         : htd::res2d_plan(c->Lr, &c->res)))
-        return HTD_OK;
+    if (std::is_same<T, double>::value) {
+        if (!htd::res2d64_plan(c->Lr, &c->res)) return HTD_OK;
+    } else if (!htd::res2d_plan(c->Lr, &c->res)) {
+        // too large for the SMs: window by window, if the second pair of state planes
+        // is there
+        if (!c->u2 || !c->u3 || !htd::res2d_win_plan(c->Lr, c->nsteps, &c->win)) return HTD_OK;
+        c->res = c->win.plan;
+    }
+    // (windows: two passes, to count their loads and stores)
+    const int tsteps = (int)(c->win.n ? std::min<long long>(c->nsteps, 2 * c->win.B) : c->nsteps);
     if (c->opt.mode == HTD_MODE_PROJECT) {
         // projection weights per phase k of the new state: cos and -sin of
         // 2 pi k / nP, rounded as for the separate accumulation kernel
@@ -750,14 +764,14 @@ htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cud
     const StepCoef<T> C = cast_coef<T>(c->C);
     for (int r = 0; r < 2; ++r) {
         if (r == 1) HTD_CUDA(cudaEventRecord(e0, s));
-        run_resident<T>(c, C, -1, -1, s, htd::Res2dProj<T>{});
+        run_resident<T>(c, C, tsteps, -1, -1, s, htd::Res2dProj<T>{});
     }
     HTD_CUDA(cudaEventRecord(e1, s));
     HTD_CUDA(cudaEventSynchronize(e1));
     HTD_CUDA(cudaGetLastError());
     float ms = 0.f;
     HTD_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-    const float us = 1e3f * ms / (float)c->nsteps;
+    const float us = 1e3f * ms / (float)tsteps;
     if (force || us < c->step_us) {
         c->use_res = true;
         c->step_us = us;
@@ -768,6 +782,7 @@ htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cud
         c->res_ab = nullptr;
         c->res_x = nullptr;
         c->res_w = nullptr;
+        c->win.n = 0;
     }
     return HTD_OK;
 }
@@ -1996,7 +2011,7 @@ htd_status htd_get_params(htd_handle h, htd_params *out)
     P.nP = h->nP;
     P.T = h->T;
     P.steps = h->nsteps;
-    P.steps_per_launch = h->use_res ? (int)h->nsteps : h->use_tb ? h->tb.B : 1;
+    P.steps_per_launch = h->use_res ? (h->win.n ? h->win.B : (int)h->nsteps) : h->use_tb ? h->tb.B : 1;
     P.tile[0] = h->use_res ? h->res.W : h->use_tb ? h->tb.TX : 0;
     P.tile[1] = h->use_res ? h->res.H : h->use_tb ? h->tb.TY : 0;
     P.tile[2] = h->use_res ? (h->esz == 8 ? 1 : 2) : h->use_tb ? (h->tb.pair ? 2 : 1) : 0;

@@ -451,7 +451,31 @@ struct Res2dInst {
     int cta0 = 0;
     RhsSet R;
     int k = 0;
+    // a window's pass: u_j, u_{j-1} (null: at rest) and, after it, u_{j+B}, u_{j+B-1}
+    // (null: not kept); owned columns and rows; the window's place in the grid of rows
+    // of gnx nodes; its first step; exchange tags already used
+    const float *s0 = nullptr, *s1 = nullptr;
+    float *o0 = nullptr, *o1 = nullptr;
+    int own[4] = {0, 0, 0, 0};
+    int gx = 0, gy = 0, gnx = 0, jbase = 0;
+    unsigned tag0 = 0;
+    int pad = 0;
 };
+
+// Windows of a grid that does not fit the SMs (htd_res2d.cu): n of `len` nodes along an axis (0: x, 1: y), B steps per pass
+struct Res2dWin {
+    int n = 0, B = 0, axis = 0, len = 0;
+    Res2dPlan plan;              // of one window
+};
+bool res2d_win_plan(const Layout &L, long long nsteps, Res2dWin *w);
+// As launch_res2d, for a grid that does not fit the SMs: passes of B steps, in each of
+// which every window in turn is loaded, run for B steps and stored.  The passes
+// alternate between the state pairs planes[0..1] and planes[2..3].
+void launch_res2d_win(const Res2dWin &w, const float *kap, const float *dco, const float *fre,
+                      const float *fim, const Layout &L, const StepCoef<float> &C, const float *ab,
+                      int nsteps, int jim, int jfin, const OutSlot *slot, unsigned long long *xbuf,
+                      int *err, float *const planes[4], cudaStream_t s,
+                      const Res2dProj<float> &P = Res2dProj<float>{});
 
 // Plans for several instances run by one launch (each on its share of the SMs), or
 // false if they do not fit the device together.

@@ -36,6 +36,14 @@
 // node pairs, and taking the halo pairs' own halves from registers, cost moves
 // (1001^2: 2.12).
 //
+// A grid that does not fit the SMs (more than about 1.5 M nodes) runs window by
+// window: strips along one axis, each loaded, run for B steps and stored, with B more
+// nodes on its inner sides (res2d_win_plan).  Against the blocked kernel, which
+// recomputes half of each tile's work in its rims and reloads everything every 4 or
+// 8 steps: 1501 x 2001 7.6 us per step (three windows, 64 steps) against 9.7 .. 10.2;
+// 2001^2 stays with the blocked kernel (10.9), whose tiles happen to fit it.  What
+// bounds a pass is the resident steps and about 30 us of launch, loads and stores.
+//
 // An exchanged value is one 64-bit word, its bits beside a tag (index of the
 // exchange + 1), so no fence orders data before a flag.  Before a CTA publishes
 // exchange e + 2 it has read its neighbours' e + 1, which they published after
@@ -49,6 +57,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 #include <vector>
 
@@ -60,6 +69,7 @@ namespace {
 
 constexpr int kThreads = 512;        // at most; 128 registers each
 constexpr int kMaxRows = 10;         // row pairs per thread, 1 .. kMaxRows
+constexpr int kWinRows = 6;          // row pairs of a window's plan, kWinRows .. kMaxRows
 constexpr int kPer = 2;              // edge nodes and ring slots per thread kept in registers
 
 __device__ __forceinline__ unsigned long long global_ns()
@@ -129,8 +139,10 @@ __device__ __forceinline__ int edge_rank(int lx, int ly, int w, int h)
 }
 
 // One run of the instance I, as the CTA of its tile (tx, ty).  kGroup: for slot I.k of
-// the handle's active list, else for its only rhs.
-template <int RPT, bool kGroup>
+// the handle's active list, else for its only rhs.  kWin: one pass over a window of a
+// larger grid (see launch_res2d_win): states from and to memory, outputs of the owned
+// nodes only.
+template <int RPT, bool kGroup, bool kWin>
 __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, const Res2dProj<float> &P)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -174,11 +186,15 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
         K[i] = 0.f;
     }
     __syncthreads();
-    // cells (lower corner lx, ly), those of the domain's nodes
+    // cells (lower corner lx, ly), those of the domain's nodes; a window's u_j
+    const float *__restrict__ s0 = kWin ? I.s0 : nullptr, *__restrict__ s1 = kWin ? I.s1 : nullptr;
+#pragma unroll 4
     for (int i = tid; i < (W + 4) * (H + 4); i += NT) {
         const int lx = i % (W + 4) - 2, ly = i / (W + 4) - 2;
-        if (x0 + lx >= -1 && x0 + lx < nx && y0 + ly >= -1 && y0 + ly < ny)
+        if (x0 + lx >= -1 && x0 + lx < nx && y0 + ly >= -1 && y0 + ly < ny) {
             K[G.at(lx, ly)] = kap[gidx(lx, ly)];
+            if (kWin && s0 && x0 + lx >= 0 && y0 + ly >= 0) U0[G.at(lx, ly)] = s0[gidx(lx, ly)];
+        }
     }
     // this thread's strip: column lx, rows ly0 + i and ly0 + RPT + i.  Nodes
     // outside the domain or beyond the ring layer have d = 0 and no forcing, so
@@ -197,12 +213,20 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
         if (has && lx <= w && la <= h && in_domain(lx, la)) {
             const int64_t g = gidx(lx, la);
             dd[i].x = dco[g];
+            if (kWin && s0) {
+                za[i].x = s0[g];
+                zb[i].x = s1[g];
+            }
             f.x = fre[g];
             f.z = fim[g];
         }
         if (has && lx <= w && lb <= h && in_domain(lx, lb)) {
             const int64_t g = gidx(lx, lb);
             dd[i].y = dco[g];
+            if (kWin && s0) {
+                za[i].y = s0[g];
+                zb[i].y = s1[g];
+            }
             f.y = fre[g];
             f.w = fim[g];
         }
@@ -245,6 +269,7 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
             EI[t] = make_int4(G.at(ex, ey), G.at(ex, ey - 1), G.at(ex, ey + 1), 0);
             const int64_t g = gidx(ex, ey);
             EC[t] = make_float4(dco[g], fre[g], fim[g], 0.f);
+            if (kWin && s0) e_prev[k] = s0[g];
         }
     }
     // ring slot k: rows -2, -1, h, h+1 over w + 4 columns, then columns -2, -1, w,
@@ -280,8 +305,9 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
     // word v (read from p) of exchange e into U0[dst], read again until it carries
     // the tag (bounded by the handle's limit; with the stall test the first wait
     // of CTA (0, 0) expects a tag no word has)
+    const unsigned tag0 = kWin ? I.tag0 : 0u;
     auto complete = [&](const unsigned long long *p, unsigned long long v, int e, int dst) {
-        unsigned want = (unsigned)(e + 1);
+        unsigned want = tag0 + (unsigned)(e + 1);
         if (e == 0 && tx == 0 && ty == 0 && *(volatile const int *)(err + 1) != 0)
             want = 0xffffffffu;
         if ((unsigned)(v >> 32) != want) {
@@ -384,16 +410,21 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
         const float ag = vfma(abj.x, e.y, vfma(-abj.y, e.z, acc));
         return vfma(e.x, vfma(-2.f, prev, ag), prev);
     };
+    auto owned = [&](int lx, int ly) {
+        return x0 + lx >= I.own[0] && x0 + lx < I.own[1] && y0 + ly >= I.own[2] && y0 + ly < I.own[3];
+    };
     // outputs of the new state of step j (tile nodes of U): snapshot, final state,
     // and in projection mode the compensated sums of the window's states (as the
     // separate accumulation kernel adds them)
     auto read_out = [&](const float *U, int j) {
         const bool acc = j >= P.j_acc;
-        const int ph = acc ? (j + 1) % P.nP : 0;
+        const int ph = acc ? ((kWin ? I.jbase : 0) + j + 1) % P.nP : 0;
         const float wc = acc ? P.w[2 * ph] : 0.f, ws = acc ? P.w[2 * ph + 1] : 0.f;
         for (int i = tid; i < w * h; i += NT) {
             const int ly = i / w, lx = i - ly * w;
-            const int64_t c = (int64_t)(y0 + ly) * nx + x0 + lx;
+            if (kWin && !owned(lx, ly)) continue;
+            const int64_t c = kWin ? (int64_t)(I.gy + y0 + ly) * I.gnx + I.gx + x0 + lx
+                                   : (int64_t)(y0 + ly) * nx + x0 + lx;
             const float v = U[G.at(lx, ly)];
             if (j + 1 == jim && slot->snap_part) slot->snap_part[2 * c] = (double)v;
             if (j + 1 == jfin && slot->final_part) slot->final_part[2 * c] = (double)v;
@@ -434,7 +465,7 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
                 const int t = tid + k * NT;
                 if (t < nE) {
                     e_prev[k] = edge_value(EI[t], EC[t], e_prev[k], abB);
-                    st_word(pub + t, e_prev[k], (unsigned)(e + 1));
+                    st_word(pub + t, e_prev[k], tag0 + (unsigned)(e + 1));
                 }
             }
         }
@@ -450,13 +481,28 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
         if (s_abort) break;
         if (reads(j + 1)) read_out(U0, j + 1);
     }
+    if (kWin && I.o0) {
+        for (int i = tid; i < w * h; i += NT) {
+            const int ly = i / w, lx = i - ly * w;
+            if (!owned(lx, ly)) continue;
+            I.o0[gidx(lx, ly)] = U0[G.at(lx, ly)];
+            I.o1[gidx(lx, ly)] = U1[G.at(lx, ly)];
+        }
+    }
 }
 
 template <int RPT>
 __global__ void __launch_bounds__(kThreads, 1)
 res2d_kernel(const __grid_constant__ Res2dInst I, const __grid_constant__ Res2dProj<float> P)
 {
-    res2d_run<RPT, false>(I, blockIdx.x, blockIdx.y, P);
+    res2d_run<RPT, false, false>(I, blockIdx.x, blockIdx.y, P);
+}
+
+template <int RPT>
+__global__ void __launch_bounds__(kThreads, 1)
+res2d_win_kernel(const __grid_constant__ Res2dInst I, const __grid_constant__ Res2dProj<float> P)
+{
+    res2d_run<RPT, false, true>(I, blockIdx.x, blockIdx.y, P);
 }
 
 // Several instances in one launch, instance i on the CTAs from inst[i].cta0 up to
@@ -477,16 +523,16 @@ res2d_group_kernel(const Res2dInst *__restrict__ inst, int n)
     const int tx = t % I.ntx, ty = t / I.ntx;
     const Res2dProj<float> P;
     switch (I.rpt) {
-    case 1: res2d_run<1, true>(I, tx, ty, P); break;
-    case 2: res2d_run<2, true>(I, tx, ty, P); break;
-    case 3: res2d_run<3, true>(I, tx, ty, P); break;
-    case 4: res2d_run<4, true>(I, tx, ty, P); break;
-    case 5: res2d_run<5, true>(I, tx, ty, P); break;
-    case 6: res2d_run<6, true>(I, tx, ty, P); break;
-    case 7: res2d_run<7, true>(I, tx, ty, P); break;
-    case 8: res2d_run<8, true>(I, tx, ty, P); break;
-    case 9: res2d_run<9, true>(I, tx, ty, P); break;
-    default: res2d_run<10, true>(I, tx, ty, P); break;
+    case 1: res2d_run<1, true, false>(I, tx, ty, P); break;
+    case 2: res2d_run<2, true, false>(I, tx, ty, P); break;
+    case 3: res2d_run<3, true, false>(I, tx, ty, P); break;
+    case 4: res2d_run<4, true, false>(I, tx, ty, P); break;
+    case 5: res2d_run<5, true, false>(I, tx, ty, P); break;
+    case 6: res2d_run<6, true, false>(I, tx, ty, P); break;
+    case 7: res2d_run<7, true, false>(I, tx, ty, P); break;
+    case 8: res2d_run<8, true, false>(I, tx, ty, P); break;
+    case 9: res2d_run<9, true, false>(I, tx, ty, P); break;
+    default: res2d_run<10, true, false>(I, tx, ty, P); break;
     }
 }
 
@@ -504,6 +550,18 @@ void with_kernel(int rpt, Fn &&fn)
     case 8: fn(res2d_kernel<8>); break;
     case 9: fn(res2d_kernel<9>); break;
     default: fn(res2d_kernel<10>); break;
+    }
+}
+
+template <typename Fn>
+void with_win_kernel(int rpt, Fn &&fn)
+{
+    switch (rpt) {
+    case 6: fn(res2d_win_kernel<6>); break;
+    case 7: fn(res2d_win_kernel<7>); break;
+    case 8: fn(res2d_win_kernel<8>); break;
+    case 9: fn(res2d_win_kernel<9>); break;
+    default: fn(res2d_win_kernel<10>); break;
     }
 }
 
@@ -543,6 +601,7 @@ bool res2d_device(int *nsm, int *avail)
                  cudaSuccess;
     };
     for (int r = 1; r <= kMaxRows; ++r) with_kernel(r, limit);
+    for (int r = kWinRows; r <= kMaxRows; ++r) with_win_kernel(r, limit);
     limit(res2d_group_kernel);
     if (!ok) (void)cudaGetLastError();
     return ok;
@@ -555,7 +614,7 @@ bool res2d_device(int *nsm, int *avail)
 // fills its latency; the edge pass about 60 per warp and pass.  Against the
 // measured times of the 14 cheapest plans at nine sizes from 101^2 to 1101^2 the
 // chosen one was within 5 % of the best.
-long long res2d_best(const Layout &L, int ctas, int avail, Res2dPlan *out)
+long long res2d_best(const Layout &L, int ctas, int avail, Res2dPlan *out, int min_rows = 1)
 {
     Res2dPlan best;
     long long best_cost = -1;
@@ -567,7 +626,7 @@ long long res2d_best(const Layout &L, int ctas, int avail, Res2dPlan *out)
         const long long H = std::max<long long>(2, (L.ny + tiles_y - 1) / tiles_y);
         const long long nty = (L.ny + H - 1) / H;
         if (H > 8192 || W > kThreads) continue;
-        for (int rpt = 1; rpt <= kMaxRows; ++rpt) {
+        for (int rpt = min_rows; rpt <= kMaxRows; ++rpt) {
             const Res2dGeom G((int)W, (int)H, rpt);
             const long long strips = (long long)G.NC * G.NB;
             const long long nedge = Res2dGeom::edges((int)W, (int)H);
@@ -602,6 +661,9 @@ long long res2d_best(const Layout &L, int ctas, int avail, Res2dPlan *out)
 
 // cost of the exchange that no work hides, per two steps (about 0.7 us)
 constexpr long long kExchangeCost = 1400;
+// cost of a window's launch, loads and stores (about 30 us; the model's cycles come
+// out some 1.35 times as long)
+constexpr long long kPassCost = 45000;
 
 }  // namespace
 
@@ -621,6 +683,57 @@ bool res2d_plan(const Layout &L, Res2dPlan *out)
         return false;
     }
     *out = best;
+    return true;
+}
+
+// Windows for a grid that does not fit the SMs: strips along one axis, each run for B
+// steps with B more nodes on its inner sides, so that what the missing neighbours
+// spoil (one node per step from the rim) never reaches the nodes it owns.  All windows
+// are equally long.  Cost per step of the whole grid: the windows' two-step costs and
+// the fixed cost of their passes.  More windows mean more rim, deeper passes wider rims
+// but fewer of them; the handle times the choice against the blocked kernel.
+bool res2d_win_plan(const Layout &L, long long nsteps, Res2dWin *out)
+{
+    int nsm = 0, avail = 0;
+    if (L.d != 2 || !res2d_device(&nsm, &avail)) return false;
+    double best = INFINITY;
+    for (int axis = 0; axis < 2; ++axis) {
+        const long long n = axis ? L.ny : L.nx, other = axis ? L.nx : L.ny;
+        for (int B = 16; B <= 96 && B <= nsteps; B += 8) {
+            for (int k = 2, fits = 0; k <= 32 && fits < 3; ++k) {
+                const long long len = (n + 2LL * B * (k - 1) + k - 1) / k;
+                if (len - 2LL * B < 32) break;         // (every window owns nodes)
+                if (len * other > 2LL * kMaxRows * kThreads * nsm) continue;
+                Layout W = L;
+                (axis ? W.ny : W.nx) = len;
+                Res2dPlan p;
+                const long long cost = res2d_best(W, nsm, avail, &p, kWinRows);
+                if (cost < 0) continue;
+                ++fits;
+                const double t = k * (0.5 * (double)(cost + kExchangeCost) + (double)kPassCost / B);
+                if (t < best) {
+                    best = t;
+                    out->n = k;
+                    out->B = B;
+                    out->axis = axis;
+                    out->len = (int)len;
+                    out->plan = p;
+                }
+            }
+        }
+    }
+    if (best == INFINITY) return false;
+    int occ = 0;
+    cudaError_t oe = cudaSuccess;
+    with_win_kernel(out->plan.rpt, [&](auto kern) {
+        oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, out->plan.threads,
+                                                           out->plan.smem);
+    });
+    if (oe != cudaSuccess || occ < 1 ||
+        (long long)out->plan.ntx * out->plan.nty > (long long)occ * nsm) {
+        (void)cudaGetLastError();
+        return false;
+    }
     return true;
 }
 
@@ -750,6 +863,71 @@ void launch_res2d(const Res2dPlan &p, const float *kap, const float *dco, const 
         launch_cooperative(kern, dim3((unsigned)p.ntx, (unsigned)p.nty), (unsigned)p.threads,
                            p.smem, s, I, P);
     });
+}
+
+void launch_res2d_win(const Res2dWin &w, const float *kap, const float *dco, const float *fre,
+                      const float *fim, const Layout &L, const StepCoef<float> &C, const float *ab,
+                      int nsteps, int jim, int jfin, const OutSlot *slot, unsigned long long *xbuf,
+                      int *err, float *const planes[4], cudaStream_t s, const Res2dProj<float> &P)
+{
+    (void)cudaMemsetAsync(xbuf, 0, w.plan.xwords * sizeof(unsigned long long), s);
+    const int n = (int)(w.axis ? L.ny : L.nx);
+    unsigned tag = 0;
+    for (int j = 0, pass = 0; j < nsteps; j += w.B, ++pass) {
+        const int steps = std::min(w.B, nsteps - j);
+        const int in = 2 * (pass & 1), to = 2 - in;
+        int own = 0;                            // first owned node of the window
+        for (int k = 0; k < w.n; ++k) {
+            const int from = std::max(0, own - w.B), end = std::min(n, from + w.len);
+            const int next = k + 1 == w.n ? n : end - w.B;
+            Res2dInst I;
+            I.L = L;
+            (w.axis ? I.L.ny : I.L.nx) = end - from;
+            const int64_t off = w.axis ? (int64_t)from * L.pitch : from;
+            I.gx = w.axis ? 0 : from;
+            I.gy = w.axis ? from : 0;
+            I.gnx = (int)L.nx;
+            I.own[0] = w.axis ? 0 : own - from;
+            I.own[1] = w.axis ? (int)L.nx : next - from;
+            I.own[2] = w.axis ? own - from : 0;
+            I.own[3] = w.axis ? next - from : (int)L.ny;
+            I.kap = kap + off;
+            I.dco = dco + off;
+            I.fre = fre + off;
+            I.fim = fim + off;
+            if (j > 0) {                        // (a run starts from rest)
+                I.s0 = planes[in] + off;
+                I.s1 = planes[in + 1] + off;
+            }
+            if (j + steps < nsteps) {
+                I.o0 = planes[to] + off;
+                I.o1 = planes[to + 1] + off;
+            }
+            I.C = C;
+            I.ab = ab + 2 * j;
+            I.nsteps = steps;
+            I.jim = jim - j;
+            I.jfin = jfin - j;
+            I.jbase = j;
+            I.slot = slot;
+            I.xbuf = xbuf;
+            I.err = err;
+            I.W = w.plan.W;
+            I.H = w.plan.H;
+            I.rpt = w.plan.rpt;
+            I.ntx = (int)((I.L.nx + I.W - 1) / I.W);
+            const int nty = (int)((I.L.ny + I.H - 1) / I.H);
+            I.tag0 = tag;
+            tag += (unsigned)(steps / 2);
+            Res2dProj<float> Q = P;
+            if (Q.acc) Q.j_acc -= j;
+            with_win_kernel(I.rpt, [&](auto kern) {
+                launch_cooperative(kern, dim3((unsigned)I.ntx, (unsigned)nty),
+                                   (unsigned)w.plan.threads, w.plan.smem, s, I, Q);
+            });
+            own = next;
+        }
+    }
 }
 
 void launch_res2d_group(const Res2dInst *inst, int n, int ctas, size_t smem,
