@@ -51,9 +51,9 @@ def test_batch_equals_single_handles(name, mode):
 
 
 def test_no_memory_for_the_resident_launch_leaves_the_handles_sequences():
-    """An allocation that fails while a batch is built is reported as before (2: out of
-    memory), except those of the resident launch, which the handles' own sequences
-    replace: same outputs."""
+    """An allocation that fails while a batch is built is reported (3: out of memory),
+    except those of the resident launch, which the handles' own sequences replace: same
+    outputs."""
     solvers, F = [], []
     for k, n in enumerate([(65, 70), (120, 33)]):
         solvers.append(htd.Solver(het_problem(2, n, T=2, layer=2, seed=30 + k), precision="mixed"))
@@ -61,16 +61,19 @@ def test_no_memory_for_the_resident_launch_leaves_the_handles_sequences():
     want = [host(s.precond(f[0])) for s, f in zip(solvers, F)]
     built = 0
     for k in range(24):
+        b = None
         htd.htd_test_fail_alloc(k)
         try:
             b = htd.Batch(solvers, [1, 1])
+            b.set_form(1)
         except htd.HtdError as e:
-            assert e.status == 2
+            assert e.status == 3
+            if b:
+                b.close()
             continue
         finally:
             htd.htd_test_fail_alloc(-1)
         built += 1
-        b.set_form(1)
         for u, w in zip(b.precond(F), want):
             assert np.array_equal(host(u)[0], w)
         b.close()
