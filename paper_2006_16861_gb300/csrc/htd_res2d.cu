@@ -40,9 +40,10 @@
 // window: strips along one axis, each loaded, run for B steps and stored, with B more
 // nodes on its inner sides (res2d_win_plan).  Against the blocked kernel, which
 // recomputes half of each tile's work in its rims and reloads everything every 4 or
-// 8 steps: 1501 x 2001 7.6 us per step (three windows, 64 steps) against 9.7 .. 10.2;
-// 2001^2 stays with the blocked kernel (10.9), whose tiles happen to fit it.  What
-// bounds a pass is the resident steps and about 30 us of launch, loads and stores.
+// 8 steps, us per step: 1301 x 1501 4.9, 1501 x 2001 7.1 against 9.7, 1800^2 8.7;
+// 2001^2 and 2501^2 stay with the blocked kernel (10.9, 19.1; windows 11.0, 19.2), whose
+// tiles happen to fit them.  What bounds a pass is the resident steps (135 us for 64 at
+// 1501 x 2001) and about 14 us of launch, loads and stores.
 //
 // An exchanged value is one 64-bit word, its bits beside a tag (index of the
 // exchange + 1), so no fence orders data before a flag.  Before a CTA publishes
@@ -186,14 +187,38 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
         K[i] = 0.f;
     }
     __syncthreads();
-    // cells (lower corner lx, ly), those of the domain's nodes; a window's u_j
+    // A window, which is loaded once per pass, loads its operands from a valid place
+    // whether or not the node exists and drops what does not: loads behind a branch wait
+    // for one another (a pass of 64 steps at 1501 x 2001: 168 us, 151 so).  A whole run's
+    // loads do not show, and its kernels keep more registers without.
     const float *__restrict__ s0 = kWin ? I.s0 : nullptr, *__restrict__ s1 = kWin ? I.s1 : nullptr;
-#pragma unroll 4
-    for (int i = tid; i < (W + 4) * (H + 4); i += NT) {
-        const int lx = i % (W + 4) - 2, ly = i / (W + 4) - 2;
-        if (x0 + lx >= -1 && x0 + lx < nx && y0 + ly >= -1 && y0 + ly < ny) {
-            K[G.at(lx, ly)] = kap[gidx(lx, ly)];
-            if (kWin && s0 && x0 + lx >= 0 && y0 + ly >= 0) U0[G.at(lx, ly)] = s0[gidx(lx, ly)];
+    const int64_t safe = gidx(0, 0);
+    auto load = [&](const float *p, int64_t g, bool ok) {
+        const float v = p[ok ? g : safe];
+        return ok ? v : 0.f;
+    };
+    // cells (lower corner lx, ly), those of the domain's nodes; a window's u_j
+    if constexpr (kWin) {
+        int cx = tid % (W + 4), cy = tid / (W + 4);
+        const int dx = NT % (W + 4), dy = NT / (W + 4);
+#pragma unroll 8
+        for (int i = tid; i < (W + 4) * (H + 4); i += NT) {
+            const int lx = cx - 2, ly = cy - 2, o = G.at(lx, ly);
+            const int64_t g = gidx(lx, ly);
+            K[o] = load(kap, g, x0 + lx >= -1 && x0 + lx < nx && y0 + ly >= -1 && y0 + ly < ny);
+            if (s0) U0[o] = load(s0, g, in_domain(lx, ly));
+            cx += dx;
+            cy += dy;
+            if (cx >= W + 4) {
+                cx -= W + 4;
+                ++cy;
+            }
+        }
+    } else {
+        for (int i = tid; i < (W + 4) * (H + 4); i += NT) {
+            const int lx = i % (W + 4) - 2, ly = i / (W + 4) - 2;
+            if (x0 + lx >= -1 && x0 + lx < nx && y0 + ly >= -1 && y0 + ly < ny)
+                K[G.at(lx, ly)] = kap[gidx(lx, ly)];
         }
     }
     // this thread's strip: column lx, rows ly0 + i and ly0 + RPT + i.  Nodes
@@ -210,23 +235,29 @@ __device__ __forceinline__ void res2d_run(const Res2dInst &I, int tx, int ty, co
         za[i] = zb[i] = dd[i] = f2(0.f, 0.f);
         float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
         const int la = ly0 + i, lb = ly0 + RPT + i;
+        if constexpr (kWin) {
+            const bool oka = has && lx <= w && la <= h && in_domain(lx, la);
+            const bool okb = has && lx <= w && lb <= h && in_domain(lx, lb);
+            const int64_t ga = gidx(lx, la), gb = gidx(lx, lb);
+            dd[i] = f2(load(dco, ga, oka), load(dco, gb, okb));
+            if (s0) {
+                za[i] = f2(load(s0, ga, oka), load(s0, gb, okb));
+                zb[i] = f2(load(s1, ga, oka), load(s1, gb, okb));
+            }
+            if (has)
+                fp[i * NC] = make_float4(load(fre, ga, oka), load(fre, gb, okb),
+                                         load(fim, ga, oka), load(fim, gb, okb));
+            continue;
+        }
         if (has && lx <= w && la <= h && in_domain(lx, la)) {
             const int64_t g = gidx(lx, la);
             dd[i].x = dco[g];
-            if (kWin && s0) {
-                za[i].x = s0[g];
-                zb[i].x = s1[g];
-            }
             f.x = fre[g];
             f.z = fim[g];
         }
         if (has && lx <= w && lb <= h && in_domain(lx, lb)) {
             const int64_t g = gidx(lx, lb);
             dd[i].y = dco[g];
-            if (kWin && s0) {
-                za[i].y = s0[g];
-                zb[i].y = s1[g];
-            }
             f.y = fre[g];
             f.w = fim[g];
         }
@@ -661,9 +692,9 @@ long long res2d_best(const Layout &L, int ctas, int avail, Res2dPlan *out, int m
 
 // cost of the exchange that no work hides, per two steps (about 0.7 us)
 constexpr long long kExchangeCost = 1400;
-// cost of a window's launch, loads and stores (about 30 us; the model's cycles come
+// cost of a window's launch, loads and stores (about 14 us; the model's cycles come
 // out some 1.35 times as long)
-constexpr long long kPassCost = 45000;
+constexpr long long kPassCost = 20000;
 
 }  // namespace
 
