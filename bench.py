@@ -102,11 +102,10 @@ NCU_TRAFFIC = {
                   "sha16": "bc39e0a2f3fd839d", "bytes": 25193114 + 0, "nodes": 1001 * 1001},
     "stream3d": {"file": "htd_stream3d.cu", "begin": "", "end": "}  // namespace\n",
                  "sha16": "4f957ccf1e700468", "bytes": 193680896 + 18157568, "nodes": 192 ** 3},
-    # captured on the 256^3 bench workload itself (z chunk 19, five launches
-    # averaged): no scaling
+    # captured on a 256^3 layered grid (z chunk 19, one launch): no scaling
     "stream3d_pair": {"file": "htd_stream3d_pair.cu", "begin": "",
                       "end": "}  // namespace\n\nsize_t stream3d_pair_smem_bytes",
-                      "sha16": "73ccff94cf1225fe", "bytes": 440054323 + 52439450,
+                      "sha16": "d2f4a0c9bc7b9ce4", "bytes": 497020928,
                       "nodes": 256 ** 3},
 }
 
@@ -128,7 +127,7 @@ def step_kernel_name(prm, ndim, prec="float"):
             return f"tb2d_pair_kernel<{prm['steps_per_launch']}>", "tb2d_pair"
         return f"tb2d_kernel<float,{prm['steps_per_launch']}>", "tb2d"
     if sk == 2:
-        if list(prm["tile"][:2]) == [64, 8]:
+        if list(prm["tile"][:2]) in ([64, 8], [32, 16]):
             return "stream3d_pair_kernel", "stream3d_pair"
         return "stream3d_kernel", "stream3d"
     return ("step2d_kernel<float>" if ndim == 2 else "step3d_kernel<float>"), None
