@@ -346,18 +346,22 @@ step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
             for (int ox = 0; ox < 3; ++ox)
                 w[2][oy][ox] = u[i + Q + (oy - 1) * P + (ox - 1)];
         const double uprev = um[i];
-        // own-node terms beside the neighbours', corners first (as in asm2d_step)
+        // Own-node terms beside the neighbours' (as in asm2d_step), and of those the small
+        // ones first: a face's term is only its mass part (the stiffness of App. A's
+        // stencil is zero there).  96^3: 8.26 ms per application, 8.36 with the faces last;
+        // error against 64-bit torch 2.2e-15 either way.
         double own = fma(a, fre[i], -b * fim[i]);
         own = fma(-2.0, uprev, own);
         own = fma(c0, w[1][1][1], own);
         own = fma(coefP[c], w[1][1][1], own);
-        double acc = coefP[13 * N + c] * w[2][2][2];
+        double acc = coefP[9 * N + c] * w[2][1][1];
 #pragma unroll
-        for (int sh = 3; sh >= 1; --sh)
+        for (int pass = 0; pass < 3; ++pass)
 #pragma unroll
-            for (int lin = 0; lin < 26; ++lin) {
+            for (int lin = 0; lin < 27; ++lin) {
                 const int oz = lin / 9, oy = lin / 3 % 3, ox = lin % 3;
-                if ((oz != 1) + (oy != 1) + (ox != 1) != sh) continue;
+                const int sh = pass == 0 ? 1 : pass == 1 ? 3 : 2;       // faces, corners, edges
+                if ((oz != 1) + (oy != 1) + (ox != 1) != sh || lin == 22) continue;
                 int64_t ci = c;
                 if (lin < 13) {
                     ci += ((int64_t)(oz - 1) * L.ny + (oy - 1)) * L.nx + (ox - 1);
