@@ -313,8 +313,15 @@ step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   RhsSet R, int zc, int nchunks)
 {
     grid_dep_begin();
-    const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
-    const int64_t iy = (int64_t)blockIdx.y * kAsmTY + threadIdx.y;
+    // (tile rows beyond grid.y's 65535 blocks follow along grid.x)
+    const unsigned gx = (unsigned)((L.nx + 31) / 32);
+    unsigned bx = blockIdx.x, by = blockIdx.y;
+    if (bx >= gx) {
+        by += bx / gx * gridDim.y;
+        bx %= gx;
+    }
+    const int64_t ix = (int64_t)bx * 32 + threadIdx.x;
+    const int64_t iy = (int64_t)by * kAsmTY + threadIdx.y;
     int rhs;
     if (!rhs_of_slot(R, (int)blockIdx.z / nchunks, rhs)) return;
     const int64_t z0 = (int64_t)(blockIdx.z % nchunks) * zc;
@@ -439,12 +446,14 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
         ++g_launches;
         return;
     }
-    const int64_t tiles = ((L.nx + 31) / 32) * ((L.ny + kAsmTY - 1) / kAsmTY) * R.slots;
+    const int64_t gx = (L.nx + 31) / 32, gy = (L.ny + kAsmTY - 1) / kAsmTY;
+    const int64_t tiles = gx * gy * R.slots;
     const int64_t want = 8 * (int64_t)sm_count();
     int zc = (int)std::min<int64_t>(16, std::max<int64_t>(1, L.nz * tiles / want));
     zc = (int)std::min<int64_t>(zc, L.nz);
     const int nchunks = (int)((L.nz + zc - 1) / zc);
-    dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + kAsmTY - 1) / kAsmTY),
+    const int64_t fold = (gy + 65534) / 65535;
+    dim3 grd((unsigned)(gx * fold), (unsigned)((gy + fold - 1) / fold),
              (unsigned)(nchunks * R.slots));
     launch_ex(step3d_asm_kernel, grd, dim3(32, kAsmTY), 0, s, overlap, u, um, out, coefP, dco, fre,
               fim, L, c0, a, b, slot, flags, R, zc, nchunks);
