@@ -741,26 +741,45 @@ htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cud
     }
     // (windows: two passes, to count their loads and stores)
     const int tsteps = (int)(c->win.n ? std::min<long long>(c->nsteps, 2 * c->win.B) : c->nsteps);
+    auto drop = [&]() {
+        cudaFree(c->res_ab);
+        cudaFree(c->res_x);
+        cudaFree(c->res_w);
+        c->res_ab = nullptr;
+        c->res_x = nullptr;
+        c->res_w = nullptr;
+        c->win.n = 0;
+    };
+    std::vector<T> w, ab(2 * (size_t)c->nsteps);
     if (c->opt.mode == HTD_MODE_PROJECT) {
         // projection weights per phase k of the new state: cos and -sin of
         // 2 pi k / nP, rounded as for the separate accumulation kernel
-        std::vector<T> w(2 * (size_t)c->nP);
+        w.resize(2 * (size_t)c->nP);
         for (int k = 0; k < c->nP; ++k) {
             const double th = 2.0 * kPi * (double)k / (double)c->nP;
             w[2 * k] = (T)std::cos(th);
             w[2 * k + 1] = (T)(-std::sin(th));
         }
-        HTD_CUDA(htd::dev_malloc(&c->res_w, sizeof(T) * w.size()));
-        HTD_CUDA(cudaMemcpy(c->res_w, w.data(), sizeof(T) * w.size(), cudaMemcpyHostToDevice));
     }
-    std::vector<T> ab(2 * (size_t)c->nsteps);
     for (long long j = 0; j < c->nsteps; ++j) {
         ab[2 * j] = (T)c->atab[j];
         ab[2 * j + 1] = (T)c->btab[j];
     }
-    HTD_CUDA(htd::dev_malloc(&c->res_ab, sizeof(T) * ab.size()));
+    cudaError_t e = cudaSuccess;
+    if (!w.empty()) e = htd::dev_malloc(&c->res_w, sizeof(T) * w.size());
+    if (e == cudaSuccess) e = htd::dev_malloc(&c->res_ab, sizeof(T) * ab.size());
+    if (e == cudaSuccess)
+        e = htd::dev_malloc(&c->res_x, sizeof(unsigned long long) * c->res.xwords);
+    if (e == cudaErrorMemoryAllocation && c->win.n) {
+        // no room for the windows' tables: the blocked kernel needs none of them
+        (void)cudaGetLastError();
+        drop();
+        return HTD_OK;
+    }
+    HTD_CUDA(e);
+    if (!w.empty())
+        HTD_CUDA(cudaMemcpy(c->res_w, w.data(), sizeof(T) * w.size(), cudaMemcpyHostToDevice));
     HTD_CUDA(cudaMemcpy(c->res_ab, ab.data(), sizeof(T) * ab.size(), cudaMemcpyHostToDevice));
-    HTD_CUDA(htd::dev_malloc(&c->res_x, sizeof(unsigned long long) * c->res.xwords));
     const StepCoef<T> C = cast_coef<T>(c->C);
     for (int r = 0; r < 2; ++r) {
         if (r == 1) HTD_CUDA(cudaEventRecord(e0, s));
@@ -778,13 +797,7 @@ htd_status try_res2d(htd_ctx *c, bool force, cudaStream_t s, cudaEvent_t e0, cud
         c->use_res = true;
         c->step_us = us;
     } else {
-        cudaFree(c->res_ab);
-        cudaFree(c->res_x);
-        cudaFree(c->res_w);
-        c->res_ab = nullptr;
-        c->res_x = nullptr;
-        c->res_w = nullptr;
-        c->win.n = 0;
+        drop();
     }
     return HTD_OK;
 }

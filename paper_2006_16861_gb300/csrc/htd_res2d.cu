@@ -723,9 +723,10 @@ bool res2d_plan(const Layout &L, Res2dPlan *out)
 // are equally long.  Cost per step of the whole grid: the windows' two-step costs and
 // the fixed cost of their passes.  More windows mean more rim, deeper passes wider rims
 // but fewer of them; the handle times the choice against the blocked kernel.
-bool res2d_win_plan(const Layout &L, long long nsteps, Res2dWin *out)
+bool res2d_win_plan(const Layout &L, long long nsteps, Res2dWin *win)
 {
     int nsm = 0, avail = 0;
+    Res2dWin w;
     if (L.d != 2 || !res2d_device(&nsm, &avail)) return false;
     double best = INFINITY;
     for (int axis = 0; axis < 2; ++axis) {
@@ -735,20 +736,20 @@ bool res2d_win_plan(const Layout &L, long long nsteps, Res2dWin *out)
                 const long long len = (n + 2LL * B * (k - 1) + k - 1) / k;
                 if (len - 2LL * B < 32) break;         // (every window owns nodes)
                 if (len * other > 2LL * kMaxRows * kThreads * nsm) continue;
-                Layout W = L;
-                (axis ? W.ny : W.nx) = len;
+                Layout S = L;
+                (axis ? S.ny : S.nx) = len;
                 Res2dPlan p;
-                const long long cost = res2d_best(W, nsm, avail, &p, kWinRows);
+                const long long cost = res2d_best(S, nsm, avail, &p, kWinRows);
                 if (cost < 0) continue;
                 ++fits;
                 const double t = k * (0.5 * (double)(cost + kExchangeCost) + (double)kPassCost / B);
                 if (t < best) {
                     best = t;
-                    out->n = k;
-                    out->B = B;
-                    out->axis = axis;
-                    out->len = (int)len;
-                    out->plan = p;
+                    w.n = k;
+                    w.B = B;
+                    w.axis = axis;
+                    w.len = (int)len;
+                    w.plan = p;
                 }
             }
         }
@@ -756,15 +757,16 @@ bool res2d_win_plan(const Layout &L, long long nsteps, Res2dWin *out)
     if (best == INFINITY) return false;
     int occ = 0;
     cudaError_t oe = cudaSuccess;
-    with_win_kernel(out->plan.rpt, [&](auto kern) {
-        oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, out->plan.threads,
-                                                           out->plan.smem);
+    with_win_kernel(w.plan.rpt, [&](auto kern) {
+        oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, w.plan.threads,
+                                                           w.plan.smem);
     });
     if (oe != cudaSuccess || occ < 1 ||
-        (long long)out->plan.ntx * out->plan.nty > (long long)occ * nsm) {
+        (long long)w.plan.ntx * w.plan.nty > (long long)occ * nsm) {
         (void)cudaGetLastError();
         return false;
     }
+    *win = w;
     return true;
 }
 
