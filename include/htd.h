@@ -512,12 +512,10 @@ void htd_test_fail_alloc(long long after);
 /* How a batch runs its preconditioner applications (filled after the first
  * application or solve; zeros before).  A batch with a group of 2-D handles
  * has two forms of a run that give the same bits: every handle's own step
- * sequence as a child graph (plain; 2-D FP32 handles whose grids fit the SMs'
- * shared memory together run as one resident-grid launch after the other
- * sequences), or the group's persistent launch beside
- * the other handles' sequences (group).  The first two rounds of a solve run
- * one form each; the one with the smaller device time per point update is
- * kept for the batch from then on. */
+ * sequence as a child graph (plain; see htd_batch_resident_desc), or the group's
+ * persistent launch beside the other handles' sequences (group).  The first
+ * rounds of a solve run one form each; the one with the smaller device time per
+ * point update is kept for the batch from then on. */
 typedef struct {
     int instances;           /* handles in the batch */
     int systems;             /* (handle, right-hand side) pairs */
@@ -528,7 +526,8 @@ typedef struct {
     int group_steps_per_task; /* recurrence steps per task (the blocked depth B) */
     int form;                /* 0 not yet decided, 1 plain, 2 group */
     double ns_per_update_plain; /* device time per point update of the timed round
-                                   in each form (0 until timed) */
+                                   in each form (0 until timed); plain: the less of
+                                   its two ways */
     double ns_per_update_group;
 } htd_batch_desc;
 htd_status htd_batch_describe(htd_batch b, htd_batch_desc *out);
@@ -538,6 +537,29 @@ htd_status htd_batch_describe(htd_batch b, htd_batch_desc *out);
  * persistent launch (HTD_ERR_ARG if the batch has no group).  Either form
  * gives the same bits. */
 htd_status htd_batch_set_form(htd_batch b, int form);
+
+/* The two ways of a plain run, with the same bits: every handle's own step sequence,
+ * or, where the grids of the batch's 2-D FP32 handles fit the SMs' shared memory
+ * together (every right-hand side that the batch carries on its share of the SMs),
+ * one resident-grid launch of those after the other handles' sequences.  Each way is
+ * timed in one round (the resident launch first), again when a round carries more
+ * systems than the timed one; a round takes the one that should be faster for the
+ * systems that still run. */
+typedef struct {
+    int systems;             /* (2-D handle, right-hand side) pairs of the resident
+                                launch (0: there is none) */
+    int ctas;                /* its CTAs, one per SM */
+    int last;                /* the last run: 0 none or handle by handle, 1 own
+                                sequences, 2 group, 3 resident launch */
+    double ns_per_update_own; /* device time per point update of the timed rounds
+                                 (0 until timed) */
+    double ns_per_update_resident;
+} htd_batch_resident_desc;
+htd_status htd_batch_describe_resident(htd_batch b, htd_batch_resident_desc *out);
+
+/* The plain form's way: 0 = the faster (the default), 1 = own sequences, 2 = the
+ * resident launch (HTD_ERR_ARG if the batch has none). */
+htd_status htd_batch_set_resident(htd_batch b, int pick);
 
 /* Static string for a status code. */
 const char *htd_status_string(htd_status s);

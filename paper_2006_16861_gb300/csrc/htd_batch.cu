@@ -22,7 +22,8 @@
 //    per run;
 //  - in the form without that persistent launch, the 2-D FP32 handles whose grids
 //    fit the SMs' shared memory together run as one resident-grid launch
-//    (htd_res2d.cu), each on its share of the SMs.
+//    (htd_res2d.cu), each on its share of the SMs, where that is faster than their
+//    own sequences (choose_form).
 //
 // The paper treats one system at a time (Sec. 5); the batch changes only the
 // schedule, not the arithmetic of any system.
@@ -89,15 +90,31 @@ struct htd_batch_s {
     cudaEvent_t tab_ev = nullptr;        // last copy of the table (guards tab_host)
     bool tab_pending = false;
     cudaEvent_t ev[2] = {nullptr, nullptr};
-    // two graphs of one run: every handle's step sequence as a child graph
-    // (exec_plain), or the group launch beside the other handles' sequences
-    // (exec); `form` is the one in use: 0 undecided (the first rounds of a
-    // solve time both), 1 plain, 2 group
-    cudaGraphExec_t exec = nullptr, exec_plain = nullptr;
-    bool graph_tried = false;
+    // The graphs of one run (kOwn, kGroup, kRes) and the device time `ms` of the timed
+    // round that advanced the most point updates, `upd`; lo_ms, lo_upd: the last timed
+    // round with fewer.  `form` is the one in use: 0 undecided (the first rounds of a
+    // solve time them), 1 plain (kOwn or kRes), 2 group.
+    struct Form {
+        cudaGraphExec_t exec = nullptr;
+        double ms = 0.0, upd = 0.0, lo_ms = 0.0, lo_upd = 0.0;
+        double ns() const { return upd > 0.0 ? 1e6 * ms / upd : 0.0; }
+        // expected time of a round with u <= upd updates: on the line through both
+        // rounds, at least in proportion; with one round, in proportion, or (fixed) all of it
+        double at(double u, bool fixed) const
+        {
+            if (lo_upd <= 0.0) return fixed ? ms : ms * (u / upd);
+            const double t = lo_ms + (ms - lo_ms) * ((u - lo_upd) / (upd - lo_upd));
+            return u < lo_upd ? std::max(t, lo_ms * (u / lo_upd)) : t;
+        }
+    } f[4];
+    bool graph_tried = false, own_tried = false;
     int form = 0;
-    int round_form = 0;                  // form of the last round launched
-    double form_ms[3] = {0.0, 0.0, 0.0};
+    int res_pick = 0;                    // plain form: 0 the faster, 1 kOwn, 2 kRes
+    int round_form = 0;                  // form of the last round launched (0: no graph)
+    // the round being timed (0: none), its updates, its events
+    int timed = 0;
+    double timed_upd = 0.0;
+    cudaEvent_t tev[2] = {nullptr, nullptr};
     // the persistent launch over the 2-D handles
     std::vector<char> in_group;          // per instance
     std::vector<int> group;              // instance indices, most levels first
@@ -111,7 +128,7 @@ struct htd_batch_s {
     unsigned long long *ghead = nullptr;
     float *gab = nullptr;
     // the 2-D handles whose grids fit the SMs together: one resident-grid launch
-    // per run in the plain form
+    // per run (kRes)
     std::vector<char> in_res;            // per instance (empty: no such launch)
     htd::Res2dInst *rinst = nullptr;
     float *rab = nullptr;
@@ -122,11 +139,16 @@ struct htd_batch_s {
 
 namespace {
 
+// Forms of a run, all with the same bits: every handle's own step sequence; the
+// group's persistent launch beside the other handles' sequences; the 2-D handles'
+// resident launch after the other handles' sequences.
+enum { kOwn = 1, kGroup = 2, kRes = 3 };
+
 void free_batch(htd_batch b)
 {
     if (!b) return;
-    if (b->exec) cudaGraphExecDestroy(b->exec);
-    if (b->exec_plain) cudaGraphExecDestroy(b->exec_plain);
+    for (htd_batch_s::Form &f : b->f)
+        if (f.exec) cudaGraphExecDestroy(f.exec);
     void *gp[] = {b->ginst, b->glev, b->goff, b->gdone, b->gabort, b->ghead, b->gab,
                   b->rinst, b->rab, b->rx};
     for (void *q : gp)
@@ -138,6 +160,8 @@ void free_batch(htd_batch b)
     if (b->tab_host) cudaFreeHost(b->tab_host);
     if (b->tab_ev) cudaEventDestroy(b->tab_ev);
     for (cudaEvent_t e : b->ev)
+        if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : b->tev)
         if (e) cudaEventDestroy(e);
     delete b;
 }
@@ -236,10 +260,11 @@ htd_status build_group(htd_batch b)
     return HTD_OK;
 }
 
-// The resident launch of the plain form: every 2-D FP32 handle (each rhs slot an
-// instance of its own), if their grids fit the SMs' shared memory together and no
-// other handle of the batch is one whose launches leave most of the GPU idle -- the
-// resident launch holds every SM, so it runs after the others, not beside them.
+// The resident launch: every 2-D FP32 handle (each right-hand side that the batch
+// carries an instance of its own: a handle's further slots never run here and would
+// only take SMs from the others), if their grids fit the SMs' shared memory together
+// and no other handle of the batch is one whose launches leave most of the GPU idle --
+// the resident launch holds every SM, so it runs after the others, not beside them.
 // Measured against the handles' own blocked sequences side by side: five handles of
 // 200^2 .. 640^2 2.04 ms per application (2.70), with a 64^3 handle of 8 rhs 2.94 (3.63).
 htd_status build_resident(htd_batch b)
@@ -247,19 +272,22 @@ htd_status build_resident(htd_batch b)
     const int ninst = (int)b->ctx.size();
     std::vector<char> in(ninst, 0);
     std::vector<htd::CtxGroupView> views;
+    std::vector<int> rhs;
     std::vector<htd::Layout> L;
     std::vector<long long> steps;
     size_t ab_n = 0;
     for (int i = 0; i < ninst; ++i) {
         htd::CtxGroupView v;
+        if (!b->ci[i].graphs) return HTD_OK;         // (it only runs from a graph)
         if (!htd::ctx_group_view(b->ctx[i], &v)) {
-            if (!htd::ctx_fills_device(b->ctx[i])) return HTD_OK;
+            if (!htd::ctx_fills_device(b->ctx[i], b->nrhs[i])) return HTD_OK;
             continue;
         }
         in[i] = 1;
         ab_n += v.ab.size();
         views.push_back(v);
-        for (int k = 0; k < v.R.slots && L.size() <= 256; ++k) {
+        rhs.push_back(b->nrhs[i]);
+        for (int k = 0; k < b->nrhs[i] && L.size() <= 256; ++k) {
             L.push_back(v.L);
             steps.push_back(v.nsteps);
         }
@@ -286,12 +314,13 @@ htd_status build_resident(htd_batch b)
     std::vector<float> ab(ab_n);
     size_t ab_at = 0, x_at = 0;
     int cta = 0;
-    for (const htd::CtxGroupView &v : views) {
+    for (size_t g = 0; g < views.size(); ++g) {
+        const htd::CtxGroupView &v = views[g];
         for (long long j = 0; j < v.nsteps; ++j) {
             ab[ab_at + 2 * j] = v.ab[j];
             ab[ab_at + 2 * j + 1] = v.ab[v.nsteps + j];
         }
-        for (int k = 0; k < v.R.slots; ++k) {
+        for (int k = 0; k < rhs[g]; ++k) {
             const htd::Res2dPlan &p = plans[inst.size()];
             htd::Res2dInst I;
             I.kap = v.kap;
@@ -372,6 +401,14 @@ htd_status make_parent(const std::vector<cudaGraph_t> &kids, cudaGraph_t last, c
         ok = false;
     }
     cudaGraphDestroy(parent);
+    // to the device now, so that the first run, which is timed, has no more to do than
+    // later ones
+    cudaStream_t cs;
+    if (ok && cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess) {
+        (void)cudaGraphUpload(*out, cs);
+        (void)cudaStreamSynchronize(cs);
+        cudaStreamDestroy(cs);
+    }
     (void)cudaGetLastError();
     return HTD_OK;
 }
@@ -401,11 +438,23 @@ cudaGraph_t capture(Run &&run)
     return g;
 }
 
-// The batch graphs.  Plain form: every handle's captured step sequence as a child
-// graph, the 2-D handles that fit the SMs together as one resident launch after
-// the others (build_resident).  Group form, when the batch has a group of 2-D
-// handles: the group launch beside the other handles' sequences.  Both give the
-// same bits; the first rounds of a solve time them and the faster one is kept.
+// Whether the graph of the handles' own sequences is there (built when first asked for)
+bool own_graph(htd_batch b)
+{
+    if (b->own_tried) return b->f[kOwn].exec != nullptr;
+    b->own_tried = true;
+    std::vector<cudaGraph_t> kids;
+    for (htd_ctx *c : b->ctx) {
+        cudaGraph_t g = htd::ctx_step_graph(c);
+        if (!g) return false;
+        kids.push_back(g);
+    }
+    if (make_parent(kids, nullptr, &b->f[kOwn].exec) != HTD_OK) b->f[kOwn].exec = nullptr;
+    return b->f[kOwn].exec != nullptr;
+}
+
+// The batch graphs (the forms above).  Where there is a resident launch, the handles'
+// own sequences are captured when choose_form first asks for them.
 htd_status build_graph(htd_batch b)
 {
     if (b->graph_tried) return HTD_OK;
@@ -413,40 +462,110 @@ htd_status build_graph(htd_batch b)
     htd_status gst = build_group(b);
     if (gst != HTD_OK) return gst;
     if ((gst = build_resident(b)) != HTD_OK) return gst;
-    std::vector<cudaGraph_t> plain, others;
+    std::vector<cudaGraph_t> beside_res, others;
     for (size_t i = 0; i < b->ctx.size(); ++i) {
-        const bool res = !b->in_res.empty() && b->in_res[i];
-        // no graphs or no capture: run the handles one by one
-        if (!b->ci[i].graphs) return HTD_OK;
-        if (res && (b->in_group[i] || b->group.empty())) continue;   // no graph of its own
+        const bool res = b->in_res.empty() || b->in_res[i];
+        const bool grp = b->group.empty() || b->in_group[i];
+        if (!b->ci[i].graphs) return HTD_OK;     // run the handles one by one
+        if (res && grp) continue;                // in neither of these graphs
         cudaGraph_t g = htd::ctx_step_graph(b->ctx[i]);
-        if (!g) return HTD_OK;
-        if (!res) plain.push_back(g);
-        if (!b->in_group[i]) others.push_back(g);
+        if (!g) return HTD_OK;                   // no capture: one by one
+        if (!res) beside_res.push_back(g);
+        if (!grp) others.push_back(g);
     }
-    cudaGraph_t rgraph = nullptr;
     if (!b->in_res.empty()) {
-        rgraph = capture([&](cudaStream_t cs) -> htd_status {
+        cudaGraph_t g = capture([&](cudaStream_t cs) -> htd_status {
             htd::launch_res2d_group(b->rinst, b->rn, b->rctas, b->rsmem, b->rx, b->rx_words, cs);
             HTD_CUDA(cudaGetLastError());
             return HTD_OK;
         });
-        if (!rgraph) return HTD_OK;
-    }
-    gst = make_parent(plain, rgraph, &b->exec_plain);
-    if (rgraph) cudaGraphDestroy(rgraph);    // the parent holds its own copy
-    if (gst != HTD_OK) return gst;
-    if (!b->group.empty()) {
-        cudaGraph_t ggraph = capture([&](cudaStream_t cs) { return run_group(b, cs); });
-        if (ggraph) {
-            others.push_back(ggraph);
-            gst = make_parent(others, nullptr, &b->exec);
-            cudaGraphDestroy(ggraph);
+        if (g) {
+            gst = make_parent(beside_res, g, &b->f[kRes].exec);
+            cudaGraphDestroy(g);                 // the parent holds its own copy
             if (gst != HTD_OK) return gst;
         }
     }
-    if (!b->exec) b->form = 1;               // no group: the plain form only
+    if (!b->f[kRes].exec && !own_graph(b)) return HTD_OK;
+    if (!b->group.empty()) {
+        cudaGraph_t g = capture([&](cudaStream_t cs) { return run_group(b, cs); });
+        if (g) {
+            others.push_back(g);
+            gst = make_parent(others, nullptr, &b->f[kGroup].exec);
+            cudaGraphDestroy(g);
+            if (gst != HTD_OK) return gst;
+        }
+    }
+    if (!b->f[kGroup].exec) b->form = 1;         // no group: the plain form only
     return HTD_OK;
+}
+
+// device time per point update of the plain form (0: not timed)
+double plain_ns(htd_batch b)
+{
+    const double own = b->f[kOwn].ns(), res = b->f[kRes].ns();
+    return own > 0.0 && (res == 0.0 || own < res) ? own : res;
+}
+
+// the time of the round being timed, once its end has been reached
+void collect_time(htd_batch b)
+{
+    if (!b->timed) return;
+    // (querying an event would end another thread's stream capture)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaEventQuery(b->tev[1]);
+    float ms = 0.f;
+    if (e == cudaSuccess && cudaEventElapsedTime(&ms, b->tev[0], b->tev[1]) == cudaSuccess && ms > 0.f) {
+        htd_batch_s::Form &f = b->f[b->timed];
+        if (b->timed_upd < f.upd) {
+            f.lo_ms = ms;
+            f.lo_upd = b->timed_upd;
+        } else {
+            f.ms = ms;
+            f.upd = b->timed_upd;
+        }
+    }
+    if (e != cudaErrorNotReady) b->timed = 0;
+    (void)cudaGetLastError();
+    (void)cudaThreadExchangeStreamCaptureMode(&mode);
+}
+
+// The form of a round that advances `upd` point updates.  A form is run once to time
+// it, and again when a round has more updates than its timed one (trial: this round
+// may be such a one); otherwise the one that should be fastest runs.  In a solve the
+// systems that still run become fewer, and every such round is timed as well
+// (Form::at).  To begin with, the own sequences' and the group's time is taken to fall
+// with them, the resident launch's to stay, as the SM shares of systems that have
+// converged stay idle: the last systems of a solve may so run their own sequences.
+// Whole solves, ms, and with own sequences only / the resident launch only: five 2-D
+// handles of 200^2 .. 640^2 (13 to 39 iterations) 64.9, 73.7 / 77.0; one of 700^2 and
+// eight of 120^2 92.4, 100.6 / 97.6.  The group is timed in solves only.
+int choose_form(htd_batch b, double upd, bool solve, bool trial)
+{
+    if (b->form == 2) return kGroup;
+    const bool res = b->f[kRes].exec && b->res_pick != 1;
+    const bool own = !res || b->res_pick != 2;
+    const bool grp = b->f[kGroup].exec && b->form == 0 && (solve || b->f[kGroup].ms > 0.0);
+    int c[3], n = 0;
+    if (res) c[n++] = kRes;
+    if (own && !res) c[n++] = kOwn;
+    if (grp) c[n++] = kGroup;
+    if (own && res) c[n++] = kOwn;
+    if (n == 1) return c[0];
+    int best = 0;
+    double best_ms = 0.0;
+    for (int k = 0; k < n; ++k) {
+        const htd_batch_s::Form &f = b->f[c[k]];
+        if (c[k] == kOwn && !(trial ? own_graph(b) : f.exec != nullptr)) continue;
+        if (trial && (f.ms == 0.0 || upd > f.upd)) return c[k];
+        if (f.ms == 0.0) continue;
+        const double ms = f.at(upd, c[k] == kRes);
+        if (!best || ms < best_ms) {
+            best = c[k];
+            best_ms = ms;
+        }
+    }
+    return best ? best : c[0];
 }
 
 // Stage every instance's vector table (input Fp[r], output Up[r] of each rhs
@@ -475,22 +594,39 @@ htd_status wait_table(htd_batch b)
 // through the batch events (read later).
 htd_status precond_round(htd_batch b, const std::vector<char> &sel,
                          const std::vector<const double2 *> &in, const std::vector<double2 *> &out,
-                         cudaStream_t s)
+                         cudaStream_t s, bool solve)
 {
     htd::NvtxRange nvtx_range("batch_round");
     const int ninst = (int)b->ctx.size();
-    HTD_CUDA(cudaEventRecord(b->ev[0], s));
     htd_status st = wait_table(b);
     if (st != HTD_OK) return st;
     std::vector<std::vector<int>> idx(ninst);
     int runs = 0;
+    double upd = 0.0;
     for (size_t k = 0; k < b->sys.size(); ++k) {
         if (!sel[k]) continue;
         const Sys &y = b->sys[k];
+        upd += (double)y.N * (double)b->ci[y.inst].nsteps * b->ci[y.inst].runs;
         idx[y.inst].push_back(y.rhs);
         b->tab_host[b->tab_off[y.inst] + y.rhs] = in[k];
         b->tab_host[b->tab_off[y.inst] + b->ci[y.inst].rcap + y.rhs] = out[k];
         runs = std::max(runs, b->ci[y.inst].runs);
+    }
+    // (a round that is being captured times nothing)
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    const bool live = cudaStreamIsCapturing(s, &capturing) == cudaSuccess &&
+                      capturing == cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    if (live) collect_time(b);
+    const bool trial = live && !b->timed;
+    const int use = choose_form(b, upd, solve, trial);
+    const htd_batch_s::Form &form = b->f[use];
+    const bool timing = trial && form.exec &&
+                        (form.ms == 0.0 || upd != form.upd);
+    HTD_CUDA(cudaEventRecord(b->ev[0], s));
+    if (timing) {
+        HTD_CUDA(cudaEventRecord(b->tev[0], s));
+        b->timed_upd = upd;
     }
     if ((st = upload_table(b, s)) != HTD_OK) return st;
     for (int run = 0; run < runs; ++run) {
@@ -509,17 +645,13 @@ htd_status precond_round(htd_batch b, const std::vector<char> &sel,
             }
         }
         if (!any) continue;
-        // undecided: the plain form first, then the group form
-        const int use = (b->form != 0) ? b->form : (b->form_ms[1] == 0.0 ? 1 : 2);
-        cudaGraphExec_t ex = (use == 2) ? b->exec : b->exec_plain;
-        if (ex) {
-            HTD_CUDA(cudaGraphLaunch(ex, s));
+        if (form.exec) {
+            HTD_CUDA(cudaGraphLaunch(form.exec, s));
             b->round_form = use;
-            for (int i = 0; i < ninst; ++i) {
-                const bool own = use == 1 ? b->in_res.empty() || !b->in_res[i] : !b->in_group[i];
-                if (own) htd::g_launches += b->ci[i].nsteps;
-            }
-            if (use == 2 || !b->in_res.empty()) htd::g_launches += 1;
+            for (int i = 0; i < ninst; ++i)
+                if (use == kOwn || !(use == kGroup ? b->in_group[i] : b->in_res[i]))
+                    htd::g_launches += b->ci[i].nsteps;
+            if (use != kOwn) htd::g_launches += 1;
         } else {
             b->round_form = 0;
             for (int i = 0; i < ninst; ++i) {
@@ -531,6 +663,10 @@ htd_status precond_round(htd_batch b, const std::vector<char> &sel,
         }
     }
     HTD_CUDA(cudaEventRecord(b->ev[1], s));
+    if (timing) {
+        HTD_CUDA(cudaEventRecord(b->tev[1], s));
+        b->timed = use;
+    }
     return HTD_OK;
 }
 
@@ -646,7 +782,7 @@ htd_status batch_gmres(htd_batch b, const void *const *F_dev, void *const *U_dev
             in[k] = y.V + (int64_t)y.j * y.N;
             out[k] = y.Z + (int64_t)y.j * y.N;
         }
-        if ((st = precond_round(b, sel, in, out, s)) != HTD_OK) return st;
+        if ((st = precond_round(b, sel, in, out, s, true)) != HTD_OK) return st;
 
         // ---- w = H Z_j built in basis slot j + 1, Gram-Schmidt against V_0..V_j:
         // pass 1 for every running system, one fetch; pass 2 for the systems
@@ -681,17 +817,13 @@ htd_status batch_gmres(htd_batch b, const void *const *F_dev, void *const *U_dev
         }
         if (any_second && (st = fetch_blocks(b, s)) != HTD_OK) return st;
         const double ms = round_ms(b);
-        if (b->form == 0 && b->round_form != 0) {
-            // the form choice: device time per point update of this round
-            double upd = 0.0;
-            for (size_t k = 0; k < ns; ++k)
-                if (sel[k]) {
-                    const htd::CtxInfo &ci = b->ci[b->sys[k].inst];
-                    upd += (double)b->sys[k].N * (double)ci.nsteps * ci.runs;
-                }
-            if (upd > 0.0 && ms > 0.0) b->form_ms[b->round_form] = 1e6 * ms / upd;   // ns per update
-            if (b->form_ms[1] > 0.0 && b->form_ms[2] > 0.0)
-                b->form = (b->form_ms[2] < b->form_ms[1]) ? 2 : 1;
+        collect_time(b);
+        if (b->form == 0 && b->f[kGroup].exec) {
+            // decided once every form that there is has been timed
+            const double plain = plain_ns(b), group = b->f[kGroup].ns();
+            const bool all = b->res_pick != 0 || !b->f[kRes].exec ||
+                             (b->f[kRes].ms > 0.0 && (b->f[kOwn].ms > 0.0 || !own_graph(b)));
+            if (all && plain > 0.0 && group > 0.0) b->form = (group < plain) ? 2 : 1;
         }
 
         // ---- Givens update on the host; finished cycles update U -------------
@@ -819,6 +951,8 @@ htd_status create_batch(int ninst, const htd_handle *handles, const int *nrhs, h
     HTD_CUDA(cudaEventCreateWithFlags(&b->tab_ev, cudaEventDisableTiming));
     HTD_CUDA(cudaEventCreate(&b->ev[0]));
     HTD_CUDA(cudaEventCreate(&b->ev[1]));
+    HTD_CUDA(cudaEventCreate(&b->tev[0]));
+    HTD_CUDA(cudaEventCreate(&b->tev[1]));
     return HTD_OK;
 }
 
@@ -839,8 +973,33 @@ htd_status htd_batch_describe(htd_batch b, htd_batch_desc *out)
         out->group_steps_per_task = b->gplan.B;
     }
     out->form = b->form;
-    out->ns_per_update_plain = b->form_ms[1];
-    out->ns_per_update_group = b->form_ms[2];
+    out->ns_per_update_plain = plain_ns(b);
+    out->ns_per_update_group = b->f[kGroup].ns();
+    return HTD_OK;
+}
+
+htd_status htd_batch_describe_resident(htd_batch b, htd_batch_resident_desc *out)
+{
+    if (!b || !out) return HTD_ERR_ARG;
+    std::memset(out, 0, sizeof(*out));
+    if (b->f[kRes].exec) {
+        out->systems = b->rn;
+        out->ctas = b->rctas;
+    }
+    out->last = b->round_form;
+    out->ns_per_update_own = b->f[kOwn].ns();
+    out->ns_per_update_resident = b->f[kRes].ns();
+    return HTD_OK;
+}
+
+htd_status htd_batch_set_resident(htd_batch b, int pick)
+{
+    if (!b || pick < 0 || pick > 2) return HTD_ERR_ARG;
+    htd_status st = build_graph(b);
+    if (st != HTD_OK) return st;
+    if (pick == 2 && !b->f[kRes].exec) return HTD_ERR_ARG;
+    if (pick == 1) (void)own_graph(b);
+    b->res_pick = pick;
     return HTD_OK;
 }
 
@@ -849,10 +1008,13 @@ htd_status htd_batch_set_form(htd_batch b, int form)
     if (!b || form < 0 || form > 2) return HTD_ERR_ARG;
     htd_status st = build_graph(b);
     if (st != HTD_OK) return st;
-    if (form == 2 && !b->exec) return HTD_ERR_ARG;
-    if (form == 1 && !b->exec_plain) return HTD_ERR_ARG;
+    if (form == 2 && !b->f[kGroup].exec) return HTD_ERR_ARG;
+    if (form == 1 && !b->f[kRes].exec && !own_graph(b)) return HTD_ERR_ARG;
     b->form = form;
-    if (form == 0) b->form_ms[1] = b->form_ms[2] = 0.0;
+    if (form == 0) {
+        for (htd_batch_s::Form &f : b->f) f.ms = f.upd = f.lo_ms = f.lo_upd = 0.0;
+        b->timed = 0;
+    }
     return HTD_OK;
 }
 
@@ -896,7 +1058,7 @@ htd_status htd_batch_apply_precond(htd_batch b, const void *const *F_dev, void *
         in[k] = static_cast<const double2 *>(F_dev[y.inst]) + (int64_t)y.rhs * y.N;
         out[k] = static_cast<double2 *>(U_dev[y.inst]) + (int64_t)y.rhs * y.N;
     }
-    return precond_round(b, sel, in, out, s);
+    return precond_round(b, sel, in, out, s, false);
 }
 
 htd_status htd_batch_gmres_solve(htd_batch b, const void *const *F_dev, void *const *U_dev,

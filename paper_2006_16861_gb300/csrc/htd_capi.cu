@@ -1863,7 +1863,7 @@ bool ctx_group_view(htd_ctx *c, CtxGroupView *out)
     return true;
 }
 
-bool ctx_fills_device(const htd_ctx *c)
+bool ctx_fills_device(const htd_ctx *c, int nrhs)
 {
     htd_params p;
     int nsm = 0;
@@ -1874,7 +1874,7 @@ bool ctx_fills_device(const htd_ctx *c)
     }
     const Layout &L = c->Lr;
     const int64_t ctas = ((L.nx + p.tile[0] - 1) / p.tile[0]) * ((L.ny + p.tile[1] - 1) / p.tile[1]) *
-                         ((L.nz + p.tile[2] - 1) / p.tile[2]) * ((c->rcap + c->s3_rpc - 1) / c->s3_rpc);
+                         ((L.nz + p.tile[2] - 1) / p.tile[2]) * ((nrhs + c->s3_rpc - 1) / c->s3_rpc);
     return ctas >= nsm;
 }
 

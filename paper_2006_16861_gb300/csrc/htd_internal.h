@@ -344,9 +344,9 @@ struct CtxGroupView {
     int rcap;
 };
 bool ctx_group_view(htd_ctx *c, CtxGroupView *out);
-// whether the handle's step launches fill the device (the streamed 3-D step with
-// at least one CTA per SM)
-bool ctx_fills_device(const htd_ctx *c);
+// whether the handle's step launches for nrhs right-hand sides fill the device (the
+// streamed 3-D step with at least one CTA per SM)
+bool ctx_fills_device(const htd_ctx *c, int nrhs);
 // zero the first state pair of every rhs slot (a run starts from rest)
 htd_status ctx_zero_states(htd_ctx *c, cudaStream_t s);
 

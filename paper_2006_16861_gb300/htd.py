@@ -37,7 +37,7 @@ EXPORTS = ("htd_default_options", "htd_create", "htd_destroy", "htd_plan", "htd_
            "htd_gmres_solve", "htd_grad", "htd_grad_td",
            "htd_gmres_solve_host", "htd_batch_create", "htd_batch_destroy",
            "htd_batch_apply_precond", "htd_batch_gmres_solve", "htd_batch_describe",
-           "htd_batch_set_form",
+           "htd_batch_set_form", "htd_batch_describe_resident", "htd_batch_set_resident",
            "htd_set_wait_limit",
            "htd_test_fail_alloc", "htd_status_string")
 
@@ -88,6 +88,15 @@ class BatchDesc(ctypes.Structure):
                 ("group_tasks", ctypes.c_longlong), ("group_steps_per_task", ctypes.c_int),
                 ("form", ctypes.c_int), ("ns_per_update_plain", ctypes.c_double),
                 ("ns_per_update_group", ctypes.c_double)]
+
+    def as_dict(self) -> dict:
+        return {f: getattr(self, f) for f, _ in self._fields_}
+
+
+class BatchResidentDesc(ctypes.Structure):
+    _fields_ = [("systems", ctypes.c_int), ("ctas", ctypes.c_int), ("last", ctypes.c_int),
+                ("ns_per_update_own", ctypes.c_double),
+                ("ns_per_update_resident", ctypes.c_double)]
 
     def as_dict(self) -> dict:
         return {f: getattr(self, f) for f, _ in self._fields_}
@@ -148,6 +157,8 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.htd_batch_gmres_solve.argtypes = [vp, vp, vp, d, i, vp, vp]
     lib.htd_batch_describe.argtypes = [vp, ctypes.POINTER(BatchDesc)]
     lib.htd_batch_set_form.argtypes = [vp, i]
+    lib.htd_batch_describe_resident.argtypes = [vp, ctypes.POINTER(BatchResidentDesc)]
+    lib.htd_batch_set_resident.argtypes = [vp, i]
     lib.htd_set_wait_limit.argtypes = [vp, ctypes.c_longlong, i]
     lib.htd_test_fail_alloc.argtypes = [ctypes.c_longlong]
     lib.htd_test_fail_alloc.restype = None
@@ -353,6 +364,20 @@ def htd_batch_set_form(batch: int, form: int) -> None:
     """0 = decide by timing the first rounds of the next solve, 1 = every
     handle's own step sequence, 2 = the group's persistent launch."""
     _check(load().htd_batch_set_form(batch, int(form)), "htd_batch_set_form")
+
+
+def htd_batch_describe_resident(batch: int) -> dict:
+    """The batch's resident launch, and how its plain runs went."""
+    out = BatchResidentDesc()
+    _check(load().htd_batch_describe_resident(batch, ctypes.byref(out)),
+           "htd_batch_describe_resident")
+    return out.as_dict()
+
+
+def htd_batch_set_resident(batch: int, pick: int) -> None:
+    """The plain form's way: 0 = the faster, 1 = own sequences, 2 = the resident
+    launch."""
+    _check(load().htd_batch_set_resident(batch, int(pick)), "htd_batch_set_resident")
 
 
 def _ptr_array(ts) -> ctypes.Array:
@@ -581,6 +606,12 @@ class Batch:
 
     def set_form(self, form: int) -> None:
         htd_batch_set_form(self.handle, form)
+
+    def describe_resident(self) -> dict:
+        return htd_batch_describe_resident(self.handle)
+
+    def set_resident(self, pick: int) -> None:
+        htd_batch_set_resident(self.handle, pick)
 
     def solve(self, Fs, Us=None, tol=1e-6, max_iters=400, stream=None,
               allow_not_converged=False):
