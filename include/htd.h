@@ -435,6 +435,17 @@ htd_status htd_grad_td(htd_handle h, int nsrc, const void *F_dev, int nrec,
                        const int64_t *rec_idx_host, const void *d_dev, int checkpoint_every,
                        void *grad_m_dev, void *grad_R_dev, double *misfit, void *stream);
 
+/* How the handle's last htd_grad_td ran (zeros before the first). */
+typedef struct {
+    int group;               /* sources that run together, at most */
+    int lean;                /* 1: one source at a time in the smaller workspace */
+    long long workspace_bytes; /* device memory of the workspace */
+    long long captures;      /* graphs captured by the handle's calls so far: a pass is
+                                captured again when the workspace, the group, the
+                                checkpoint interval or the wanted gradients change */
+} htd_grad_td_desc;
+htd_status htd_grad_td_describe(htd_handle h, htd_grad_td_desc *out);
+
 /*
  * Batches.  The paper solves one right-hand side of one problem at a time
  * (Sec. 5); these calls run many independent systems together: several

@@ -193,11 +193,16 @@ struct htd_ctx {
     // htd_grad_td workspace (checkpoints, segment states, multipliers), grown on demand
     void *td_ws = nullptr;
     size_t td_ws_bytes = 0;
+    // its receiver residuals: apart, so that another number of receivers leaves the
+    // workspace, and with it the captured passes, in place
+    double2 *td_res = nullptr;
+    size_t td_res_cap = 0;
+    htd_grad_td_desc td_desc{};
     // captured passes of htd_grad_td: a group's forward pass and, per real run, its
     // backward sweep, for the workspace and settings of the last call (two group
     // sizes: whole groups and the last one)
     struct TdGraph {
-        long long key[5] = {0, 0, 0, 0, 0};
+        long long key[4] = {0, 0, 0, 0};
         cudaGraphExec_t ex[3] = {nullptr, nullptr, nullptr};
         long long launches[3] = {0, 0, 0};
     } td_graph[2];
@@ -246,7 +251,7 @@ void free_ctx(htd_ctx *c)
     void *dev[] = {c->kap, c->dco, c->fre, c->fim, c->u0, c->u1, c->kap64, c->imH, c->coefP, c->coefI, c->V, c->Z,
                    c->w, c->t, c->r, c->partial, c->hdev, c->slot, c->Fh, c->Uh, c->u2, c->u3,
                    c->err_dev, c->gU, c->gMu, c->gR, c->gres, c->grec, c->act_dev,
-                   c->acc, c->td_ws, c->res_ab, c->res_x, c->res_w};
+                   c->acc, c->td_ws, c->td_res, c->res_ab, c->res_x, c->res_w};
     for (void *p : dev)
         if (p) cudaFree(p);
     if (c->hhost) cudaFreeHost(c->hhost);
@@ -1076,6 +1081,7 @@ htd_status replay(htd_ctx *c, cudaGraphExec_t *ex, long long *launches, cudaStre
         }
         *launches = htd::g_launches - before;
         htd::g_launches = before;
+        c->td_desc.captures++;
         if (!ok || cudaGraphInstantiate(ex, g, 0) != cudaSuccess) *ex = nullptr;
         if (g) cudaGraphDestroy(g);
         cudaStreamDestroy(cs);
@@ -1106,10 +1112,10 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
     int g = 1, nlam = (int)C + 2;
     size_t npl = (size_t)(2 * nseg + C + 2 + nlam + 4);
     int64_t nsum = ncell + N;
-    const size_t vec = sizeof(double2) * ((size_t)nrec * nsrc + 1) + sizeof(int) * (1 + htd::kMaxRhs);
+    const size_t act_bytes = sizeof(int) * (1 + htd::kMaxRhs);
     auto bytes = [&](int k) {
         return (plane * npl + sizeof(double) * (size_t)nsum + sizeof(double2) * (size_t)N +
-                sizeof(OutSlot)) * k + vec;
+                sizeof(OutSlot)) * k + act_bytes;
     };
     while (g < std::min(nsrc, htd::kMaxRhs) && bytes(g + 1) <= kTdGroupBytes &&
            5 * plane * (g + 1) <= kTdHotBytes)
@@ -1135,6 +1141,9 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
         c->td_ws_bytes = bytes(g);
     }
     const bool lean = nsum == 0;
+    c->td_desc.group = g;
+    c->td_desc.lean = lean;
+    c->td_desc.workspace_bytes = (long long)c->td_ws_bytes;
     const int64_t sstride = (int64_t)npl * L.total;         // from source to source
     T *base = static_cast<T *>(c->td_ws);
     auto P = [&](long long k) { return base + (size_t)k * L.total; };
@@ -1146,9 +1155,16 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
     double2 *U = reinterpret_cast<double2 *>(base + (size_t)sstride * g);      // per source
     OutSlot *slots = reinterpret_cast<OutSlot *>(U + (size_t)N * g);
     double *sums = reinterpret_cast<double *>(slots + g);
-    double2 *resd = reinterpret_cast<double2 *>(sums + (((size_t)nsum * g + 1) & ~(size_t)1));
-    int *act = reinterpret_cast<int *>(resd + (size_t)nrec * nsrc);   // (resd: receiver
-                                                                      // residuals of all sources)
+    int *act = reinterpret_cast<int *>(sums + (size_t)nsum * g);
+    const size_t nres = (size_t)nrec * nsrc;                // receiver residuals of all sources
+    if (nres > c->td_res_cap) {
+        if (c->td_res) cudaFree(c->td_res);
+        c->td_res = nullptr;
+        c->td_res_cap = 0;
+        HTD_CUDA(htd::dev_malloc((void **)&c->td_res, sizeof(double2) * nres));
+        c->td_res_cap = nres;
+    }
+    double2 *resd = c->td_res;
     // Table 1 in 2-D: the forward pass ends in the application's own result, bit for
     // bit (every 2-D kernel evaluates the same expression), so it gives U itself
     const bool forward_U = want && !lean && c->d == 2 && runs == 1;
@@ -1172,7 +1188,7 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
         if (n == 1) return cudaMemsetAsync(p, 0, plane * planes, t);
         return cudaMemset2DAsync(p, sizeof(T) * sstride, 0, plane * planes, n, t);
     };
-    std::vector<double2> res(nrec > 0 ? (size_t)nrec * nsrc : 1);
+    std::vector<double2> res(std::max<size_t>(nres, 1));
     for (int first = 0; first < nsrc; first += g) {
         const int n = std::min(g, nsrc - first);
         HTD_CUDA(zero(are, 2, n, s));                        // are, aim adjacent
@@ -1262,9 +1278,8 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
             return HTD_OK;
         };
         // the captured passes of this workspace, group size and settings
-        const long long key[5] = {(long long)(intptr_t)c->td_ws, ((long long)g << 32) | n, C,
-                                  (gms ? 1 : 0) | (gRs ? 2 : 0) | (want ? 4 : 0),
-                                  (long long)(intptr_t)act};
+        const long long key[4] = {(long long)(intptr_t)c->td_ws, ((long long)g << 32) | n, C,
+                                  (gms ? 1 : 0) | (gRs ? 2 : 0) | (want ? 4 : 0)};
         htd_ctx::TdGraph &tg = c->td_graph[n == g ? 0 : 1];
         if (std::memcmp(tg.key, key, sizeof(key)) != 0) {
             for (cudaGraphExec_t &x : tg.ex) {
@@ -1292,11 +1307,11 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
         HTD_CUDA(cudaGetLastError());
     }
     if (nrec > 0)
-        HTD_CUDA(cudaMemcpyAsync(res.data(), resd, sizeof(double2) * nrec * nsrc,
+        HTD_CUDA(cudaMemcpyAsync(res.data(), resd, sizeof(double2) * nres,
                                  cudaMemcpyDeviceToHost, s));
     HTD_CUDA(cudaStreamSynchronize(s));
     double J = 0.0;
-    for (size_t k = 0; k < (size_t)nrec * nsrc; ++k)
+    for (size_t k = 0; k < nres; ++k)
         J += 0.5 * (res[k].x * res[k].x + res[k].y * res[k].y);
     *misfit = J;
     return std::isfinite(J) ? HTD_OK : HTD_ERR_NONFINITE;
@@ -2243,6 +2258,13 @@ htd_status htd_grad_td(htd_handle h, int nsrc, const void *F_dev, int nrec,
         }
     }
     return st;
+}
+
+htd_status htd_grad_td_describe(htd_handle h, htd_grad_td_desc *out)
+{
+    if (!h || !out) return HTD_ERR_ARG;
+    *out = h->td_desc;
+    return HTD_OK;
 }
 
 const char *htd_status_string(htd_status s)

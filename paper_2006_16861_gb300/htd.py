@@ -34,7 +34,7 @@ LAUNCH_NO_OVERLAP, LAUNCH_NO_GRAPH, LAUNCH_NO_GROUP = 1, 2, 4
 #: every function include/htd.h declares (checked by the ABI test)
 EXPORTS = ("htd_default_options", "htd_create", "htd_destroy", "htd_plan", "htd_get_params",
            "htd_apply_precond", "htd_apply_H", "htd_residual_norm", "htd_residual_norm_noalloc",
-           "htd_gmres_solve", "htd_grad", "htd_grad_td",
+           "htd_gmres_solve", "htd_grad", "htd_grad_td", "htd_grad_td_describe",
            "htd_gmres_solve_host", "htd_batch_create", "htd_batch_destroy",
            "htd_batch_apply_precond", "htd_batch_gmres_solve", "htd_batch_describe",
            "htd_batch_set_form", "htd_batch_describe_resident", "htd_batch_set_resident",
@@ -88,6 +88,14 @@ class BatchDesc(ctypes.Structure):
                 ("group_tasks", ctypes.c_longlong), ("group_steps_per_task", ctypes.c_int),
                 ("form", ctypes.c_int), ("ns_per_update_plain", ctypes.c_double),
                 ("ns_per_update_group", ctypes.c_double)]
+
+    def as_dict(self) -> dict:
+        return {f: getattr(self, f) for f, _ in self._fields_}
+
+
+class GradTdDesc(ctypes.Structure):
+    _fields_ = [("group", ctypes.c_int), ("lean", ctypes.c_int),
+                ("workspace_bytes", ctypes.c_longlong), ("captures", ctypes.c_longlong)]
 
     def as_dict(self) -> dict:
         return {f: getattr(self, f) for f, _ in self._fields_}
@@ -151,6 +159,7 @@ def load(build_if_missing: bool = True) -> ctypes.CDLL:
     lib.htd_grad.argtypes = [vp, i, vp, i, vp, vp, d, i, vp, vp, ctypes.POINTER(d), vp,
                              ctypes.POINTER(SolveInfo)]
     lib.htd_grad_td.argtypes = [vp, i, vp, i, vp, vp, i, vp, vp, ctypes.POINTER(d), vp]
+    lib.htd_grad_td_describe.argtypes = [vp, ctypes.POINTER(GradTdDesc)]
     lib.htd_batch_create.argtypes = [i, vp, vp, ctypes.POINTER(vp)]
     lib.htd_batch_destroy.argtypes = [vp]
     lib.htd_batch_apply_precond.argtypes = [vp, vp, vp, vp]
@@ -425,6 +434,13 @@ def htd_grad_td(handle: int, F, rec_idx: np.ndarray, d, grad_m=None, grad_R=None
                             _stream_ptr(stream))
     _check(st, "htd_grad_td")
     return J.value
+
+
+def htd_grad_td_describe(handle: int) -> dict:
+    """How the handle's last htd_grad_td ran."""
+    out = GradTdDesc()
+    _check(load().htd_grad_td_describe(handle, ctypes.byref(out)), "htd_grad_td_describe")
+    return out.as_dict()
 
 
 def htd_set_wait_limit(handle: int, limit_ns: int, stall_test: bool = False) -> None:
