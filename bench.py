@@ -85,10 +85,10 @@ def launch_words(prm):
     spl = max(1, int(prm.get("steps_per_launch", 1) or 1))
     return WORDS_ONE_STEP if spl == 1 else WORDS_BLOCKED
 # FLOPs per point update as the step kernels compute them (FMA = 2).  FP32: 2-D
-# 12 FMA + 11 add + 6 mul; 3-D 57 FMA + 21 add/mul.  FP64: 2-D 12 FMA + 20
-# add/mul; 3-D as FP32.
+# 12 FMA + 11 add + 6 mul; 3-D 57 FMA + 21 add/mul.  FP64, from the assembled
+# stencil: 2-D 12 FMA + 3 add/mul; 3-D 30 FMA + 3 add/mul.
 F32_FLOPS_PER_UPDATE = {2: 41, 3: 135}
-FP64_FLOPS_PER_UPDATE = {2: 44, 3: 135}
+FP64_FLOPS_PER_UPDATE = {2: 27, 3: 63}
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture, valid only for the kernel source it was taken on: the sha256 prefix
@@ -118,10 +118,13 @@ def step_kernel_name(prm, ndim, prec="float"):
     recurrence precision, "float" or "double")."""
     sk = prm.get("step_kernel")
     if sk == 4:
-        p = "" if prec == "float" else "double,"
-        return f"res2d_kernel<{p}{prm['tile'][0]}x{prm['tile'][1]}>", None
+        form = ("res2d64" if prec == "double" else
+                "res2d" if prm["steps_per_launch"] == prm["steps"] else "res2d_win")
+        return f"{form}_kernel<{prm['tile'][0]}x{prm['tile'][1]}>", None
+    if sk == 3:
+        return ("abd_step2d_kernel" if ndim == 2 else "abd_step_kernel") + f"<{prec}>", None
     if prec == "double":
-        return f"step{ndim}d_kernel<double>", None
+        return f"step{ndim}d_asm_kernel", None
     if sk == 1:
         if prm["tile"][2] == 2:
             return f"tb2d_pair_kernel<{prm['steps_per_launch']}>", "tb2d_pair"
@@ -130,7 +133,7 @@ def step_kernel_name(prm, ndim, prec="float"):
         if list(prm["tile"][:2]) in ([64, 8], [32, 16]):
             return "stream3d_pair_kernel", "stream3d_pair"
         return "stream3d_kernel", "stream3d"
-    return ("step2d_kernel<float>" if ndim == 2 else "step3d_kernel<float>"), None
+    return f"step{ndim}d_kernel", None
 
 
 def ncu_traffic(key, nodes):
@@ -907,6 +910,7 @@ def run_ours(args):
     if args.fp64_steps > 0:
         s64 = htd.Solver(p, precision="fp64", mode="table1", krylov="fgmres",
                          restart=args.restart)
+        kern64 = step_kernel_name(s64.params, p.ndim, "double")[0]
         t = []
         for _ in range(args.fp64_steps):
             flush.fill_(3)
@@ -919,11 +923,11 @@ def run_ours(args):
         fp64_ms = allmax(statistics.mean(t))
         s64.close()
         # the FP64 step kernel against the FP64 pipe (it is ALU-bound on GB300):
-        # FLOPs per point update of step2d/step3d as written (FMA = 2)
+        # FLOPs per point update as written (FMA = 2)
         fp_upd = FP64_FLOPS_PER_UPDATE[p.ndim]
         upd = N * fp64_info["steps"]
         tflops = fp_upd * upd / (fp64_info["ms_precond"] * 1e-3) / 1e12
-        fp64_roof = {"bound": "alu", "kernel": f"step{p.ndim}d_kernel<double>",
+        fp64_roof = {"bound": "alu", "kernel": kern64,
                      "achieved": tflops, "peak": pk["fp64_tflops"], "unit": "TFLOP/s",
                      "frac": tflops / pk["fp64_tflops"], "flops_per_update": fp_upd,
                      "peak_kind": f"FP64 pipe derived: 2 DFMA per clock per SM x {pk['nsm']} "
