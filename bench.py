@@ -93,8 +93,9 @@ FP64_FLOPS_PER_UPDATE = {2: 27, 3: 63}
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from one ncu
 # capture, valid only for the kernel source it was taken on: the sha256 prefix
 # of the kernel's region of its file (from `begin`, or the file start, up to
-# `end`), so that edits elsewhere in the file keep the record; scaled by node
-# count to other grid sizes.  The captures are summarised under profiles/.
+# `end`), so that edits elsewhere in the file keep the record; and only for the
+# captured grid size (how much of a grid stays in L2 differs from size to size).
+# The captures are summarised under profiles/.
 NCU_TRAFFIC = {
     # 2-D 1001^2 bench leg, five launches averaged (the grid stays in L2)
     "tb2d_pair": {"file": "htd_tblock.cu", "begin": "// Node-pair form of tb2d_kernel (FP32)",
@@ -102,7 +103,7 @@ NCU_TRAFFIC = {
                   "sha16": "bc39e0a2f3fd839d", "bytes": 25193114 + 0, "nodes": 1001 * 1001},
     "stream3d": {"file": "htd_stream3d.cu", "begin": "", "end": "}  // namespace\n",
                  "sha16": "4f957ccf1e700468", "bytes": 193680896 + 18157568, "nodes": 192 ** 3},
-    # captured on a 256^3 layered grid (z chunk 19, one launch): no scaling
+    # captured on a 256^3 layered grid (64 x 8 tiles, z chunk 19, one launch)
     "stream3d_pair": {"file": "htd_stream3d_pair.cu", "begin": "",
                       "end": "}  // namespace\n\nsize_t stream3d_pair_smem_bytes",
                       "sha16": "d2f4a0c9bc7b9ce4", "bytes": 497020928,
@@ -130,18 +131,20 @@ def step_kernel_name(prm, ndim, prec="float"):
             return f"tb2d_pair_kernel<{prm['steps_per_launch']}>", "tb2d_pair"
         return f"tb2d_kernel<float,{prm['steps_per_launch']}>", "tb2d"
     if sk == 2:
-        if list(prm["tile"][:2]) in ([64, 8], [32, 16]):
+        if list(prm["tile"][:2]) == [64, 8]:
             return "stream3d_pair_kernel", "stream3d_pair"
+        if list(prm["tile"][:2]) == [32, 16]:            # no capture of these tiles
+            return "stream3d_pair_kernel", None
         return "stream3d_kernel", "stream3d"
     return f"step{ndim}d_kernel", None
 
 
 def ncu_traffic(key, nodes):
     """Measured DRAM bytes per launch for `nodes` nodes, or None if the kernel
-    source changed since the capture."""
+    source changed since the capture or the capture has another size."""
     import hashlib
     rec = NCU_TRAFFIC.get(key)
-    if rec is None:
+    if rec is None or nodes != rec["nodes"]:
         return None
     path = os.path.join(ROOT, "paper_2006_16861_gb300", "csrc", rec["file"])
     try:
@@ -153,7 +156,7 @@ def ncu_traffic(key, nodes):
         return None
     if hashlib.sha256(text[i:j].encode()).hexdigest()[:16] != rec["sha16"]:
         return None
-    return rec["bytes"] * nodes / rec["nodes"]
+    return rec["bytes"]
 
 
 def parse_args(argv=None):
