@@ -722,10 +722,13 @@ template <typename T>
 htd_status upload_recurrence(htd_ctx *c, const std::vector<double> &qkap, const std::vector<double> &dcoef)
 {
     const Layout &L = c->Lr;
-    std::vector<T> a(L.total, (T)0), b(L.total, (T)0);
-    for (size_t i = 0; i < (size_t)L.total; ++i) { a[i] = (T)qkap[i]; b[i] = (T)dcoef[i]; }
-    HTD_CUDA(cudaMemcpy(c->kap, a.data(), sizeof(T) * L.total, cudaMemcpyHostToDevice));
-    HTD_CUDA(cudaMemcpy(c->dco, b.data(), sizeof(T) * L.total, cudaMemcpyHostToDevice));
+    std::vector<T> a(L.total);
+    auto upload = [&](void *to, const std::vector<double> &from) {
+        for (size_t i = 0; i < (size_t)L.total; ++i) a[i] = (T)from[i];
+        return cudaMemcpy(to, a.data(), sizeof(T) * L.total, cudaMemcpyHostToDevice);
+    };
+    if (c->kap) HTD_CUDA(upload(c->kap, qkap));
+    HTD_CUDA(upload(c->dco, dcoef));
     return HTD_OK;
 }
 
@@ -1526,6 +1529,7 @@ htd_status create_impl(const htd_grid *grid, const double *c_cell, const double 
     c->rcap = opt.max_rhs;
     void **shared_arrs[] = {&c->kap, &c->dco};
     for (void **pp : shared_arrs) {
+        if (pp == &c->kap && !mixed && !abd) continue;   // FP64 I_acd steps from coefP
         HTD_CUDA(htd::dev_malloc(pp, bytes));
         HTD_CUDA(cudaMemset(*pp, 0, bytes));
     }
