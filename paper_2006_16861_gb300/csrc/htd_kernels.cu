@@ -68,15 +68,17 @@ __device__ __forceinline__ void grid_dep_begin()
 // One step in 2-D, FP32: u_{j+1} -> out (which may be the plane um of u_{j-1}).  A
 // thread takes ROWS nodes of one column, so that a node costs 4.5 loads of u_j and 2.5
 // of q*kappa (nine and four with one row), all of them issued before the first sum.
-// ROWS = 4 where that leaves two blocks per SM, else 1.  force: without it the step has no forcing (a = b = 0: the adjoint
-// between its read-out steps).
-template <int ROWS>
+// ROWS = 4 where that leaves two blocks per SM, else 1.  kForce: without it the step has
+// no forcing (a = b = 0: the adjoint between its read-out steps); a parameter of the
+// kernel, and the rows' clamping for one row too, put a branch and 64-bit minima before the
+// loads: 401^2 2.73 us per step, 2.24 so.
+template <int ROWS, bool kForce>
 __global__ void __launch_bounds__(256)
 step2d_kernel(const float *__restrict__ u, const float *um, float *out,
               const float *__restrict__ kap, const float *__restrict__ dco,
               const float *__restrict__ fre, const float *__restrict__ fim, Layout L,
               StepCoef<float> C, float a, float b, const OutSlot *__restrict__ slot, int flags,
-              RhsSet R, bool force)
+              RhsSet R)
 {
     grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
@@ -99,7 +101,8 @@ step2d_kernel(const float *__restrict__ u, const float *um, float *out,
     float w[ROWS + 2][3], k[ROWS + 1][2], um1[ROWS], d[ROWS], fr[ROWS], fi[ROWS];
     int64_t at[ROWS + 2];                   // u row r - 1
 #pragma unroll
-    for (int r = 0; r < ROWS + 2; ++r) at[r] = i0 + (min(iy0 + r - 1, L.ny) - iy0) * P;
+    for (int r = 0; r < ROWS + 2; ++r)
+        at[r] = i0 + (ROWS == 1 ? r - 1 : min(iy0 + r - 1, L.ny) - iy0) * P;
 #pragma unroll
     for (int r = 0; r < ROWS + 2; ++r)
 #pragma unroll
@@ -112,7 +115,7 @@ step2d_kernel(const float *__restrict__ u, const float *um, float *out,
     for (int r = 0; r < ROWS; ++r) {
         um1[r] = um[at[r + 1]];
         d[r] = dco[at[r + 1]];
-        if (force) {
+        if (kForce) {
             fr[r] = fre[at[r + 1]];
             fi[r] = fim[at[r + 1]];
         }
@@ -129,7 +132,7 @@ step2d_kernel(const float *__restrict__ u, const float *um, float *out,
                              a1[0] + a1[2], a2[0] + a2[2], k[r][0] + k[r][1],
                              k[r + 1][0] + k[r + 1][1]);
         // acc + a Re F - b Im F as two FMAs (the blocked kernels round the same way)
-        if (force) ag = vfma(a, fr[r], vfma(-b, fi[r], ag));
+        if (kForce) ag = vfma(a, fr[r], vfma(-b, fi[r], ag));
         const float unew = vfma(d[r], vfma(-2.f, um1[r], ag), um1[r]);
         out[at[r + 1]] = unew;
         if (flags) {
@@ -146,12 +149,13 @@ step2d_kernel(const float *__restrict__ u, const float *um, float *out,
 // L1, the plane below and the node's own plane from registers).
 constexpr int kZChunk = 16;
 
+template <bool kForce>
 __global__ void __launch_bounds__(256)
 step3d_kernel(const float *__restrict__ u, const float *um, float *out,
               const float *__restrict__ kap, const float *__restrict__ dco,
               const float *__restrict__ fre, const float *__restrict__ fim, Layout L,
               StepCoef<float> C, float a, float b, const OutSlot *__restrict__ slot, int flags,
-              RhsSet R, int nchunks, bool force)
+              RhsSet R, int nchunks)
 {
     typedef float T;
     grid_dep_begin();
@@ -231,7 +235,7 @@ step3d_kernel(const float *__restrict__ u, const float *um, float *out,
                     acc += coef * w[oz][oy][ox];
                 }
         const int64_t i = (iz + 1) * Q + col;
-        const T g = force ? a * fre[i] - b * fim[i] : 0.f;
+        const T g = kForce ? a * fre[i] - b * fim[i] : 0.f;
         const T d = dco[i];
         const T uprev = um[i];
         const T unew = d * (acc + g - T(2) * uprev) + uprev;
@@ -263,20 +267,28 @@ void launch_step(const Layout &L, const float *u, const float *um, float *out, c
     const unsigned gx = (unsigned)((L.nx + 31) / 32);
     if (L.d == 2) {
         const int64_t blocks4 = gx * ((L.ny + 31) / 32) * R.slots;
-        if (blocks4 >= 2 * (int64_t)sm_count()) {
-            dim3 grd(gx, (unsigned)((L.ny + 31) / 32), (unsigned)R.slots);
-            launch_ex(step2d_kernel<4>, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre,
-                      fim, L, C, a, b, slot, flags, R, force);
+        const bool four = blocks4 >= 2 * (int64_t)sm_count();
+        const dim3 grd(gx, (unsigned)(four ? (L.ny + 31) / 32 : (L.ny + 7) / 8), (unsigned)R.slots);
+        auto go = [&](auto kern) {
+            launch_ex(kern, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre, fim, L, C, a,
+                      b, slot, flags, R);
+        };
+        if (four) {
+            if (force) go(step2d_kernel<4, true>);
+            else go(step2d_kernel<4, false>);
         } else {
-            dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
-            launch_ex(step2d_kernel<1>, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre,
-                      fim, L, C, a, b, slot, flags, R, force);
+            if (force) go(step2d_kernel<1, true>);
+            else go(step2d_kernel<1, false>);
         }
     } else {
         const int nchunks = (int)((L.nz + kZChunk - 1) / kZChunk);
         dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)(nchunks * R.slots));
-        launch_ex(step3d_kernel, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre, fim, L,
-                  C, a, b, slot, flags, R, nchunks, force);
+        auto go = [&](auto kern) {
+            launch_ex(kern, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre, fim, L, C, a,
+                      b, slot, flags, R, nchunks);
+        };
+        if (force) go(step3d_kernel<true>);
+        else go(step3d_kernel<false>);
     }
     ++g_launches;
 }
