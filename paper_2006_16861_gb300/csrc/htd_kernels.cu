@@ -26,6 +26,9 @@
 // cs_s = q 2^{d-s} S_s; the stored per-cell coefficient is q * kappa.
 #include <cuda_runtime.h>
 #include <algorithm>
+#include <mutex>
+#include <type_traits>
+#include <vector>
 
 #include "htd_internal.h"
 
@@ -56,13 +59,83 @@ static int sm_count()
 // recurrence step
 // ---------------------------------------------------------------------------
 
-// Programmatic dependent launch (no-op for an ordinary launch): the next kernel of
-// the stream may be scheduled as this one's blocks retire; from here on everything
-// the previous kernel wrote is visible.
-__device__ __forceinline__ void grid_dep_begin()
+// Programmatic dependent launch (no-ops for an ordinary launch): what the previous kernel
+// wrote is visible after grid_dep_wait; the next kernel of the stream may be scheduled
+// once every block of this one has called grid_dep_launch.
+__device__ __forceinline__ void grid_dep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ void grid_dep_launch()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// kEarly: let the next kernel in at once, else only after the wait (launch_step_kernel)
+template <bool kEarly>
+__device__ __forceinline__ void grid_dep_begin()
+{
+    if (kEarly) grid_dep_launch();
+    grid_dep_wait();
+    if (!kEarly) grid_dep_launch();
+}
+
+// Blocks of `kern` with `threads` threads that the device holds at once (0: unknown)
+template <typename Kern>
+static int64_t resident_blocks(Kern kern, int threads)
+{
+    struct Entry {
+        const void *kern;
+        int dev, occ;
+    };
+    static std::mutex lock;
+    static std::vector<Entry> seen;
+    int dev = 0, occ = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    const void *key = reinterpret_cast<const void *>(kern);
+    const std::lock_guard<std::mutex> hold(lock);
+    for (const Entry &e : seen)
+        if (e.kern == key && e.dev == dev) return (int64_t)e.occ * sm_count();
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, threads, 0) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    seen.push_back({key, dev, occ});
+    return (int64_t)occ * sm_count();
+}
+
+// How a one-step launch overlaps the one before it, by the share of the device's
+// resident blocks that a step takes:
+//  - up to a half (both steps' blocks fit, and are spread before the first has ended): the
+//    next step is let in after the wait, so that no more than one waits.  Let in before it,
+//    several waiting grids filled the SMs, and a new grid's blocks went where old ones
+//    happened to end, several to one SM.  us per step, after / before the wait / no overlap:
+//    FP64 2-D 0.17 share 2.63 / 6.1 / 2.78, 0.42 4.72 / 7.0 / 4.87; I_abd FP64 0.19 6.2 / 12.7 /
+//    6.4; FP32 2-D 0.40 1.89 / 2.40 / 2.11;
+//  - from `full` on: before the wait, as the next step's blocks only take up what the last
+//    blocks leave.  FP64 2-D 1.38 10.84 / 10.77 / 10.98, 801^2 (2.9) 19.08 / 18.99 / 19.24;
+//  - between: no overlap; part of the next step's blocks wait in the gaps and the rest crowd.
+//    FP64 2-D 0.53 7.79 / 7.73 / 5.86, 0.73 7.81 / 7.75 / 6.93; FP32 2-D 0.55 2.53 / 2.52 /
+//    2.26; I_abd FP32 3-D 0.63 3.82 / 3.73 / 3.15.
+// `full` is where the last two meet: kFull32, kFull64, and kFullAbd64 for the 2-D I_abd
+// step, which has its coefficients to load before the wait.
+constexpr double kFull32 = 0.8, kFull64 = 1.2, kFullAbd64 = 0.7;
+
+// Launches `early` (the kernel that lets the next one in before the wait) or `late` (after
+// it), otherwise the same
+template <typename Kern, typename... Args>
+static void launch_step_kernel(Kern early, Kern late, double full, dim3 grid, dim3 threads,
+                               cudaStream_t s, bool overlap, Args &&...args)
+{
+    const double blocks = (double)grid.x * grid.y * grid.z;
+    const double fit = overlap ? (double)resident_blocks(late, (int)(threads.x * threads.y)) : 0.0;
+    const bool first = fit > 0.0 && blocks >= full * fit;
+    launch_ex(first ? early : late, grid, threads, 0, s, first || 2.0 * blocks <= fit,
+              static_cast<Args &&>(args)...);
 }
 
 // One step in 2-D, FP32: u_{j+1} -> out (which may be the plane um of u_{j-1}).  A
@@ -72,7 +145,7 @@ __device__ __forceinline__ void grid_dep_begin()
 // no forcing (a = b = 0: the adjoint between its read-out steps); a parameter of the
 // kernel, and the rows' clamping for one row too, put a branch and 64-bit minima before the
 // loads: 401^2 2.73 us per step, 2.24 so.
-template <int ROWS, bool kForce>
+template <int ROWS, bool kForce, bool kEarly>
 __global__ void __launch_bounds__(256)
 step2d_kernel(const float *__restrict__ u, const float *um, float *out,
               const float *__restrict__ kap, const float *__restrict__ dco,
@@ -80,7 +153,7 @@ step2d_kernel(const float *__restrict__ u, const float *um, float *out,
               StepCoef<float> C, float a, float b, const OutSlot *__restrict__ slot, int flags,
               RhsSet R)
 {
-    grid_dep_begin();
+    grid_dep_begin<kEarly>();
     const int64_t ix = (int64_t)blockIdx.x * 32 + threadIdx.x;
     const int64_t iy0 = ((int64_t)blockIdx.y * 8 + threadIdx.y) * ROWS;
     int rhs;
@@ -158,7 +231,6 @@ step3d_kernel(const float *__restrict__ u, const float *um, float *out,
               RhsSet R, int nchunks)
 {
     typedef float T;
-    grid_dep_begin();
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -269,23 +341,24 @@ void launch_step(const Layout &L, const float *u, const float *um, float *out, c
         const int64_t blocks4 = gx * ((L.ny + 31) / 32) * R.slots;
         const bool four = blocks4 >= 2 * (int64_t)sm_count();
         const dim3 grd(gx, (unsigned)(four ? (L.ny + 31) / 32 : (L.ny + 7) / 8), (unsigned)R.slots);
-        auto go = [&](auto kern) {
-            launch_ex(kern, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre, fim, L, C, a,
-                      b, slot, flags, R);
+        auto go = [&](auto early, auto late) {
+            launch_step_kernel(early, late, kFull32, grd, dim3(32, 8), s, overlap, u, um, out, kap,
+                               dco, fre, fim, L, C, a, b, slot, flags, R);
         };
         if (four) {
-            if (force) go(step2d_kernel<4, true>);
-            else go(step2d_kernel<4, false>);
+            if (force) go(step2d_kernel<4, true, true>, step2d_kernel<4, true, false>);
+            else go(step2d_kernel<4, false, true>, step2d_kernel<4, false, false>);
         } else {
-            if (force) go(step2d_kernel<1, true>);
-            else go(step2d_kernel<1, false>);
+            if (force) go(step2d_kernel<1, true, true>, step2d_kernel<1, true, false>);
+            else go(step2d_kernel<1, false, true>, step2d_kernel<1, false, false>);
         }
     } else {
         const int nchunks = (int)((L.nz + kZChunk - 1) / kZChunk);
         dim3 grd(gx, (unsigned)((L.ny + 7) / 8), (unsigned)(nchunks * R.slots));
+        // (never overlapped: few long blocks, 120^3 22.9 us per step so, 18.5 in stream order)
         auto go = [&](auto kern) {
-            launch_ex(kern, grd, dim3(32, 8), 0, s, overlap, u, um, out, kap, dco, fre, fim, L, C, a,
-                      b, slot, flags, R, nchunks);
+            launch_ex(kern, grd, dim3(32, 8), 0, s, false, u, um, out, kap, dco, fre, fim, L, C, a, b,
+                      slot, flags, R, nchunks);
         };
         if (force) go(step3d_kernel<true>);
         else go(step3d_kernel<false>);
@@ -319,7 +392,7 @@ constexpr int kAsmTY = 4;
 
 // (kFold: tile rows beyond grid.y's 65535 blocks follow along grid.x; a form of its own,
 // as the index arithmetic cost the others up to 1.7 %)
-template <bool kFold>
+template <bool kFold, bool kEarly>
 __global__ void __launch_bounds__(32 * kAsmTY)
 step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   const double *__restrict__ coefP, const double *__restrict__ dco,
@@ -327,7 +400,7 @@ step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   double c0, double a, double b, const OutSlot *__restrict__ slot, int flags,
                   RhsSet R, int zc, int nchunks)
 {
-    grid_dep_begin();
+    grid_dep_begin<kEarly>();
     unsigned bx = blockIdx.x, by = blockIdx.y;
     if (kFold) {
         const unsigned gx = (unsigned)((L.nx + 31) / 32);
@@ -409,6 +482,7 @@ step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
 
 // the 2-D form: one node per thread, 16 FP64 operations (the cell form: 33);
 // 801^2: 18.9 us per step (cell form: 43 us), 14.3 us at the FP64 pipe's rate
+template <bool kEarly>
 __global__ void __launch_bounds__(256)
 step2d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   const double *__restrict__ coefP, const double *__restrict__ dco,
@@ -416,7 +490,7 @@ step2d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
                   double c0, double a, double b, const OutSlot *__restrict__ slot, int flags,
                   RhsSet R)
 {
-    grid_dep_begin();
+    grid_dep_begin<kEarly>();
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -455,8 +529,9 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
 {
     if (L.d == 2) {
         dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
-        launch_ex(step2d_asm_kernel, grd, dim3(32, 8), 0, s, overlap, u, um, out, coefP, dco, fre,
-                  fim, L, c0, a, b, slot, flags, R);
+        launch_step_kernel(step2d_asm_kernel<true>, step2d_asm_kernel<false>, kFull64, grd,
+                           dim3(32, 8), s, overlap, u, um, out, coefP, dco, fre, fim, L, c0, a, b,
+                           slot, flags, R);
         ++g_launches;
         return;
     }
@@ -469,12 +544,12 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
     const int64_t fold = (gy + 65534) / 65535;
     dim3 grd((unsigned)(gx * fold), (unsigned)((gy + fold - 1) / fold),
              (unsigned)(nchunks * R.slots));
-    auto go = [&](auto kern) {
-        launch_ex(kern, grd, dim3(32, kAsmTY), 0, s, overlap, u, um, out, coefP, dco, fre, fim, L, c0,
-                  a, b, slot, flags, R, zc, nchunks);
+    auto go = [&](auto early, auto late) {
+        launch_step_kernel(early, late, kFull64, grd, dim3(32, kAsmTY), s, overlap, u, um, out, coefP,
+                           dco, fre, fim, L, c0, a, b, slot, flags, R, zc, nchunks);
     };
-    if (fold > 1) go(step3d_asm_kernel<true>);
-    else go(step3d_asm_kernel<false>);
+    if (fold > 1) go(step3d_asm_kernel<true, true>, step3d_asm_kernel<true, false>);
+    else go(step3d_asm_kernel<false, true>, step3d_asm_kernel<false, false>);
     ++g_launches;
 }
 
@@ -495,14 +570,14 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
 // sum_o M_s (sum of damp over the shared cells) w_{beta+o}).  Reads u_{n-1} at
 // the neighbours in the cell case, so u_{n+1} goes to a third plane.
 
-template <typename T, bool kCell>
+template <typename T, bool kCell, bool kEarly>
 __global__ void __launch_bounds__(256)
 abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict__ out,
                 const T *__restrict__ kap, const T *__restrict__ damp,
                 const T *__restrict__ fre, const T *__restrict__ fim, Layout L, StepCoef<T> C,
                 T a, T b, T cth, const OutSlot *__restrict__ slot, int flags, RhsSet R, int nz)
 {
-    grid_dep_begin();
+    grid_dep_begin<kEarly>();
     const int64_t ix = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t iy = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     int rhs;
@@ -571,7 +646,7 @@ abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict
 // the expressions and their order are abd_step_kernel's.  ROWS: the most of 4, 2, 1
 // that leaves two blocks per SM.  401^2 cell damping: 2.0 us per step (two rows), 3.0 with
 // the per-node loads of the 3-D form.
-template <typename T, bool kCell, int ROWS>
+template <typename T, bool kCell, int ROWS, bool kEarly>
 __global__ void __launch_bounds__(256)
 abd_step2d_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict__ out,
                   const T *__restrict__ kap, const T *__restrict__ damp,
@@ -596,7 +671,7 @@ abd_step2d_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restri
         }
 #pragma unroll
     for (int r = 0; r < ROWS; ++r) dn[r] = !kCell && in ? damp[at[r + 1]] : T(0);
-    grid_dep_begin();
+    grid_dep_begin<kEarly>();
     int rhs;
     if (!rhs_of_slot(R, (int)blockIdx.z, rhs)) return;
     if (!in) return;
@@ -674,25 +749,37 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
         };
         const int rows = fits(4) ? 4 : fits(2) ? 2 : 1;
         const dim3 grd2(gx, (unsigned)blocks(rows), (unsigned)R.slots);
-        auto go = [&](auto kern) {
-            launch_ex(kern, grd2, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, L, C, a, b,
-                      cth, slot, flags, R);
+        auto go = [&](auto early, auto late) {
+            // (FP32: always before the wait, as the coefficients that the next steps load
+            // meanwhile are then half of a step: 401^2 cell 2.29 us, 2.57 after it, 2.76 in
+            // stream order; 0.8 to 0.96 of stream order from 60^2 to 1200^2)
+            if constexpr (sizeof(T) == 4)
+                launch_ex(early, grd2, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, L, C, a,
+                          b, cth, slot, flags, R);
+            else
+                launch_step_kernel(early, late, kFullAbd64, grd2, blk, s, overlap, u, um, out, kap,
+                                   damp, fre, fim, L, C, a, b, cth, slot, flags, R);
         };
-        if (cell) {
-            if (rows == 4) go(abd_step2d_kernel<T, true, 4>);
-            else if (rows == 2) go(abd_step2d_kernel<T, true, 2>);
-            else go(abd_step2d_kernel<T, true, 1>);
-        } else {
-            if (rows == 4) go(abd_step2d_kernel<T, false, 4>);
-            else if (rows == 2) go(abd_step2d_kernel<T, false, 2>);
-            else go(abd_step2d_kernel<T, false, 1>);
-        }
-    } else if (cell) {
-        launch_ex(abd_step_kernel<T, true>, grd, blk, 0, s, overlap, u, um, out, kap, damp, fre,
-                  fim, L, C, a, b, cth, slot, flags, R, nz);
+        auto with_rows = [&](auto cellc, auto rowsc) {
+            constexpr bool kCell = decltype(cellc)::value;
+            constexpr int ROWS = decltype(rowsc)::value;
+            go(abd_step2d_kernel<T, kCell, ROWS, true>,
+               abd_step2d_kernel<T, kCell, ROWS, sizeof(T) == 4>);
+        };
+        auto with_cell = [&](auto cellc) {
+            if (rows == 4) with_rows(cellc, std::integral_constant<int, 4>{});
+            else if (rows == 2) with_rows(cellc, std::integral_constant<int, 2>{});
+            else with_rows(cellc, std::integral_constant<int, 1>{});
+        };
+        if (cell) with_cell(std::true_type{});
+        else with_cell(std::false_type{});
     } else {
-        launch_ex(abd_step_kernel<T, false>, grd, blk, 0, s, overlap, u, um, out, kap, damp, fre,
-                  fim, L, C, a, b, cth, slot, flags, R, nz);
+        auto go = [&](auto early, auto late) {
+            launch_step_kernel(early, late, sizeof(T) == 8 ? kFull64 : kFull32, grd, blk, s, overlap,
+                               u, um, out, kap, damp, fre, fim, L, C, a, b, cth, slot, flags, R, nz);
+        };
+        if (cell) go(abd_step_kernel<T, true, true>, abd_step_kernel<T, true, false>);
+        else go(abd_step_kernel<T, false, true>, abd_step_kernel<T, false, false>);
     }
     ++g_launches;
 }
