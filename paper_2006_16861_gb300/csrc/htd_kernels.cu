@@ -122,7 +122,7 @@ static int64_t resident_blocks(Kern kern, int threads)
 //    FP64 2-D 0.53 7.79 / 7.73 / 5.86, 0.73 7.81 / 7.75 / 6.93; FP32 2-D 0.55 2.53 / 2.52 /
 //    2.26; I_abd FP32 3-D 0.63 3.82 / 3.73 / 3.15.
 // `full` is where the last two meet: kFull32, kFull64, and kFullAbd64 for the 2-D I_abd
-// step, which has its coefficients to load before the wait.
+// step with several rows per thread, which has many coefficients to load before the wait.
 constexpr double kFull32 = 0.8, kFull64 = 1.2, kFullAbd64 = 0.7;
 
 // Launches `early` (the kernel that lets the next one in before the wait) or `late` (after
@@ -644,8 +644,8 @@ abd_step_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict
 // The 2-D step, ROWS nodes of a column per thread with all operands loaded before
 // the first sum (a row of u_n and u_{n-1} serves the nodes above and below it too);
 // the expressions and their order are abd_step_kernel's.  ROWS: the most of 4, 2, 1
-// that leaves two blocks per SM.  401^2 cell damping: 2.0 us per step (two rows), 3.0 with
-// the per-node loads of the 3-D form.
+// that leaves two blocks per SM, or in FP64 the best balanced one of those.  401^2 cell
+// damping: 2.0 us per step (two rows), 3.0 with the per-node loads of the 3-D form.
 template <typename T, bool kCell, int ROWS, bool kEarly>
 __global__ void __launch_bounds__(256)
 abd_step2d_kernel(const T *__restrict__ u, const T *__restrict__ um, T *__restrict__ out,
@@ -747,7 +747,19 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
         auto fits = [&](int rows) {
             return gx * blocks(rows) * R.slots >= 2 * (int64_t)sm_count();
         };
-        const int rows = fits(4) ? 4 : fits(2) ? 2 : 1;
+        int rows = fits(4) ? 4 : fits(2) ? 2 : 1;
+        if (sizeof(T) == 8) {
+            // FP64: the pipe of the SM with the most blocks sets the time; a node costs 0.83
+            // with two rows and 0.8 with four of what it costs with one (560^2 node damping:
+            // 23.7, 22.3 and 25.5 us per step with 1, 2, 4 rows)
+            const double node[5] = {0.0, 1.0, 0.83, 0.0, 0.8};
+            auto cost = [&](int k) {
+                const int64_t nsm = sm_count(), n = gx * blocks(k) * R.slots;
+                return (double)((n + nsm - 1) / nsm) * k * node[k];
+            };
+            for (int k = rows / 2; k >= 1; k /= 2)
+                if (cost(k) < cost(rows)) rows = k;
+        }
         const dim3 grd2(gx, (unsigned)blocks(rows), (unsigned)R.slots);
         auto go = [&](auto early, auto late) {
             // (FP32: always before the wait, as the coefficients that the next steps load
@@ -757,8 +769,9 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
                 launch_ex(early, grd2, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, L, C, a,
                           b, cth, slot, flags, R);
             else
-                launch_step_kernel(early, late, kFullAbd64, grd2, blk, s, overlap, u, um, out, kap,
-                                   damp, fre, fim, L, C, a, b, cth, slot, flags, R);
+                launch_step_kernel(early, late, rows == 1 ? kFull64 : kFullAbd64, grd2, blk, s,
+                                   overlap, u, um, out, kap, damp, fre, fim, L, C, a, b, cth, slot,
+                                   flags, R);
         };
         auto with_rows = [&](auto cellc, auto rowsc) {
             constexpr bool kCell = decltype(cellc)::value;

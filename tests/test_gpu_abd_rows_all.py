@@ -2,9 +2,10 @@
 device's SM count.
 
 The launcher takes the most of 4, 2 and 1 rows per thread that leave two blocks (32
-columns, 8 threads of rows) per SM.  For each count one grid just inside the rule, with
-a last row that ends inside a thread's rows.  Tolerances of test_gpu_abd: 1e-10 (FP64),
-5e-5 (mixed).
+columns, 8 threads of rows) per SM; in FP64 the one of those whose SM with the most blocks
+has the least to do, a node costing 1, 0.83, 0.8 with 1, 2, 4 rows.  For each count one
+grid just inside the rule, with a last row that ends inside a thread's rows.  Tolerances
+of test_gpu_abd: 1e-10 (FP64), 5e-5 (mixed).
 """
 import pytest
 
@@ -27,16 +28,21 @@ def blocks(ny, rows):
     return -(-NX // 32) * -(-ny // (8 * rows))
 
 
-def rule(ny):
+def rule(ny, precision):
     """The row count that the launcher takes for ny x NX nodes."""
-    want = 2 * torch.cuda.get_device_properties(0).multi_processor_count
-    return next((r for r in (4, 2) if blocks(ny, r) >= want), 1)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rows = next((r for r in (4, 2) if blocks(ny, r) >= 2 * sms), 1)
+    if precision == "fp64":
+        node = {1: 1.0, 2: 0.83, 4: 0.8}
+        rows = min((r for r in (4, 2, 1) if r <= rows),
+                   key=lambda r: -(-blocks(ny, r) // sms) * r * node[r])
+    return rows
 
 
-def grid_rows(rows, rest):
+def grid_rows(rows, rest, precision):
     """The fewest grid rows for which the rule takes `rows`, `rest` more than whole threads."""
     ny = rest
-    while rule(ny) != rows:
+    while rule(ny, precision) != rows:
         ny += rows
     return ny
 
@@ -45,8 +51,8 @@ def grid_rows(rows, rest):
 @pytest.mark.parametrize("damping", ["node", "cell"])
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 def test_abd_rows_match_the_oracle(rows, rest, damping, precision):
-    ny = grid_rows(rows, rest) if rows > 1 else 37
-    assert rule(ny) == rows and ny % rows == rest
+    ny = grid_rows(rows, rest, precision) if rows > 1 else 37
+    assert rule(ny, precision) == rows and ny % rows == rest
     p = abd_problem(2, (ny, NX), T=1)
     s = htd.Solver(p, precision=precision, integrator="abd", damping=damping, restart=2)
     assert s.params["step_kernel"] == 3
