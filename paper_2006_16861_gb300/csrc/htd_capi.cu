@@ -1218,7 +1218,7 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
         if (!forward_U && (rst = residuals()) != HTD_OK) return rst;
         if (!want) continue;
         // the sources of the group as the rhs slots of a step launch
-        set.slots = n;
+        set.slots = set.sure = n;
         set.act = nullptr;
         if (n > 1) {
             std::vector<int> idx(n);

@@ -147,10 +147,12 @@ struct OutSlot {
 // capture).  act == null: a single rhs, index 0, slot 0.  The per-rhs planes
 // (u_j, u_{j-1}, Re F, Im F, the second state pair of the blocked kernel) lie
 // `stride` elements apart; q*kappa and d are shared by all rhs; the output
-// slot of rhs r is slot[r].
+// slot of rhs r is slot[r].  `sure`: slots that are active in every launch (for the
+// launchers' rules; a captured sequence does not know its list).
 struct RhsSet {
     const int *act = nullptr;
     int slots = 1;
+    int sure = 1;
     int64_t stride = 0;
 };
 

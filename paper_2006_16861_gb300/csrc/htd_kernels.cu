@@ -121,19 +121,24 @@ static int64_t resident_blocks(Kern kern, int threads)
 //  - between: no overlap; part of the next step's blocks wait in the gaps and the rest crowd.
 //    FP64 2-D 0.53 7.79 / 7.73 / 5.86, 0.73 7.81 / 7.75 / 6.93; FP32 2-D 0.55 2.53 / 2.52 /
 //    2.26; I_abd FP32 3-D 0.63 3.82 / 3.73 / 3.15.
-// `full` is where the last two meet: kFull32, kFull64, and kFullAbd64 for the 2-D I_abd
-// step with several rows per thread, which has many coefficients to load before the wait.
-constexpr double kFull32 = 0.8, kFull64 = 1.2, kFullAbd64 = 0.7;
+// `full` is where the last two meet: kFull32, kFull64, and kFullRows for the 2-D steps with
+// several rows per thread (FP32 600^2, 0.79: 2.90 / 3.17 before the wait / no overlap).
+// Slots that may be idle count for the first rule, and for the second only where their
+// blocks alone are kManyWaves times what the device holds: of 8 right-hand sides with 2
+// active, before the wait / in stream order, ms per application: I_abd FP64 150 x 170 (1.2)
+// 2.81 / 2.04, FP64 (1.0) 1.03 / 0.68; FP32 401^2 (3.0) 0.70 / 0.78.
+constexpr double kFull32 = 0.8, kFull64 = 1.2, kFullRows = 0.7, kManyWaves = 2.5;
 
 // Launches `early` (the kernel that lets the next one in before the wait) or `late` (after
 // it), otherwise the same
 template <typename Kern, typename... Args>
 static void launch_step_kernel(Kern early, Kern late, double full, dim3 grid, dim3 threads,
-                               cudaStream_t s, bool overlap, Args &&...args)
+                               const RhsSet &R, cudaStream_t s, bool overlap, Args &&...args)
 {
     const double blocks = (double)grid.x * grid.y * grid.z;
     const double fit = overlap ? (double)resident_blocks(late, (int)(threads.x * threads.y)) : 0.0;
-    const bool first = fit > 0.0 && blocks >= full * fit;
+    const bool first = fit > 0.0 && (blocks * R.sure >= full * fit * R.slots ||
+                                     blocks >= kManyWaves * fit);
     launch_ex(first ? early : late, grid, threads, 0, s, first || 2.0 * blocks <= fit,
               static_cast<Args &&>(args)...);
 }
@@ -342,8 +347,8 @@ void launch_step(const Layout &L, const float *u, const float *um, float *out, c
         const bool four = blocks4 >= 2 * (int64_t)sm_count();
         const dim3 grd(gx, (unsigned)(four ? (L.ny + 31) / 32 : (L.ny + 7) / 8), (unsigned)R.slots);
         auto go = [&](auto early, auto late) {
-            launch_step_kernel(early, late, kFull32, grd, dim3(32, 8), s, overlap, u, um, out, kap,
-                               dco, fre, fim, L, C, a, b, slot, flags, R);
+            launch_step_kernel(early, late, four ? kFullRows : kFull32, grd, dim3(32, 8), R, s,
+                               overlap, u, um, out, kap, dco, fre, fim, L, C, a, b, slot, flags, R);
         };
         if (four) {
             if (force) go(step2d_kernel<4, true, true>, step2d_kernel<4, true, false>);
@@ -530,7 +535,7 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
     if (L.d == 2) {
         dim3 grd((unsigned)((L.nx + 31) / 32), (unsigned)((L.ny + 7) / 8), (unsigned)R.slots);
         launch_step_kernel(step2d_asm_kernel<true>, step2d_asm_kernel<false>, kFull64, grd,
-                           dim3(32, 8), s, overlap, u, um, out, coefP, dco, fre, fim, L, c0, a, b,
+                           dim3(32, 8), R, s, overlap, u, um, out, coefP, dco, fre, fim, L, c0, a, b,
                            slot, flags, R);
         ++g_launches;
         return;
@@ -545,8 +550,8 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
     dim3 grd((unsigned)(gx * fold), (unsigned)((gy + fold - 1) / fold),
              (unsigned)(nchunks * R.slots));
     auto go = [&](auto early, auto late) {
-        launch_step_kernel(early, late, kFull64, grd, dim3(32, kAsmTY), s, overlap, u, um, out, coefP,
-                           dco, fre, fim, L, c0, a, b, slot, flags, R, zc, nchunks);
+        launch_step_kernel(early, late, kFull64, grd, dim3(32, kAsmTY), R, s, overlap, u, um, out,
+                           coefP, dco, fre, fim, L, c0, a, b, slot, flags, R, zc, nchunks);
     };
     if (fold > 1) go(step3d_asm_kernel<true, true>, step3d_asm_kernel<true, false>);
     else go(step3d_asm_kernel<false, true>, step3d_asm_kernel<false, false>);
@@ -744,17 +749,19 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
     if (L.d == 2) {
         const unsigned gx = (unsigned)((L.nx + 31) / 32);
         auto blocks = [&](int rows) { return (L.ny + 8 * rows - 1) / (8 * rows); };
-        auto fits = [&](int rows) {
-            return gx * blocks(rows) * R.slots >= 2 * (int64_t)sm_count();
-        };
+        // FP64 counts the right-hand sides that are sure to be active: with 2 of 8 active,
+        // 150 x 170 cell damping took 3.1 ms per application with two rows, 2.1 with one; with
+        // one of 8, 401^2 7.8 with four, 6.4 with two
+        const int64_t rhs = sizeof(T) == 8 ? R.sure : R.slots;
+        auto fits = [&](int rows) { return gx * blocks(rows) * rhs >= 2 * (int64_t)sm_count(); };
         int rows = fits(4) ? 4 : fits(2) ? 2 : 1;
         if (sizeof(T) == 8) {
-            // FP64: the pipe of the SM with the most blocks sets the time; a node costs 0.83
-            // with two rows and 0.8 with four of what it costs with one (560^2 node damping:
-            // 23.7, 22.3 and 25.5 us per step with 1, 2, 4 rows)
+            // the pipe of the SM with the most blocks sets the time; a node costs 0.83 with two
+            // rows and 0.8 with four of what it costs with one (560^2 node damping: 23.7, 22.3
+            // and 25.5 us per step with 1, 2, 4 rows)
             const double node[5] = {0.0, 1.0, 0.83, 0.0, 0.8};
             auto cost = [&](int k) {
-                const int64_t nsm = sm_count(), n = gx * blocks(k) * R.slots;
+                const int64_t nsm = sm_count(), n = gx * blocks(k) * rhs;
                 return (double)((n + nsm - 1) / nsm) * k * node[k];
             };
             for (int k = rows / 2; k >= 1; k /= 2)
@@ -769,7 +776,7 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
                 launch_ex(early, grd2, blk, 0, s, overlap, u, um, out, kap, damp, fre, fim, L, C, a,
                           b, cth, slot, flags, R);
             else
-                launch_step_kernel(early, late, rows == 1 ? kFull64 : kFullAbd64, grd2, blk, s,
+                launch_step_kernel(early, late, rows == 1 ? kFull64 : kFullRows, grd2, blk, R, s,
                                    overlap, u, um, out, kap, damp, fre, fim, L, C, a, b, cth, slot,
                                    flags, R);
         };
@@ -788,8 +795,9 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
         else with_cell(std::false_type{});
     } else {
         auto go = [&](auto early, auto late) {
-            launch_step_kernel(early, late, sizeof(T) == 8 ? kFull64 : kFull32, grd, blk, s, overlap,
-                               u, um, out, kap, damp, fre, fim, L, C, a, b, cth, slot, flags, R, nz);
+            launch_step_kernel(early, late, sizeof(T) == 8 ? kFull64 : kFull32, grd, blk, R, s,
+                               overlap, u, um, out, kap, damp, fre, fim, L, C, a, b, cth, slot,
+                               flags, R, nz);
         };
         if (cell) go(abd_step_kernel<T, true, true>, abd_step_kernel<T, true, false>);
         else go(abd_step_kernel<T, false, true>, abd_step_kernel<T, false, false>);

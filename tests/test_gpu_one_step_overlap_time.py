@@ -23,7 +23,9 @@ NODE, CELL = (dict(integrator="abd", damping=d) for d in ("node", "cell"))
 CASES = [((333, 127), "fp64", dict(tblock=1)), ((350, 350), "fp64", dict(tblock=1)),
          ((401, 401), "mixed", dict(tblock=1)), ((333, 127), "fp64", NODE),
          ((350, 350), "fp64", CELL), ((401, 401), "mixed", NODE), ((48, 48, 48), "mixed", NODE),
-         ((90, 80, 70), "mixed", dict(s3_kernel=htd.S3_ZMARCH)), ((30, 40, 50), "fp64", {})]
+         ((90, 80, 70), "mixed", dict(s3_kernel=htd.S3_ZMARCH)), ((30, 40, 50), "fp64", {}),
+         # one of eight right-hand sides active: most blocks of a launch are idle
+         ((170, 150), "fp64", dict(CELL, max_rhs=8)), ((300, 200), "fp64", dict(max_rhs=8))]
 
 
 @pytest.mark.parametrize("n,precision,kw", CASES,
