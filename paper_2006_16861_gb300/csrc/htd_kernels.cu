@@ -121,13 +121,14 @@ static int64_t resident_blocks(Kern kern, int threads)
 //  - between: no overlap; part of the next step's blocks wait in the gaps and the rest crowd.
 //    FP64 2-D 0.53 7.79 / 7.73 / 5.86, 0.73 7.81 / 7.75 / 6.93; FP32 2-D 0.55 2.53 / 2.52 /
 //    2.26; I_abd FP32 3-D 0.63 3.82 / 3.73 / 3.15.
-// `full` is where the last two meet: kFull32, kFull64, and kFullRows for the 2-D steps with
+// `full` is where the last two meet: kFull (FP64 3-D 0.79 7.9 / 7.0 before the wait / no overlap,
+// 0.85 7.36 / 7.52), kFull64 for the other FP64 steps, and kFullRows for the 2-D steps with
 // several rows per thread (FP32 600^2, 0.79: 2.90 / 3.17 before the wait / no overlap).
 // Slots that may be idle count for the first rule, and for the second only where their
 // blocks alone are kManyWaves times what the device holds: of 8 right-hand sides with 2
 // active, before the wait / in stream order, ms per application: I_abd FP64 150 x 170 (1.2)
 // 2.81 / 2.04, FP64 (1.0) 1.03 / 0.68; FP32 401^2 (3.0) 0.70 / 0.78.
-constexpr double kFull32 = 0.8, kFull64 = 1.2, kFullRows = 0.7, kManyWaves = 2.5;
+constexpr double kFull = 0.8, kFull64 = 1.2, kFullRows = 0.7, kManyWaves = 2.5;
 
 // Launches `early` (the kernel that lets the next one in before the wait) or `late` (after
 // it), otherwise the same
@@ -347,7 +348,7 @@ void launch_step(const Layout &L, const float *u, const float *um, float *out, c
         const bool four = blocks4 >= 2 * (int64_t)sm_count();
         const dim3 grd(gx, (unsigned)(four ? (L.ny + 31) / 32 : (L.ny + 7) / 8), (unsigned)R.slots);
         auto go = [&](auto early, auto late) {
-            launch_step_kernel(early, late, four ? kFullRows : kFull32, grd, dim3(32, 8), R, s,
+            launch_step_kernel(early, late, four ? kFullRows : kFull, grd, dim3(32, 8), R, s,
                                overlap, u, um, out, kap, dco, fre, fim, L, C, a, b, slot, flags, R);
         };
         if (four) {
@@ -550,7 +551,7 @@ void launch_step_asm(const Layout &L, const double *u, const double *um, double 
     dim3 grd((unsigned)(gx * fold), (unsigned)((gy + fold - 1) / fold),
              (unsigned)(nchunks * R.slots));
     auto go = [&](auto early, auto late) {
-        launch_step_kernel(early, late, kFull64, grd, dim3(32, kAsmTY), R, s, overlap, u, um, out,
+        launch_step_kernel(early, late, kFull, grd, dim3(32, kAsmTY), R, s, overlap, u, um, out,
                            coefP, dco, fre, fim, L, c0, a, b, slot, flags, R, zc, nchunks);
     };
     if (fold > 1) go(step3d_asm_kernel<true, true>, step3d_asm_kernel<true, false>);
@@ -795,7 +796,7 @@ void launch_abd_step(const Layout &L, const T *u, const T *um, T *out, const T *
         else with_cell(std::false_type{});
     } else {
         auto go = [&](auto early, auto late) {
-            launch_step_kernel(early, late, sizeof(T) == 8 ? kFull64 : kFull32, grd, blk, R, s,
+            launch_step_kernel(early, late, sizeof(T) == 8 ? kFull64 : kFull, grd, blk, R, s,
                                overlap, u, um, out, kap, damp, fre, fim, L, C, a, b, cth, slot,
                                flags, R, nz);
         };
