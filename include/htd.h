@@ -257,10 +257,11 @@ typedef struct {
                                 windows of a larger grid; 0 in htd_plan, which does not
                                 look at the device) */
     int tile[3];             /* owned tile (x, y) of the blocked or resident-grid
-                                2-D step kernel and its columns per thread (1, or
-                                2: node pairs in paired FP32 instructions), or
-                                column tile and z chunk of the streamed 3-D one; 0
-                                if unused */
+                                2-D step kernel and the nodes that a thread updates
+                                together (1, or 2: pairs in paired FP32
+                                instructions, of one row in the blocked kernel, of
+                                one column in the resident one), or column tile and
+                                z chunk of the streamed 3-D one; 0 if unused */
     int ctas_per_sm;         /* resident CTAs per SM of that kernel */
     int waves;               /* waves of CTAs per launch of that kernel */
     int step_kernel;         /* recurrence kernel in use: 0 one step per launch
@@ -423,9 +424,10 @@ htd_status htd_grad(htd_handle h, int nsrc, const void *F_dev, int nrec,
  *               segment is recomputed once on the way back; 0 chooses
  *               ceil(sqrt(2 T n_P)).  Device memory 2 ceil(T n_P / C) + 2 C + 8
  *               state planes and the two gradients in FP64 for each of the
- *               sources that run together (as many as fit 1 GiB, at least one);
- *               where that does not fit the device, 2 ceil(T n_P / C) + C + 6
- *               planes (the handle keeps the largest workspace asked).
+ *               sources that run together (as many as keep that within 1 GiB and
+ *               five state planes each within 24 MiB, at least one); where that
+ *               does not fit the device, 2 ceil(T n_P / C) + C + 6 planes (the
+ *               handle keeps the largest workspace asked, htd_grad_td_describe).
  * The states and multipliers are in the handle's recurrence precision (FP32 in
  * mixed mode), the gradient sums in FP64.  Synchronises the stream.  Errors:
  * HTD_ERR_ARG (bad sizes or indices, mode PROJECT), HTD_ERR_OOM, HTD_ERR_CUDA,

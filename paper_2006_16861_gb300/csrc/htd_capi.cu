@@ -1046,9 +1046,9 @@ htd_status autotune_s3_zchunk(htd_ctx *c, const htd::RhsSet &R = htd::RhsSet{})
 
 // Misfit of the preconditioner's own output and its gradient through the
 // recurrence (htd_grad_td).  Per source U = P F by the handle's fast path for the
-// misfit (2-D Table 1 runs take it from the forward pass); then, for a group of sources at once (a one-step launch of one source
-// leaves most of the GPU idle at the sizes of an inversion), per real run a forward
-// pass of one-step launches that keeps (u_j, u_{j-1}) every C steps, and a backward
+// misfit (2-D Table 1 runs take it from the forward pass); then, for a group of sources
+// at once (a one-step launch of one source leaves most of the GPU idle at the sizes of
+// an inversion), per real run a forward pass of one-step launches that keeps (u_j, u_{j-1}) every C steps, and a backward
 // sweep over the segments from the last: recompute the segment's states from its
 // checkpoint, run the adjoint recurrence (the same step kernel on the multipliers,
 // forcing -dJ/du_k at the read-out steps) keeping the segment's multipliers, and add
@@ -1058,12 +1058,15 @@ htd_status autotune_s3_zchunk(htd_ctx *c, const htd::RhsSet &R = htd::RhsSet{})
 // Where not even one source's fits, one source at a time with two multiplier
 // planes, a gradient launch per step into gm and gR, and the handle's forcing
 // planes: 2 ceil(N/C) + C + 6 planes.
-// Measured on GB300, 512^2 mixed, 768 steps, 4 sources: 17.2 ms; one source at a time,
+// Measured on GB300, 512^2 mixed, 768 steps, 4 sources: 15.7 ms; one source at a time,
 // launch by launch, 86.8.
 constexpr size_t kTdGroupBytes = (size_t)1 << 30;   // a group's workspace, at most (or one source's)
-// planes that a group's steps read and write, at most: 512^2 (5.7 MB per source) took
-// 9.0, 6.4 and 7.1 ms per source in groups of 2, 4 and 7 -- beyond, a step's operands
-// no longer stay in L2 beside the states it leaves behind
+// Planes that a group's steps read and write (five per source), at most.  Mixed, ms per
+// call at 12 / 24 / 48 / 96 MiB (groups of as many sources): 8 sources 300^2 11.3 / 7.9 / 7.9 /
+// 7.9 (5, 8, 8, 8), 512^2 40.6 / 31.9 / 32.0 / 32.0 (2, 4, 6, 6), 800^2 131.8 / 131.9 / 113.0 /
+// 112.9 (1, 1, 2, 2); 4 sources 64^3 16.8 / 10.8 / 7.7 / 7.6 (1, 2, 4, 4); FP64 300^2 52.6 /
+// 48.7 / 45.1 / 45.1.  So half of it is too little and twice as much no worse on any of
+// these, for up to twice the workspace; kTdGroupBytes ends the groups from there on.
 constexpr size_t kTdHotBytes = (size_t)24 << 20;
 
 // Replays a pass of htd_grad_td from graph `*ex`, capturing it first if need be; run

@@ -107,7 +107,7 @@ struct Asm9 {
 };
 
 // u_{j+1} at a node in FP64: one multiply-add per neighbour, the small corner terms
-// first, and the own-node terms beside them (16 operations).  Summed apart, the
+// first, and the own-node terms beside them (15 operations).  Summed apart, the
 // neighbours' rounding stays at their size: the misfit of a 512^2 run came out with a
 // rounding noise of 3.3e-15 of its value against 5.9e-15 in one chain and 4.6e-15
 // with the cell form.  The one-step and the resident-grid kernel share it, so their

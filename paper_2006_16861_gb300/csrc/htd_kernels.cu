@@ -392,8 +392,8 @@ void launch_step(const Layout &L, const float *u, const float *um, float *out, c
 // A thread marches up a column of zc planes with the 3 x 3 x 3 window of u in
 // registers; zc is chosen by the launcher so that every SM gets about eight
 // blocks (the last wave of an FP64-bound kernel costs as much as it holds).
-// Measured on GB300, 96^3: 59 us per step (cell form: 179 us), 76 % of the
-// FP64 pipe's 45 us.
+// Measured on GB300, 96^3: 57.4 us per step (cell form: 179 us); the FP64 pipe alone
+// would take 46.4 us, 0.81 of it (0.90 at 256^3).
 constexpr int kAsmTY = 4;
 
 // (kFold: tile rows beyond grid.y's 65535 blocks follow along grid.x; a form of its own,
@@ -486,8 +486,8 @@ step3d_asm_kernel(const double *__restrict__ u, const double *um, double *out,
     }
 }
 
-// the 2-D form: one node per thread, 16 FP64 operations (the cell form: 33);
-// 801^2: 18.9 us per step (cell form: 43 us), 14.3 us at the FP64 pipe's rate
+// the 2-D form: one node per thread, 15 FP64 operations (the cell form: 33);
+// 801^2: 19.0 us per step (cell form: 41 us), 15.3 us at the FP64 pipe's rate
 template <bool kEarly>
 __global__ void __launch_bounds__(256)
 step2d_asm_kernel(const double *__restrict__ u, const double *um, double *out,

@@ -27,8 +27,8 @@
 // slower at every size (257 x 193: 0.87 us per step against 0.75).
 //
 // What bounds it: on small grids the exchange (257 x 193: 0.45 us per step
-// without its wait, 0.72 with it), on large ones shared memory (69 % of its
-// wavefronts at 1001^2), FP32 (47 %) and issue (46 %) together.  Measured on
+// without its wait, 0.72 with it), on large ones shared memory (63 % of its
+// wavefronts at 1001^2), FP32 (47 %) and issue (49 %) together.  Measured on
 // GB300, us per step, against one exchange per step with every operand in
 // shared memory: 0.72 / 1.6 at 257 x 193, 1.90 / 2.34 at 1001^2.  Holding the
 // forcing and the cells in registers as well (256 threads) spilled from 8 rows up
