@@ -258,8 +258,8 @@ void free_ctx(htd_ctx *c)
     delete c;
 }
 
-// Consecutive step launches overlap (programmatic dependent launch) unless the handle's options say
-// HTD_LAUNCH_NO_OVERLAP.
+// Consecutive step launches may overlap (programmatic dependent launch; the one-step
+// kernels where it pays) unless the handle's options say HTD_LAUNCH_NO_OVERLAP.
 bool step_overlap(const htd_ctx *c)
 {
     return !(c->opt.launch & HTD_LAUNCH_NO_OVERLAP);

@@ -234,8 +234,8 @@ void launch_ex(void (*kern)(KArgs...), dim3 grd, dim3 threads, size_t smem, cuda
 
 // One FP32 step u_{j+1} -> out from u = u_j and um = u_{j-1} (out may be um); force
 // false: no forcing (a = b = 0).  overlap (here and below): the launch may start
-// while the kernel before it drains; the one-step kernels wait for it before they
-// read or write a state.
+// while the kernel before it drains, if the launcher finds that this pays; the
+// one-step kernels wait for it before they read or write a state.
 void launch_step(const Layout &L, const float *u, const float *um, float *out, const float *kap,
                  const float *dco, const float *fre, const float *fim, const StepCoef<float> &C,
                  float a, float b, const OutSlot *slot, int flags, cudaStream_t s,
