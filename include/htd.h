@@ -425,9 +425,11 @@ htd_status htd_grad(htd_handle h, int nsrc, const void *F_dev, int nrec,
  *               ceil(sqrt(2 T n_P)).  Device memory 2 ceil(T n_P / C) + 2 C + 8
  *               state planes and the two gradients in FP64 for each of the
  *               sources that run together (as many as keep that within 1 GiB and
- *               five state planes each within 24 MiB, at least one); where that
- *               does not fit the device, 2 ceil(T n_P / C) + C + 6 planes (the
- *               handle keeps the largest workspace asked, htd_grad_td_describe).
+ *               five state planes each within 24 MiB, at least one; a source
+ *               that needs more than 1 GiB takes min(C, 8) in place of one C);
+ *               where that does not fit the device, 2 ceil(T n_P / C) + C + 6
+ *               planes (the handle keeps the largest workspace asked,
+ *               htd_grad_td_describe).
  * The states and multipliers are in the handle's recurrence precision (FP32 in
  * mixed mode), the gradient sums in FP64.  Synchronises the stream.  Errors:
  * HTD_ERR_ARG (bad sizes or indices, mode PROJECT), HTD_ERR_OOM, HTD_ERR_CUDA,

@@ -1055,6 +1055,8 @@ htd_status autotune_s3_zchunk(htd_ctx *c, const htd::RhsSet &R = htd::RhsSet{})
 // the segment's gradient terms in one launch.  The sums are kept per source and
 // added in order, so the gradient depends neither on C nor on the group.
 // Workspace of a group: per source 2 ceil(N/C) + 2 (C + 2) + 4 planes and the sums.
+// A source alone that would need more than kTdGroupBytes keeps kTdFewLam multipliers and
+// adds its gradient terms that many at a time, with the same bits.
 // Where not even one source's fits, one source at a time with two multiplier
 // planes, a gradient launch per step into gm and gR, and the handle's forcing
 // planes: 2 ceil(N/C) + C + 6 planes.
@@ -1068,6 +1070,10 @@ constexpr size_t kTdGroupBytes = (size_t)1 << 30;   // a group's workspace, at m
 // 48.7 / 45.1 / 45.1.  So half of it is too little and twice as much no worse on any of
 // these, for up to twice the workspace; kTdGroupBytes ends the groups from there on.
 constexpr size_t kTdHotBytes = (size_t)24 << 20;
+
+// 200^3 mixed, 128 steps, one source: 2.40 GB and 39.8 ms (a segment's 16 at a time 2.73
+// and 39.2, 4 at a time 2.23 and 41.7; a launch per step 49.5)
+constexpr long long kTdFewLam = 8;
 
 // Replays a pass of htd_grad_td from graph `*ex`, capturing it first if need be; run
 // directly where that fails or the handle's options ask for no graphs.
@@ -1123,6 +1129,10 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
         return (plane * npl + sizeof(double) * (size_t)nsum + sizeof(double2) * (size_t)N +
                 sizeof(OutSlot)) * k + act_bytes;
     };
+    if (bytes(1) > kTdGroupBytes && C > kTdFewLam) {
+        npl -= (size_t)(C - kTdFewLam);
+        nlam = (int)kTdFewLam + 2;
+    }
     while (g < std::min(nsrc, htd::kMaxRhs) && bytes(g + 1) <= kTdGroupBytes &&
            5 * plane * (g + 1) <= kTdHotBytes)
         ++g;
@@ -1260,6 +1270,7 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
                 for (long long j = s0 - 1; j < s1; ++j)
                     one_step<T>(c, seg_of(j, s0), seg_of(j - 1, s0), seg_of(j + 1, s0), fre, fim, Cf,
                                 (T)c->atab[j], (T)c->btab[j], slots, 0, t, set);
+                long long first = s1;                  // first of the terms not yet added
                 for (long long k = s1; k >= s0; --k) {
                     // forcing -dJ/du_k: Table 1 reads Re U at N and Im U at jim; EXACT
                     // reads Re U (run 0) or Im U (run 1) at N
@@ -1275,10 +1286,12 @@ htd_status grad_td_impl(htd_ctx *c, int nsrc, const double2 *F, int nrec, const 
                     if (lean)
                         htd::launch_grad_td<T>(L, c->M, cm, cR, lam, nlam, seg, sstride, 1, s0, k, k,
                                                gms, gRs, 0, t);
+                    else if (k == s0 || first - k + 1 == nlam - 2) {
+                        htd::launch_grad_td<T>(L, c->M, cm, cR, lam, nlam, seg, sstride, n, s0, first,
+                                               k, gms, gRs, nsum, t);
+                        first = k - 1;
+                    }
                 }
-                if (!lean)
-                    htd::launch_grad_td<T>(L, c->M, cm, cR, lam, nlam, seg, sstride, n, s0, s1, s0,
-                                           gms, gRs, nsum, t);
             }
             HTD_CUDA(cudaGetLastError());
             return HTD_OK;
