@@ -722,9 +722,8 @@ template <typename T>
 htd_status upload_recurrence(htd_ctx *c, const std::vector<double> &qkap, const std::vector<double> &dcoef)
 {
     const Layout &L = c->Lr;
-    std::vector<T> a(L.total);
     auto upload = [&](void *to, const std::vector<double> &from) {
-        for (size_t i = 0; i < (size_t)L.total; ++i) a[i] = (T)from[i];
+        const std::vector<T> a(from.begin(), from.end());
         return cudaMemcpy(to, a.data(), sizeof(T) * L.total, cudaMemcpyHostToDevice);
     };
     if (c->kap) HTD_CUDA(upload(c->kap, qkap));
